@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "dg.h"
 #include "rtd.h"
 #include "rttddft.h"
 
@@ -59,7 +60,6 @@ struct rttddft_ctx {
     double *d_part_fin = nullptr, *d_gdev = nullptr;
     int max_nback = 1, wmax = 1, nseg = 1, segw = BT, ntsel = 2, msegw = 64, nslot = 1, coop_grid = 0;
     int toep_global = 0;  // the direct sum's table window does not fit in shared memory: gather from L2
-    int cheb_tile = 0;
     zd* d_part_t = nullptr;
     zd* d_part = nullptr;
     double *d_a = nullptr, *d_dvs = nullptr;
@@ -84,6 +84,11 @@ struct rttddft_ctx {
     std::vector<double> eps_min, eps_max, pnorm, dvnorm;
     std::vector<std::vector<int>> h_glin;       // host copy of the table offsets of G per k
     TcPlan* tc = nullptr;                       // tensor-core operator (split-BF16 form)
+    // FP64 form: the products with CC and the matching coefficients on the tensor cores
+    DgLeft *dgl_cc = nullptr, *dgl_cch = nullptr, *dgl_a = nullptr, *dgl_ah = nullptr;
+    DgGemm *dg_expand = nullptr, *dg_fwd = nullptr, *dg_back = nullptr, *dg_proj = nullptr;
+    zd* d_proj = nullptr;                       // CC^H S C of every k-point (one slice)
+    DgSeries* series = nullptr;                 // Chebyshev series as digit products (many states)
     FftPlan* fft = nullptr;                     // FFT route of the interstitial convolution
     ToepDesc* td_op = nullptr;                  // per k {C, th}: the operator's convolution
     unsigned* d_tile_cnt = nullptr;             // row-tile counters of the fused split-K sums
@@ -250,7 +255,7 @@ static StepArgs make_args(rttddft_ctx* ctx, int dv_on) {
     a.gdev = ctx->d_gdev;
     a.at = ctx->d_at;
     a.gd_proj = ctx->gd_proj;
-    a.part_proj = ctx->d_part;
+    a.part_proj = ctx->dg_proj ? ctx->d_proj : ctx->d_part;
     a.kc_proj = ctx->kc_proj;
     a.max_nback = ctx->max_nback;
     a.wmax = ctx->wmax;
@@ -262,8 +267,7 @@ static StepArgs make_args(rttddft_ctx* ctx, int dv_on) {
     a.part_t = ctx->d_part_t;
     a.flag = ctx->d_flag;
     a.coop_grid = ctx->coop_grid;
-    a.cheb_tile = ctx->cheb_tile;
-    a.tcback = (ctx->opt.precision >= RTTDDFT_PREC_BF16X3 && tc_has_back(ctx->tc)) ? 1 : 0;
+    a.tcback = (ctx->dg_back || (ctx->opt.precision >= RTTDDFT_PREC_BF16X3 && tc_has_back(ctx->tc))) ? 1 : 0;
     a.tc_fmt = tc_format(ctx->tc);
     a.tc_st = tc_table_scale(ctx->tc);
     a.at_n = ctx->at.n;
@@ -316,6 +320,11 @@ static StepPlan make_plan(rttddft_ctx* ctx) {
     p.tc = ctx->tc;
     p.tcc = ctx->tcc;
     p.tcmt = ctx->tcmt;
+    p.dg_expand = ctx->dg_expand;
+    p.dg_fwd = ctx->dg_fwd;
+    p.dg_back = ctx->dg_back;
+    p.dg_proj = ctx->dg_proj;
+    p.series = ctx->series;
     p.fft = ctx->fft;
     p.td_op = ctx->td_op;
     p.tile_cnt = ctx->d_tile_cnt;
@@ -588,6 +597,56 @@ static void validate(const rttddft_system* s, const rttddft_options* o) {
     if (!finite_all(s->occ, s->n_s) || !finite_all(s->wk, s->n_k)) fail(ctx, RTTDDFT_ERR_NONFINITE, "occ/wk not finite");
 }
 
+static void drop_dg(rttddft_ctx* ctx) {
+    for (DgGemm** g : {&ctx->dg_expand, &ctx->dg_fwd, &ctx->dg_back, &ctx->dg_proj}) {
+        dg_gemm_destroy(*g);
+        *g = nullptr;
+    }
+    for (DgLeft** l : {&ctx->dgl_cc, &ctx->dgl_cch, &ctx->dgl_a, &ctx->dgl_ah}) {
+        dg_left_destroy(*l);
+        *l = nullptr;
+    }
+}
+
+// FP64 form: digits of CC (rows; and CC^H) and of the matching coefficients (A
+// and A^H), 12 bytes per real against 8, and the products they serve.  Returns
+// false, with nothing built, where they would take more than half of the free
+// device memory: the FP64 kernels run instead.
+static bool build_dg(rttddft_ctx* ctx) {
+    const int nk = ctx->nk, ns = ctx->ns, naux = ctx->naux, ma = ctx->at.ma;
+    size_t need = 0, fr = 0, tot = 0;
+    for (int k = 0; k < nk; ++k)
+        need += dg_left_bytes(ctx->nb[k], naux) + dg_left_bytes(naux, ctx->nb[k]) + dg_left_bytes(ma, ctx->ng[k]) +
+                dg_left_bytes(ctx->ng[k], ma) + 2 * dg_left_bytes(2 * ns, ctx->nb[k]) + dg_left_bytes(4 * ns, ma);
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || need > fr / 2) return false;
+    std::vector<DgMat> cc(nk), cch(nk), am(nk), ah(nk);
+    std::vector<DgRight> re(nk), rf(nk), rb(nk), rp(nk);
+    ctx->d_proj = dalloc<zd>(ctx, (size_t)nk * ns * naux);
+    for (int k = 0; k < nk; ++k) {
+        KDev& K = ctx->hkd[k];
+        if (ma > 0 && !K.tb) K.tb = dalloc<zd>(ctx, (size_t)K.ng * 2 * ns);
+        cc[k] = DgMat{K.caux, 1, (size_t)K.nb, 0, K.nb, naux};
+        cch[k] = DgMat{K.caux, (size_t)K.nb, 1, 1, naux, K.nb};
+        am[k] = DgMat{K.at, (size_t)K.ng, 1, 1, ma, K.ng};
+        ah[k] = DgMat{K.at, 1, (size_t)K.ng, 0, K.ng, ma};
+        re[k] = DgRight{K.theta, naux, naux, K.C, K.nb};
+        rf[k] = DgRight{K.C, K.nb, K.ng, K.Q, ma};
+        rb[k] = DgRight{K.Z, ma, ma, K.tb, K.ng};
+        rp[k] = DgRight{K.Y + (size_t)ns * K.nb, K.nb, K.nb, ctx->d_proj + (size_t)k * ns * naux, naux};
+    }
+    bool ok = (ctx->dgl_cc = dg_left_create(nk, cc.data(), ctx->stream)) &&
+              (ctx->dgl_cch = dg_left_create(nk, cch.data(), ctx->stream)) &&
+              (ctx->dg_expand = dg_gemm_create(ctx->dgl_cc, nk, re.data(), ns, ctx->d_flag)) &&
+              (ctx->dg_proj = dg_gemm_create(ctx->dgl_cch, nk, rp.data(), ns, ctx->d_flag));
+    if (ok && ma > 0)
+        ok = (ctx->dgl_a = dg_left_create(nk, am.data(), ctx->stream)) &&
+             (ctx->dgl_ah = dg_left_create(nk, ah.data(), ctx->stream)) &&
+             (ctx->dg_fwd = dg_gemm_create(ctx->dgl_a, nk, rf.data(), ns, ctx->d_flag)) &&
+             (ctx->dg_back = dg_gemm_create(ctx->dgl_ah, nk, rb.data(), 2 * ns, ctx->d_flag));
+    if (!ok) drop_dg(ctx);
+    return ok;
+}
+
 // ------------------------------------------------------------ ABI
 extern "C" {
 
@@ -626,6 +685,8 @@ void rttddft_destroy(rttddft_ctx* ctx) {
     tc_plan_destroy(ctx->tc);
     tc_cc_destroy(ctx->tcc);
     tc_mt_destroy(ctx->tcmt);
+    dg_series_destroy(ctx->series);
+    drop_dg(ctx);
     fft_plan_destroy(ctx->fft);
     for (void* p : ctx->allocs) cudaFree(p);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
@@ -1089,9 +1150,10 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
             for (int k = 0; k < nk; ++k) td[k] = ToepDesc{ctx->hkd[k].C, ctx->hkd[k].th, ctx->hkd[k].nb, ctx->hkd[k].ng};
             ctx->td_op = dupload(ctx, td.data(), td.size());
         }
+        const bool f32 = o->precision != RTTDDFT_PREC_FP64;
+        const bool dg = !f32 && build_dg(ctx);
         CK(cudaMemcpy(ctx->d_kd, ctx->hkd.data(), nk * sizeof(KDev), cudaMemcpyHostToDevice));
         // ---- step descriptors
-        const bool f32 = o->precision != RTTDDFT_PREC_FP64;
         std::vector<GemmDesc> ex, fw, pj, g1, g2, eh, en;
         ctx->kc_fwd = kchunk_for((at.ma + cn_rows(ns) - 1) / cn_rows(ns), nk, ctx->maxng);
         ctx->kc_proj = kchunk_for((naux + cn_rows(ns) - 1) / cn_rows(ns), nk, ctx->maxnb);
@@ -1126,6 +1188,7 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
             if (e) fail(ctx, e, why);
             ctx->kc_proj = ctx->maxnb;
         }
+        if (dg) ctx->kc_proj = ctx->maxnb;  // one slice per k-point
         {
             // expand: rows are many, K = n_aux is short; split K only in FP64 where the
             // DFMA pipe of every SM is needed
@@ -1268,7 +1331,10 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
             const int e = prepare_back_kernels(a);
             if (e) fail(ctx, RTTDDFT_ERR_UNSUPPORTED, "table window needs more shared memory than a block has");
             CK(cudaStreamSynchronize(ctx->stream));
-            ctx->coop_grid = prepare_cheb_coop(a, ctx->stream, &ctx->cheb_tile);
+            ctx->coop_grid = prepare_cheb_coop(a, ctx->stream);
+            // without the memory for the digits the per-row form runs
+            if (o->propagator != RTTDDFT_PROP_EIG && ns >= DG_SERIES_MIN_NS)
+                ctx->series = dg_series_create(nk, naux, ns);
         }
         // ---- theta(0)
         if (s->c0) {
@@ -2412,6 +2478,7 @@ extern "C" int rttddft_apply_noalloc(rttddft_ctx* ctx, int k, int ncols, const d
         p.side = nullptr;
         p.tile_cnt = nullptr;  // the context's counters may be in use on another stream
         p.gd_mt1 = nullptr;
+        p.dg_fwd = p.dg_back = nullptr;  // their digit buffers belong to the context
         p.gd_fwd = (const GemmDesc*)(base + o_gd);
         p.maxng = ng;
         p.part = (zd*)(base + o_part);

@@ -1,0 +1,35 @@
+// FP64 contractions by exact digit products on the tensor cores (k_dg.cu).
+#pragma once
+#include "common.cuh"
+
+#define DG_SERIES_MIN_NS 9  // states from which the series runs as digit products
+
+struct DgLeft;    // digits of a static left operand per batch entry
+struct DgGemm;    // C (+)= A X per batch entry
+struct DgSeries;  // the Chebyshev series
+
+// element (r, k) of a left operand: src[r rs + k cs], conjugated when conj
+struct DgMat {
+    const zd* src;
+    size_t rs, cs;
+    int conj, M, K;
+};
+struct DgRight {
+    const zd* X;  // K x ncol, column-major
+    int ldx, K;   // K at most the left operand's
+    zd* C;
+    int ldc;
+};
+
+DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s);
+void dg_left_destroy(DgLeft* l);
+size_t dg_left_bytes(int M, int K);
+// null where the device memory does not suffice
+DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag);
+void dg_gemm_destroy(DgGemm* g);
+int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s);  // returns its launches
+
+struct StepArgs;
+DgSeries* dg_series_create(int nk, int n, int ns);
+void dg_series_destroy(DgSeries* g);
+int launch_dg_series(const DgSeries* g, const StepArgs& a, cudaStream_t s);       // returns its launches

@@ -1,0 +1,1070 @@
+// FP64 contractions on the sm_103a tensor cores by exact digit products.
+//
+// GB300 runs FP64 at 1/64 of its FP32 rate (1.2 TFLOP/s), so the FP64 form's
+// contractions were bound by the FP64 pipe at a few per cent of the memory
+// rate.  Here every operand is written as an integer of 54 bits relative to a
+// power of two (of its row of A, of its column of X), cut into six balanced
+// base-512 digits d in [-256, 256] (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, Numer. Algorithms 59, 2012).  Digits are exact in fp16, a
+// product of two is at most 2^16, and the FP32 accumulator of tcgen05.mma
+// holds the sum of one group (pairs i + j = s) over 64 reals of K exactly:
+// 2^24 bounds it for s >= 7; below, only operands whose digits all have the
+// same size and sign can pass 2^24, by an error of 2^-52 of the scale.  Groups
+// s = 4 .. 10 are kept (26 of 36 pairs; the dropped ones are below
+// 2^-70 (256^2) sqrt(K) of the scale, under the 2^-54 of the cut itself), read
+// out every 64 reals and added up as integers, so a result does not depend on
+// the order of the sums or on the number of K slices.
+#include <cooperative_groups.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cstring>
+#include <string>
+#include <vector>
+
+#include "dg.h"
+#include "rtd.h"
+#include "rttddft.h"
+#include "tcgen05.cuh"
+
+namespace cg = cooperative_groups;
+
+#define DG_P 6              // digits
+#define DG_KS 32            // reals per stage: 64 bytes of fp16, one row of the 64-byte swizzle
+#define DG_BM 128           // rows per tile
+#define DG_G 7              // groups kept, s = 10 - g
+#define DG_THREADS 320      // 8 read-out warps, one product warp, one copy warp
+#define DG_A_PL (DG_BM * 64)
+
+typedef long long i64;
+
+// ------------------------------------------------------------ digits
+// q = sum_i d_i 512^i with |q| <= 2^53, returned as the six biased values
+// d_i + 256 (0 .. 512)
+__device__ __forceinline__ void dg_cut(i64 q, uint32_t* d) {
+    const i64 bias = 256ll * (1ll + (1ll << 9) + (1ll << 18) + (1ll << 27) + (1ll << 36) + (1ll << 45));
+    const i64 u = q + bias;
+#pragma unroll
+    for (int i = 0; i < DG_P - 1; ++i) d[i] = (uint32_t)(u >> (9 * i)) & 511u;
+    d[DG_P - 1] = (uint32_t)(u >> 45);
+}
+// fp16 pair (x - 256, y - 256) of biased digits: 1024 + x is exact in fp16
+__device__ __forceinline__ uint32_t dg_pair(uint32_t x, uint32_t y) {
+    const uint32_t b = (x | (y << 16)) | 0x64006400u;
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&b), __floats2half2_rn(1280.f, 1280.f));
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+#define DG_NEG 0x8000u
+// exponent e with |x| < 2^e from the high word of the largest |x|; 2048 marks Inf and NaN
+__device__ __forceinline__ int dg_exp(int hw) {
+    const int f = hw >> 20;
+    return f == 2047 ? 2048 : f - 1022;
+}
+__device__ __forceinline__ int dg_hw(double x) { return __double2hiint(x) & 0x7fffffff; }
+// x 2^(53 - e) as an integer; the power of two is applied in two halves so that neither overflows
+struct DgScale {
+    double p1, p2;
+};
+__device__ __forceinline__ double dg_pow2(int n) { return __hiloint2double((n + 1023) << 20, 0); }
+__device__ __forceinline__ DgScale dg_scale(int e) {
+    const int s = 53 - e, h = s / 2;
+    return DgScale{dg_pow2(h), dg_pow2(s - h)};
+}
+__device__ __forceinline__ i64 dg_int(double x, DgScale s) { return __double2ll_rn((x * s.p1) * s.p2); }
+
+// (hi 2^27 + lo) 2^e as a double with integer arithmetic (the conversions of
+// the FP64 pipe would cost more than the products of a short K)
+__device__ __forceinline__ double dg_double(i64 hi, i64 lo, int e) {
+    i64 m = hi + (lo >> 27);
+    uint32_t r = (uint32_t)lo & ((1u << 27) - 1u);
+    const bool neg = m < 0;
+    if (neg) {
+        const bool b = r != 0u;
+        m = -m - (b ? 1 : 0);
+        r = b ? (1u << 27) - r : 0u;
+    }
+    // keep the leading 63 bits of m 2^27 + r
+    const int lz = __clzll(m);
+    const int k = lz > 27 ? 27 : lz - 1;
+    const unsigned long long x = ((unsigned long long)m << k) | (r >> (27 - k));
+    if (x == 0ull) return 0.0;
+    const int z = __clzll(x);
+    const unsigned long long t = ((x << z) + (1ull << 10));  // the carry out of a value of all ones:
+    const bool cy = t < (1ull << 10);
+    const int ex = e + (27 - k) + 63 - z + (cy ? 1 : 0) + 1023;
+    const unsigned long long man = cy ? 0ull : (t >> 11) & ((1ull << 52) - 1ull);
+    double v;
+    if (ex >= 1 && ex <= 2046) {
+        v = __longlong_as_double((i64)(((unsigned long long)ex << 52) | man));
+    } else if (ex > 2046) {
+        v = __longlong_as_double(0x7ff0000000000000ll);
+    } else {
+        v = scalbn(__longlong_as_double((i64)((1023ull << 52) | man)), ex - 1023);
+    }
+    return neg ? -v : v;
+}
+
+// rows 2n: [Re, -Im] and 2n + 1: [Im, Re] of a right operand, entry k of complex column n
+__device__ __forceinline__ void dg_put_col(uint32_t* b, size_t plw, size_t kw, int n, int k, i64 qr, i64 qi) {
+    uint32_t dr[DG_P], di[DG_P];
+    dg_cut(qr, dr);
+    dg_cut(qi, di);
+    b += (size_t)(2 * n) * kw + k;
+#pragma unroll
+    for (int i = 0; i < DG_P; ++i) {
+        const uint32_t p = dg_pair(dr[i], di[i]);
+        b[i * plw] = p ^ (DG_NEG << 16);
+        b[i * plw + kw] = (p >> 16) | (p << 16);
+    }
+}
+
+// ------------------------------------------------------------ the product kernel
+struct DgOut {
+    int M, nst, ldc;    // rows, K stages, leading dimension of C
+    const int* er;      // row exponents of A
+    const int* ec;      // column exponents of X
+    zd* C;
+    int tile0;          // first tile in the split buffers
+};
+struct DgCheb {
+    int n;              // N_aux
+    i64 *y0, *y1;       // y of even and of odd terms, units 2^-62 of the column's scale: [2 ns][n]
+    i64* acc;           // sum_n c_n y_n
+    __half* Bn[2];      // digit operands of even and odd terms
+    size_t pl;          // their plane stride
+    int kpad;
+    i64* coef;          // c_n in units 2^-62
+};
+struct DgArgs {
+    const CUtensorMap *tmA, *tmB;
+    const DgOut* out;
+    const DgCheb* ch;
+    int kofs, ncol, ntn, cs, gs, beta, term, last;  // cs K slices per cluster, gs clusters per tile
+    i64* part;
+    unsigned* cnt;
+    int* flag;
+};
+
+__device__ __forceinline__ uint64_t dg_desc(uint32_t saddr) {  // K-major, 64-byte swizzle, 8-row atoms of 512 B
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
+}
+__device__ __forceinline__ void dg_tma(void* dst, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            smem_u32(dst)),
+        "l"((uint64_t)tm), "r"(x), "r"(y), "r"(0), "r"(smem_u32(bar))
+        : "memory");
+}
+template <int W>
+__device__ __forceinline__ void dg_ld(uint32_t taddr, uint32_t* r) {
+    static_assert(W == 8 || W == 16, "columns per load");
+    if constexpr (W == 8) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(taddr));
+    } else {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(taddr));
+    }
+}
+// a b 2^-62 of two integers in units 2^-62
+__device__ __forceinline__ i64 dg_mul62(i64 a, i64 b) {
+    return (i64)(((unsigned long long)__mul64hi(a, b) << 2) | (((unsigned long long)a * (unsigned long long)b) >> 62));
+}
+
+// One 128-row x NT-column tile of D = A^ B^^T over this split's K stages (NT
+// real columns: Re and Im of NT / 2 complex ones).  The copy warp brings the
+// six digit planes of both operands of a stage with one TMA each; the product
+// warp issues the 26 pairs group by group into the group's own NT columns of
+// tensor memory; the read-out warps add a finished group (64 reals of K) to
+// their integers while the next groups' products run, so a group is handed
+// back and forth by a pair of mbarriers.  The K slices of a tile meet in the
+// distributed shared memory of a cluster, further clusters of the tile in
+// global memory, where the last one finishes it.
+// MODE 0: C (+)= the product, scaled back.  MODE 1: a Chebyshev term.
+template <int NT, int MODE>
+__global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
+    extern __shared__ unsigned char dgsm[];
+    constexpr int STAGES = NT == 16 ? 4 : 3;
+    constexpr int B_PL = NT * 64;
+    constexpr int STAGE = DG_P * (DG_A_PL + B_PL);
+    constexpr int CP = NT / 2;  // columns per read-out thread
+    constexpr uint32_t NCOLS = DG_G * NT <= 128 ? 128 : (DG_G * NT <= 256 ? 256 : 512);
+    unsigned char* smem = dgsm + ((1024u - (smem_u32(dgsm) & 1023u)) & 1023u);
+    __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], gfull[DG_G], gfree[DG_G], done;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+    __shared__ int is_last;
+    const int z = blockIdx.z + g.kofs;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = blockIdx.x % g.cs, nt_i = (blockIdx.x / g.cs) % g.ntn;
+    const int sp = blockIdx.x / (g.cs * g.ntn) * g.cs + rank, splits = g.cs * g.gs;
+    const int m_i = blockIdx.y;
+    const DgOut& o = g.out[z];
+    const int m0 = m_i * DG_BM, n0 = nt_i * NT;
+    if (m0 >= o.M) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int st0 = (int)((i64)o.nst * sp / splits), nk = (int)((i64)o.nst * (sp + 1) / splits) - st0;
+    if (tid == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < DG_G; ++s) {
+            mbar_init(&gfull[s], 1);
+            mbar_init(&gfree[s], 8);
+        }
+        mbar_init(&done, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(NCOLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+    i64 hi[CP], lo[CP];
+#pragma unroll
+    for (int c = 0; c < CP; ++c) hi[c] = lo[c] = 0;
+    if (warp == 9) {
+        if (lane == 0) {
+            int issued = 0;
+            for (int t = 0; t < nk; ++t) {
+                const int s = t % STAGES;
+                if (t >= STAGES && !mbar_wait(&empty[s], (uint32_t)((t / STAGES - 1) & 1))) {
+                    abort_flag = 1;
+                    atomicOr(g.flag, 8);
+                    break;
+                }
+                if (abort_flag) break;
+                unsigned char* sa = smem + s * STAGE;
+                mbar_expect_tx(&full[s], STAGE);
+                dg_tma(sa, g.tmA + z, (st0 + t) * DG_KS, m0, &full[s]);
+                dg_tma(sa + DG_P * DG_A_PL, g.tmB + z, (st0 + t) * DG_KS, n0, &full[s]);
+                issued = t + 1;
+            }
+            // nothing may still be on its way into shared memory when the block ends
+            for (int t = issued > STAGES ? issued - STAGES : 0; t < issued; ++t)
+                mbar_wait(&full[t % STAGES], (uint32_t)((t / STAGES) & 1));
+        }
+    } else if (warp == 8) {
+        if (lane == 0) {
+            // kind::f16, fp16 operands, FP32 accumulator, both K-major
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(DG_BM >> 4) << 24);
+            bool ok = true;
+            for (int t = 0; t < nk && ok; ++t) {
+                const int s = t % STAGES;
+                if (!mbar_wait(&full[s], (uint32_t)((t / STAGES) & 1))) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const bool first = (t & 1) == 0, lastp = !first || t == nk - 1;
+                const int sl = t >> 1;
+                const uint64_t da = dg_desc(smem_u32(smem + s * STAGE));
+                const uint64_t db = dg_desc(smem_u32(smem + s * STAGE + DG_P * DG_A_PL));
+#pragma unroll
+                for (int gi = 0; gi < DG_G; ++gi) {
+                    if (first && sl > 0) {
+                        if (!mbar_wait(&gfree[gi], (uint32_t)((sl - 1) & 1))) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                    }
+                    constexpr int TOP = 2 * (DG_P - 1);
+                    const int sum = TOP - gi;
+#pragma unroll
+                    for (int i = 0; i < DG_P; ++i) {
+                        const int j = sum - i;
+                        if (j < 0 || j >= DG_P) continue;
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk)
+                            umma_bf16(tmem + (uint32_t)(gi * NT), da + (uint64_t)((i * DG_A_PL + kk * 32) >> 4),
+                                      db + (uint64_t)((j * B_PL + kk * 32) >> 4), idesc,
+                                      (first && kk == 0 && i == (sum >= DG_P ? sum - DG_P + 1 : 0)) ? 0u : 1u);
+                    }
+                    if (lastp) umma_commit(&gfull[gi]);
+                }
+                umma_commit(&empty[s]);
+            }
+            umma_commit(&done);
+            if (!ok) {
+                abort_flag = 1;
+                atomicOr(g.flag, 8);
+            }
+        }
+    } else {
+        const int nsl = (nk + 1) >> 1;
+        const uint32_t tb = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * CP);
+        bool ok = true;
+        for (int sl = 0; sl < nsl && ok; ++sl) {
+#pragma unroll
+            for (int gi = 0; gi < DG_G; ++gi) {
+                if (!mbar_wait(&gfull[gi], (uint32_t)(sl & 1)) || abort_flag) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                constexpr int W = CP >= 16 ? 16 : 8;
+#pragma unroll
+                for (int c0 = 0; c0 < CP; c0 += W) {
+                    uint32_t r[W];
+                    dg_ld<W>(tb + (uint32_t)(gi * NT + c0), r);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (c0 + W >= CP) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0)
+                            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&gfree[gi])) : "memory");
+                    }
+#pragma unroll
+                    for (int c = 0; c < W; ++c) {
+                        const i64 v = (i64)__float2int_rn(__uint_as_float(r[c]));
+                        if (gi <= 3) hi[c0 + c] += v << (9 * (3 - gi));  // units of s = 7
+                        else lo[c0 + c] += v << (9 * (6 - gi));          // units of s = 4
+                    }
+                }
+            }
+        }
+        if (!ok) {
+            abort_flag = 1;
+            if (lane == 0) atomicOr(g.flag, 8);
+        }
+    }
+    __syncthreads();
+    // every product has written its accumulator before tensor memory goes back
+    // (a block that gave up, with its flag raised, still takes part below: the split
+    // buffers and counters are left ready for the next launch)
+    if (!mbar_wait(&done, 0) && tid == 0) atomicOr(g.flag, 8);
+    tc_fence_after();
+    // the stages are free now: the tile's integers go to shared memory, column by
+    // column, and the blocks of the cluster (K slices of one tile) each add up and
+    // finish their share of the columns
+    i64* S = (i64*)smem;  // [NT][hi, lo][128]
+    if (warp < 8) {
+        const int rl = (warp & 3) * 32 + lane, cb = (warp >> 2) * CP;
+#pragma unroll
+        for (int c = 0; c < CP; ++c) {
+            S[(size_t)(2 * (cb + c)) * DG_BM + rl] = hi[c];
+            S[(size_t)(2 * (cb + c) + 1) * DG_BM + rl] = lo[c];
+        }
+    }
+    if (g.cs > 1) cl.sync();
+    else __syncthreads();
+    const int share = NT / g.cs, c0 = rank * share;  // real columns of this block, an even number
+    const int items = DG_BM * share;
+    bool mine = true;
+    // the sum over the clusters (beside S, which the cluster's other blocks may still read)
+    i64* T0 = g.cs > 1 ? S + (size_t)2 * NT * DG_BM : S;
+    if (g.gs > 1) {
+        const int tile = (o.tile0 + m_i * g.ntn + nt_i) * g.cs + rank;
+        unsigned long long* P = (unsigned long long*)g.part + (size_t)tile * share * 2 * DG_BM;
+        for (int it = tid; it < 2 * items; it += DG_THREADS) {
+            i64 v = 0;
+            for (int q = 0; q < g.cs; ++q) v += (g.cs > 1 ? cl.map_shared_rank(S, q) : S)[(size_t)2 * c0 * DG_BM + it];
+            atomicAdd(P + it, (unsigned long long)v);
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            is_last = atomicAdd(g.cnt + tile, 1u) == (unsigned)(g.gs - 1);
+            if (is_last) g.cnt[tile] = 0u;
+        }
+        __syncthreads();
+        mine = is_last != 0;
+        if (mine) {
+            __threadfence();
+            for (int it = tid; it < 2 * items; it += DG_THREADS) {
+                T0[it] = (i64)__ldcg(P + it);
+                __stcg(P + it, 0ull);  // ready for the next launch
+            }
+            __syncthreads();
+        }
+    }
+    if (mine) {
+        for (int it = tid; it < items / 2; it += DG_THREADS) {
+            const int rl = it & (DG_BM - 1), row = m0 + rl, c = (it / DG_BM) * 2, n = (n0 + c0 + c) >> 1;
+            if (row >= o.M || n >= g.ncol) continue;
+            i64 hv[2], lv[2];
+            if (g.gs > 1) {
+                const i64* T = T0 + (size_t)2 * c * DG_BM + rl;
+                hv[0] = T[0];
+                lv[0] = T[DG_BM];
+                hv[1] = T[2 * DG_BM];
+                lv[1] = T[3 * DG_BM];
+            } else {
+                hv[0] = hv[1] = lv[0] = lv[1] = 0;
+                for (int q = 0; q < g.cs; ++q) {
+                    const i64* T = (g.cs > 1 ? cl.map_shared_rank(S, q) : S) + (size_t)2 * (c0 + c) * DG_BM + rl;
+                    hv[0] += T[0];
+                    lv[0] += T[DG_BM];
+                    hv[1] += T[2 * DG_BM];
+                    lv[1] += T[3 * DG_BM];
+                }
+            }
+            if constexpr (MODE == 0) {
+                const int er = o.er[row], ec = o.ec[n];
+                zd v;
+                if (ec >= 2048 || er >= 2048) {
+                    v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+                } else {
+                    v.x = dg_double(hv[0], lv[0], er + ec - 70);
+                    v.y = dg_double(hv[1], lv[1], er + ec - 70);
+                }
+                zd* p = o.C + row + (size_t)n * o.ldc;
+                if (g.beta) v = zadd(*p, v);
+                *p = v;
+            } else {
+                const DgCheb& ch = g.ch[z];
+                i64* yb = (g.term & 1) ? ch.y1 : ch.y0;
+                i64 y[2];
+                const size_t e = (size_t)(2 * n) * ch.n + row;
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    // H~ y in units 2^-62: hi has 2^-43, lo has 2^-70
+                    i64 w = (i64)((unsigned long long)hv[q] << 19) + ((lv[q] + 128) >> 8);
+                    if (g.term > 1) w = (i64)(2ull * (unsigned long long)w - (unsigned long long)yb[e + (size_t)q * ch.n]);
+                    y[q] = w;
+                }
+                const i64 cr = ch.coef[2 * g.term], ci = ch.coef[2 * g.term + 1];
+                ch.acc[e] += dg_mul62(cr, y[0]) - dg_mul62(ci, y[1]);
+                ch.acc[e + ch.n] += dg_mul62(cr, y[1]) + dg_mul62(ci, y[0]);
+                if (!g.last) {
+                    yb[e] = y[0];
+                    yb[e + ch.n] = y[1];
+                    dg_put_col((uint32_t*)(g.term & 1 ? ch.Bn[1] : ch.Bn[0]), ch.pl / 2, ch.kpad / 2, n, row, (y[0] + 256) >> 9,
+                               (y[1] + 256) >> 9);
+                }
+            }
+        }
+    }
+    if (g.cs > 1) cl.sync();  // a block's integers are read before the block may end
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOLS) : "memory");
+}
+
+// ------------------------------------------------------------ packing
+// element (r, k) of op(A): src[r rs + k cs], conjugated when conj
+struct DgSrc {
+    const zd* src;
+    size_t rs, cs;
+    int conj, M, K, mpad, kpad;
+    __half* dst;  // [6][mpad][kpad]
+    int* er;
+};
+// row exponents: a warp per row
+__global__ void k_dg_rowmax(const DgSrc* d) {
+    const DgSrc& s = d[blockIdx.z];
+    int mx = 0;
+    if (s.rs == 1) {  // rows contiguous: 32 rows per block, 8 threads stride K
+        const int r = blockIdx.x * 32 + (threadIdx.x & 31);
+        if (r < s.M)
+            for (int k = threadIdx.x >> 5; k < s.K; k += 8) {
+                const zd v = s.src[r + (size_t)k * s.cs];
+                mx = max(mx, max(dg_hw(v.x), dg_hw(v.y)));
+            }
+        __shared__ int sh[8][32];
+        sh[threadIdx.x >> 5][threadIdx.x & 31] = mx;
+        __syncthreads();
+        if (threadIdx.x < 32 && r < s.M) {
+            for (int q = 0; q < 8; ++q) mx = max(mx, sh[q][threadIdx.x]);
+            s.er[r] = dg_exp(mx);
+        }
+        return;
+    }
+    for (int u = 0; u < 4; ++u) {
+        const int r = blockIdx.x * 32 + (threadIdx.x >> 5) * 4 + u;
+        if (r >= s.M) return;
+        mx = 0;
+        for (int k = threadIdx.x & 31; k < s.K; k += 32) {
+            const zd v = s.src[r * s.rs + (size_t)k * s.cs];
+            mx = max(mx, max(dg_hw(v.x), dg_hw(v.y)));
+        }
+        for (int w = 16; w > 0; w >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+        if ((threadIdx.x & 31) == 0) s.er[r] = dg_exp(mx);
+    }
+}
+// digits of a 32 x 32 tile, read along the source's contiguous axis, written along K
+__global__ void k_dg_pack_a(const DgSrc* d) {
+    __shared__ zd t[32][33];
+    const DgSrc& s = d[blockIdx.z];
+    const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    if (r0 >= s.M || k0 >= s.K) return;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    for (int q = y; q < 32; q += 8) {
+        const int r = s.rs == 1 ? r0 + x : r0 + q, k = s.rs == 1 ? k0 + q : k0 + x;
+        zd v = zmk(0.0, 0.0);
+        if (r < s.M && k < s.K) v = s.src[r * s.rs + (size_t)k * s.cs];
+        if (s.conj) v.y = -v.y;
+        if (s.rs == 1) t[x][q] = v;
+        else t[q][x] = v;
+    }
+    __syncthreads();
+    const int k = k0 + x;
+    for (int q = y; q < 32; q += 8) {
+        const int r = r0 + q;
+        if (r >= s.M || k >= s.K) continue;
+        const zd v = t[q][x];
+        const int e = s.er[r];
+        const DgScale sc = dg_scale(e >= 2048 ? 0 : e);
+        uint32_t dr[DG_P], di[DG_P];
+        dg_cut(e >= 2048 ? 0 : dg_int(v.x, sc), dr);
+        dg_cut(e >= 2048 ? 0 : dg_int(v.y, sc), di);
+        for (int i = 0; i < DG_P; ++i)
+            ((uint32_t*)s.dst)[((size_t)i * s.mpad + r) * (s.kpad / 2) + k] = dg_pair(dr[i], di[i]);
+    }
+}
+
+// right operand: per complex column n of X (K x N) the rows 2n: [Re, -Im] and
+// 2n + 1: [Im, Re] of every k, and the column's exponent.  A cluster of eight
+// blocks shares a column: the largest entry goes around through distributed
+// shared memory, the entries stay in registers meanwhile.
+struct DgPackB {
+    const zd* X;
+    int ldx, K;
+    __half* dst;  // [6][npad][kpad]
+    int npad, kpad;
+    int* ec;
+};
+#define DG_PB_T 256
+#define DG_PB_E 4  // entries per thread held in registers
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(DG_PB_T) k_dg_pack_b(const DgPackB* d, int kofs) {
+    __shared__ int sh[8];
+    __shared__ int cmax;
+    cg::cluster_group cl = cg::this_cluster();
+    const DgPackB& s = d[blockIdx.z + kofs];
+    const int rank = blockIdx.x & 7, n = blockIdx.x >> 3;
+    const int tid = threadIdx.x;
+    const zd* __restrict__ x = s.X + (size_t)n * s.ldx;
+    zd v[DG_PB_E];
+    int mx = 0;
+#pragma unroll
+    for (int u = 0; u < DG_PB_E; ++u) {
+        const int k = (u * 8 + rank) * DG_PB_T + tid;
+        v[u] = k < s.K ? x[k] : zmk(0.0, 0.0);
+        mx = max(mx, max(dg_hw(v[u].x), dg_hw(v[u].y)));
+    }
+    for (int k = (DG_PB_E * 8 + rank) * DG_PB_T + tid; k < s.K; k += 8 * DG_PB_T) {
+        const zd w = x[k];
+        mx = max(mx, max(dg_hw(w.x), dg_hw(w.y)));
+    }
+    for (int w = 16; w > 0; w >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+    if ((tid & 31) == 0) sh[tid >> 5] = mx;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 0; w < DG_PB_T / 32; ++w) mx = max(mx, sh[w]);
+        cmax = mx;
+    }
+    cl.sync();
+    mx = 0;
+    for (int w = 0; w < 8; ++w) mx = max(mx, *cl.map_shared_rank(&cmax, w));
+    cl.sync();  // a block's value is read before the block may end
+    const int e = dg_exp(mx);
+    if (rank == 0 && tid == 0) s.ec[n] = e;
+    const bool bad = e >= 2048;
+    const DgScale sc = dg_scale(bad ? 0 : e);
+    auto put = [&](int k, zd w) {
+        dg_put_col((uint32_t*)s.dst, (size_t)s.npad * (s.kpad / 2), s.kpad / 2, n, k, bad ? 0 : dg_int(w.x, sc),
+                   bad ? 0 : dg_int(w.y, sc));
+    };
+#pragma unroll
+    for (int u = 0; u < DG_PB_E; ++u) {
+        const int k = (u * 8 + rank) * DG_PB_T + tid;
+        if (k < s.K) put(k, v[u]);
+    }
+    for (int k = (DG_PB_E * 8 + rank) * DG_PB_T + tid; k < s.K; k += 8 * DG_PB_T) put(k, x[k]);
+}
+
+// ------------------------------------------------------------ host side
+struct DgPool {  // device memory of a plan
+    std::vector<void*> p;
+    bool ok = true;
+    void* get(size_t bytes, bool zero) {
+        void* q = nullptr;
+        if (!ok || cudaMalloc(&q, std::max<size_t>(bytes, 16)) != cudaSuccess) {
+            cudaGetLastError();
+            ok = false;
+            return nullptr;
+        }
+        p.push_back(q);
+        if (zero && cudaMemset(q, 0, std::max<size_t>(bytes, 16)) != cudaSuccess) ok = false;
+        return q;
+    }
+    template <typename T>
+    T* up(const std::vector<T>& v) {
+        T* q = (T*)get(v.size() * sizeof(T), false);
+        if (q && cudaMemcpy(q, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+        return q;
+    }
+    void drop() {
+        for (void* q : p) cudaFree(q);
+        p.clear();
+    }
+};
+static int dg_up(int n, int m) { return (n + m - 1) / m * m; }
+static int dg_nt(int ncol) { return 2 * ncol <= 16 ? 16 : (2 * ncol <= 32 ? 32 : 64); }
+static int dg_kpad(int K) { return dg_up(2 * K, DG_KS); }
+
+// digit planes [6][rows][kpad] of fp16, box of 32 reals x box_rows rows x 6 planes
+static bool dg_tmap(CUtensorMap* tm, const void* base, int kpad, int rows, int box_rows) {
+    encode_fn_t enc = get_encode();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)kpad, (cuuint64_t)rows, DG_P};
+    cuuint64_t str[2] = {(cuuint64_t)kpad * 2, (cuuint64_t)kpad * 2 * rows};
+    cuuint32_t box[3] = {DG_KS, (cuuint32_t)box_rows, DG_P};
+    cuuint32_t es[3] = {1, 1, 1};
+    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, str, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+template <int NT>
+static constexpr int dg_smem() {
+    return (NT == 16 ? 4 : 3) * DG_P * (DG_A_PL + NT * 64) + 1024;
+}
+template <int MODE>
+static const void* dg_fn(int NT, int* smem) {
+    *smem = NT == 16 ? dg_smem<16>() : (NT == 32 ? dg_smem<32>() : dg_smem<64>());
+    return NT == 16 ? (const void*)k_dg<16, MODE> : (NT == 32 ? (const void*)k_dg<32, MODE> : (const void*)k_dg<64, MODE>);
+}
+template <int MODE>
+static cudaError_t dg_attr(int NT) {
+    int sm;
+    const void* f = dg_fn<MODE>(NT, &sm);
+    return raise_smem(f, sm);
+}
+template <int MODE>
+static void dg_launch(int NT, int mt, int nk, DgArgs a, cudaStream_t s) {
+    int sm;
+    const void* f = dg_fn<MODE>(NT, &sm);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.cs * a.ntn * a.gs, mt, nk);
+    cfg.blockDim = dim3(DG_THREADS);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = a.cs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    void* args[1] = {&a};
+    cudaLaunchKernelExC(&cfg, f, args);
+}
+// K slices so that the waves of blocks are short.  In units of one stage's
+// products (about 0.9 us) a block costs its stages, a start and a read-out worth
+// about four, one more for the cluster's exchange and three where clusters
+// meet in global memory.  Clusters of eight leave a few of the 152 SMs idle.
+static void dg_splits(int tiles, int nst, int* cs, int* gs) {
+    double tb = 1e30;
+    *cs = *gs = 1;
+    for (int c = 1; c <= 8; c *= 2)
+        for (int q = 1; q <= 32 && c * q <= std::max(1, nst); ++q) {
+            const int room = c == 8 ? 136 : 152;
+            const double t = (double)((tiles * c * q + room - 1) / room) *
+                             ((nst + c * q - 1) / (c * q) + 4.0 + (c > 1 ? 1.0 : 0.0) + (q > 1 ? 3.0 : 0.0));
+            if (t < tb * 0.97) {
+                tb = t;
+                *cs = c;
+                *gs = q;
+            }
+        }
+}
+
+struct DgLeft {
+    DgPool pool;
+    std::vector<CUtensorMap> tm;
+    std::vector<int> M, K, kpad;
+    std::vector<int*> er;
+};
+struct DgGemm {
+    DgPool pool;
+    int nk = 0, ncol = 0, NT = 0, ntn = 0, mt = 0, cs = 1, gs = 1;
+    CUtensorMap *tmA = nullptr, *tmB = nullptr;
+    DgOut* out = nullptr;
+    DgPackB* pb = nullptr;
+    i64* part = nullptr;
+    unsigned* cnt = nullptr;
+    int* flag = nullptr;
+};
+
+void dg_left_destroy(DgLeft* l) {
+    if (!l) return;
+    l->pool.drop();
+    delete l;
+}
+void dg_gemm_destroy(DgGemm* g) {
+    if (!g) return;
+    g->pool.drop();
+    delete g;
+}
+
+DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s) {
+    DgLeft* l = new DgLeft();
+    std::vector<DgSrc> src(nk);
+    int mm = 1, mk = 1;
+    for (int k = 0; k < nk && l->pool.ok; ++k) {
+        const int mp = dg_up(m[k].M, DG_BM), kp = dg_kpad(m[k].K);
+        DgSrc& d = src[k];
+        d.src = m[k].src;
+        d.rs = m[k].rs;
+        d.cs = m[k].cs;
+        d.conj = m[k].conj;
+        d.M = m[k].M;
+        d.K = m[k].K;
+        d.mpad = mp;
+        d.kpad = kp;
+        d.dst = (__half*)l->pool.get((size_t)DG_P * mp * kp * sizeof(__half), true);
+        d.er = (int*)l->pool.get(mp * sizeof(int), true);
+        CUtensorMap t;
+        if (l->pool.ok && !dg_tmap(&t, d.dst, kp, mp, DG_BM)) l->pool.ok = false;
+        l->tm.push_back(t);
+        l->M.push_back(m[k].M);
+        l->K.push_back(m[k].K);
+        l->kpad.push_back(kp);
+        l->er.push_back(d.er);
+        mm = std::max(mm, m[k].M);
+        mk = std::max(mk, m[k].K);
+    }
+    DgSrc* ds = l->pool.ok ? l->pool.up(src) : nullptr;
+    if (l->pool.ok) {
+        k_dg_rowmax<<<dim3((mm + 31) / 32, 1, nk), 256, 0, s>>>(ds);
+        k_dg_pack_a<<<dim3((mk + 31) / 32, (mm + 31) / 32, nk), 256, 0, s>>>(ds);
+        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) l->pool.ok = false;
+    }
+    if (!l->pool.ok) {
+        dg_left_destroy(l);
+        return nullptr;
+    }
+    return l;
+}
+
+// device bytes of dg_left_create
+size_t dg_left_bytes(int M, int K) { return (size_t)DG_P * dg_up(M, DG_BM) * dg_kpad(K) * sizeof(__half); }
+
+DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag) {
+    DgGemm* g = new DgGemm();
+    g->nk = nk;
+    g->ncol = ncol;
+    g->NT = dg_nt(ncol);
+    g->ntn = (2 * ncol + g->NT - 1) / g->NT;
+    g->flag = flag;
+    const int np = g->ntn * g->NT;
+    std::vector<CUtensorMap> tb(nk);
+    std::vector<DgOut> out(nk);
+    std::vector<DgPackB> pb(nk);
+    int tiles = 0, nst = 1;
+    for (int k = 0; k < nk && g->pool.ok; ++k) {
+        const int kp = dg_kpad(r[k].K);
+        pb[k].X = r[k].X;
+        pb[k].ldx = r[k].ldx;
+        pb[k].K = r[k].K;
+        pb[k].dst = (__half*)g->pool.get((size_t)DG_P * np * kp * sizeof(__half), true);
+        pb[k].npad = np;
+        pb[k].kpad = kp;
+        pb[k].ec = (int*)g->pool.get(ncol * sizeof(int), true);
+        if (g->pool.ok && !dg_tmap(&tb[k], pb[k].dst, kp, np, g->NT)) g->pool.ok = false;
+        out[k].M = l->M[k];
+        out[k].nst = kp / DG_KS;
+        out[k].ldc = r[k].ldc;
+        out[k].er = l->er[k];
+        out[k].ec = pb[k].ec;
+        out[k].C = r[k].C;
+        out[k].tile0 = tiles;
+        const int mt = (l->M[k] + DG_BM - 1) / DG_BM;
+        g->mt = std::max(g->mt, mt);
+        tiles += mt * g->ntn;
+        nst = std::max(nst, out[k].nst);
+    }
+    dg_splits(std::max(tiles, 1), nst, &g->cs, &g->gs);
+    if (g->gs > 1) {
+        g->part = (i64*)g->pool.get((size_t)tiles * g->NT * 2 * DG_BM * sizeof(i64), true);
+        g->cnt = (unsigned*)g->pool.get((size_t)tiles * g->cs * sizeof(unsigned), true);
+    }
+    if (g->pool.ok) {
+        std::vector<CUtensorMap> ta(l->tm.begin(), l->tm.begin() + nk);
+        g->tmA = g->pool.up(ta);
+        g->tmB = g->pool.up(tb);
+        g->out = g->pool.up(out);
+        g->pb = g->pool.up(pb);
+    }
+    if (!g->pool.ok || dg_attr<0>(g->NT) != cudaSuccess) {
+        dg_gemm_destroy(g);
+        return nullptr;
+    }
+    return g;
+}
+
+// C (+)= A X for entries kofs .. kofs + nk - 1
+int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s) {
+    k_dg_pack_b<<<dim3(8 * g->ncol, 1, nk), DG_PB_T, 0, s>>>(g->pb, kofs);
+    DgArgs a{};
+    a.tmA = g->tmA;
+    a.tmB = g->tmB;
+    a.out = g->out;
+    a.kofs = kofs;
+    a.ncol = g->ncol;
+    a.ntn = g->ntn;
+    a.cs = g->cs;
+    a.gs = g->gs;
+    a.beta = beta;
+    a.part = g->part;
+    a.cnt = g->cnt;
+    a.flag = g->flag;
+    dg_launch<0>(g->NT, g->mt, nk, a, s);
+    return 2;
+}
+
+// ------------------------------------------------------------ Chebyshev series
+// The series with H~ y_{n-1} as digit products, one launch per term, for
+// DG_SERIES_MIN_NS states and more.  In FP64 its rate was the FP64 pipe's (16
+// k-points of N_aux 300, N_s 60: 9.0 GFLOP in 8.3 ms; 2 k-points 1.91 ms), here
+// the 2 k-points take 0.29 ms, bound by the 14 launches of a few stages each.
+// Below nine states the cooperative per-row form has the shorter chain.  H~ = (HH - lam_c) / lam_h has norm <= 1, so its entries take the scale
+// 1; a column of theta takes the power of two above its 2-norm, which bounds
+// every y_n.  y_n, the recurrence and the sum are integers in units of 2^-62
+// of that scale: nothing is rounded between the terms but the digits' cut.
+struct DgSeriesK {
+    KDev const* kd;
+    __half* A;       // [6][mpad][kpad]
+    int mpad, kpad;
+    int* bad;        // per row: HH not finite
+    int* ec;
+};
+struct DgSeries {
+    DgPool pool;
+    int nk = 0, n = 0, ns = 0, NT = 0, ntn = 0, mt = 0, cs = 1, gs = 1;
+    CUtensorMap *tmA = nullptr, *tmB[2] = {nullptr, nullptr};
+    DgOut* out = nullptr;
+    DgCheb* ch = nullptr;
+    DgSeriesK* sk = nullptr;
+    i64* part = nullptr;
+    unsigned* cnt = nullptr;
+};
+
+// digits of row i of H~ (HH as in k_hsub; HH is Hermitian, so row i is read
+// as the conjugate of the contiguous column i)
+__global__ void __launch_bounds__(128) k_dg_hsub(StepArgs a, const DgSeriesK* sk) {
+    const DgSeriesK& S = sk[blockIdx.z];
+    const KDev& K = a.kd[blockIdx.z];
+    const int n = a.naux, i = blockIdx.x;
+    DevState* st = a.st;
+    const double* av = a.a + 3 * (size_t)st->cstep;
+    const double ax = av[0], ay = av[1], az = av[2];
+    const double aa = (ax * ax + ay * ay + az * az) * a.half_inv_c2;
+    if (i == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
+        st->bar = 0u;
+        if (!a.dv_on) {
+            st->cur_a[0] = ax;
+            st->cur_a[1] = ay;
+            st->cur_a[2] = az;
+            st->cur_s = 0.0;
+            st->cur_aa = aa;
+        }
+    }
+    const double lc = K.lam[0], ilh = K.lam[2];
+    const double al[3] = {ax * a.inv_c, ay * a.inv_c, az * a.inv_c};
+    const size_t nn = (size_t)n * n;
+    const DgScale sc = dg_scale(0);
+    int bad = 0;
+    for (int j = threadIdx.x; j < n; j += 128) {
+        const size_t e = (size_t)i * n + j;
+        zd v = zmk(0.0, 0.0);
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+            if (al[l] != 0.0) v = zadd(v, zscale(K.psub[l * nn + e], al[l]));
+        if (i == j) v.x += K.eps[i] + aa;
+        if (a.dv_on) v = zadd(v, K.dvsub[e]);
+        if (i == j) v.x -= lc;
+        v = zscale(v, ilh);
+        if (dg_hw(v.x) >= 0x7ff00000 || dg_hw(v.y) >= 0x7ff00000) bad = 1;
+        // |H~_ij| <= 1; a step beyond its bounds (reported by its flag) stays in range
+        v.x = fmin(fmax(v.x, -1.0), 1.0);
+        v.y = fmin(fmax(v.y, -1.0), 1.0);
+        uint32_t dr[DG_P], di[DG_P];
+        dg_cut(dg_int(v.x, sc), dr);
+        dg_cut(dg_int(-v.y, sc), di);
+#pragma unroll
+        for (int q = 0; q < DG_P; ++q)
+            ((uint32_t*)S.A)[((size_t)q * S.mpad + i) * (S.kpad / 2) + j] = dg_pair(dr[q], di[q]);
+    }
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) S.bad[i] = bad;
+}
+
+// y_0 = theta in units of its column's scale, its digits, and c_0 y_0
+__global__ void __launch_bounds__(128) k_dg_y0(StepArgs a, const DgSeriesK* sk, const DgCheb* chs) {
+    __shared__ double sh[4];
+    const DgSeriesK& S = sk[blockIdx.z];
+    const DgCheb& ch = chs[blockIdx.z];
+    const KDev& K = a.kd[blockIdx.z];
+    const int n = a.naux, c = blockIdx.x, tid = threadIdx.x;
+    const zd* th = K.theta + (size_t)c * n;
+    // the norm of theta / 2^e with e from its largest entry: no overflow in the squares
+    int mx = 0;
+    for (int i = tid; i < n; i += 128) mx = max(mx, max(dg_hw(th[i].x), dg_hw(th[i].y)));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    __shared__ int smx[4];
+    if ((tid & 31) == 0) smx[tid >> 5] = mx;
+    __syncthreads();
+    mx = max(max(smx[0], smx[1]), max(smx[2], smx[3]));
+    int e = dg_exp(mx);
+    const bool bad = e >= 2048;
+    if (bad) e = 0;
+    const DgScale s0 = dg_scale(e);
+    double q = 0.0;
+    for (int i = tid; i < n; i += 128) {
+        const double x = (th[i].x * s0.p1) * s0.p2, y = (th[i].y * s0.p1) * s0.p2;  // 2^53 at most
+        q += x * x + y * y;
+    }
+    q = warp_sum(q);
+    if ((tid & 31) == 0) sh[tid >> 5] = q;
+    __syncthreads();
+    q = sqrt(sh[0] + sh[1] + sh[2] + sh[3]);
+    // the power of two above the norm, less a rounding error's room at exact powers
+    const int en = q > 0.0 ? dg_exp(dg_hw(q * (1.0 - 1e-12))) : 53;
+    e += en - 53;
+    if (tid == 0) S.ec[c] = bad ? 2048 : e;
+    const int s = 62 - e, h = s / 2;
+    const double p1 = dg_pow2(max(-1000, min(1000, h))), p2 = dg_pow2(max(-1000, min(1000, s - h)));
+    // the coefficients in units 2^-62 (|c_n| < 2), once per k-point and by every block for c_0
+    const double one62 = 4611686018427387904.0;
+    const i64 cr = __double2ll_rn(K.coef[0].x * one62), ci = __double2ll_rn(K.coef[0].y * one62);
+    if (c == 0)
+        for (int i = tid; i < a.nterms; i += 128) {
+            ch.coef[2 * i] = __double2ll_rn(K.coef[i].x * one62);
+            ch.coef[2 * i + 1] = __double2ll_rn(K.coef[i].y * one62);
+        }
+    for (int i = tid; i < n; i += 128) {
+        const i64 yr = bad ? 0 : __double2ll_rn((th[i].x * p1) * p2), yi = bad ? 0 : __double2ll_rn((th[i].y * p1) * p2);
+        const size_t x = (size_t)(2 * c) * n + i;
+        ch.y0[x] = yr;
+        ch.y0[x + n] = yi;
+        ch.acc[x] = dg_mul62(cr, yr) - dg_mul62(ci, yi);
+        ch.acc[x + n] = dg_mul62(cr, yi) + dg_mul62(ci, yr);
+        dg_put_col((uint32_t*)ch.Bn[0], ch.pl / 2, ch.kpad / 2, c, i, (yr + 256) >> 9, (yi + 256) >> 9);
+    }
+}
+
+// theta = phase x sum; a k-point whose HH is not finite gives NaN
+__global__ void __launch_bounds__(128) k_dg_theta(StepArgs a, const DgSeriesK* sk, const DgCheb* chs) {
+    const DgSeriesK& S = sk[blockIdx.z];
+    const DgCheb& ch = chs[blockIdx.z];
+    const KDev& K = a.kd[blockIdx.z];
+    const int n = a.naux, c = blockIdx.x, tid = threadIdx.x;
+    const int e = S.ec[c];
+    int bad = e >= 2048;
+    for (int i = tid; i < n; i += 128) bad |= S.bad[i];
+    bad = __syncthreads_or(bad);
+    const zd ph = (a.prop == 0) ? zmk(K.lam[3], K.lam[4]) : zmk(1.0, 0.0);
+    const int s = bad ? 0 : e - 62, h = s / 2;
+    const double p1 = dg_pow2(max(-1000, min(1000, h))), p2 = dg_pow2(max(-1000, min(1000, s - h)));
+    for (int i = tid; i < n; i += 128) {
+        const size_t x = (size_t)(2 * c) * n + i;
+        zd v = zmul(ph, zmk((double)ch.acc[x], (double)ch.acc[x + n]));
+        v = zmk((v.x * p1) * p2, (v.y * p1) * p2);
+        if (bad) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+        K.theta[i + (size_t)c * n] = v;
+    }
+}
+
+void dg_series_destroy(DgSeries* g) {
+    if (!g) return;
+    g->pool.drop();
+    delete g;
+}
+
+DgSeries* dg_series_create(int nk, int n, int ns) {
+    DgSeries* g = new DgSeries();
+    g->nk = nk;
+    g->n = n;
+    g->ns = ns;
+    g->NT = dg_nt(ns);
+    g->ntn = (2 * ns + g->NT - 1) / g->NT;
+    g->mt = (n + DG_BM - 1) / DG_BM;
+    const int np = g->ntn * g->NT, mp = g->mt * DG_BM, kp = dg_kpad(n);
+    std::vector<CUtensorMap> ta(nk), tb0(nk), tb1(nk);
+    std::vector<DgOut> out(nk);
+    std::vector<DgCheb> ch(nk);
+    std::vector<DgSeriesK> sk(nk);
+    for (int k = 0; k < nk && g->pool.ok; ++k) {
+        sk[k].A = (__half*)g->pool.get((size_t)DG_P * mp * kp * sizeof(__half), true);
+        sk[k].mpad = mp;
+        sk[k].kpad = kp;
+        sk[k].bad = (int*)g->pool.get(n * sizeof(int), true);
+        sk[k].ec = (int*)g->pool.get(ns * sizeof(int), true);
+        DgCheb& c = ch[k];
+        c.n = n;
+        c.y0 = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
+        c.y1 = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
+        c.acc = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
+        for (int q = 0; q < 2; ++q) c.Bn[q] = (__half*)g->pool.get((size_t)DG_P * np * kp * sizeof(__half), true);
+        c.pl = (size_t)np * kp;
+        c.kpad = kp;
+        c.coef = (i64*)g->pool.get((size_t)2 * RTD_MAX_TERMS * sizeof(i64), true);
+        out[k].M = n;
+        out[k].nst = kp / DG_KS;
+        out[k].ldc = 0;
+        out[k].er = nullptr;
+        out[k].ec = nullptr;
+        out[k].C = nullptr;
+        out[k].tile0 = k * g->mt * g->ntn;
+        if (g->pool.ok && (!dg_tmap(&ta[k], sk[k].A, kp, mp, DG_BM) || !dg_tmap(&tb0[k], c.Bn[0], kp, np, g->NT) ||
+                           !dg_tmap(&tb1[k], c.Bn[1], kp, np, g->NT)))
+            g->pool.ok = false;
+    }
+    const int tiles = nk * g->mt * g->ntn;
+    dg_splits(tiles, kp / DG_KS, &g->cs, &g->gs);
+    if (g->gs > 1) {
+        g->part = (i64*)g->pool.get((size_t)tiles * g->NT * 2 * DG_BM * sizeof(i64), true);
+        g->cnt = (unsigned*)g->pool.get((size_t)tiles * g->cs * sizeof(unsigned), true);
+    }
+    if (g->pool.ok) {
+        g->tmA = g->pool.up(ta);
+        g->tmB[0] = g->pool.up(tb0);
+        g->tmB[1] = g->pool.up(tb1);
+        g->out = g->pool.up(out);
+        g->ch = g->pool.up(ch);
+        g->sk = g->pool.up(sk);
+    }
+    if (!g->pool.ok || dg_attr<1>(g->NT) != cudaSuccess) {
+        dg_series_destroy(g);
+        return nullptr;
+    }
+    return g;
+}
+
+int launch_dg_series(const DgSeries* g, const StepArgs& a, cudaStream_t s) {
+    k_dg_hsub<<<dim3(g->n, 1, g->nk), 128, 0, s>>>(a, g->sk);
+    k_dg_y0<<<dim3(g->ns, 1, g->nk), 128, 0, s>>>(a, g->sk, g->ch);
+    DgArgs d{};
+    d.tmA = g->tmA;
+    d.out = g->out;
+    d.ch = g->ch;
+    d.ncol = g->ns;
+    d.ntn = g->ntn;
+    d.cs = g->cs;
+    d.gs = g->gs;
+    d.part = g->part;
+    d.cnt = g->cnt;
+    d.flag = a.flag;
+    for (int t = 1; t < a.nterms; ++t) {
+        d.tmB = g->tmB[(t - 1) & 1];
+        d.term = t;
+        d.last = t == a.nterms - 1;
+        dg_launch<1>(g->NT, g->mt, g->nk, d, s);
+    }
+    k_dg_theta<<<dim3(g->ns, 1, g->nk), 128, 0, s>>>(a, g->sk, g->ch);
+    return a.nterms + 2;
+}

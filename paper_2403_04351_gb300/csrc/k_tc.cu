@@ -11,7 +11,6 @@
 // shared memory by TMA (cp.async.bulk.tensor, 128-byte swizzle, K-major),
 // issued by one thread through a four-stage mbarrier pipeline; every wait
 // is bounded and raises flag bit 3 instead of hanging.
-#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -21,97 +20,12 @@
 #include <vector>
 
 #include "rtd.h"
+#include "tcgen05.cuh"
 #include "rttddft.h"
 
 #define TC_BM 128
 #define TC_BK 64  // bf16 per K block = 128 bytes, one swizzle row
 #define TC_STAGES 4
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// The dynamic shared-memory attribute is global per kernel and shared by every
-// context of the process: raise it to `bytes`, never lower it.
-static cudaError_t raise_smem(const void* f, int bytes) {
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, f);
-    if (e != cudaSuccess) return e;
-    if (fa.maxDynamicSharedSizeBytes >= bytes) return cudaSuccess;
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* b, uint32_t phase) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(b)), "r"(phase)
-        : "memory");
-    return ok != 0;
-}
-// bounded wait on an mbarrier phase: false after about 2^31 SM cycles (~1 s)
-__device__ bool mbar_wait(uint64_t* b, uint32_t phase) {
-    const long long t0 = clock64();
-    while (!mbar_try_wait(b, phase))
-        if (clock64() - t0 > (1ll << 31)) return false;
-    return true;
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            smem_u32(dst)),
-        "l"((uint64_t)tm), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row atoms 1024 B apart
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-    d |= (uint64_t)1 << 16;                  // leading byte offset (unused for this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;        // stride byte offset
-    d |= (uint64_t)1 << 46;                  // descriptor version
-    d |= (uint64_t)2 << 61;                  // 128-byte swizzle
-    return d;
-}
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accum) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            tmem_d),
-        "l"(da), "l"(db), "r"(idesc), "r"(accum)
-        : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// D (TMEM) (+)= A (TMEM, 128 lanes = rows, 16 packed bf16/fp16 K values in 8
-// columns) x B (shared-memory descriptor)
-__device__ __forceinline__ void umma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t accum) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(
-            tmem_d),
-        "r"(tmem_a), "l"(db), "r"(idesc), "r"(accum)
-        : "memory");
-}
-// a warp's 32 lanes x W consecutive 32-bit TMEM columns from W registers per thread
-template <int W>
-__device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t* v) {
-    if constexpr (W == 8)
-        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-                     "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                     : "memory");
-    else
-        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v[0]),
-                     "r"(v[1]), "r"(v[2]), "r"(v[3])
-                     : "memory");
-}
 
 // D[split][m][n] (FP32, row-major M x N) = sum over this split's K blocks
 // of A^ B^^T; grid (M tiles, K splits, N tiles).
@@ -297,23 +211,6 @@ __global__ void k_tc_combine(const float* __restrict__ D, int splits, int M, int
 }
 
 // ------------------------------------------------------------ host side
-typedef CUresult (*encode_fn_t)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static encode_fn_t get_encode() {
-    static encode_fn_t fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (encode_fn_t)p;
-    }
-    return fn;
-}
-
 // 2-D bf16 tensor map, rows of `inner` elements (row pitch `pitch_elems`),
 // box of 64 x box_rows elements, 128-byte swizzle
 static int tc_tmap(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t rows, uint64_t pitch_elems,

@@ -147,7 +147,6 @@ struct StepArgs {
     int tc_fmt;               // tensor-core operand format: 1 bf16, 0 fp16
     int ith;                  // the interstitial sum arrives in K.th (tensor cores or FFT)
     int hartree;              // the potential change is the Hartree potential of the density (FFT route)
-    int cheb_tile;            // the cooperative series runs as k_cheb_tile (4 < N_s <= 64)
     double tc_st;             // scale of the split table (fp16 range)
     double mt_u;              // muffin-tin part of the density feedback: dh = mt_u (n - n0) (0: off)
     const zd* mtn0;           //   reference muffin-tin density matrices n_a(0) (atom blocks at boff)
@@ -211,6 +210,8 @@ struct StepPlan {
     const struct TcPlan* tc;  // tensor-core operator plan (split-BF16 form) or null
     const struct TcCC* tcc;   // tensor-core expansion and projection (split forms, many states) or null
     const struct TcMT* tcmt;  // tensor-core muffin-tin blocks (split-BF16 form, many states) or null
+    const struct DgGemm *dg_expand, *dg_fwd, *dg_back, *dg_proj;  // FP64 products on the tensor cores, or null
+    const struct DgSeries* series;  // Chebyshev series as digit products (many states) or null
     const struct FftPlan* fft;  // FFT route of the interstitial convolution or null
     unsigned* tile_cnt;         // zeroed row-tile counters of the fused split-K sums (or null)
     cudaStream_t side;          // second stream for work that overlaps the main chain (or null)
@@ -233,8 +234,7 @@ void launch_step(const StepArgs& a, const StepPlan& p, cudaStream_t s, int* nlau
 int launch_operator_pass(const StepArgs& a, const StepPlan& p, cudaStream_t s, TraceHook* tr = nullptr);
 int prepare_back_kernels(const StepArgs& a);
 // blocks for the cooperative Chebyshev launch if it can be captured in a graph, else 0
-// tile: set to 1 when the series for many states runs in tiles of HH rows (k_cheb_tile)
-int prepare_cheb_coop(const StepArgs& a, cudaStream_t s, int* tile);
+int prepare_cheb_coop(const StepArgs& a, cudaStream_t s);
 void launch_cheb_coop(const StepArgs& a, cudaStream_t s);
 void launch_prep_coef(const StepArgs& a, cudaStream_t s);
 void launch_subspace_current(const StepArgs& a, int set_gs, cudaStream_t s);

@@ -1,0 +1,84 @@
+"""The FP64 contractions by exact digit products on the tensor cores, at the
+edges of their tiles (128 rows, 16/32/64 real columns, K in stages of 32
+reals and slices of 64), against plain FP64."""
+import numpy as np
+import pytest
+import scipy.linalg as sla
+
+from paper_2403_04351_gb300 import Context
+from synth import make_system, tiny_config
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_aux,n_s", [(16, 9), (33, 16), (128, 17), (129, 32), (145, 33), (300, 64), (97, 70)])
+def test_series_of_many_states(n_aux, n_s):
+    """theta' = exp(-i HH dt) theta for states of very different norms and for
+    a zero column.  The digits' cut (2^-54 of the norm per factor and term,
+    sqrt(2 n) entries, about 15 terms) stays below 2e-14 of a column's norm;
+    the reference's own rounding is of the same size."""
+    s = make_system(tiny_config(n_g=max(n_aux, 60), n_s=n_s, n_aux=n_aux, n_k=2, kgrid=(2, 1, 1)))
+    rng = np.random.default_rng(n_aux)
+    ctx = Context(s, graph_steps=1)
+    a = np.array([[1.0, -2.0, 3.0], [0.5, 4.0, 0.0]])
+    want = []
+    for k in range(2):
+        th = rng.standard_normal((n_aux, n_s)) + 1j * rng.standard_normal((n_aux, n_s))
+        th *= 10.0 ** rng.integers(-30, 30, n_s)[None, :]
+        th[:, 1] = 0.0
+        th[:, 2] = np.eye(n_aux)[:, n_aux - 1]
+        ctx.set_state(k, th)
+        _, eps, pp = ctx.get_aux(k)
+        for v in a:
+            h = np.diag(eps + v @ v / (2 * s["c_light"] ** 2)) + np.tensordot(v / s["c_light"], pp, 1)
+            th = sla.expm(-1j * s["dt"] * h) @ th
+        want.append(th)
+    ctx.step(a)
+    for k in range(2):
+        got = ctx.get_state(k)
+        assert np.all(got[:, 1] == 0.0)
+        norm = np.linalg.norm(want[k], axis=0)
+        norm[1] = 1.0
+        assert np.max(np.linalg.norm(got - want[k], axis=0) / norm) < 4e-14
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_g,n_s,n_atoms", [(40, 1, 1), (128, 8, 2), (129, 9, 1), (255, 17, 3), (300, 33, 2), (65, 64, 0)])
+@pytest.mark.parametrize("route", ["toeplitz", "fft"])
+def test_operator_and_projection(n_g, n_s, n_atoms, route):
+    """FP64 operator on columns of very different sizes (and a zero one), and
+    the expansion and projection of a step, against the explicit matrices.
+    The cut is 2^-54 of a row's and of a column's largest entry: entrywise
+    2^-53 sqrt(K) of their product and below, here 1e-13 of the row's and
+    column's norms with the three products in a row."""
+    from oracle.rttddft_oracle import explicit_operators, hamiltonian
+    from systems import free_electron_system
+    if n_atoms:
+        s = make_system(tiny_config(n_g=n_g, n_atoms=n_atoms, lmax=2, n_lo_per_atom=3, n_s=n_s, n_aux=max(n_s, 12)))
+    else:
+        s = free_electron_system(n_g=n_g, n_s=n_s, n_aux=n_s)
+    rng = np.random.default_rng(n_g)
+    ctx = Context(s, interstitial=route)
+    ops = explicit_operators(s, 0)
+    nb = ops["nb"]
+    x = rng.standard_normal((nb, n_s + 1)) + 1j * rng.standard_normal((nb, n_s + 1))
+    x *= 10.0 ** rng.integers(-100, 100, n_s + 1)[None, :]
+    x[:, 0] = 0.0
+    a = np.array([0.4, -0.9, 1.3])
+    hx, sx = ctx.apply(0, x, a)
+    h = hamiltonian(ops, a, s["c_light"])
+    assert np.all(hx[:, 0] == 0.0) and np.all(sx[:, 0] == 0.0)
+    size = np.linalg.norm(x[:, 1:], axis=0)
+    assert np.max(np.abs(hx - h @ x)[:, 1:] / (np.linalg.norm(h, axis=1)[:, None] * size)) < 1e-13
+    assert np.max(np.abs(sx - ops["S"] @ x)[:, 1:] / (np.linalg.norm(ops["S"], axis=1)[:, None] * size)) < 1e-13
+    if n_s > 1:
+        x[1, 1] = np.nan
+        assert np.all(np.isnan(ctx.apply(0, x, a)[0][:, 1]))
+    ctx.step(a[None, :])
+    o = ctx.observables()
+    th, c = ctx.get_state(0, with_c=True)
+    cc = ctx.get_aux(0)[0]
+    e = 2.0 * np.real(np.vdot(cc @ th, h @ (cc @ th)))
+    assert abs(o["energy"][0] - e) < 1e-12 * max(1.0, abs(e))
+    assert o["resid"][0] < 1e-12 and o["norm_dev"][0] < 1e-12
+    ctx.close()
