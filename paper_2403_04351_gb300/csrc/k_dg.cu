@@ -7,12 +7,13 @@
 // base-512 digits d in [-256, 256] (the error-free splitting of Ozaki, Ogita,
 // Oishi and Rump, Numer. Algorithms 59, 2012).  Digits are exact in fp16, a
 // product of two is at most 2^16, and the FP32 accumulator of tcgen05.mma
-// holds the sum of one group (pairs i + j = s) over 64 reals of K exactly:
-// 2^24 bounds it for s >= 7; below, only operands whose digits all have the
-// same size and sign can pass 2^24, by an error of 2^-52 of the scale.  Groups
-// s = 4 .. 10 are kept (26 of 36 pairs; the dropped ones are below
-// 2^-70 (256^2) sqrt(K) of the scale, under the 2^-54 of the cut itself), read
-// out every 64 reals and added up as integers, so a result does not depend on
+// holds the sum of a group (the pairs i + j = s) exactly up to 2^24: over 256
+// reals of K for s = 10 (one pair), 128 for s = 9, 64 for s = 8 and 7.  s = 6 is
+// read out every 128, s = 5 and 4 every 512: their sums pass 2^24 only where
+// nearly all digits have the largest size and one sign, by a rounding of 2^-52
+// of the scale where the result itself is 2^5 of it.  The groups s = 4 .. 10
+// are kept (26 of 36 pairs; the dropped ones are below the 2^-54 of the cut
+// itself), read out and added up as integers, so a result does not depend on
 // the order of the sums or on the number of K slices.
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
@@ -32,9 +33,13 @@ namespace cg = cooperative_groups;
 #define DG_P 6              // digits
 #define DG_KS 32            // reals per stage: 64 bytes of fp16, one row of the 64-byte swizzle
 #define DG_BM 128           // rows per tile
-#define DG_G 7              // groups kept, s = 10 - g
+#define DG_S0 4             // smallest i + j kept
+#define DG_G 7              // groups kept, s = DG_S0 + g, NT columns of tensor memory each
 #define DG_THREADS 320      // 8 read-out warps, one product warp, one copy warp
 #define DG_A_PL (DG_BM * 64)
+
+// slices of 64 reals that a group collects before it is read out
+__host__ __device__ constexpr int dg_run(int g) { return g == 6 ? 4 : (g == 5 || g == 2 ? 2 : (g < 2 ? 8 : 1)); }
 
 typedef long long i64;
 
@@ -104,23 +109,34 @@ __device__ __forceinline__ double dg_double(i64 hi, i64 lo, int e) {
     return neg ? -v : v;
 }
 
+// Operands lie tile by tile as a block of k_dg takes them: per tile of RT rows
+// and stage of 16 complex k, six planes of RT rows of 64 bytes, the 16-byte
+// chunks of a row permuted as the 64-byte swizzle wants them.  A stage is one
+// contiguous copy (as boxes of a row-major array, 64 bytes a row, the copies
+// gave 4.9 TB/s over the chip).  Word (two fp16) of row r, complex k, plane 0;
+// the planes are RT 16 words apart.
+__host__ __device__ __forceinline__ size_t dg_word(int r, int k, int RT, int nst) {
+    const int rr = r % RT;
+    return (((size_t)(r / RT) * nst + (k >> 4)) * DG_P * RT + rr) * 16 + ((((k >> 2) & 3) ^ ((rr >> 1) & 3)) << 2) + (k & 3);
+}
 // rows 2n: [Re, -Im] and 2n + 1: [Im, Re] of a right operand, entry k of complex column n
-__device__ __forceinline__ void dg_put_col(uint32_t* b, size_t plw, size_t kw, int n, int k, i64 qr, i64 qi) {
+__device__ __forceinline__ void dg_put_col(uint32_t* b, int NT, int nst, int n, int k, i64 qr, i64 qi) {
     uint32_t dr[DG_P], di[DG_P];
     dg_cut(qr, dr);
     dg_cut(qi, di);
-    b += (size_t)(2 * n) * kw + k;
+    b += dg_word(2 * n, k, NT, nst);
 #pragma unroll
     for (int i = 0; i < DG_P; ++i) {
         const uint32_t p = dg_pair(dr[i], di[i]);
-        b[i * plw] = p ^ (DG_NEG << 16);
-        b[i * plw + kw] = (p >> 16) | (p << 16);
+        b[(size_t)i * NT * 16] = p ^ (DG_NEG << 16);
+        b[(size_t)i * NT * 16 + 16] = (p >> 16) | (p << 16);
     }
 }
 
 // ------------------------------------------------------------ the product kernel
 struct DgOut {
-    int M, nst, ldc;    // rows, K stages, leading dimension of C
+    const unsigned char *A, *B;  // operands of the product
+    int M, nst, nsta, ldc;       // rows, K stages of X and of A (at least as many), leading dimension of C
     const int* er;      // row exponents of A
     const int* ec;      // column exponents of X
     zd* C;
@@ -130,13 +146,11 @@ struct DgCheb {
     int n;              // N_aux
     i64 *y0, *y1;       // y of even and of odd terms, units 2^-62 of the column's scale: [2 ns][n]
     i64* acc;           // sum_n c_n y_n
-    __half* Bn[2];      // digit operands of even and odd terms
-    size_t pl;          // their plane stride
-    int kpad;
+    uint32_t* Bn[2];    // digit operands of even and odd terms
+    int nst;
     i64* coef;          // c_n in units 2^-62
 };
 struct DgArgs {
-    const CUtensorMap *tmA, *tmB;
     const DgOut* out;
     const DgCheb* ch;
     int kofs, ncol, ntn, cs, gs, beta, term, last;  // cs K slices per cluster, gs clusters per tile
@@ -149,11 +163,10 @@ __device__ __forceinline__ uint64_t dg_desc(uint32_t saddr) {  // K-major, 64-by
     return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
            ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
-__device__ __forceinline__ void dg_tma(void* dst, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
+__device__ __forceinline__ void dg_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
-            smem_u32(dst)),
-        "l"((uint64_t)tm), "r"(x), "r"(y), "r"(0), "r"(smem_u32(bar))
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
 }
 template <int W>
@@ -178,11 +191,14 @@ __device__ __forceinline__ i64 dg_mul62(i64 a, i64 b) {
 
 // One 128-row x NT-column tile of D = A^ B^^T over this split's K stages (NT
 // real columns: Re and Im of NT / 2 complex ones).  The copy warp brings the
-// six digit planes of both operands of a stage with one TMA each; the product
-// warp issues the 26 pairs group by group into the group's own NT columns of
-// tensor memory; the read-out warps add a finished group (64 reals of K) to
-// their integers while the next groups' products run, so a group is handed
-// back and forth by a pair of mbarriers.  The K slices of a tile meet in the
+// six digit planes of both operands of a stage with one bulk copy each.  A group has
+// its own NT columns of tensor memory in the order of s, and X's digit planes
+// lie one after another in shared memory, so digit i of A meets a run of X's
+// digits in one product of up to N = 256 (9 instructions per 16 reals for
+// NT = 64 instead of 26, 6 for fewer columns: a product reads A's 128 rows once
+// whatever its N).  The read-out warps add a finished group (64 reals of K) to
+// their integers while the products of the others run; a group is handed back
+// and forth by a pair of mbarriers.  The K slices of a tile meet in the
 // distributed shared memory of a cluster, further clusters of the tile in
 // global memory, where the last one finishes it.
 // MODE 0: C (+)= the product, scaled back.  MODE 1: a Chebyshev term.
@@ -238,6 +254,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
     if (warp == 9) {
         if (lane == 0) {
             int issued = 0;
+            const unsigned char* ga = o.A + ((size_t)m_i * o.nsta + st0) * (DG_P * DG_A_PL);
+            const unsigned char* gb = (MODE == 0 ? o.B : (const unsigned char*)g.ch[z].Bn[(g.term - 1) & 1]) +
+                                      ((size_t)nt_i * o.nst + st0) * (DG_P * B_PL);
             for (int t = 0; t < nk; ++t) {
                 const int s = t % STAGES;
                 if (t >= STAGES && !mbar_wait(&empty[s], (uint32_t)((t / STAGES - 1) & 1))) {
@@ -248,8 +267,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
                 if (abort_flag) break;
                 unsigned char* sa = smem + s * STAGE;
                 mbar_expect_tx(&full[s], STAGE);
-                dg_tma(sa, g.tmA + z, (st0 + t) * DG_KS, m0, &full[s]);
-                dg_tma(sa + DG_P * DG_A_PL, g.tmB + z, (st0 + t) * DG_KS, n0, &full[s]);
+                dg_copy(sa, ga + (size_t)t * (DG_P * DG_A_PL), DG_P * DG_A_PL, &full[s]);
+                dg_copy(sa + DG_P * DG_A_PL, gb + (size_t)t * (DG_P * B_PL), DG_P * B_PL, &full[s]);
                 issued = t + 1;
             }
             // nothing may still be on its way into shared memory when the block ends
@@ -259,7 +278,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
     } else if (warp == 8) {
         if (lane == 0) {
             // kind::f16, fp16 operands, FP32 accumulator, both K-major
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(DG_BM >> 4) << 24);
+            const uint32_t idesc0 = (1u << 4) | ((uint32_t)(DG_BM >> 4) << 24);
+            constexpr int WMAX = 256 / NT < DG_P ? 256 / NT : DG_P;  // digits of X per product
             bool ok = true;
             for (int t = 0; t < nk && ok; ++t) {
                 const int s = t % STAGES;
@@ -272,28 +292,48 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
                 const int sl = t >> 1;
                 const uint64_t da = dg_desc(smem_u32(smem + s * STAGE));
                 const uint64_t db = dg_desc(smem_u32(smem + s * STAGE + DG_P * DG_A_PL));
+                // digit i of A times the digits j .. j + w - 1 of X in one product of N = w NT
+                auto mma = [&](int kk, int i, int j, int w, uint32_t acc) {
+                    umma_bf16(tmem + (uint32_t)((i + j - DG_S0) * NT), da + (uint64_t)((i * DG_A_PL + kk * 32) >> 4),
+                              db + (uint64_t)((j * B_PL + kk * 32) >> 4),
+                              idesc0 | ((uint32_t)((w * NT) >> 3) << 17), acc);
+                };
+                if (first) {
+                    // the slice's first products, a group at a time: a group that starts anew waits
+                    // for its read-out and overwrites its columns
 #pragma unroll
-                for (int gi = 0; gi < DG_G; ++gi) {
-                    if (first && sl > 0) {
-                        if (!mbar_wait(&gfree[gi], (uint32_t)((sl - 1) & 1))) {
-                            ok = false;
-                            break;
+                    for (int q = DG_G - 1; q >= 0; --q) {
+                        const bool anew = (sl & (dg_run(q) - 1)) == 0;
+                        if (anew && sl > 0) {
+                            if (!mbar_wait(&gfree[q], (uint32_t)((sl / dg_run(q) - 1) & 1))) {
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
                         }
-                        tc_fence_after();
+                        if (q > 0) mma(0, 5, q + DG_S0 - 5, 1, anew ? 0u : 1u);
+                        else mma(0, 4, 0, 1, anew ? 0u : 1u);
                     }
-                    constexpr int TOP = 2 * (DG_P - 1);
-                    const int sum = TOP - gi;
+                    if (!ok) break;
+                }
 #pragma unroll
-                    for (int i = 0; i < DG_P; ++i) {
-                        const int j = sum - i;
-                        if (j < 0 || j >= DG_P) continue;
+                for (int i = DG_P - 1; i >= 0; --i) {
 #pragma unroll
-                        for (int kk = 0; kk < 2; ++kk)
-                            umma_bf16(tmem + (uint32_t)(gi * NT), da + (uint64_t)((i * DG_A_PL + kk * 32) >> 4),
-                                      db + (uint64_t)((j * B_PL + kk * 32) >> 4), idesc,
-                                      (first && kk == 0 && i == (sum >= DG_P ? sum - DG_P + 1 : 0)) ? 0u : 1u);
+                    for (int kk = 0; kk < 2; ++kk) {
+                        int j = i < DG_S0 ? DG_S0 - i : 0;
+                        if (first && kk == 0) {
+                            if (i == 5) continue;
+                            if (i == 4) j = 1;
+                        }
+#pragma unroll
+                        for (; j < DG_P; j += WMAX) mma(kk, i, j, DG_P - j < WMAX ? DG_P - j : WMAX, 1u);
                     }
-                    if (lastp) umma_commit(&gfull[gi]);
+                    // the largest group that digit i reaches is complete (the smallest two with digit 0)
+                    if (lastp) {
+                        const int q = i + DG_P - 1 - DG_S0;
+                        if (t == nk - 1 || (sl & (dg_run(q) - 1)) == dg_run(q) - 1) umma_commit(&gfull[q]);
+                        if (i == 0 && (t == nk - 1 || (sl & (dg_run(0) - 1)) == dg_run(0) - 1)) umma_commit(&gfull[0]);
+                    }
                 }
                 umma_commit(&empty[s]);
             }
@@ -309,8 +349,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
         bool ok = true;
         for (int sl = 0; sl < nsl && ok; ++sl) {
 #pragma unroll
-            for (int gi = 0; gi < DG_G; ++gi) {
-                if (!mbar_wait(&gfull[gi], (uint32_t)(sl & 1)) || abort_flag) {
+            for (int gi = DG_G - 1; gi >= 0; --gi) {
+                if (sl != nsl - 1 && (sl & (dg_run(gi) - 1)) != dg_run(gi) - 1) continue;
+                if (!mbar_wait(&gfull[gi], (uint32_t)((sl / dg_run(gi)) & 1)) || abort_flag) {
                     ok = false;
                     break;
                 }
@@ -330,8 +371,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
 #pragma unroll
                     for (int c = 0; c < W; ++c) {
                         const i64 v = (i64)__float2int_rn(__uint_as_float(r[c]));
-                        if (gi <= 3) hi[c0 + c] += v << (9 * (3 - gi));  // units of s = 7
-                        else lo[c0 + c] += v << (9 * (6 - gi));          // units of s = 4
+                        if (gi >= 3) hi[c0 + c] += v << (9 * (gi - 3));  // units of s = 7
+                        else lo[c0 + c] += v << (9 * gi);                // units of s = 4
                     }
                 }
             }
@@ -442,8 +483,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
                 if (!g.last) {
                     yb[e] = y[0];
                     yb[e + ch.n] = y[1];
-                    dg_put_col((uint32_t*)(g.term & 1 ? ch.Bn[1] : ch.Bn[0]), ch.pl / 2, ch.kpad / 2, n, row, (y[0] + 256) >> 9,
-                               (y[1] + 256) >> 9);
+                    dg_put_col(ch.Bn[g.term & 1], NT, ch.nst, n, row, (y[0] + 256) >> 9, (y[1] + 256) >> 9);
                 }
             }
         }
@@ -460,8 +500,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
 struct DgSrc {
     const zd* src;
     size_t rs, cs;
-    int conj, M, K, mpad, kpad;
-    __half* dst;  // [6][mpad][kpad]
+    int conj, M, K, nst;
+    uint32_t* dst;  // tiles of 128 rows
     int* er;
 };
 // row exponents: a warp per row
@@ -523,7 +563,7 @@ __global__ void k_dg_pack_a(const DgSrc* d) {
         dg_cut(e >= 2048 ? 0 : dg_int(v.x, sc), dr);
         dg_cut(e >= 2048 ? 0 : dg_int(v.y, sc), di);
         for (int i = 0; i < DG_P; ++i)
-            ((uint32_t*)s.dst)[((size_t)i * s.mpad + r) * (s.kpad / 2) + k] = dg_pair(dr[i], di[i]);
+            s.dst[dg_word(r, k, DG_BM, s.nst) + (size_t)i * DG_BM * 16] = dg_pair(dr[i], di[i]);
     }
 }
 
@@ -533,9 +573,8 @@ __global__ void k_dg_pack_a(const DgSrc* d) {
 // shared memory, the entries stay in registers meanwhile.
 struct DgPackB {
     const zd* X;
-    int ldx, K;
-    __half* dst;  // [6][npad][kpad]
-    int npad, kpad;
+    int ldx, K, NT, nst;
+    uint32_t* dst;  // tiles of NT rows
     int* ec;
 };
 #define DG_PB_T 256
@@ -576,8 +615,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(DG_PB_T) k_dg_pack_b
     const bool bad = e >= 2048;
     const DgScale sc = dg_scale(bad ? 0 : e);
     auto put = [&](int k, zd w) {
-        dg_put_col((uint32_t*)s.dst, (size_t)s.npad * (s.kpad / 2), s.kpad / 2, n, k, bad ? 0 : dg_int(w.x, sc),
-                   bad ? 0 : dg_int(w.y, sc));
+        dg_put_col(s.dst, s.NT, s.nst, n, k, bad ? 0 : dg_int(w.x, sc), bad ? 0 : dg_int(w.y, sc));
     };
 #pragma unroll
     for (int u = 0; u < DG_PB_E; ++u) {
@@ -615,20 +653,9 @@ struct DgPool {  // device memory of a plan
 };
 static int dg_up(int n, int m) { return (n + m - 1) / m * m; }
 static int dg_nt(int ncol) { return 2 * ncol <= 16 ? 16 : (2 * ncol <= 32 ? 32 : 64); }
-static int dg_kpad(int K) { return dg_up(2 * K, DG_KS); }
+static int dg_nst(int K) { return (2 * K + DG_KS - 1) / DG_KS; }
+static size_t dg_bytes(int rows, int K) { return (size_t)DG_P * rows * dg_nst(K) * 64; }
 
-// digit planes [6][rows][kpad] of fp16, box of 32 reals x box_rows rows x 6 planes
-static bool dg_tmap(CUtensorMap* tm, const void* base, int kpad, int rows, int box_rows) {
-    encode_fn_t enc = get_encode();
-    if (!enc) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)kpad, (cuuint64_t)rows, DG_P};
-    cuuint64_t str[2] = {(cuuint64_t)kpad * 2, (cuuint64_t)kpad * 2 * rows};
-    cuuint32_t box[3] = {DG_KS, (cuuint32_t)box_rows, DG_P};
-    cuuint32_t es[3] = {1, 1, 1};
-    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, str, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 template <int NT>
 static constexpr int dg_smem() {
     return (NT == 16 ? 4 : 3) * DG_P * (DG_A_PL + NT * 64) + 1024;
@@ -684,14 +711,11 @@ static void dg_splits(int tiles, int nst, int* cs, int* gs) {
 
 struct DgLeft {
     DgPool pool;
-    std::vector<CUtensorMap> tm;
-    std::vector<int> M, K, kpad;
-    std::vector<int*> er;
+    std::vector<DgSrc> src;
 };
 struct DgGemm {
     DgPool pool;
     int nk = 0, ncol = 0, NT = 0, ntn = 0, mt = 0, cs = 1, gs = 1;
-    CUtensorMap *tmA = nullptr, *tmB = nullptr;
     DgOut* out = nullptr;
     DgPackB* pb = nullptr;
     i64* part = nullptr;
@@ -712,32 +736,24 @@ void dg_gemm_destroy(DgGemm* g) {
 
 DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s) {
     DgLeft* l = new DgLeft();
-    std::vector<DgSrc> src(nk);
+    l->src.resize(nk);
     int mm = 1, mk = 1;
-    for (int k = 0; k < nk && l->pool.ok; ++k) {
-        const int mp = dg_up(m[k].M, DG_BM), kp = dg_kpad(m[k].K);
-        DgSrc& d = src[k];
+    for (int k = 0; k < nk; ++k) {
+        DgSrc& d = l->src[k];
         d.src = m[k].src;
         d.rs = m[k].rs;
         d.cs = m[k].cs;
         d.conj = m[k].conj;
         d.M = m[k].M;
         d.K = m[k].K;
-        d.mpad = mp;
-        d.kpad = kp;
-        d.dst = (__half*)l->pool.get((size_t)DG_P * mp * kp * sizeof(__half), true);
+        d.nst = dg_nst(m[k].K);
+        const int mp = dg_up(m[k].M, DG_BM);
+        d.dst = (uint32_t*)l->pool.get(dg_bytes(mp, m[k].K), true);
         d.er = (int*)l->pool.get(mp * sizeof(int), true);
-        CUtensorMap t;
-        if (l->pool.ok && !dg_tmap(&t, d.dst, kp, mp, DG_BM)) l->pool.ok = false;
-        l->tm.push_back(t);
-        l->M.push_back(m[k].M);
-        l->K.push_back(m[k].K);
-        l->kpad.push_back(kp);
-        l->er.push_back(d.er);
         mm = std::max(mm, m[k].M);
         mk = std::max(mk, m[k].K);
     }
-    DgSrc* ds = l->pool.ok ? l->pool.up(src) : nullptr;
+    DgSrc* ds = l->pool.ok ? l->pool.up(l->src) : nullptr;
     if (l->pool.ok) {
         k_dg_rowmax<<<dim3((mm + 31) / 32, 1, nk), 256, 0, s>>>(ds);
         k_dg_pack_a<<<dim3((mk + 31) / 32, (mm + 31) / 32, nk), 256, 0, s>>>(ds);
@@ -751,7 +767,7 @@ DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s) {
 }
 
 // device bytes of dg_left_create
-size_t dg_left_bytes(int M, int K) { return (size_t)DG_P * dg_up(M, DG_BM) * dg_kpad(K) * sizeof(__half); }
+size_t dg_left_bytes(int M, int K) { return dg_bytes(dg_up(M, DG_BM), K); }
 
 DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag) {
     DgGemm* g = new DgGemm();
@@ -761,28 +777,29 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
     g->ntn = (2 * ncol + g->NT - 1) / g->NT;
     g->flag = flag;
     const int np = g->ntn * g->NT;
-    std::vector<CUtensorMap> tb(nk);
     std::vector<DgOut> out(nk);
     std::vector<DgPackB> pb(nk);
     int tiles = 0, nst = 1;
-    for (int k = 0; k < nk && g->pool.ok; ++k) {
-        const int kp = dg_kpad(r[k].K);
+    for (int k = 0; k < nk; ++k) {
+        const DgSrc& d = l->src[k];
         pb[k].X = r[k].X;
         pb[k].ldx = r[k].ldx;
         pb[k].K = r[k].K;
-        pb[k].dst = (__half*)g->pool.get((size_t)DG_P * np * kp * sizeof(__half), true);
-        pb[k].npad = np;
-        pb[k].kpad = kp;
+        pb[k].NT = g->NT;
+        pb[k].nst = dg_nst(r[k].K);
+        pb[k].dst = (uint32_t*)g->pool.get(dg_bytes(np, r[k].K), true);
         pb[k].ec = (int*)g->pool.get(ncol * sizeof(int), true);
-        if (g->pool.ok && !dg_tmap(&tb[k], pb[k].dst, kp, np, g->NT)) g->pool.ok = false;
-        out[k].M = l->M[k];
-        out[k].nst = kp / DG_KS;
+        out[k].A = (const unsigned char*)d.dst;
+        out[k].B = (const unsigned char*)pb[k].dst;
+        out[k].M = d.M;
+        out[k].nst = pb[k].nst;
+        out[k].nsta = d.nst;
         out[k].ldc = r[k].ldc;
-        out[k].er = l->er[k];
+        out[k].er = d.er;
         out[k].ec = pb[k].ec;
         out[k].C = r[k].C;
         out[k].tile0 = tiles;
-        const int mt = (l->M[k] + DG_BM - 1) / DG_BM;
+        const int mt = (d.M + DG_BM - 1) / DG_BM;
         g->mt = std::max(g->mt, mt);
         tiles += mt * g->ntn;
         nst = std::max(nst, out[k].nst);
@@ -793,9 +810,6 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
         g->cnt = (unsigned*)g->pool.get((size_t)tiles * g->cs * sizeof(unsigned), true);
     }
     if (g->pool.ok) {
-        std::vector<CUtensorMap> ta(l->tm.begin(), l->tm.begin() + nk);
-        g->tmA = g->pool.up(ta);
-        g->tmB = g->pool.up(tb);
         g->out = g->pool.up(out);
         g->pb = g->pool.up(pb);
     }
@@ -810,8 +824,6 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
 int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s) {
     k_dg_pack_b<<<dim3(8 * g->ncol, 1, nk), DG_PB_T, 0, s>>>(g->pb, kofs);
     DgArgs a{};
-    a.tmA = g->tmA;
-    a.tmB = g->tmB;
     a.out = g->out;
     a.kofs = kofs;
     a.ncol = g->ncol;
@@ -837,15 +849,14 @@ int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s) 
 // of that scale: nothing is rounded between the terms but the digits' cut.
 struct DgSeriesK {
     KDev const* kd;
-    __half* A;       // [6][mpad][kpad]
-    int mpad, kpad;
+    uint32_t* A;     // digits of H~, tiles of 128 rows
+    int nst, NT;
     int* bad;        // per row: HH not finite
     int* ec;
 };
 struct DgSeries {
     DgPool pool;
     int nk = 0, n = 0, ns = 0, NT = 0, ntn = 0, mt = 0, cs = 1, gs = 1;
-    CUtensorMap *tmA = nullptr, *tmB[2] = {nullptr, nullptr};
     DgOut* out = nullptr;
     DgCheb* ch = nullptr;
     DgSeriesK* sk = nullptr;
@@ -897,7 +908,7 @@ __global__ void __launch_bounds__(128) k_dg_hsub(StepArgs a, const DgSeriesK* sk
         dg_cut(dg_int(-v.y, sc), di);
 #pragma unroll
         for (int q = 0; q < DG_P; ++q)
-            ((uint32_t*)S.A)[((size_t)q * S.mpad + i) * (S.kpad / 2) + j] = dg_pair(dr[q], di[q]);
+            S.A[dg_word(i, j, DG_BM, S.nst) + (size_t)q * DG_BM * 16] = dg_pair(dr[q], di[q]);
     }
     bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) S.bad[i] = bad;
@@ -953,7 +964,7 @@ __global__ void __launch_bounds__(128) k_dg_y0(StepArgs a, const DgSeriesK* sk, 
         ch.y0[x + n] = yi;
         ch.acc[x] = dg_mul62(cr, yr) - dg_mul62(ci, yi);
         ch.acc[x + n] = dg_mul62(cr, yi) + dg_mul62(ci, yr);
-        dg_put_col((uint32_t*)ch.Bn[0], ch.pl / 2, ch.kpad / 2, c, i, (yr + 256) >> 9, (yi + 256) >> 9);
+        dg_put_col(ch.Bn[0], S.NT, ch.nst, c, i, (yr + 256) >> 9, (yi + 256) >> 9);
     }
 }
 
@@ -993,15 +1004,14 @@ DgSeries* dg_series_create(int nk, int n, int ns) {
     g->NT = dg_nt(ns);
     g->ntn = (2 * ns + g->NT - 1) / g->NT;
     g->mt = (n + DG_BM - 1) / DG_BM;
-    const int np = g->ntn * g->NT, mp = g->mt * DG_BM, kp = dg_kpad(n);
-    std::vector<CUtensorMap> ta(nk), tb0(nk), tb1(nk);
+    const int np = g->ntn * g->NT, nst = dg_nst(n);
     std::vector<DgOut> out(nk);
     std::vector<DgCheb> ch(nk);
     std::vector<DgSeriesK> sk(nk);
-    for (int k = 0; k < nk && g->pool.ok; ++k) {
-        sk[k].A = (__half*)g->pool.get((size_t)DG_P * mp * kp * sizeof(__half), true);
-        sk[k].mpad = mp;
-        sk[k].kpad = kp;
+    for (int k = 0; k < nk; ++k) {
+        sk[k].A = (uint32_t*)g->pool.get(dg_bytes(g->mt * DG_BM, n), true);
+        sk[k].nst = nst;
+        sk[k].NT = g->NT;
         sk[k].bad = (int*)g->pool.get(n * sizeof(int), true);
         sk[k].ec = (int*)g->pool.get(ns * sizeof(int), true);
         DgCheb& c = ch[k];
@@ -1009,31 +1019,22 @@ DgSeries* dg_series_create(int nk, int n, int ns) {
         c.y0 = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
         c.y1 = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
         c.acc = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
-        for (int q = 0; q < 2; ++q) c.Bn[q] = (__half*)g->pool.get((size_t)DG_P * np * kp * sizeof(__half), true);
-        c.pl = (size_t)np * kp;
-        c.kpad = kp;
+        for (int q = 0; q < 2; ++q) c.Bn[q] = (uint32_t*)g->pool.get(dg_bytes(np, n), true);
+        c.nst = nst;
         c.coef = (i64*)g->pool.get((size_t)2 * RTD_MAX_TERMS * sizeof(i64), true);
+        out[k] = DgOut{};
+        out[k].A = (const unsigned char*)sk[k].A;
         out[k].M = n;
-        out[k].nst = kp / DG_KS;
-        out[k].ldc = 0;
-        out[k].er = nullptr;
-        out[k].ec = nullptr;
-        out[k].C = nullptr;
+        out[k].nst = out[k].nsta = nst;
         out[k].tile0 = k * g->mt * g->ntn;
-        if (g->pool.ok && (!dg_tmap(&ta[k], sk[k].A, kp, mp, DG_BM) || !dg_tmap(&tb0[k], c.Bn[0], kp, np, g->NT) ||
-                           !dg_tmap(&tb1[k], c.Bn[1], kp, np, g->NT)))
-            g->pool.ok = false;
     }
     const int tiles = nk * g->mt * g->ntn;
-    dg_splits(tiles, kp / DG_KS, &g->cs, &g->gs);
+    dg_splits(tiles, nst, &g->cs, &g->gs);
     if (g->gs > 1) {
         g->part = (i64*)g->pool.get((size_t)tiles * g->NT * 2 * DG_BM * sizeof(i64), true);
         g->cnt = (unsigned*)g->pool.get((size_t)tiles * g->cs * sizeof(unsigned), true);
     }
     if (g->pool.ok) {
-        g->tmA = g->pool.up(ta);
-        g->tmB[0] = g->pool.up(tb0);
-        g->tmB[1] = g->pool.up(tb1);
         g->out = g->pool.up(out);
         g->ch = g->pool.up(ch);
         g->sk = g->pool.up(sk);
@@ -1049,7 +1050,6 @@ int launch_dg_series(const DgSeries* g, const StepArgs& a, cudaStream_t s) {
     k_dg_hsub<<<dim3(g->n, 1, g->nk), 128, 0, s>>>(a, g->sk);
     k_dg_y0<<<dim3(g->ns, 1, g->nk), 128, 0, s>>>(a, g->sk, g->ch);
     DgArgs d{};
-    d.tmA = g->tmA;
     d.out = g->out;
     d.ch = g->ch;
     d.ncol = g->ns;
@@ -1060,7 +1060,6 @@ int launch_dg_series(const DgSeries* g, const StepArgs& a, cudaStream_t s) {
     d.cnt = g->cnt;
     d.flag = a.flag;
     for (int t = 1; t < a.nterms; ++t) {
-        d.tmB = g->tmB[(t - 1) & 1];
         d.term = t;
         d.last = t == a.nterms - 1;
         dg_launch<1>(g->NT, g->mt, g->nk, d, s);
