@@ -87,6 +87,11 @@ struct rttddft_ctx {
     // FP64 form: the products with CC and the matching coefficients on the tensor cores
     DgLeft *dgl_cc = nullptr, *dgl_cch = nullptr, *dgl_a = nullptr, *dgl_ah = nullptr;
     DgGemm *dg_expand = nullptr, *dg_fwd = nullptr, *dg_back = nullptr, *dg_proj = nullptr;
+    DgLeft *dgl_mt = nullptr, *dgl_dh = nullptr, *dgl_lh = nullptr;  // muffin-tin stacks, dh, L^H
+    DgGemm *dg_mt = nullptr, *dg_mtd = nullptr, *dg_dvw = nullptr, *dg_dvg = nullptr, *dg_dvi = nullptr;
+    zd* d_mtd = nullptr;
+    int mtd_stride = 0;
+    std::vector<zd*> dv_t, dv_w;                // per k T = dV~ * CC_G and W = dh L of the rebuild
     zd* d_proj = nullptr;                       // CC^H S C of every k-point (one slice)
     DgSeries* series = nullptr;                 // Chebyshev series as digit products (many states)
     FftPlan* fft = nullptr;                     // FFT route of the interstitial convolution
@@ -280,6 +285,9 @@ static StepArgs make_args(rttddft_ctx* ctx, int dv_on) {
     a.mtv = ctx->d_mtv;
     a.mtv_stride = ctx->mtv_stride;
     a.mtw_stride = ctx->mtw_stride;
+    a.mtd = ctx->d_mtd;
+    a.mtd_stride = ctx->mtd_stride;
+    a.mt64 = ctx->dg_mt ? 1 : 0;
     return a;
 }
 
@@ -324,6 +332,12 @@ static StepPlan make_plan(rttddft_ctx* ctx) {
     p.dg_fwd = ctx->dg_fwd;
     p.dg_back = ctx->dg_back;
     p.dg_proj = ctx->dg_proj;
+    p.dg_mt = ctx->dg_mt;
+    p.dg_mtd = ctx->dg_mtd;
+    p.dgl_dh = ctx->dgl_dh;
+    p.dg_dvw = ctx->dg_dvw;
+    p.dg_dvg = ctx->dg_dvg;
+    p.dg_dvi = ctx->dg_dvi;
     p.series = ctx->series;
     p.fft = ctx->fft;
     p.td_op = ctx->td_op;
@@ -598,11 +612,12 @@ static void validate(const rttddft_system* s, const rttddft_options* o) {
 }
 
 static void drop_dg(rttddft_ctx* ctx) {
-    for (DgGemm** g : {&ctx->dg_expand, &ctx->dg_fwd, &ctx->dg_back, &ctx->dg_proj}) {
+    for (DgGemm** g : {&ctx->dg_expand, &ctx->dg_fwd, &ctx->dg_back, &ctx->dg_proj, &ctx->dg_mt, &ctx->dg_mtd, &ctx->dg_dvw,
+                       &ctx->dg_dvg, &ctx->dg_dvi}) {
         dg_gemm_destroy(*g);
         *g = nullptr;
     }
-    for (DgLeft** l : {&ctx->dgl_cc, &ctx->dgl_cch, &ctx->dgl_a, &ctx->dgl_ah}) {
+    for (DgLeft** l : {&ctx->dgl_cc, &ctx->dgl_cch, &ctx->dgl_a, &ctx->dgl_ah, &ctx->dgl_mt, &ctx->dgl_dh, &ctx->dgl_lh}) {
         dg_left_destroy(*l);
         *l = nullptr;
     }
@@ -643,8 +658,101 @@ static bool build_dg(rttddft_ctx* ctx) {
              (ctx->dgl_ah = dg_left_create(nk, ah.data(), ctx->stream)) &&
              (ctx->dg_fwd = dg_gemm_create(ctx->dgl_a, nk, rf.data(), ns, ctx->d_flag)) &&
              (ctx->dg_back = dg_gemm_create(ctx->dgl_ah, nk, rb.data(), 2 * ns, ctx->d_flag));
+    const AtomTab& at = ctx->at;
+    if (ok && at.n > 0 && (long long)nk * at.n <= 65535) {
+        // the muffin-tin stacks [h; o; p_x; p_y; p_z] of every atom, static; their products per (k, atom)
+        zd* stk = dalloc<zd>(ctx, 5 * ctx->nblk);
+        ctx->mtw_stride = 5 * ctx->maxm * ns;
+        ctx->d_mtw = dalloc<zd>(ctx, (size_t)nk * at.n * ctx->mtw_stride);
+        std::vector<DgMat> mm;
+        std::vector<DgRight> rm;
+        for (int al = 0; al < at.n; ++al) {
+            const int m = at.m[al];
+            zd* g = stk + 5 * at.boff[al];
+            const zd* blk[5] = {ctx->d_h + at.boff[al], ctx->d_o + at.boff[al], ctx->d_p + 3 * at.boff[al],
+                                ctx->d_p + 3 * at.boff[al] + (size_t)m * m, ctx->d_p + 3 * at.boff[al] + 2 * (size_t)m * m};
+            for (int q = 0; q < 5; ++q)
+                CK(cudaMemcpy2DAsync(g + (size_t)q * m, (size_t)5 * m * sizeof(zd), blk[q], (size_t)m * sizeof(zd),
+                                     (size_t)m * sizeof(zd), m, cudaMemcpyDeviceToDevice, ctx->stream));
+            mm.push_back(DgMat{g, 1, (size_t)5 * m, 0, 5 * m, m});
+        }
+        for (int k = 0; k < nk; ++k)
+            for (int al = 0; al < at.n; ++al) {
+                KDev& K = ctx->hkd[k];
+                DgRight r{K.Q + at.aoff[al], ma, at.m[al], ctx->d_mtw + ((size_t)k * at.n + al) * ctx->mtw_stride, 5 * at.m[al]};
+                r.X2 = K.C + K.ng + at.looff[al];
+                r.ldx2 = K.nb;
+                r.K1 = at.na[al];
+                rm.push_back(r);
+            }
+        ok = (ctx->dgl_mt = dg_left_create(at.n, mm.data(), ctx->stream)) &&
+             (ctx->dg_mt = dg_gemm_create(ctx->dgl_mt, nk * at.n, rm.data(), ns, ctx->d_flag, at.n));
+        CK(cudaStreamSynchronize(ctx->stream));
+        dfree(ctx, stk);
+    }
     if (!ok) drop_dg(ctx);
     return ok;
+}
+
+// The potential-change rebuild (dh L, L^H W, CC_G^H T) as digit products, in
+// every form, and dh times [Q; C_lo] in the FP64 form.  Needs dv_t, dv_w, d_dh
+// and K.dvsub; nothing is built where the memory does not suffice.
+static void build_dv_dg(rttddft_ctx* ctx) {
+    const int nk = ctx->nk, ns = ctx->ns, naux = ctx->naux;
+    const AtomTab& at = ctx->at;
+    if ((long long)nk * std::max(at.n, 1) > 65535) return;
+    size_t need = 0, fr = 0, tot = 0;
+    for (int k = 0; k < nk; ++k)
+        need += dg_left_bytes(naux, ctx->nb[k]) + dg_left_bytes(2 * naux, ctx->ng[k]) + 3 * dg_left_bytes(2 * naux, at.lrows + 1);
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || need > fr / 2) return;
+    bool ok = true;
+    if (!ctx->dgl_cch) {
+        std::vector<DgMat> cch(nk);
+        for (int k = 0; k < nk; ++k)
+            cch[k] = DgMat{ctx->hkd[k].caux, (size_t)ctx->nb[k], 1, 1, naux, ctx->nb[k]};
+        ok = (ctx->dgl_cch = dg_left_create(nk, cch.data(), ctx->stream));
+    }
+    std::vector<DgRight> ri(nk);
+    for (int k = 0; k < nk; ++k) ri[k] = DgRight{ctx->dv_t[k], ctx->ng[k], ctx->ng[k], ctx->hkd[k].dvsub, naux};
+    DgGemm *gi = nullptr, *gw = nullptr, *gg = nullptr, *gd = nullptr;
+    if (ok && ctx->d_dh && at.n > 0) {
+        std::vector<DgMat> dh, lh(nk);
+        std::vector<DgRight> rw, rg(nk), rd;
+        ctx->mtd_stride = ctx->maxm * ns;
+        if (ctx->dg_mt) ctx->d_mtd = dalloc<zd>(ctx, (size_t)nk * at.n * ctx->mtd_stride);
+        for (int al = 0; al < at.n; ++al)
+            dh.push_back(DgMat{ctx->d_dh + at.boff[al], 1, (size_t)at.m[al], 0, at.m[al], at.m[al]});
+        for (int k = 0; k < nk; ++k) {
+            KDev& K = ctx->hkd[k];
+            for (int al = 0; al < at.n; ++al) {
+                rw.push_back(DgRight{K.lloc + at.loff[al], at.lrows, at.m[al], ctx->dv_w[k] + at.loff[al], at.lrows});
+                DgRight r{K.Q + at.aoff[al], at.ma, at.m[al], ctx->d_mtd + ((size_t)k * at.n + al) * ctx->mtd_stride, at.m[al]};
+                r.X2 = K.C + K.ng + at.looff[al];
+                r.ldx2 = K.nb;
+                r.K1 = at.na[al];
+                rd.push_back(r);
+            }
+            lh[k] = DgMat{K.lloc, (size_t)at.lrows, 1, 1, naux, at.lrows};
+            rg[k] = DgRight{ctx->dv_w[k], at.lrows, at.lrows, K.dvsub, naux};
+            rg[k].scale = &ctx->d_st->cur_s;
+        }
+        ok = (ctx->dgl_dh = dg_left_create(at.n, dh.data(), ctx->stream)) &&
+             (ctx->dgl_lh = dg_left_create(nk, lh.data(), ctx->stream)) &&
+             (gw = dg_gemm_create(ctx->dgl_dh, nk * at.n, rw.data(), naux, ctx->d_flag, at.n)) &&
+             (gg = dg_gemm_create(ctx->dgl_lh, nk, rg.data(), naux, ctx->d_flag)) &&
+             (!ctx->dg_mt || (gd = dg_gemm_create(ctx->dgl_dh, nk * at.n, rd.data(), ns, ctx->d_flag, at.n)));
+    }
+    ok = ok && (gi = dg_gemm_create(ctx->dgl_cch, nk, ri.data(), naux, ctx->d_flag));
+    if (ok) {
+        ctx->dg_dvi = gi;
+        ctx->dg_dvw = gw;
+        ctx->dg_dvg = gg;
+        ctx->dg_mtd = gd;
+        if (gw) launch_dg_gemm(gw, 0, nk * at.n, 0, ctx->stream);  // L's digits stay
+        CK(cudaStreamSynchronize(ctx->stream));
+        return;
+    }
+    for (DgGemm* g : {gi, gw, gg, gd}) dg_gemm_destroy(g);
 }
 
 // ------------------------------------------------------------ ABI
@@ -1383,6 +1491,7 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
                 KDev& K = ctx->hkd[k];
                 K.dvsub = dalloc<zd>(ctx, (size_t)naux * naux);
                 zd* T = dalloc<zd>(ctx, (size_t)K.ng * naux);
+                ctx->dv_t.push_back(T);
                 td.push_back(ToepDesc{K.caux, T, K.nb, K.ng});
                 GemmDesc d{};
                 d.A = K.caux;
@@ -1460,6 +1569,7 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
                 }
                 ctx->gd_mty = upload_descs(ctx, gy);
             }
+            build_dv_dg(ctx);
             CK(cudaMemcpy(ctx->d_kd, ctx->hkd.data(), nk * sizeof(KDev), cudaMemcpyHostToDevice));
             for (int k = 0; k < nk; ++k) ctx->dvnorm[k] = o->hartree_bound;
             ctx->dv_set = true;
@@ -1852,6 +1962,7 @@ static void build_mt_rebuild(rttddft_ctx* ctx) {
     for (int k = 0; k < nk; ++k) {
         KDev& K = ctx->hkd[k];
         zd* W = dalloc<zd>(ctx, (size_t)std::max(at.lrows, 1) * naux);
+        ctx->dv_w.push_back(W);
         for (int a = 0; a < at.n; ++a) {
             GemmDesc d{};
             d.A = ctx->d_dh + at.boff[a];
@@ -1929,6 +2040,7 @@ int rttddft_set_dv(rttddft_ctx* ctx, const double* dh, const double* dvtab) {
                 KDev& K = ctx->hkd[k];
                 K.dvsub = dalloc<zd>(ctx, (size_t)naux * naux);
                 zd* T = dalloc<zd>(ctx, (size_t)K.ng * naux);
+                ctx->dv_t.push_back(T);
                 td.push_back(ToepDesc{K.caux, T, K.nb, K.ng});
                 GemmDesc d{};
                 d.A = K.caux;
@@ -1976,6 +2088,8 @@ int rttddft_set_dv(rttddft_ctx* ctx, const double* dh, const double* dvtab) {
         }
         if (at.n > 0) CK(cudaMemcpy(ctx->d_dh, dh, nblk * sizeof(zd), cudaMemcpyHostToDevice));
         if (ctx->d_dh32) launch_convert_f32(ctx->d_dh, ctx->d_dh32, nblk, ctx->stream);
+        if (!ctx->dv_set) build_dv_dg(ctx);
+        else if (ctx->dgl_dh) launch_dg_left(ctx->dgl_dh, ctx->stream);
         CK(cudaMemcpy(ctx->d_dvtab, dvtab, ctx->nvt * sizeof(zd), cudaMemcpyHostToDevice));
         if (ctx->tc && !ctx->fft) {
             double vmax = 0.0;
@@ -2478,7 +2592,7 @@ extern "C" int rttddft_apply_noalloc(rttddft_ctx* ctx, int k, int ncols, const d
         p.side = nullptr;
         p.tile_cnt = nullptr;  // the context's counters may be in use on another stream
         p.gd_mt1 = nullptr;
-        p.dg_fwd = p.dg_back = nullptr;  // their digit buffers belong to the context
+        p.dg_fwd = p.dg_back = p.dg_mt = p.dg_mtd = nullptr;  // their digit buffers belong to the context
         p.gd_fwd = (const GemmDesc*)(base + o_gd);
         p.maxng = ng;
         p.part = (zd*)(base + o_part);

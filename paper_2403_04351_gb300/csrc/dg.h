@@ -19,15 +19,19 @@ struct DgRight {
     int ldx, K;   // K at most the left operand's
     zd* C;
     int ldc;
+    const zd* X2 = nullptr;          // rows K1 .. K - 1 of X from here, or null
+    int ldx2 = 0, K1 = 0;
+    const double* scale = nullptr;   // device factor on the product, or null
 };
 
 DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s);
+int launch_dg_left(const DgLeft* l, cudaStream_t s);  // cut the operand anew; returns its launches
 void dg_left_destroy(DgLeft* l);
 size_t dg_left_bytes(int M, int K);
-// null where the device memory does not suffice
-DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag);
+// null where the device memory does not suffice; lmod > 0: entry k takes the left operand k % lmod
+DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag, int lmod = 0);
 void dg_gemm_destroy(DgGemm* g);
-int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s);  // returns its launches
+int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s, bool packed = false);  // returns its launches
 
 struct StepArgs;
 DgSeries* dg_series_create(int nk, int n, int ns);

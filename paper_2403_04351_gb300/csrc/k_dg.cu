@@ -140,6 +140,7 @@ struct DgOut {
     const int* er;      // row exponents of A
     const int* ec;      // column exponents of X
     zd* C;
+    const double* scale;  // factor on the product, or null
     int tile0;          // first tile in the split buffers
 };
 struct DgCheb {
@@ -462,6 +463,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
                     v.x = dg_double(hv[0], lv[0], er + ec - 70);
                     v.y = dg_double(hv[1], lv[1], er + ec - 70);
                 }
+                if (o.scale) v = zscale(v, *o.scale);
                 zd* p = o.C + row + (size_t)n * o.ldc;
                 if (g.beta) v = zadd(*p, v);
                 *p = v;
@@ -572,8 +574,8 @@ __global__ void k_dg_pack_a(const DgSrc* d) {
 // blocks shares a column: the largest entry goes around through distributed
 // shared memory, the entries stay in registers meanwhile.
 struct DgPackB {
-    const zd* X;
-    int ldx, K, NT, nst;
+    const zd *X, *X2;  // rows 0 .. K1 - 1 from X, the others from X2
+    int ldx, ldx2, K1, K, NT, nst;
     uint32_t* dst;  // tiles of NT rows
     int* ec;
 };
@@ -587,16 +589,18 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(DG_PB_T) k_dg_pack_b
     const int rank = blockIdx.x & 7, n = blockIdx.x >> 3;
     const int tid = threadIdx.x;
     const zd* __restrict__ x = s.X + (size_t)n * s.ldx;
+    const zd* __restrict__ x2 = s.X2 + (size_t)n * s.ldx2 - s.K1;
+    auto get = [&](int k) { return k < s.K1 ? x[k] : x2[k]; };
     zd v[DG_PB_E];
     int mx = 0;
 #pragma unroll
     for (int u = 0; u < DG_PB_E; ++u) {
         const int k = (u * 8 + rank) * DG_PB_T + tid;
-        v[u] = k < s.K ? x[k] : zmk(0.0, 0.0);
+        v[u] = k < s.K ? get(k) : zmk(0.0, 0.0);
         mx = max(mx, max(dg_hw(v[u].x), dg_hw(v[u].y)));
     }
     for (int k = (DG_PB_E * 8 + rank) * DG_PB_T + tid; k < s.K; k += 8 * DG_PB_T) {
-        const zd w = x[k];
+        const zd w = get(k);
         mx = max(mx, max(dg_hw(w.x), dg_hw(w.y)));
     }
     for (int w = 16; w > 0; w >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, w));
@@ -622,7 +626,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(DG_PB_T) k_dg_pack_b
         const int k = (u * 8 + rank) * DG_PB_T + tid;
         if (k < s.K) put(k, v[u]);
     }
-    for (int k = (DG_PB_E * 8 + rank) * DG_PB_T + tid; k < s.K; k += 8 * DG_PB_T) put(k, x[k]);
+    for (int k = (DG_PB_E * 8 + rank) * DG_PB_T + tid; k < s.K; k += 8 * DG_PB_T) put(k, get(k));
 }
 
 // ------------------------------------------------------------ host side
@@ -712,6 +716,8 @@ static void dg_splits(int tiles, int nst, int* cs, int* gs) {
 struct DgLeft {
     DgPool pool;
     std::vector<DgSrc> src;
+    DgSrc* d_src = nullptr;
+    int mm = 1, mk = 1;
 };
 struct DgGemm {
     DgPool pool;
@@ -734,10 +740,17 @@ void dg_gemm_destroy(DgGemm* g) {
     delete g;
 }
 
+// cut the source's present values
+int launch_dg_left(const DgLeft* l, cudaStream_t s) {
+    const int nk = (int)l->src.size();
+    k_dg_rowmax<<<dim3((l->mm + 31) / 32, 1, nk), 256, 0, s>>>(l->d_src);
+    k_dg_pack_a<<<dim3((l->mk + 31) / 32, (l->mm + 31) / 32, nk), 256, 0, s>>>(l->d_src);
+    return 2;
+}
+
 DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s) {
     DgLeft* l = new DgLeft();
     l->src.resize(nk);
-    int mm = 1, mk = 1;
     for (int k = 0; k < nk; ++k) {
         DgSrc& d = l->src[k];
         d.src = m[k].src;
@@ -750,13 +763,12 @@ DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s) {
         const int mp = dg_up(m[k].M, DG_BM);
         d.dst = (uint32_t*)l->pool.get(dg_bytes(mp, m[k].K), true);
         d.er = (int*)l->pool.get(mp * sizeof(int), true);
-        mm = std::max(mm, m[k].M);
-        mk = std::max(mk, m[k].K);
+        l->mm = std::max(l->mm, m[k].M);
+        l->mk = std::max(l->mk, m[k].K);
     }
-    DgSrc* ds = l->pool.ok ? l->pool.up(l->src) : nullptr;
+    if (l->pool.ok) l->d_src = l->pool.up(l->src);
     if (l->pool.ok) {
-        k_dg_rowmax<<<dim3((mm + 31) / 32, 1, nk), 256, 0, s>>>(ds);
-        k_dg_pack_a<<<dim3((mk + 31) / 32, (mm + 31) / 32, nk), 256, 0, s>>>(ds);
+        launch_dg_left(l, s);
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) l->pool.ok = false;
     }
     if (!l->pool.ok) {
@@ -769,7 +781,7 @@ DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s) {
 // device bytes of dg_left_create
 size_t dg_left_bytes(int M, int K) { return dg_bytes(dg_up(M, DG_BM), K); }
 
-DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag) {
+DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag, int lmod) {
     DgGemm* g = new DgGemm();
     g->nk = nk;
     g->ncol = ncol;
@@ -781,9 +793,12 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
     std::vector<DgPackB> pb(nk);
     int tiles = 0, nst = 1;
     for (int k = 0; k < nk; ++k) {
-        const DgSrc& d = l->src[k];
+        const DgSrc& d = l->src[lmod > 0 ? k % lmod : k];
         pb[k].X = r[k].X;
         pb[k].ldx = r[k].ldx;
+        pb[k].X2 = r[k].X2 ? r[k].X2 : r[k].X;
+        pb[k].ldx2 = r[k].X2 ? r[k].ldx2 : r[k].ldx;
+        pb[k].K1 = r[k].X2 ? r[k].K1 : r[k].K;
         pb[k].K = r[k].K;
         pb[k].NT = g->NT;
         pb[k].nst = dg_nst(r[k].K);
@@ -798,6 +813,7 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
         out[k].er = d.er;
         out[k].ec = pb[k].ec;
         out[k].C = r[k].C;
+        out[k].scale = r[k].scale;
         out[k].tile0 = tiles;
         const int mt = (d.M + DG_BM - 1) / DG_BM;
         g->mt = std::max(g->mt, mt);
@@ -820,9 +836,9 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
     return g;
 }
 
-// C (+)= A X for entries kofs .. kofs + nk - 1
-int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s) {
-    k_dg_pack_b<<<dim3(8 * g->ncol, 1, nk), DG_PB_T, 0, s>>>(g->pb, kofs);
+// C (+)= A X for entries kofs .. kofs + nk - 1; packed: X's digits are those of the last call
+int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s, bool packed) {
+    if (!packed) k_dg_pack_b<<<dim3(8 * g->ncol, 1, nk), DG_PB_T, 0, s>>>(g->pb, kofs);
     DgArgs a{};
     a.out = g->out;
     a.kofs = kofs;
@@ -835,7 +851,7 @@ int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s) 
     a.cnt = g->cnt;
     a.flag = g->flag;
     dg_launch<0>(g->NT, g->mt, nk, a, s);
-    return 2;
+    return packed ? 1 : 2;
 }
 
 // ------------------------------------------------------------ Chebyshev series

@@ -686,59 +686,93 @@ __global__ void k_mt_gather(StepArgs a) {
     }
 }
 
-__global__ void __launch_bounds__(128) k_mt_epi(StepArgs a) {
+// 32 rows x 8 column groups per block: the FP64 chain of a row's shares is
+// N_s / 8 columns long (one thread per row: 26 us at N_s 60 whatever the number of rows)
+__global__ void __launch_bounds__(256) k_mt_epi(StepArgs a) {
+    __shared__ double red[8][32][5];
     const int k = blockIdx.z, al = blockIdx.y;
     const AtomTab& at = *a.at;
     if (al >= at.n) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, cg = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
     const int m = at.m[al], na = at.na[al];
-    if (i >= m) return;
+    if (blockIdx.x * 32 >= m) return;
     const KDev& K = a.kd[k];
     const int ns = a.ns, nb = K.nb, ma = at.ma, ng = K.ng;
     const int aoff = at.aoff[al], lo0 = ng + at.looff[al];
     const size_t ent = (size_t)(a.kofs + k) * at.n + al;  // kofs: single-k operator calls
     const zd* W = a.mtw + ent * a.mtw_stride;
-    const zd* V = a.mtv + ent * a.mtv_stride;
     const size_t ld = (size_t)5 * m;
+    const DevState* st = a.st;
+    const double cx = st->cur_a[0] * a.inv_c, cy = st->cur_a[1] * a.inv_c, cz = st->cur_a[2] * a.inv_c;
+    const double aa = st->cur_aa, sdv = st->cur_s;
+    const bool dvm = a.mt64 && a.dh && sdv != 0.0;
+    const zd* D = dvm ? a.mtd + ent * a.mtd_stride : nullptr;
     double jc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int c = 0; c < ns; ++c) {
-        const zd* w = W + (size_t)c * ld;
-        const zd zh = w[i], zs = w[m + i];
-        const zd x = V[i + (size_t)c * m];
-        const double f = a.occ[c];
-        if (i < na) {
-            K.Z[aoff + i + (size_t)c * ma] = zh;
-            K.Z[aoff + i + (size_t)(ns + c) * ma] = zs;
-        } else {
-            const int r = lo0 + (i - na);
-            K.Y[r + (size_t)c * nb] = zh;
-            K.Y[r + (size_t)(ns + c) * nb] = zs;
-            jc[3] += f * (x.x * zh.x + x.y * zh.y);
-            jc[4] += f * (x.x * zs.x + x.y * zs.y);
-        }
-#pragma unroll
-        for (int l = 0; l < 3; ++l) {
-            const zd pv = w[(2 + l) * m + i];
-            jc[l] += f * (x.x * pv.x + x.y * pv.y);
+    if (i < m) {
+        for (int c = cg; c < ns; c += 8) {
+            const zd* w = W + (size_t)c * ld;
+            zd zh = w[i];
+            const zd zs = w[m + i], px = w[2 * m + i], py = w[3 * m + i], pz = w[4 * m + i];
+            if (a.mt64) {
+                zh = zadd(zh, zadd(zadd(zscale(px, cx), zscale(py, cy)), zadd(zscale(pz, cz), zscale(zs, aa))));
+                if (dvm) zh = zadd(zh, zscale(D[i + (size_t)c * m], sdv));
+            }
+            const double f = a.occ[c];
+            zd x;
+            if (i < na) {
+                x = K.Q[aoff + i + (size_t)c * ma];
+                K.Z[aoff + i + (size_t)c * ma] = zh;
+                K.Z[aoff + i + (size_t)(ns + c) * ma] = zs;
+                x = zscale(x, f);
+            } else {
+                const int r = lo0 + (i - na);
+                x = zscale(K.C[r + (size_t)c * nb], f);
+                K.Y[r + (size_t)c * nb] = zh;
+                K.Y[r + (size_t)(ns + c) * nb] = zs;
+                jc[3] += x.x * zh.x + x.y * zh.y;
+                jc[4] += x.x * zs.x + x.y * zs.y;
+            }
+            jc[0] += x.x * px.x + x.y * px.y;
+            jc[1] += x.x * py.x + x.y * py.y;
+            jc[2] += x.x * pz.x + x.y * pz.y;
         }
     }
-    double* pj = a.part_jmt + ((size_t)k * at.lrows + at.loff[al] + i) * 5;
 #pragma unroll
-    for (int q = 0; q < 5; ++q) pj[q] = jc[q];
+    for (int q = 0; q < 5; ++q) red[cg][lane][q] = jc[q];
+    __syncthreads();
+    if (threadIdx.x < 160) {
+        const int r = threadIdx.x / 5, q = threadIdx.x % 5;
+        if (blockIdx.x * 32 + r < m) {
+            double t = red[0][r][q];
+            for (int g = 1; g < 8; ++g) t += red[g][r][q];
+            a.part_jmt[((size_t)k * at.lrows + at.loff[al] + blockIdx.x * 32 + r) * 5 + q] = t;
+        }
+    }
 }
 
+// the FP64 form's muffin-tin products as digit products (dh among them when the change is on)
+static bool mt_digits(const StepArgs& a, const StepPlan& p) { return p.dg_mt && (!a.dh || p.dg_mtd); }
 static int launch_mt_gemm(const StepArgs& a, const StepPlan& p, cudaStream_t s) {
+    if (mt_digits(a, p)) {
+        // FP64 form: [h; o; p_x; p_y; p_z] (and dh) times [Q; C_lo] as digit products; h_eff X
+        // is their combination
+        int nl = launch_dg_gemm(p.dg_mt, a.kofs * a.at_n, a.nk * a.at_n, 0, s) + 1;
+        if (a.dh) nl += launch_dg_gemm(p.dg_mtd, a.kofs * a.at_n, a.nk * a.at_n, 0, s);
+        k_mt_epi<<<dim3((a.at_maxm + 31) / 32, a.at_n, a.nk), 256, 0, s>>>(a);
+        return nl;
+    }
     if (p.tcmt) {
         // split-BF16 form: the stacks formed in FP64 and the products on the tensor cores
         k_mt_gather<<<dim3((a.at_maxm * a.ns + 255) / 256, a.at_n, a.nk), 256, 0, s>>>(a);
         const int nl = launch_tc_mt(p.tcmt, a, s);
-        k_mt_epi<<<dim3((a.at_maxm + 127) / 128, a.at_n, a.nk), 128, 0, s>>>(a);
+        k_mt_epi<<<dim3((a.at_maxm + 31) / 32, a.at_n, a.nk), 256, 0, s>>>(a);
         return nl + 2;
     }
     k_mt_form<<<dim3(64, a.at_n), 256, 0, s>>>(a);
     k_mt_gather<<<dim3((a.at_maxm * a.ns + 255) / 256, a.at_n, a.nk), 256, 0, s>>>(a);
     launch_gemm_nn(p.gd_mt1, a.nk * a.at_n, 5 * a.at_maxm, a.at_maxm, a.ns, 0, nullptr, 0, true, nullptr, s);
-    k_mt_epi<<<dim3((a.at_maxm + 127) / 128, a.at_n, a.nk), 128, 0, s>>>(a);
+    k_mt_epi<<<dim3((a.at_maxm + 31) / 32, a.at_n, a.nk), 256, 0, s>>>(a);
     return 4;
 }
 
@@ -1859,7 +1893,7 @@ int launch_operator_pass(const StepArgs& a, const StepPlan& p, cudaStream_t s, T
             }
         }
     }
-    if (a.lrows > 0 && f32 && p.gd_mt1 && a.mtg) {
+    if (a.lrows > 0 && ((f32 && p.gd_mt1 && a.mtg) || mt_digits(a, p))) {
         nl += launch_mt_gemm(a, p, s);
         mark(tr, "local_mt", s);
     } else if (a.lrows > 0) {
@@ -1901,10 +1935,36 @@ int launch_operator_pass(const StepArgs& a, const StepPlan& p, cudaStream_t s, T
 }
 
 // Eq. v_MT and Eq. v_interstitial rebuilt from the scaled blocks:
-// dVV = L^H (s dh) L + CC_G^H (s dV~ * CC_G).  In the tensor-core forms the
-// interstitial convolution runs on tcgen05 (split-BF16) and its projection in
-// FP32; otherwise both in FP64.  Returns the launches.
+// dVV = L^H (s dh) L + CC_G^H (s dV~ * CC_G), as digit products where the context
+// holds the digits.  Without them: in the tensor-core forms the interstitial
+// convolution runs on tcgen05 (split-BF16) and its projection in FP32; otherwise
+// both in FP64.  Returns the launches.
 static int launch_dv_rebuild(const StepArgs& a, const StepPlan& p, cudaStream_t s, TraceHook* tr) {
+    if (p.dg_dvi) {
+        // digit products in every form; T by FFT, by the direct sum or on tcgen05 as the form has it
+        int nl = 0, beta = 0;
+        if (p.dg_dvw && (!a.hartree || a.mt_u != 0.0)) {
+            if (a.hartree) nl += launch_dg_left(p.dgl_dh, s);  // the step's dh
+            nl += launch_dg_gemm(p.dg_dvw, 0, a.nk * a.at_n, 0, s, true);  // L is fixed: its digits are
+            nl += launch_dg_gemm(p.dg_dvg, 0, a.nk, 0, s);
+            mark(tr, "dv_mt_blocks", s);
+            beta = 1;
+        }
+        if (p.fft) {
+            const int l = launch_fft_conv(p.fft, p.td_dv, a.kofs, a.nk, a.naux, 1, 1, &a.st->cur_s, s);
+            if (!a.hartree) nl += l;  // counted by the caller
+        } else if (a.prec >= 2 && p.tc && tc_dv_ready(p.tc)) {
+            launch_tc_dv_toeplitz(p.tc, a, p.td_dv, s);
+            nl += 2 * tc_dv_tiles(p.tc);
+        } else {
+            launch_toeplitz(a.kd, p.td_dv, a.nk, p.maxng, a.naux, a.dvtab, a.vt_center, 0, 0, &a.st->cur_s, s);
+            ++nl;
+        }
+        mark(tr, "dv_interstitial", s);
+        nl += launch_dg_gemm(p.dg_dvi, 0, a.nk, beta, s);
+        mark(tr, "dv_interstitial_project", s);
+        return nl;
+    }
     if (a.hartree) {
         // dVV = [sum_a L^H dh_a L] + CC_G^H (dV~ * CC_G) with dV~ (and dh, when the
         // muffin-tin part is on) from the previous step's density

@@ -161,6 +161,8 @@ struct StepArgs {
     zd* mtw;                  //   per (k, atom) its product with [Q; C_lo] (5m x N_s, stride mtw_stride)
     zd* mtv;                  //   per (k, atom) the gathered [Q; C_lo] (m x N_s, stride mtv_stride)
     int mtw_stride, mtv_stride;
+    zd* mtd;                  //   FP64 form: its product with dh (m x N_s, stride mtd_stride)
+    int mtd_stride, mt64;     //   mt64: mtw holds [h; o; p] [Q; C_lo], h_eff is combined by k_mt_epi
 };
 #define ZT_MIN_N 16           // columns from which the FP32 contractions take the 64 x 64 tiled kernel
 #define JRHO_MIN_NS 8         // above this many states the subspace current goes through rho = theta F theta^H
@@ -211,6 +213,9 @@ struct StepPlan {
     const struct TcCC* tcc;   // tensor-core expansion and projection (split forms, many states) or null
     const struct TcMT* tcmt;  // tensor-core muffin-tin blocks (split-BF16 form, many states) or null
     const struct DgGemm *dg_expand, *dg_fwd, *dg_back, *dg_proj;  // FP64 products on the tensor cores, or null
+    const struct DgGemm *dg_mt, *dg_mtd;        // FP64 muffin-tin stacks, and dh, times [Q; C_lo]
+    const struct DgLeft* dgl_dh;                // dh of every atom
+    const struct DgGemm *dg_dvw, *dg_dvg, *dg_dvi;  // potential change: dh L, L^H W, CC_G^H T (all forms)
     const struct DgSeries* series;  // Chebyshev series as digit products (many states) or null
     const struct FftPlan* fft;  // FFT route of the interstitial convolution or null
     unsigned* tile_cnt;         // zeroed row-tile counters of the fused split-K sums (or null)

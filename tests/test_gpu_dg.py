@@ -82,3 +82,29 @@ def test_operator_and_projection(n_g, n_s, n_atoms, route):
     assert abs(o["energy"][0] - e) < 1e-12 * max(1.0, abs(e))
     assert o["resid"][0] < 1e-12 and o["norm_dev"][0] < 1e-12
     ctx.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-11), ("fp32", 1e-5)])
+@pytest.mark.parametrize("n_aux,n_s,n_atoms,n_k", [(12, 1, 1, 1), (65, 17, 2, 2), (130, 33, 3, 1)])
+def test_rebuilt_potential_change(prec, tol, n_aux, n_s, n_atoms, n_k):
+    """dVV rebuilt over four steps, with the pattern replaced after two, against
+    the explicit matrices (the FP32 form's T carries FP32 accuracy)."""
+    from oracle import Oracle
+    from synth import dv_scale_samples, make_dv, pulse_samples
+    s = make_system(tiny_config(n_g=200, n_atoms=n_atoms, lmax=2, n_lo_per_atom=3, n_s=n_s, n_aux=n_aux, n_k=n_k,
+                                kgrid=(n_k, 1, 1)))
+    a, sc = pulse_samples(s, n_steps=4, a0=5.0), dv_scale_samples(4, s["dt"], freq=3.0)
+    pats = make_dv(s, amp=0.3), make_dv(s, amp=0.2, seed_offset=3)
+    ctx = Context(s, precision=prec, graph_steps=2)
+    th = None
+    for i, dv in enumerate(pats):
+        r = Oracle(s, dv=dv).run(a[2 * i:2 * i + 2], s["dt"], dv_scale=sc[2 * i:2 * i + 2], thetas=th)
+        th = r["theta"]
+        ctx.set_dv(dv)
+        ctx.step(a[2 * i:2 * i + 2], sc[2 * i:2 * i + 2])
+    o = ctx.observables()
+    for k in range(n_k):
+        d = ctx.get_state(k) - th[k]
+        assert np.linalg.norm(d) / np.linalg.norm(th[k]) < tol
+    assert np.max(np.abs(o["energy"][2:] - r["E"]) / np.abs(r["E"])) < tol
+    ctx.close()
