@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cmath>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -155,34 +156,53 @@ __global__ void __launch_bounds__(128, 1)
 }
 
 // ------------------------------------------------------------ operand packing
+// hi and lo of v from v rounded once to FP32 (the two keep 16 of its 24 bits):
+// the same split in FP64 arithmetic ran on the 1/64-rate pipe, 40 us of a
+// 9917 x 300 operand
 __device__ __forceinline__ void split_bf16(double v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
-    hi = __double2bfloat16(v);
-    lo = __double2bfloat16(v - (double)__bfloat162float(hi));
+    const float w = (float)v;
+    hi = __float2bfloat16_rn(w);
+    lo = __float2bfloat16_rn(w - __bfloat162float(hi));
 }
 
 // A^ rows r < R (K-major, Kp columns): [Re v | Im v | 0 pad], v = A[r, k]
-// (mode 0) or conj(A[k, r]) (mode 1), A complex column-major with ld.
-__global__ void k_tc_pack_a(const zd* __restrict__ A, int ld, int R, int K, int Kp, int mode,
-                            __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
-    const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (e >= (size_t)R * Kp) return;
-    const int r = (int)(e / Kp), kp = (int)(e % Kp);
-    double v = 0.0;
-    if (kp < 2 * K) {
-        const int k = kp < K ? kp : kp - K;
-        const zd a = (mode == 0) ? A[r + (size_t)k * ld] : zconj(A[k + (size_t)r * ld]);
-        v = (kp < K) ? a.x : a.y;
+// (mode 0) or conj(A[k, r]) (mode 1), A complex column-major with ld.  A block
+// turns a 32 x 32 tile through shared memory, so that it is read along A's
+// columns and written along K (read along K, a 9917 x 300 operand took 32 bytes
+// of memory traffic per entry and pass).
+__global__ void __launch_bounds__(256) k_tc_pack_a(const zd* __restrict__ A, int ld, int R, int K, int Kp, int mode,
+                                                   __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+    __shared__ zd t[32][33];
+    const int k0 = blockIdx.y * 32, r0 = blockIdx.x * 32;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    for (int q = y; q < 32; q += 8) {
+        const int r = mode == 0 ? r0 + x : r0 + q, k = mode == 0 ? k0 + q : k0 + x;
+        zd v = zmk(0.0, 0.0);
+        if (r < R && k < K) v = mode == 0 ? A[r + (size_t)k * ld] : zconj(A[k + (size_t)r * ld]);
+        if (mode == 0) t[x][q] = v;
+        else t[q][x] = v;
     }
-    split_bf16(v, hi[e], lo[e]);
+    __syncthreads();
+    for (int q = y; q < 32; q += 8) {
+        const int r = r0 + q, k = k0 + x;
+        if (r >= R) continue;
+        const size_t row = (size_t)r * Kp;
+        if (k < K) {
+            split_bf16(t[q][x].x, hi[row + k], lo[row + k]);
+            split_bf16(t[q][x].y, hi[row + K + k], lo[row + K + k]);
+        }
+        if (blockIdx.y == 0)
+            for (int kp = 2 * K + x; kp < Kp; kp += 32) hi[row + kp] = lo[row + kp] = __float2bfloat16_rn(0.f);
+    }
 }
 
 // B^ rows n' < Rp (K-major, Kp columns) from X (K x N complex, column-major):
 // n' < N: [Re X_n | -Im X_n], N <= n' < 2N: [Im X_n | Re X_n], else 0.
 __global__ void k_tc_pack_b(const zd* __restrict__ X, int ldx, int K, int N, int Kp, int Rp,
                             __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
-    const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (e >= (size_t)Rp * Kp) return;
-    const int r = (int)(e / Kp), kp = (int)(e % Kp);
+    const int kp = blockIdx.y * 256 + threadIdx.x, r = blockIdx.x;
+    if (kp >= Kp) return;
+    const size_t e = (size_t)r * Kp + kp;
     double v = 0.0;
     if (r < 2 * N && kp < 2 * K) {
         const int n = r < N ? r : r - N;
@@ -194,20 +214,31 @@ __global__ void k_tc_pack_b(const zd* __restrict__ X, int ldx, int K, int N, int
     split_bf16(v, hi[e], lo[e]);
 }
 
-// C[m, n] (+)= sum_s D[s][m][n] + i D[s][m][N + n]  (FP64 sums)
-__global__ void k_tc_combine(const float* __restrict__ D, int splits, int M, int Nc, int Dn, zd* __restrict__ C,
-                             int ldc, int beta_add) {
-    const int e = blockIdx.x * 256 + threadIdx.x;
-    if (e >= M * Nc) return;
-    const int m = e % M, n = e / M;
-    double re = 0.0, im = 0.0;
-    for (int s = 0; s < splits; ++s) {
-        const float* d = D + ((size_t)s * M + m) * Dn;
-        re += (double)d[n];
-        im += (double)d[Nc + n];
+// C[m, n] (+)= sum_s D[s][m][n] + i D[s][m][N + n]  (FP64 sums), 32 x 32 tiles
+// turned through shared memory: D is read along its rows, C written along its columns
+__global__ void __launch_bounds__(256) k_tc_combine(const float* __restrict__ D, int splits, int M, int Nc, int Dn,
+                                                    zd* __restrict__ C, int ldc, int beta_add) {
+    __shared__ zd t[32][33];
+    const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    for (int q = y; q < 32; q += 8) {
+        const int m = m0 + q, n = n0 + x;
+        if (m >= M || n >= Nc) continue;
+        double re = 0.0, im = 0.0;
+        for (int s = 0; s < splits; ++s) {
+            const float* d = D + ((size_t)s * M + m) * Dn;
+            re += (double)d[n];
+            im += (double)d[Nc + n];
+        }
+        t[q][x] = zmk(re, im);
     }
-    zd* c = C + m + (size_t)n * ldc;
-    *c = beta_add ? zadd(*c, zmk(re, im)) : zmk(re, im);
+    __syncthreads();
+    for (int q = y; q < 32; q += 8) {
+        const int m = m0 + x, n = n0 + q;
+        if (m >= M || n >= Nc) continue;
+        zd* c = C + m + (size_t)n * ldc;
+        *c = beta_add ? zadd(*c, t[x][q]) : t[x][q];
+    }
 }
 
 // ------------------------------------------------------------ host side
@@ -238,6 +269,33 @@ static int tc_launch(const CUtensorMap& ah, const CUtensorMap& al, const CUtenso
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+// Stream-ordered workspace from a pool of the library, one per device, which
+// keeps up to 128 MiB between calls (the driver takes back what is above that at
+// the next synchronization; six cudaMalloc and cudaFree a call cost 0.3 ms).
+static cudaError_t zg_alloc(void** p, size_t bytes, int dev, cudaStream_t s) {
+    static std::mutex mu;
+    static cudaMemPool_t pools[64];
+    cudaMemPool_t pool = nullptr;
+    if (dev >= 0 && dev < 64) {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!pools[dev]) {
+            cudaMemPoolProps pr = {};
+            pr.allocType = cudaMemAllocationTypePinned;
+            pr.location.type = cudaMemLocationTypeDevice;
+            pr.location.id = dev;
+            unsigned long long keep = 128ull << 20;
+            cudaMemPool_t q = nullptr;
+            if (cudaMemPoolCreate(&q, &pr) == cudaSuccess) {
+                cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep);
+                pools[dev] = q;
+            }
+            cudaGetLastError();
+        }
+        pool = pools[dev];
+    }
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+}
+
 // One split-BF16 complex GEMM C = op(A) X (A: M x K for op N, K x M for op C;
 // X: K x N; all complex FP64 column-major on the device), with its own
 // workspace.  Returns an RTTDDFT_* code; synchronizes the stream.
@@ -260,58 +318,65 @@ int tc_zgemm(int opA, int M, int N, int K, const zd* A, int lda, const zd* X, in
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    int splits = (2 * nsm + mt * ntile - 1) / (mt * ntile);
-    splits = std::max(1, std::min(splits, std::max(1, total / 4)));
+    // K slices: one block runs per SM, so the blocks come in waves of nsm; a block costs its K
+    // blocks and about ten more for its start, its read-out and its share of D.  A slice's FP32
+    // sum is kept to 32 K blocks (2048 reals) where more slices than that cost nothing.
+    int splits = 1;
+    {
+        double best = 1e30;
+        const int smax = std::max(1, std::min(total / 4, (4 * nsm + mt * ntile - 1) / (mt * ntile)));
+        for (int sp = 1; sp <= smax; ++sp) {
+            const int kbs = (total + sp - 1) / sp;
+            const double t = (double)((mt * ntile * sp + nsm - 1) / nsm) * (kbs + 10.0) * (kbs > 32 && sp < smax ? 4.0 : 1.0);
+            if (t < best) {
+                best = t;
+                splits = sp;
+            }
+        }
+    }
     const int kbs = (total + splits - 1) / splits;
     splits = (total + kbs - 1) / kbs;
     const size_t mrows = (size_t)mt * TC_BM;
-    __nv_bfloat16 *ah = nullptr, *al = nullptr, *bh = nullptr, *bl = nullptr;
-    float* D = nullptr;
-    int* flag = nullptr;
-    int rc = RTTDDFT_OK;
-    if (cudaMalloc(&ah, mrows * Kp * 2) != cudaSuccess || cudaMalloc(&al, mrows * Kp * 2) != cudaSuccess ||
-        cudaMalloc(&bh, (size_t)Rp * Kp * 2) != cudaSuccess || cudaMalloc(&bl, (size_t)Rp * Kp * 2) != cudaSuccess ||
-        cudaMalloc(&D, (size_t)splits * M * Dn * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&flag, sizeof(int)) != cudaSuccess) {
+    // one workspace from the library's pool, carved; the rows of the left operand past M are
+    // left as they are: their products are not stored
+    const size_t na = mrows * Kp * 2, nb = (size_t)Rp * Kp * 2, nd = (size_t)splits * M * Dn * sizeof(float);
+    auto up = [](size_t n) { return (n + 1023) & ~(size_t)1023; };
+    unsigned char* ws = nullptr;
+    if (zg_alloc((void**)&ws, 2 * up(na) + 2 * up(nb) + up(nd) + 1024, dev, s) != cudaSuccess) {
         cudaGetLastError();
-        rc = RTTDDFT_ERR_OOM;
+        return RTTDDFT_ERR_OOM;
     }
-    if (rc == RTTDDFT_OK) {
-        cudaMemsetAsync(flag, 0, sizeof(int), s);
-        cudaMemsetAsync(ah, 0, mrows * Kp * 2, s);
-        cudaMemsetAsync(al, 0, mrows * Kp * 2, s);
-        k_tc_pack_a<<<(unsigned)(((size_t)M * Kp + 255) / 256), 256, 0, s>>>(A, lda, M, K, Kp, opA, ah, al);
-        k_tc_pack_b<<<(unsigned)(((size_t)Rp * Kp + 255) / 256), 256, 0, s>>>(X, ldx, K, N, Kp, Rp, bh, bl);
-        CUtensorMap tah, tal, tbh, tbl;
-        if (tc_tmap(&tah, ah, Kp, mrows, Kp, TC_BM) || tc_tmap(&tal, al, Kp, mrows, Kp, TC_BM) ||
-            tc_tmap(&tbh, bh, Kp, Rp, Kp, NT) || tc_tmap(&tbl, bl, Kp, Rp, Kp, NT)) {
-            rc = RTTDDFT_ERR_CUDA;
-        } else {
-            dim3 grid(mt, splits, ntile);
-            int lr = 0;
-            switch (NT) {
+    __nv_bfloat16 *ah = (__nv_bfloat16*)ws, *al = (__nv_bfloat16*)(ws + up(na));
+    __nv_bfloat16 *bh = (__nv_bfloat16*)(ws + 2 * up(na)), *bl = (__nv_bfloat16*)(ws + 2 * up(na) + up(nb));
+    float* D = (float*)(ws + 2 * up(na) + 2 * up(nb));
+    int* flag = (int*)(ws + 2 * up(na) + 2 * up(nb) + up(nd));
+    int rc = RTTDDFT_OK;
+    cudaMemsetAsync(flag, 0, sizeof(int), s);
+    k_tc_pack_a<<<dim3((M + 31) / 32, (K + 31) / 32), 256, 0, s>>>(A, lda, M, K, Kp, opA, ah, al);
+    k_tc_pack_b<<<dim3(Rp, (Kp + 255) / 256), 256, 0, s>>>(X, ldx, K, N, Kp, Rp, bh, bl);
+    CUtensorMap tah, tal, tbh, tbl;
+    if (tc_tmap(&tah, ah, Kp, mrows, Kp, TC_BM) || tc_tmap(&tal, al, Kp, mrows, Kp, TC_BM) ||
+        tc_tmap(&tbh, bh, Kp, Rp, Kp, NT) || tc_tmap(&tbl, bl, Kp, Rp, Kp, NT)) {
+        rc = RTTDDFT_ERR_CUDA;
+    } else {
+        dim3 grid(mt, splits, ntile);
+        int lr = 0;
+        switch (NT) {
 #define RTD_TC(n) \
     case n: lr = tc_launch<n>(tah, tal, tbh, tbl, nkb2, kbs, grid, D, M, Dn, flag, s); break;
-                RTD_TC(16) RTD_TC(32) RTD_TC(48) RTD_TC(64) RTD_TC(80) RTD_TC(96) RTD_TC(112) RTD_TC(128)
-                RTD_TC(144) RTD_TC(160) RTD_TC(176) RTD_TC(192) RTD_TC(208) RTD_TC(224) RTD_TC(240) RTD_TC(256)
+            RTD_TC(16) RTD_TC(32) RTD_TC(48) RTD_TC(64) RTD_TC(80) RTD_TC(96) RTD_TC(112) RTD_TC(128)
+            RTD_TC(144) RTD_TC(160) RTD_TC(176) RTD_TC(192) RTD_TC(208) RTD_TC(224) RTD_TC(240) RTD_TC(256)
 #undef RTD_TC
-                default: lr = -1;
-            }
-            if (lr) rc = RTTDDFT_ERR_CUDA;
-            else k_tc_combine<<<(M * N + 255) / 256, 256, 0, s>>>(D, splits, M, N, Dn, C, ldc, beta_add);
+            default: lr = -1;
         }
+        if (lr) rc = RTTDDFT_ERR_CUDA;
+        else k_tc_combine<<<dim3((M + 31) / 32, (N + 31) / 32), 256, 0, s>>>(D, splits, M, N, Dn, C, ldc, beta_add);
     }
     int hflag = 0;
+    if (cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = RTTDDFT_ERR_CUDA;
+    cudaFreeAsync(ws, s);
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) rc = RTTDDFT_ERR_CUDA;
-    if (rc == RTTDDFT_OK && cudaMemcpy(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-        rc = RTTDDFT_ERR_CUDA;
     if (rc == RTTDDFT_OK && (hflag & 8)) rc = RTTDDFT_ERR_TIMEOUT;
-    cudaFree(ah);
-    cudaFree(al);
-    cudaFree(bh);
-    cudaFree(bl);
-    cudaFree(D);
-    cudaFree(flag);
     return rc;
 }
 
