@@ -55,6 +55,8 @@ struct rttddft_ctx {
     double tc_st = 1.0;         // its fp16 scale
     double *d_occ = nullptr, *d_wk = nullptr, *d_lam = nullptr;
     DevState* d_st = nullptr;
+    unsigned char* d_cheb_sync = nullptr;
+    int cheb_cl = 0;
     double* d_rec = nullptr;
     double *d_part_jmt = nullptr, *d_part_full = nullptr, *d_part_post = nullptr;
     double *d_part_fin = nullptr, *d_gdev = nullptr;
@@ -272,6 +274,8 @@ static StepArgs make_args(rttddft_ctx* ctx, int dv_on) {
     a.part_t = ctx->d_part_t;
     a.flag = ctx->d_flag;
     a.coop_grid = ctx->coop_grid;
+    a.cheb_cl = ctx->cheb_cl;
+    a.cheb_sync = ctx->d_cheb_sync;
     a.tcback = (ctx->dg_back || (ctx->opt.precision >= RTTDDFT_PREC_BF16X3 && tc_has_back(ctx->tc))) ? 1 : 0;
     a.tc_fmt = tc_format(ctx->tc);
     a.tc_st = tc_table_scale(ctx->tc);
@@ -943,6 +947,8 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
         ctx->d_st = dalloc<DevState>(ctx, 1);
         CK(cudaMemset(ctx->d_st, 0, sizeof(DevState)));
         ctx->d_flag = dalloc<int>(ctx, 1);
+        ctx->d_cheb_sync = dalloc<unsigned char>(ctx, cheb_sync_bytes(nk, naux));
+        CK(cudaMemset(ctx->d_cheb_sync, 0, cheb_sync_bytes(nk, naux)));
         ctx->d_rec = dalloc<double>(ctx, (size_t)o->max_record * RTD_REC_STRIDE);
         ctx->d_lam = dalloc<double>(ctx, LAM_N * (size_t)nk);
         ctx->max_nback = (ctx->maxng + BKB - 1) / BKB;
@@ -1439,10 +1445,10 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
             const int e = prepare_back_kernels(a);
             if (e) fail(ctx, RTTDDFT_ERR_UNSUPPORTED, "table window needs more shared memory than a block has");
             CK(cudaStreamSynchronize(ctx->stream));
-            ctx->coop_grid = prepare_cheb_coop(a, ctx->stream);
-            // without the memory for the digits the per-row form runs
-            if (o->propagator != RTTDDFT_PROP_EIG && ns >= DG_SERIES_MIN_NS)
-                ctx->series = dg_series_create(nk, naux, ns);
+            ctx->coop_grid = prepare_cheb_coop(a, ctx->stream, &ctx->cheb_cl);
+            // many states or rows: digit products; without the memory for the digits one launch
+            // per term
+            if (o->propagator != RTTDDFT_PROP_EIG && ctx->coop_grid == 0) ctx->series = dg_series_create(nk, naux, ns);
         }
         // ---- theta(0)
         if (s->c0) {

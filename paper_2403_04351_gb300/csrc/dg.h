@@ -2,8 +2,6 @@
 #pragma once
 #include "common.cuh"
 
-#define DG_SERIES_MIN_NS 9  // states from which the series runs as digit products
-
 struct DgLeft;    // digits of a static left operand per batch entry
 struct DgGemm;    // C (+)= A X per batch entry
 struct DgSeries;  // the Chebyshev series

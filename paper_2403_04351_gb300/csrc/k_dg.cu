@@ -855,16 +855,15 @@ int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s, 
 }
 
 // ------------------------------------------------------------ Chebyshev series
-// The series with H~ y_{n-1} as digit products, one launch per term, for
-// DG_SERIES_MIN_NS states and more.  In FP64 its rate was the FP64 pipe's (16
-// k-points of N_aux 300, N_s 60: 9.0 GFLOP in 8.3 ms; 2 k-points 1.91 ms), here
-// the 2 k-points take 0.29 ms, bound by the 14 launches of a few stages each.
-// Below nine states the cooperative per-row form has the shorter chain.  H~ = (HH - lam_c) / lam_h has norm <= 1, so its entries take the scale
+// The series with H~ y_{n-1} as digit products, one launch per term, for more
+// states or rows than k_cheb_coop takes.  In FP64 its rate was the FP64 pipe's (16
+// k-points of N_aux 300, N_s 60: 9.0 GFLOP in 8.3 ms; 2 k-points 1.91 ms); here the
+// 2 k-points take 0.27 ms, bound by the 14 launches of a few stages each.
+// H~ = (HH - lam_c) / lam_h has norm <= 1, so its entries take the scale
 // 1; a column of theta takes the power of two above its 2-norm, which bounds
 // every y_n.  y_n, the recurrence and the sum are integers in units of 2^-62
 // of that scale: nothing is rounded between the terms but the digits' cut.
 struct DgSeriesK {
-    KDev const* kd;
     uint32_t* A;     // digits of H~, tiles of 128 rows
     int nst, NT;
     int* bad;        // per row: HH not finite
@@ -891,7 +890,6 @@ __global__ void __launch_bounds__(128) k_dg_hsub(StepArgs a, const DgSeriesK* sk
     const double ax = av[0], ay = av[1], az = av[2];
     const double aa = (ax * ax + ay * ay + az * az) * a.half_inv_c2;
     if (i == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
-        st->bar = 0u;
         if (!a.dv_on) {
             st->cur_a[0] = ax;
             st->cur_a[1] = ay;

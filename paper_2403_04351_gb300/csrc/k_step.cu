@@ -12,6 +12,7 @@
 #include "dg.h"
 #include "rtd.h"
 
+#include <algorithm>
 #include <cstdlib>
 
 __device__ __forceinline__ double dsq(double x) { return x * x; }
@@ -57,7 +58,6 @@ __global__ void k_hsub(StepArgs a) {
     const double ax = av[0], ay = av[1], az = av[2];
     const double aa = (ax * ax + ay * ay + az * az) * a.half_inv_c2;
     if (blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
-        st->bar = 0u;
         if (!a.dv_on) {
             st->cur_a[0] = ax;
             st->cur_a[1] = ay;
@@ -148,174 +148,569 @@ __global__ void __launch_bounds__(128) k_cheb(StepArgs a, int nt, int last) {
     }
 }
 
-// Grid-wide barrier of a cooperative launch: a monotone arrival counter in
-// device memory (zeroed by k_hsub before the launch); a block waits until
-// the counter reaches `target`.  The wait is bounded: after about 0.3 s it
-// raises flag bit 2 (reported as ERR_TIMEOUT) and returns false, so a launch
-// can never hang.
+// ------------------------------------------------------------ cooperative series
+// The whole series of few states in one cooperative launch, one block per row
+// (k, i) of HH.  An FP64 instruction of a warp holds its sub-partition for 64
+// cycles on GB300 whatever the number of active lanes, so a term's dot product,
+// sums and update took 3 us; here they run on the integer pipe (a series of N_aux
+// 200, N_s 2: 82 -> 48 us; N_aux 240, N_s 7: 111 -> 73 us).  H~ = (HH - lam_c) / lam_h has norm <= 1 and takes units of 2^-58, a
+// column of theta the power of two above its 2-norm (which bounds every y_n),
+// y_n units of 2^-57 of it.  An operand is held as hi 2^28 + lo; a product keeps
+// hi hi and hi lo + lo hi (the dropped lo lo is below 2^-61), summed exactly in
+// 64 bits, so a term's error is the cut of its operands, 2^-58 of the norm, below
+// FP64's own.  The recurrence and sum_n c_n y_n are integers in units of 2^-59.
+//
+// Per term y_n goes around through L2 (two slots of 16 bytes per entry) and a
+// grid barrier follows.  The barrier has CS_CNT arrival counters on lines of
+// their own (one counter serialises its arrivals); a warp polls them all.
+// (Entries that carry a tag of their term and are polled themselves, one trip
+// instead of three, measured slower: 65 against 46 us at N_aux 200, N_s 2; stores
+// to lines under polling are held up.)  The wait is bounded: it raises flag bit 2
+// (reported as ERR_TIMEOUT).  The last block to leave sets the counters back.
+#define CS_THREADS 128
+#define CS_CNT 16
+#define CS_MAXC 128  // coefficients kept in shared memory at a time
+struct ChebSync {
+    unsigned cnt[CS_CNT][32];
+    unsigned left;
+    unsigned bad;  // HH of some k-point is not finite (a NaN or infinite pulse or change)
+    unsigned pad[30];
+};
+typedef long long i64;
+__device__ __forceinline__ int2 cs_split(i64 q) {  // q = hi 2^28 + lo
+    const int lo = (int)(q << 36 >> 36);
+    return make_int2((int)((q - lo) >> 28), lo);
+}
+__device__ __forceinline__ double cs_pow2(int n) { return __hiloint2double((n + 1023) << 20, 0); }
+// x 2^(f - e) rounded to an integer, |x| < 2^e, f <= 62, with integer arithmetic
+__device__ __forceinline__ i64 cs_fix(double x, int e, int f) {
+    const i64 b = __double_as_longlong(x);
+    const int ex = (int)(b >> 52) & 2047;
+    if (ex == 0) return 0;  // zero, or below 2^-1022: nothing of it is left at this scale
+    i64 m = (b & ((1ll << 52) - 1)) | (1ll << 52);
+    const int sh = ex - 1075 + f - e;
+    m = sh >= 0 ? m << sh : (sh < -54 ? 0 : (m + (1ll << (-sh - 1))) >> -sh);
+    return b < 0 ? -m : m;
+}
+// |x| 2^-e for the norm's estimate, from the high word (relative error 2^-20, small values 0)
+__device__ __forceinline__ float cs_small(double x, int e) {
+    const int hw = __double2hiint(x) & 0x7fffffff;
+    const int ex = (hw >> 20) - 1023 - e;
+    return ex < -100 ? 0.f : __int_as_float(((ex + 127) << 23) | ((hw & 0xfffff) << 3));
+}
+// (A, B) += x y and -= x y of two cut numbers: A holds hi hi, B the mixed products
+__device__ __forceinline__ void cs_fma(i64& A, i64& B, int2 x, int2 y) {
+    A += (i64)x.x * y.x;
+    B += (i64)x.x * y.y;
+    B += (i64)x.y * y.x;
+}
+__device__ __forceinline__ void cs_fms(i64& A, i64& B, int2 x, int2 y) {
+    A -= (i64)x.x * y.x;
+    B -= (i64)x.x * y.y;
+    B -= (i64)x.y * y.x;
+}
+// a b 2^-62
+__device__ __forceinline__ i64 cs_mul62(i64 a, i64 b) {
+    return (i64)(((unsigned long long)__mul64hi(a, b) << 2) | (((unsigned long long)a * (unsigned long long)b) >> 62));
+}
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ bool grid_barrier(unsigned* count, unsigned target, int* flag) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // release: the block's writes (ordered before by the bar.sync above)
-        // become visible to every block that acquires the count
-        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(count), "r"(1u) : "memory");
-        int ok = 1;
-        unsigned long long it = 0;
-        while (ld_acquire_gpu(count) < target) {
-            if (++it > (1ull << 22)) {
-                atomicOr(flag, 4);
-                ok = 0;
-                break;
-            }
-            __nanosleep(32);
-        }
-        s_ok = ok;
+
+// phase x sum of c_n y_n (units 2^-59 of the column's scale 2^e) as theta
+__device__ __forceinline__ zd cs_result(const StepArgs& a, const KDev& K, i64 sr, i64 si, int e, bool bad) {
+    const zd ph = (a.prop == 0) ? zmk(K.lam[3], K.lam[4]) : zmk(1.0, 0.0);
+    zd t = zmul(ph, zmk((double)sr, (double)si));
+    const int s = min(e, 1024) - 59, h = s / 2;
+    const double p1 = cs_pow2(h), p2 = cs_pow2(s - h);
+    t = zmk((t.x * p1) * p2, (t.y * p1) * p2);
+    if (e >= 1024 || bad) t.x = t.y = __longlong_as_double(0x7ff8000000000000ll);
+    return t;
+}
+// (A, B)[0, 1] += conj(h) y
+__device__ __forceinline__ void cs_mac(i64* A, i64* B, int2 hr, int2 hi, int4 y) {
+    const int2 yr = make_int2(y.x, y.y), yi = make_int2(y.z, y.w);
+    cs_fma(A[0], B[0], hr, yr);
+    cs_fma(A[0], B[0], hi, yi);
+    cs_fma(A[1], B[1], hr, yi);
+    cs_fms(A[1], B[1], hi, yr);
+}
+// the step's pulse in units of lam_h; `first` stores the step's A and |A|^2/(2c^2) as k_hsub does
+struct CsPulse {
+    double al[3], diag, ilh;
+};
+__device__ __forceinline__ CsPulse cs_pulse(const StepArgs& a, const KDev& K, bool first) {
+    DevState* st = a.st;
+    const double* av = a.a + 3 * (size_t)st->cstep;
+    const double ax = av[0], ay = av[1], az = av[2];
+    const double aa = (ax * ax + ay * ay + az * az) * a.half_inv_c2;
+    if (first && !a.dv_on) {
+        st->cur_a[0] = ax;
+        st->cur_a[1] = ay;
+        st->cur_a[2] = az;
+        st->cur_s = 0.0;
+        st->cur_aa = aa;
     }
-    __syncthreads();
-    return s_ok != 0;
+    CsPulse p;
+    p.ilh = K.lam[2];
+    p.al[0] = ax * a.inv_c * p.ilh;
+    p.al[1] = ay * a.inv_c * p.ilh;
+    p.al[2] = az * a.inv_c * p.ilh;
+    p.diag = aa - K.lam[0];
+    return p;
+}
+// the stored column i, entry j, of H~ cut into (re hi, re lo, im hi, im lo); it is
+// the conjugate of row i (HH is Hermitian)
+__device__ __forceinline__ int4 cs_hentry(const StepArgs& a, const KDev& K, const CsPulse& p, int i, int j, bool& bad) {
+    const int n = a.naux;
+    const size_t nn = (size_t)n * n, e = (size_t)i * n + j;
+    zd v = zmk(0.0, 0.0);
+    if (a.dv_on) v = zscale(K.dvsub[e], p.ilh);
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+        if (p.al[l] != 0.0) {
+            const zd q = K.psub[l * nn + e];
+            v.x = fma(q.x, p.al[l], v.x);
+            v.y = fma(q.y, p.al[l], v.y);
+        }
+    if (i == j) v.x += (K.eps[i] + p.diag) * p.ilh;
+    const int hx = __double2hiint(v.x) & 0x7fffffff, hy = __double2hiint(v.y) & 0x7fffffff;
+    bad |= hx >= 0x7ff00000 || hy >= 0x7ff00000;
+    // |H~_ij| <= 1; a step beyond its bounds (reported by its flag) stays in range
+    const int2 r = cs_split(hx >= 0x40000000 ? 1ll << 58 : cs_fix(v.x, 0, 58));
+    const int2 m = cs_split(hy >= 0x40000000 ? 1ll << 58 : cs_fix(v.y, 0, 58));
+    return make_int4(r.x, r.y, m.x, m.y);
 }
 
-// The whole Chebyshev series in one cooperative launch.  A block of two
-// warps owns rows (k, i) = blockIdx.x + r gridDim.x for all terms; its lanes
-// stride a row's dot products and reduce them with WarpHalvingSum (the FP64
-// pipe, not memory, bounds a term on GB300).  Only the newest vector y_{n-1}
-// is exchanged through global memory (two slots, read through L2 with
-// ld.global.cg); each block keeps y_{n-1}, y_{n-2} and the partial sum of
-// its own rows in shared memory.  A grid barrier separates the terms (per-block
-// epoch flags polled by every block measured slower on GB300: 107 against 80 us
-// per series at N_aux = 200).
-#define CHEB_THREADS 64
-#define CHEB_JU 4  // row entries per thread held at once (n_aux <= 256 in one pass)
-template <int NT>
-__global__ void __launch_bounds__(CHEB_THREADS) k_cheb_coop(StepArgs a, int direct) {
+// NT columns (N_s <= NT), JU entries of the row per thread.  The thread's entries of
+// y_(n-1) come into its part of shared memory all at once (cp.async: no registers
+// for loads in flight).
+template <int NT, int JU>
+__global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepArgs a, ChebSync* sy) {
+    constexpr int CW = NT < 4 ? NT : 4;  // columns at a time (registers)
     constexpr int V = 2 * NT;
-    __shared__ double red[CHEB_THREADS / 32][V];
-    extern __shared__ zd cst[];  // [rows of the block][3][ns]: y_{n-1}, y_{n-2}, partial sum
+    extern __shared__ int4 ysm[];  // [N_s][N_aux]
+    __shared__ i64 red[CS_THREADS / 32][V];
+    __shared__ i64 cf[CS_MAXC][2];
+    __shared__ int smx[CS_THREADS / 32][NT];
+    __shared__ float snm[CS_THREADS / 32][NT];
     const int n = a.naux, ns = a.ns;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const size_t vs = (size_t)n * ns;
-    const int nrow = a.nk * n;
-    // direct: every block owns one row and n <= CHEB_JU * CHEB_THREADS, so the
-    // block builds its row of HH(t_k) (Eq. auxiliary_hamiltonian_with_parts)
-    // once, in registers, instead of reading a matrix formed by k_hsub
-    zd hrow[CHEB_JU];
-    if (direct && blockIdx.x < nrow) {
-        const int k = blockIdx.x / n, i = blockIdx.x % n;
-        const KDev& K = a.kd[k];
-        DevState* st = a.st;
-        const double* av = a.a + 3 * (size_t)st->cstep;
-        const double ax = av[0], ay = av[1], az = av[2];
-        const double aa = (ax * ax + ay * ay + az * az) * a.half_inv_c2;
-        if (blockIdx.x == 0 && tid == 0 && !a.dv_on) {
-            st->cur_a[0] = ax;
-            st->cur_a[1] = ay;
-            st->cur_a[2] = az;
-            st->cur_s = 0.0;
-            st->cur_aa = aa;
+    const int k = blockIdx.x / n, i = blockIdx.x % n;
+    const KDev& K = a.kd[k];
+    int2 hr[JU], hi[JU];
+    {
+        // row i of HH(t_k) (Eq. auxiliary_hamiltonian_with_parts)
+        const CsPulse pu = cs_pulse(a, K, blockIdx.x == 0 && tid == 0);
+        bool bad = false;
+#pragma unroll
+        for (int u = 0; u < JU; ++u) {
+            const int j = tid + u * CS_THREADS;
+            const int4 h = j < n ? cs_hentry(a, K, pu, i, j, bad) : make_int4(0, 0, 0, 0);
+            hr[u] = make_int2(h.x, h.y);
+            hi[u] = make_int2(h.z, h.w);
         }
-        const size_t nn = (size_t)n * n;
-        const double al[3] = {ax * a.inv_c, ay * a.inv_c, az * a.inv_c};
-#pragma unroll
-        for (int u = 0; u < CHEB_JU; ++u) {
-            const int j = tid + u * CHEB_THREADS;
-            zd v = zmk(0.0, 0.0);
-            if (j < n) {
-                const size_t e = (size_t)i * n + j;  // the storage element (row j, column i) of k_hsub
-#pragma unroll
-                for (int l = 0; l < 3; ++l)
-                    if (al[l] != 0.0) v = zadd(v, zscale(K.psub[l * nn + e], al[l]));
-                if (i == j) v.x += K.eps[i] + aa;
-                if (a.dv_on) v = zadd(v, K.dvsub[e]);
-            }
-            hrow[u] = v;
+        if (bad) {
+            atomicOr(&sy->bad, 1u);
+            __threadfence();
         }
     }
+    for (int t = tid; t < min(a.nterms, CS_MAXC); t += CS_THREADS) {
+        cf[t][0] = __double2ll_rn(K.coef[t].x * 4611686018427387904.0);
+        cf[t][1] = __double2ll_rn(K.coef[t].y * 4611686018427387904.0);
+    }
+    // the scale of every column of theta: the power of two above its 2-norm
+    int e[NT];
+    {
+        int mx[NT];
+#pragma unroll
+        for (int c = 0; c < NT; ++c) mx[c] = 0;
+#pragma unroll
+        for (int u = 0; u < JU; ++u) {
+            const int j = tid + u * CS_THREADS;
+#pragma unroll
+            for (int c = 0; c < NT; ++c) {
+                if (j >= n || c >= ns) continue;
+                const zd t = K.theta[j + (size_t)c * n];
+                mx[c] = max(mx[c], max(__double2hiint(t.x) & 0x7fffffff, __double2hiint(t.y) & 0x7fffffff));
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NT; ++c) {
+            mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
+            if (lane == 0) smx[warp][c] = mx[c];
+        }
+        __syncthreads();
+        float q[NT];
+#pragma unroll
+        for (int c = 0; c < NT; ++c) {
+            q[c] = 0.f;
+            int m = 0;
+#pragma unroll
+            for (int w = 0; w < CS_THREADS / 32; ++w) m = max(m, smx[w][c]);
+            e[c] = (m >> 20) - 1023;
+        }
+#pragma unroll
+        for (int u = 0; u < JU; ++u) {
+            const int j = tid + u * CS_THREADS;
+#pragma unroll
+            for (int c = 0; c < NT; ++c) {
+                if (j >= n || c >= ns) continue;
+                const zd t = K.theta[j + (size_t)c * n];
+                const float x = cs_small(t.x, e[c]), y = cs_small(t.y, e[c]);
+                q[c] += x * x + y * y;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NT; ++c) {
+            for (int o = 16; o > 0; o >>= 1) q[c] += __shfl_xor_sync(0xffffffffu, q[c], o);
+            if (lane == 0) snm[warp][c] = q[c];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < NT; ++c) {
+            float t = 0.f;
+#pragma unroll
+            for (int w = 0; w < CS_THREADS / 32; ++w) t += snm[w][c];
+            // a column that is not finite: e = 1024 and more, answered with NaN at the end
+            if (e[c] < 1024) e[c] += ((__float_as_int(sqrtf(t) * 1.00001f) >> 23) & 255) - 126;
+        }
+    }
+    // the block's own entries of the recurrence: thread c of the first warp
+    const int oc = tid;
+    const bool own = tid < NT && oc < ns;
+    int eo = 0;
+#pragma unroll
+    for (int c = 0; c < NT; ++c)
+        if (oc == c) eo = e[c];
+    const size_t oe = i + (size_t)oc * n;
+    i64 y1r = 0, y1i = 0, y2r = 0, y2i = 0, sr = 0, si = 0;
+    if (own && eo < 1024) {
+        const zd t = K.theta[oe];
+        y1r = cs_fix(t.x, eo, 59);
+        y1i = cs_fix(t.y, eo, 59);
+        sr = cs_mul62(cf[0][0], y1r) - cs_mul62(cf[0][1], y1i);
+        si = cs_mul62(cf[0][0], y1i) + cs_mul62(cf[0][1], y1r);
+    }
+    unsigned mycnt = 0;  // blocks that arrive at the counter this lane polls
+    if (lane < CS_CNT) mycnt = (gridDim.x - lane + CS_CNT - 1) / CS_CNT;
+    int4* ring = (int4*)K.ring;
+    bool ok = true;
     for (int nt = 1; nt < a.nterms; ++nt) {
-        const int last = (nt == a.nterms - 1);
-        int r = 0;
-        for (int q = blockIdx.x; q < nrow; q += gridDim.x, ++r) {
-            const int k = q / n, i = q % n;
-            const KDev& K = a.kd[k];
-            const zd* __restrict__ H = K.hsub + (size_t)i * n;
-            const zd* yin = (nt == 1) ? K.theta : K.ring + ((nt - 1) & 1) * vs;
-            zd* yout = K.ring + (nt & 1) * vs;
-            zd* y1 = cst + (size_t)r * 3 * ns;
-            zd* y2 = y1 + ns;
-            zd* ac = y2 + ns;
-            for (int n0 = 0; n0 < ns; n0 += NT) {
-                // operands of the update first, so their latency overlaps the dot products
-                const bool upd = tid < NT && n0 + tid < ns;
-                zd yi = zmk(0.0, 0.0), cn = zmk(0.0, 0.0), c0 = zmk(0.0, 0.0);
-                double lc = 0.0, ilh = 0.0;
-                if (upd) {
-                    yi = (nt == 1) ? K.theta[i + (size_t)(n0 + tid) * n] : y1[n0 + tid];
-                    cn = K.coef[nt];
-                    if (nt == 1) c0 = K.coef[0];
-                    lc = K.lam[0];
-                    ilh = K.lam[2];
-                }
-                zd acc[NT];
+        const bool last = nt == a.nterms - 1;
+        const int4* yin = ring + ((nt - 1) & 1) * vs;
+        if (nt >= CS_MAXC && nt % CS_MAXC == 0) {
+            __syncthreads();
+            for (int t = tid; t < min(a.nterms - nt, CS_MAXC); t += CS_THREADS) {
+                cf[t][0] = __double2ll_rn(K.coef[nt + t].x * 4611686018427387904.0);
+                cf[t][1] = __double2ll_rn(K.coef[nt + t].y * 4611686018427387904.0);
+            }
+            __syncthreads();
+        }
 #pragma unroll
-                for (int c = 0; c < NT; ++c) acc[c] = zmk(0.0, 0.0);
-                for (int j0 = tid; j0 < n; j0 += CHEB_JU * CHEB_THREADS) {
-                    zd hv[CHEB_JU], yv[CHEB_JU][NT];
+        for (int u = 0; u < JU; ++u) {
+            const int j = tid + u * CS_THREADS;
 #pragma unroll
-                    for (int u = 0; u < CHEB_JU; ++u) {
-                        const int j = j0 + u * CHEB_THREADS;
-                        const bool ok = j < n;
-                        hv[u] = direct ? hrow[u] : (ok ? H[j] : zmk(0.0, 0.0));
-#pragma unroll
-                        for (int c = 0; c < NT; ++c)
-                            yv[u][c] = (ok && n0 + c < ns) ? __ldcg(yin + j + (size_t)(n0 + c) * n) : zmk(0.0, 0.0);
-                    }
-#pragma unroll
-                    for (int u = 0; u < CHEB_JU; ++u)
-#pragma unroll
-                        for (int c = 0; c < NT; ++c) zfmac(acc[c], hv[u], yv[u][c]);
-                }
-                double v[V];
-#pragma unroll
-                for (int c = 0; c < NT; ++c) {
-                    v[2 * c] = acc[c].x;
-                    v[2 * c + 1] = acc[c].y;
-                }
-                warp_sum_store<double, V>(v, lane, red[warp]);
-                __syncthreads();
-                if (upd) {
-                    const int c = n0 + tid;
-                    zd sm = zmk(red[0][2 * tid], red[0][2 * tid + 1]);
-#pragma unroll
-                    for (int w = 1; w < CHEB_THREADS / 32; ++w) sm = zadd(sm, zmk(red[w][2 * tid], red[w][2 * tid + 1]));
-                    const zd w = zscale(zsub(sm, zscale(yi, lc)), ilh);
-                    zd y, s;
-                    if (nt == 1) {
-                        y = w;
-                        s = zadd(zmul(c0, yi), zmul(cn, y));
-                    } else {
-                        y = zsub(zscale(w, 2.0), y2[c]);
-                        s = zadd(ac[c], zmul(cn, y));
-                    }
-                    y2[c] = yi;
-                    y1[c] = y;
-                    if (last) {
-                        const zd ph = (a.prop == 0) ? zmk(K.lam[3], K.lam[4]) : zmk(1.0, 0.0);
-                        K.theta[i + (size_t)c * n] = zmul(ph, s);
-                    } else {
-                        yout[i + (size_t)c * n] = y;
-                        ac[c] = s;
+            for (int c = 0; c < NT; ++c) {
+                if (j >= n || c >= ns) continue;
+                int4* d = ysm + j + (size_t)c * n;
+                if (nt > 1) {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(d)),
+                                 "l"(yin + j + (size_t)c * n)
+                                 : "memory");
+                } else {
+                    *d = make_int4(0, 0, 0, 0);
+                    if (e[c] < 1024) {
+                        const zd t = K.theta[j + (size_t)c * n];
+                        const int2 p = cs_split(cs_fix(t.x, e[c], 57)), r = cs_split(cs_fix(t.y, e[c], 57));
+                        *d = make_int4(p.x, p.y, r.x, r.y);
                     }
                 }
-                __syncthreads();
             }
         }
-        if (!last && !grid_barrier(&a.st->bar, (unsigned)nt * gridDim.x, a.flag)) return;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+        for (int h = 0; h < NT; h += CW) {
+            i64 A[2 * CW], B[2 * CW];
+#pragma unroll
+            for (int v = 0; v < 2 * CW; ++v) A[v] = B[v] = 0;
+#pragma unroll
+            for (int u = 0; u < JU; ++u) {
+                const int j = tid + u * CS_THREADS;
+                if (j >= n) continue;
+#pragma unroll
+                for (int q = 0; q < CW; ++q)
+                    if (h + q < ns) cs_mac(A + 2 * q, B + 2 * q, hr[u], hi[u], ysm[j + (size_t)(h + q) * n]);
+            }
+#pragma unroll
+            for (int v = 0; v < 2 * CW; ++v) A[v] += (B[v] + (1ll << 27)) >> 28;  // units 2^-59
+            warp_sum_store<i64, 2 * CW>(A, lane, &red[warp][2 * h]);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            i64 yr = 0, yi = 0;
+            if (own) {
+                yr = red[0][2 * tid];
+                yi = red[0][2 * tid + 1];
+#pragma unroll
+                for (int w = 1; w < CS_THREADS / 32; ++w) {
+                    yr += red[w][2 * tid];
+                    yi += red[w][2 * tid + 1];
+                }
+                if (nt > 1) {
+                    yr = 2 * yr - y2r;
+                    yi = 2 * yi - y2i;
+                }
+                y2r = y1r;
+                y2i = y1i;
+                y1r = yr;
+                y1i = yi;
+                if (!last) {
+                    const int2 p = cs_split((yr + 2) >> 2), q = cs_split((yi + 2) >> 2);
+                    __stcg(ring + (nt & 1) * vs + oe, make_int4(p.x, p.y, q.x, q.y));
+                }
+            }
+            if (!last) {
+                // release: the warp's stores become visible to every block that acquires the count
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&sy->cnt[blockIdx.x % CS_CNT][0]), "r"(1u)
+                                 : "memory");
+            }
+            if (own) {
+                const i64 cr = cf[nt % CS_MAXC][0], ci = cf[nt % CS_MAXC][1];
+                sr += cs_mul62(cr, yr) - cs_mul62(ci, yi);
+                si += cs_mul62(cr, yi) + cs_mul62(ci, yr);
+            }
+            if (!last) {
+                const unsigned want = mycnt * (unsigned)nt;
+                bool there = lane >= CS_CNT;
+                unsigned it = 0;
+                while (true) {
+                    if (!there) there = ld_acquire_gpu(&sy->cnt[lane][0]) >= want;
+                    if (__all_sync(0xffffffffu, there)) break;
+                    if (++it > (1u << 20)) {
+                        ok = false;
+                        break;
+                    }
+                }
+            }
+        }
+        if (!last) {
+            ok = !__syncthreads_or(!ok);
+            if (!ok) break;
+        }
     }
+    if (!ok && tid == 0) atomicOr(a.flag, 4);
+    // (every block read theta before it wrote its y_1, so theta may be written now)
+    if (ok && own) {
+        K.theta[oe] = cs_result(a, K, sr, si, eo, *(volatile unsigned*)&sy->bad != 0u);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(&sy->left, 1u) == gridDim.x - 1) {
+            // every block has read what it needs
+            for (int c = 0; c < CS_CNT; ++c) sy->cnt[c][0] = 0u;
+            sy->bad = 0u;
+            sy->left = 0u;
+        }
+    }
+}
+
+// The same series with one cluster of 16 blocks per k-point, for up to CL_MAXN
+// rows.  A warp owns a row of H~ (in registers, cut by k_cs_rows on all SMs); y_n
+// goes to the shared memory of all 16 blocks by st.async, whose bytes complete
+// the receiving block's mbarrier: one trip through the cluster's network per term
+// instead of a grid barrier and two trips through L2.  The products bound it, at
+// 1.4 cycles each on an SM (twelve 32-bit multiply-adds).  Two slots and mbarriers: a
+// warp sends y_(n+2) after all of y_(n+1) has arrived, and every warp sends its
+// entries of y_(n+1) after it has read y_n.  Waits are bounded as elsewhere.
+#define CL_N 16
+#define CL_MAXN 256
+#define CL_THREADS 512
+__global__ void __launch_bounds__(128) k_cs_rows(StepArgs a, int* rowbad) {
+    const int k = blockIdx.y, i = blockIdx.x, n = a.naux;
+    const KDev& K = a.kd[k];
+    const CsPulse pu = cs_pulse(a, K, i == 0 && k == 0 && threadIdx.x == 0);
+    bool bad = false;
+    for (int j = threadIdx.x; j < n; j += 128) ((int4*)K.hsub)[(size_t)i * n + j] = cs_hentry(a, K, pu, i, j, bad);
+    const int any = __syncthreads_or(bad);
+    if (threadIdx.x == 0) rowbad[(size_t)k * n + i] = any;
+}
+__device__ __forceinline__ bool cl_wait(uint64_t* b, unsigned parity) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(b);
+    const long long t0 = clock64();
+    while (true) {
+        unsigned ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(s), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if (clock64() - t0 > (1ll << 31)) return false;
+    }
+}
+template <int NT>
+__global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int* rowbad) {
+    constexpr int CW = NT < 4 ? NT : 4, JU = CL_MAXN / 32;
+    extern __shared__ int4 csm[];  // [2][N_s][N_aux] y, then the coefficients
+    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ i64 red[CL_THREADS / 32][2 * NT];
+    __shared__ int4 snd[CL_THREADS / 32][NT];
+    __shared__ int es[NT];
+    const int n = a.naux, ns = a.ns;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x % CL_N, k = blockIdx.x / CL_N;
+    const KDev& K = a.kd[k];
+    const int i = warp * CL_N + rank;
+    const bool act = i < n;
+    const size_t vs = (size_t)n * ns;
+    i64* cf = (i64*)(csm + 2 * vs);
+    const unsigned bytes = (unsigned)(vs * sizeof(int4));
+    if (tid == 0) {
+        for (int q = 0; q < 2; ++q) {
+            const unsigned b = (unsigned)__cvta_generic_to_shared(&bar[q]);
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    int2 hr[JU], hi[JU];
+#pragma unroll
+    for (int u = 0; u < JU; ++u) {
+        const int j = lane + 32 * u;
+        const int4 h = act && j < n ? ((const int4*)K.hsub)[(size_t)i * n + j] : make_int4(0, 0, 0, 0);
+        hr[u] = make_int2(h.x, h.y);
+        hi[u] = make_int2(h.z, h.w);
+    }
+    for (int t = tid; t < a.nterms; t += CL_THREADS) {
+        cf[2 * t] = __double2ll_rn(K.coef[t].x * 4611686018427387904.0);
+        cf[2 * t + 1] = __double2ll_rn(K.coef[t].y * 4611686018427387904.0);
+    }
+    if (warp < ns) {  // a warp per column: the power of two above its 2-norm
+        const zd* th = K.theta + (size_t)warp * n;
+        int m = 0;
+        for (int j = lane; j < n; j += 32) m = max(m, max(__double2hiint(th[j].x) & 0x7fffffff, __double2hiint(th[j].y) & 0x7fffffff));
+        m = __reduce_max_sync(0xffffffffu, m);
+        int e = (m >> 20) - 1023;
+        float q = 0.f;
+        for (int j = lane; j < n; j += 32) {
+            const float x = cs_small(th[j].x, e), y = cs_small(th[j].y, e);
+            q += x * x + y * y;
+        }
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (e < 1024) e += ((__float_as_int(sqrtf(q) * 1.00001f) >> 23) & 255) - 126;
+        if (lane == 0) es[warp] = e;
+    }
+    bool bad = false;
+    for (int j = tid; j < n; j += CL_THREADS) bad |= rowbad[(size_t)k * n + j] != 0;
+    bad = __syncthreads_or(bad);
+    for (int t = tid; t < (int)vs; t += CL_THREADS) {
+        const int c = t / n, e = es[c];
+        const zd v = K.theta[t];
+        int2 p = make_int2(0, 0), q = make_int2(0, 0);
+        if (e < 1024) {
+            p = cs_split(cs_fix(v.x, e, 57));
+            q = cs_split(cs_fix(v.y, e, 57));
+        }
+        csm[t] = make_int4(p.x, p.y, q.x, q.y);
+    }
+    const bool own = act && lane < ns;
+    const int eo = lane < ns ? es[lane] : 0;
+    const size_t oe = i + (size_t)lane * n;
+    i64 y1r = 0, y1i = 0, y2r = 0, y2i = 0, sr = 0, si = 0;
+    if (own && eo < 1024) {
+        const zd t = K.theta[oe];
+        y1r = cs_fix(t.x, eo, 59);
+        y1i = cs_fix(t.y, eo, 59);
+        sr = cs_mul62(cf[0], y1r) - cs_mul62(cf[1], y1i);
+        si = cs_mul62(cf[0], y1i) + cs_mul62(cf[1], y1r);
+    }
+    // every block's mbarriers stand before anything is sent
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    __syncthreads();
+    bool ok = true;
+    if (act) {
+        for (int nt = 1; nt < a.nterms; ++nt) {
+            const bool last = nt == a.nterms - 1;
+            const int4* y = csm + ((nt - 1) & 1) * vs;
+            if (nt > 1) {
+                const int m = nt - 1;  // y_m
+                if (!cl_wait(&bar[m & 1], (unsigned)((m - 1) >> 1 & 1))) {
+                    ok = false;
+                    break;
+                }
+                // armed for y_(m + 2), which no warp sends before this block's y_(m + 1)
+                if (tid == 0)
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
+                                     (unsigned)__cvta_generic_to_shared(&bar[m & 1])),
+                                 "r"(bytes)
+                                 : "memory");
+            }
+#pragma unroll
+            for (int h = 0; h < NT; h += CW) {
+                i64 A[2 * CW], B[2 * CW];
+#pragma unroll
+                for (int v = 0; v < 2 * CW; ++v) A[v] = B[v] = 0;
+#pragma unroll
+                for (int u = 0; u < JU; ++u) {
+                    const int j = lane + 32 * u;
+                    if (j >= n) continue;
+#pragma unroll
+                    for (int q = 0; q < CW; ++q)
+                        if (h + q < ns) cs_mac(A + 2 * q, B + 2 * q, hr[u], hi[u], y[j + (size_t)(h + q) * n]);
+                }
+#pragma unroll
+                for (int v = 0; v < 2 * CW; ++v) A[v] += (B[v] + (1ll << 27)) >> 28;  // units 2^-59
+                warp_sum_store<i64, 2 * CW>(A, lane, &red[warp][2 * h]);
+            }
+            __syncwarp();
+            i64 yr = 0, yi = 0;
+            if (own) {
+                yr = red[warp][2 * lane];
+                yi = red[warp][2 * lane + 1];
+                if (nt > 1) {
+                    yr = 2 * yr - y2r;
+                    yi = 2 * yi - y2i;
+                }
+                y2r = y1r;
+                y2i = y1i;
+                y1r = yr;
+                y1i = yi;
+                const int2 p = cs_split((yr + 2) >> 2), q = cs_split((yi + 2) >> 2);
+                snd[warp][lane] = make_int4(p.x, p.y, q.x, q.y);
+            }
+            __syncwarp();
+            if (!last) {
+                const unsigned mb = (unsigned)__cvta_generic_to_shared(&bar[nt & 1]);
+                for (int t = lane; t < CL_N * ns; t += 32) {
+                    const int c = t / CL_N, d = t % CL_N;
+                    const int4 v = snd[warp][c];
+                    const unsigned dst = (unsigned)__cvta_generic_to_shared(csm + (nt & 1) * vs + i + (size_t)c * n);
+                    unsigned rd, rb;
+                    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(dst), "r"(d));
+                    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(mb), "r"(d));
+                    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(rd),
+                                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(rb)
+                                 : "memory");
+                }
+            }
+            if (own) {
+                const i64 cr = cf[2 * nt], ci = cf[2 * nt + 1];
+                sr += cs_mul62(cr, yr) - cs_mul62(ci, yi);
+                si += cs_mul62(cr, yi) + cs_mul62(ci, yr);
+            }
+        }
+        if (!ok && lane == 0) atomicOr(a.flag, 4);
+        if (ok && own) K.theta[oe] = cs_result(a, K, sr, si, eo, bad);
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // Chebyshev coefficients of the call, per k-point.
@@ -1448,7 +1843,6 @@ __device__ void finalize_body(const StepArgs& a, int set_gs) {
     st->rec_count = pre_rec + 1;
     st->gstep += 1;
     st->cstep += 1;
-    st->bar = 0u;  // the next step's cooperative series counts from zero
 }
 
 __global__ void __launch_bounds__(256) k_finalize(StepArgs a, int set_gs) { finalize_body(a, set_gs); }
@@ -1666,63 +2060,106 @@ void launch_phase_fix(const KDev* kd, int nk, int naux, zd* const* extra, const 
 }
 
 // ------------------------------------------------------------ orchestration
-// the cooperative series forms its own rows of HH when each block owns one
-// row and the row fits the registers of the block's threads
-int cheb_direct(const StepArgs& a) {
-    return (a.coop_grid >= a.nk * a.naux && a.naux <= CHEB_JU * CHEB_THREADS && a.ns <= 4) ? 1 : 0;
+static const void* cheb_coop_fn(const StepArgs& a) {
+    const bool two = a.naux <= 2 * CS_THREADS;
+    if (a.ns <= 2) return two ? (const void*)k_cheb_coop<2, 2> : (const void*)k_cheb_coop<2, 4>;
+    if (a.ns <= 4) return two ? (const void*)k_cheb_coop<4, 2> : (const void*)k_cheb_coop<4, 4>;
+    return two ? (const void*)k_cheb_coop<8, 2> : (const void*)k_cheb_coop<8, 4>;
 }
-// per-row state of the cooperative series: 3 ns complex per row of a block
-static size_t cheb_coop_smem(const StepArgs& a, int grid) {
-    const int nrow = a.nk * a.naux;
-    const int rows = grid > 0 ? (nrow + grid - 1) / grid : 0;
-    return (size_t)rows * 3 * a.ns * sizeof(zd);
+static const void* cheb_cl_fn(const StepArgs& a) {
+    return a.ns <= 2 ? (const void*)k_cheb_cl<2> : (a.ns <= 4 ? (const void*)k_cheb_cl<4> : (const void*)k_cheb_cl<8>);
 }
+// the cluster's shared memory: two slots of y and the coefficients
+static size_t cheb_cl_smem(const StepArgs& a, int nterms) { return ((size_t)2 * a.naux * a.ns + nterms) * sizeof(int4); }
+static size_t cheb_coop_smem(const StepArgs& a) { return (size_t)a.naux * a.ns * sizeof(int4); }
 static cudaError_t launch_cheb_coop_raw(const StepArgs& a, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.coop_grid);
-    cfg.blockDim = dim3(CHEB_THREADS);
-    cfg.dynamicSmemBytes = cheb_coop_smem(a, a.coop_grid);
-    cfg.stream = s;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
+    cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const int direct = cheb_direct(a);
-    if (a.ns <= 2) return cudaLaunchKernelEx(&cfg, k_cheb_coop<2>, a, direct);
-    if (a.ns <= 4) return cudaLaunchKernelEx(&cfg, k_cheb_coop<4>, a, direct);
-    return cudaLaunchKernelEx(&cfg, k_cheb_coop<8>, a, direct);
+    StepArgs arg = a;
+    if (a.cheb_cl) {
+        int* rowbad = (int*)a.cheb_sync;
+        k_cs_rows<<<dim3(a.naux, a.nk), 128, 0, s>>>(a, rowbad);
+        cfg.gridDim = dim3(CL_N * a.nk);
+        cfg.blockDim = dim3(CL_THREADS);
+        cfg.dynamicSmemBytes = cheb_cl_smem(a, a.nterms);
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CL_N;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        void* args[2] = {&arg, &rowbad};
+        return cudaLaunchKernelExC(&cfg, cheb_cl_fn(a), args);
+    }
+    cfg.gridDim = dim3(a.nk * a.naux);
+    cfg.blockDim = dim3(CS_THREADS);
+    cfg.dynamicSmemBytes = cheb_coop_smem(a);
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    ChebSync* sy = (ChebSync*)a.cheb_sync;
+    void* args[2] = {&arg, &sy};
+    return cudaLaunchKernelExC(&cfg, cheb_coop_fn(a), args);
 }
-void launch_cheb_coop(const StepArgs& a, cudaStream_t s) { launch_cheb_coop_raw(a, s); }
+int launch_cheb_coop(const StepArgs& a, cudaStream_t s) {
+    launch_cheb_coop_raw(a, s);
+    return a.cheb_cl ? 2 : 1;
+}
+size_t cheb_sync_bytes(int nk, int naux) { return std::max(sizeof(ChebSync), (size_t)nk * naux * sizeof(int)); }
 
-// Blocks for the cooperative series: all must be resident at once (the
-// launch guarantees it or fails), and the launch must be capturable in a
-// graph on this driver; otherwise 0 (one launch per term).
-int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s) {
+static cudaError_t grow_smem(const void* f, size_t bytes) {  // the attribute is shared by every context: never lowered
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaFuncGetAttributes(&fa, f);
+    if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// Blocks of the one-launch series for at most eight states, or 0; *cl: 1 for the
+// cluster form.  16 SMs take 1.4 cycles per product of a row's entry and a
+// column, so the cluster form is the faster one only while N_aux^2 N_s / 16 is
+// small (N_aux 32, N_s 8: 41 us a series against 57 of the grid form; N_aux 200,
+// N_s 2: 75 against 48; N_aux 240, N_s 7: 246 against 73).  The grid form has all
+// its blocks resident at once (the launch guarantees it or fails) and must be
+// capturable in a graph on this driver.
+#define CL_WORK 2000
+int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s, int* cl) {
     int dev = 0, coop = 0, nsm = 0, per_sm = 0;
+    *cl = 0;
+    if (a0.ns > 8 || a0.naux > 4 * CS_THREADS) return 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    StepArgs a = a0;
+    if (a.naux >= CL_N && a.naux <= CL_MAXN && (a.naux + CL_N - 1) / CL_N * a.naux * a.ns <= CL_WORK) {
+        const void* f = cheb_cl_fn(a);
+        const size_t sm = cheb_cl_smem(a, RTD_MAX_TERMS);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        cfg.gridDim = dim3(CL_N);
+        cfg.blockDim = dim3(CL_THREADS);
+        cfg.dynamicSmemBytes = sm;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CL_N;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int ncl = 0;
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            grow_smem(f, sm) == cudaSuccess && cudaOccupancyMaxActiveClusters(&ncl, f, &cfg) == cudaSuccess && ncl > 0) {
+            *cl = 1;
+            return CL_N * a.nk;
+        }
+        cudaGetLastError();
+    }
+    a.cheb_cl = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (!coop || nsm <= 0) return 0;
-    // one block per row while the rows last, at most four blocks per SM
-    // (more blocks would lengthen the barrier's arrival chain)
-    const int nrow = a0.nk * a0.naux;
-    int grid = nrow < 4 * nsm ? nrow : 4 * nsm;
-    const size_t smem = cheb_coop_smem(a0, grid);
-    const void* fn = a0.ns <= 2 ? (const void*)k_cheb_coop<2>
-                                : (a0.ns <= 4 ? (const void*)k_cheb_coop<4> : (const void*)k_cheb_coop<8>);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    const long long grid = (long long)a.nk * a.naux;
+    cudaError_t e = grow_smem(cheb_coop_fn(a), cheb_coop_smem(a));
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cheb_coop_fn(a), CS_THREADS, cheb_coop_smem(a));
+    if (e != cudaSuccess || per_sm <= 0 || grid > (long long)per_sm * nsm) {
         cudaGetLastError();
         return 0;
     }
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, CHEB_THREADS, smem);
-    if (e != cudaSuccess || per_sm <= 0 || grid > per_sm * nsm) {
-        cudaGetLastError();
-        return 0;
-    }
-    StepArgs a = a0;
-    a.coop_grid = grid;
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
@@ -1738,7 +2175,7 @@ int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s) {
     }
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
-    return ok ? grid : 0;
+    return ok ? (int)grid : 0;
 }
 
 void launch_set_cur(const StepArgs& a, cudaStream_t s) { k_set_cur<<<1, 1, 0, s>>>(a); }
@@ -2047,7 +2484,7 @@ void launch_step(const StepArgs& a, const StepPlan& p, cudaStream_t s, int* nlau
             nl += 1 + launch_dv_rebuild(a, p, s, tr);
         }
     }
-    if (!p.series && !(a.prop != 1 && a.coop_grid > 0 && cheb_direct(a))) {
+    if (!p.series && !(a.prop != 1 && a.coop_grid > 0)) {
         k_hsub<<<dim3((nn + 255) / 256, 1, a.nk), 256, 0, s>>>(a);
         mark(tr, "hsub", s);
         ++nl;
@@ -2064,9 +2501,8 @@ void launch_step(const StepArgs& a, const StepPlan& p, cudaStream_t s, int* nlau
         mark(tr, "eig_apply", s);
         nl += 4;
     } else if (a.coop_grid > 0) {
-        launch_cheb_coop(a, s);
+        nl += launch_cheb_coop(a, s);
         mark(tr, "chebyshev_series", s);
-        ++nl;
     } else {
         dim3 g(a.naux, 1, a.nk);
         for (int t = 1; t < a.nterms; ++t) {

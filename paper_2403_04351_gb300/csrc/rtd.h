@@ -141,6 +141,8 @@ struct StepArgs {
     zd* part_t;               // [nk][nslot][2 NT][maxng] slot partial sums
     int* flag;                // device error flags (bit 0 Jacobi, 1 bounds, 2 barrier)
     int coop_grid;            // blocks of the cooperative Chebyshev launch (0: per-term launches)
+    int cheb_cl;              // the series runs in one cluster per k-point
+    void* cheb_sync;          // barrier counters of the grid form (zero between launches), row flags of the cluster form
     int kofs;                 // k-point of kd[0] (single-k operator calls), 0 in the step
     int tcback;               // the back-projection runs on the tensor cores (split-BF16 form)
     int at_n, at_maxm;        // atoms, and the largest local block m = N_A + n_lo
@@ -238,9 +240,10 @@ void launch_step(const StepArgs& a, const StepPlan& p, cudaStream_t s, int* nlau
                  TraceHook* tr = nullptr);
 int launch_operator_pass(const StepArgs& a, const StepPlan& p, cudaStream_t s, TraceHook* tr = nullptr);
 int prepare_back_kernels(const StepArgs& a);
-// blocks for the cooperative Chebyshev launch if it can be captured in a graph, else 0
-int prepare_cheb_coop(const StepArgs& a, cudaStream_t s);
-void launch_cheb_coop(const StepArgs& a, cudaStream_t s);
+// blocks of the one-launch Chebyshev series for few states, or 0; cl: it runs in clusters
+int prepare_cheb_coop(const StepArgs& a, cudaStream_t s, int* cl);
+int launch_cheb_coop(const StepArgs& a, cudaStream_t s);
+size_t cheb_sync_bytes(int nk, int naux);
 void launch_prep_coef(const StepArgs& a, cudaStream_t s);
 void launch_subspace_current(const StepArgs& a, int set_gs, cudaStream_t s);
 void launch_set_cur(const StepArgs& a, cudaStream_t s);
