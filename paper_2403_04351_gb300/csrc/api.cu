@@ -55,6 +55,8 @@ struct rttddft_ctx {
     double tc_st = 1.0;         // its fp16 scale
     double *d_occ = nullptr, *d_wk = nullptr, *d_lam = nullptr;
     DevState* d_st = nullptr;
+    unsigned char* adj_ws = nullptr;  // workspace of the adjoint, kept between calls up to 256 MiB
+    size_t adj_cap = 0;
     unsigned char* d_cheb_sync = nullptr;
     int cheb_cl = 0;
     double* d_rec = nullptr;
@@ -2277,7 +2279,12 @@ int rttddft_trace_steps(rttddft_ctx* ctx, int nsteps, const double* a_samples, c
 int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const double* dv_scale,
                     const double* gdir, int ckpt_every, double* grad, double* dmu_out) {
     if (!ctx) return RTTDDFT_ERR_ARG;
-    std::vector<void*> tmp;
+    auto drop = [&] {
+        if (ctx->adj_cap <= ((size_t)256 << 20)) return;
+        dfree(ctx, ctx->adj_ws);
+        ctx->adj_ws = nullptr;
+        ctx->adj_cap = 0;
+    };
     DevState saved{};
     std::vector<zd*> theta_saved;
     bool restore = false;
@@ -2316,35 +2323,62 @@ int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const
         if (dv_scale) CK(cudaMemcpy(ctx->d_dvs, hs.data(), nsteps * sizeof(double), cudaMemcpyHostToDevice));
         // save the state the call must leave unchanged
         CK(cudaMemcpy(&saved, ctx->d_st, sizeof(DevState), cudaMemcpyDeviceToHost));
-        for (int k = 0; k < nk; ++k) {
-            zd* b = dalloc<zd>(ctx, vs);
-            tmp.push_back(b);
-            theta_saved.push_back(b);
-            CK(cudaMemcpy(b, ctx->hkd[k].theta, vs * sizeof(zd), cudaMemcpyDeviceToDevice));
-        }
-        restore = true;
         const int N = ctx->nterms;
-        const int K = ckpt_every;
+        const int K = std::min(ckpt_every, nsteps);
         const int nseg = (nsteps + K - 1) / K;
-        auto alloc = [&](size_t n) {
-            zd* p = dalloc<zd>(ctx, n);
-            tmp.push_back(p);
-            return p;
-        };
-        zd* ckpt = alloc((size_t)nseg * nk * vs);   // theta at the start of every segment
-        zd* hist = alloc((size_t)(K + 1) * nk * vs);  // theta over the current segment
-        zd* Yh = alloc((size_t)nk * N * vs);
-        zd* Yb = alloc((size_t)nk * N * vs);
-        zd* lam = alloc((size_t)nk * vs);
-        const int gblk = std::max(1, std::min(64, (naux * naux + 255) / 256));
-        double* gpart = dalloc<double>(ctx, (size_t)nk * gblk * 4);
-        tmp.push_back(gpart);
-        double* nrm = dalloc<double>(ctx, (size_t)nk * naux);
-        tmp.push_back(nrm);
         const int dv_on = dv_scale ? 1 : 0;
         StepArgs a = make_args(ctx, dv_on);
-        a.coop_grid = 0;
         StepPlan p = make_plan(ctx);
+        // few states: the segment's pass keeps the Chebyshev vectors of its steps and the reversed
+        // recurrence runs in one launch; otherwise one step's vectors at a time, a launch per term
+        bool fast = adj_series_fits(a);
+        const int gblk = std::max(1, std::min(304, (naux * naux + 255) / 256));
+        const size_t ng = (size_t)nk * gblk * 4, nn = (size_t)nk * naux;
+        if (fast && (size_t)K * nk * N * vs * sizeof(zd) > ((size_t)64 << 20)) {
+            size_t fr = 0, tot = 0;
+            CK(cudaMemGetInfo(&fr, &tot));
+            fast = (size_t)K * nk * N * vs * sizeof(zd) < fr / 4;
+        }
+        // one workspace, kept for the next call while it is small
+        unsigned char* ws = nullptr;
+        size_t off = 0;
+        auto take = [&](size_t bytes) {
+            const size_t at = off;
+            off += (bytes + 255) & ~(size_t)255;
+            return ws + at;
+        };
+        zd *th0 = nullptr, *ckpt = nullptr, *hist = nullptr, *Yh = nullptr, *Yb = nullptr, *lam = nullptr;
+        double *gpart = nullptr, *nrm = nullptr, *jdev = nullptr;
+        void* sync = nullptr;
+        for (int pass = 0; pass < 2; ++pass) {
+            off = 0;
+            th0 = (zd*)take((size_t)nk * vs * sizeof(zd));                 // the state to leave unchanged
+            ckpt = (zd*)take((size_t)nseg * nk * vs * sizeof(zd));         // theta at the start of every segment
+            hist = (zd*)take((size_t)(K + 1) * nk * vs * sizeof(zd));      // theta over the current segment
+            Yh = (zd*)take((size_t)(fast ? K : 1) * nk * N * vs * sizeof(zd));
+            Yb = (zd*)take((size_t)nk * N * vs * sizeof(zd));
+            lam = (zd*)take((size_t)nk * vs * sizeof(zd));
+            // per step of a segment, and of the whole pass the current: read back once
+            gpart = (double*)take((size_t)K * ng * sizeof(double));
+            nrm = (double*)take((size_t)K * nn * sizeof(double));
+            jdev = (double*)take(3 * (size_t)nsteps * sizeof(double));
+            sync = take(adj_sync_bytes());
+            if (pass) break;
+            if (off > ctx->adj_cap) {
+                dfree(ctx, ctx->adj_ws);
+                ctx->adj_ws = nullptr;
+                ctx->adj_cap = 0;
+                ctx->adj_ws = dalloc<unsigned char>(ctx, off);
+                ctx->adj_cap = off;
+            }
+            ws = ctx->adj_ws;
+        }
+        CK(cudaMemsetAsync(sync, 0, adj_sync_bytes(), st));
+        for (int k = 0; k < nk; ++k) {
+            theta_saved.push_back(th0 + (size_t)k * vs);
+            CK(cudaMemcpyAsync(theta_saved[k], ctx->hkd[k].theta, vs * sizeof(zd), cudaMemcpyDeviceToDevice, st));
+        }
+        restore = true;
         auto copy_theta = [&](zd* dst /* nk * vs */, bool to_theta) {
             for (int k = 0; k < nk; ++k) {
                 if (to_theta) CK(cudaMemcpyAsync(ctx->hkd[k].theta, dst + (size_t)k * vs, vs * sizeof(zd), cudaMemcpyDeviceToDevice, st));
@@ -2352,96 +2386,101 @@ int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const
             }
         };
         const double om = ctx->omega, dt = ctx->opt.dt, c = ctx->c;
-        // current of the propagated theta at t_m (host sum of the row partials)
-        std::vector<double> post((size_t)nk * naux * POST_STRIDE), wk(nk);
-        CK(cudaMemcpy(wk.data(), ctx->d_wk, nk * sizeof(double), cudaMemcpyDeviceToHost));
-        auto current = [&](double out[3]) {
-            launch_subspace_j(a, st);
-            KCHECK();
-            CK(cudaMemcpyAsync(post.data(), ctx->d_part_post, post.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
-            for (int l = 0; l < 3; ++l) {
-                double v = 0.0;
-                for (int k = 0; k < nk; ++k)
-                    for (int i = 0; i < naux; ++i) v += wk[k] * post[((size_t)k * naux + i) * POST_STRIDE + 1 + l];
-                out[l] = -v / om;
-            }
-        };
-        // ---- forward pass: checkpoints and the dipole increment
-        double dmu[3] = {0, 0, 0}, jprev[3] = {saved.jind_prev[0], saved.jind_prev[1], saved.jind_prev[2]};
+        // ---- forward pass: checkpoints and the current of every step (its sample is that of the step just taken)
         for (int m = 0; m < nsteps; ++m) {
             if (m % K == 0) copy_theta(ckpt + (size_t)(m / K) * nk * vs, false);
-            // the current uses the sample of the step just taken
-            launch_propagate_only(a, p, m, st);
+            launch_propagate_only(a, p, m, nullptr, nullptr, st);
+            launch_subspace_j(a, st);
+            launch_adj_current(a, jdev + 3 * (size_t)m, st);
             KCHECK();
-            double J[3];
-            current(J);
-            for (int l = 0; l < 3; ++l) {
-                const double jind = J[l] - saved.j_gs[l];
-                dmu[l] += om * dt * 0.5 * (jprev[l] + jind);
-                jprev[l] = jind;
-            }
         }
-        if (dmu_out)
-            for (int l = 0; l < 3; ++l) dmu_out[l] = dmu[l];
         // ---- reverse sweep, segment by segment
         for (size_t q = 0; q < na; ++q) grad[q] = 0.0;
         launch_zero(lam, (size_t)nk * vs, st);
-        std::vector<double> hg((size_t)nk * gblk * 4), hn((size_t)nk * naux), lamh(2 * nk);
+        std::vector<double> hg((size_t)K * ng), hn((size_t)K * nn);
         std::vector<double> lamc(LAM_N * nk);
-        CK(cudaMemcpy(lamc.data(), ctx->d_lam, lamc.size() * sizeof(double), cudaMemcpyDeviceToHost));
+        CK(cudaMemcpyAsync(lamc.data(), ctx->d_lam, lamc.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
         for (int sg = nseg - 1; sg >= 0; --sg) {
             const int s0 = sg * K, s1 = std::min(nsteps, s0 + K);
             copy_theta(ckpt + (size_t)sg * nk * vs, true);
             copy_theta(hist, false);
             for (int m = s0; m < s1; ++m) {
-                launch_propagate_only(a, p, m, st);
+                launch_propagate_only(a, p, m, sync, fast ? Yh + (size_t)(m - s0) * nk * N * vs : nullptr, st);
                 copy_theta(hist + (size_t)(m - s0 + 1) * nk * vs, false);
             }
             KCHECK();
             for (int m = s1; m > s0; --m) {
                 const double* am = ha.data() + 3 * (size_t)(m - 1);
+                const size_t q = (size_t)(m - 1 - s0);  // the step within the segment
                 // source from J(t_m): weight of t_m in the trapezoid sum of dmu
                 const double wm = om * dt * (m == nsteps ? 0.5 : 1.0);
                 const double sm = (gdir[0] * am[0] + gdir[1] * am[1] + gdir[2] * am[2]) / c;
-                launch_adj_jterm(a, lam, hist + (size_t)(m - s0) * nk * vs, gdir, sm, -2.0 * wm / om, nrm, st);
+                launch_adj_jterm(a, lam, hist + (q + 1) * nk * vs, gdir, sm, -2.0 * wm / om, nrm + q * nn, st);
+                // propagator of step m-1 (its sample, its potential change)
+                launch_hsub_only(a, p, m - 1, !fast, st);
+                zd* Y = Yh;
+                if (fast) {
+                    Y = Yh + q * nk * N * vs;
+                    launch_adj_series(a, sync, Yb, lam, st);
+                } else {
+                    // recompute the Chebyshev vectors from theta_{m-1}
+                    for (int k = 0; k < nk; ++k)
+                        CK(cudaMemcpyAsync(Yh + (size_t)k * N * vs, hist + q * nk * vs + (size_t)k * vs, vs * sizeof(zd),
+                                           cudaMemcpyDeviceToDevice, st));
+                    for (int t = 1; t < N; ++t) launch_adj_fwd_term(a, Yh, N, t, st);
+                    launch_adj_bwd_init(a, Yb, lam, N, st);
+                    for (int t = N - 1; t >= 1; --t) launch_adj_bwd_term(a, Yb, N, t, st);
+                }
+                launch_adj_grad(a, Y, Yb, N, gpart + q * ng, gblk, st);
+                if (!fast)
+                    // lam_{m-1} = theta-bar = ybar_0
+                    for (int k = 0; k < nk; ++k)
+                        CK(cudaMemcpyAsync(lam + (size_t)k * vs, Yb + (size_t)k * N * vs, vs * sizeof(zd),
+                                           cudaMemcpyDeviceToDevice, st));
                 KCHECK();
-                CK(cudaMemcpyAsync(hn.data(), nrm, hn.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-                // propagator of step m-1: recompute the Chebyshev vectors from theta_{m-1}
-                launch_hsub_only(a, p, m - 1, st);
-                for (int k = 0; k < nk; ++k)
-                    CK(cudaMemcpyAsync(Yh + (size_t)k * N * vs, hist + (size_t)(m - 1 - s0) * nk * vs + (size_t)k * vs,
-                                       vs * sizeof(zd), cudaMemcpyDeviceToDevice, st));
-                for (int t = 1; t < N; ++t) launch_adj_fwd_term(a, Yh, N, t, st);
-                launch_adj_bwd_init(a, Yb, lam, N, st);
-                for (int t = N - 1; t >= 1; --t) launch_adj_bwd_term(a, Yb, N, t, st);
-                launch_adj_grad(a, Yh, Yb, N, gpart, gblk, st);
-                KCHECK();
-                CK(cudaMemcpyAsync(hg.data(), gpart, hg.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-                // lam_{m-1} = theta-bar = ybar_0
-                for (int k = 0; k < nk; ++k)
-                    CK(cudaMemcpyAsync(lam + (size_t)k * vs, Yb + (size_t)k * N * vs, vs * sizeof(zd),
-                                       cudaMemcpyDeviceToDevice, st));
-                CK(cudaStreamSynchronize(st));
+            }
+            const size_t cnt = (size_t)(s1 - s0);
+            CK(cudaMemcpyAsync(hg.data(), gpart, cnt * ng * sizeof(double), cudaMemcpyDeviceToHost, st));
+            CK(cudaMemcpyAsync(hn.data(), nrm, cnt * nn * sizeof(double), cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            for (int m = s1; m > s0; --m) {
+                const double* am = ha.data() + 3 * (size_t)(m - 1);
+                const size_t q = (size_t)(m - 1 - s0);
+                const double wm = om * dt * (m == nsteps ? 0.5 : 1.0);
                 double nm = 0.0;
-                for (double x : hn) nm += x;
+                for (size_t x = 0; x < nn; ++x) nm += hn[q * nn + x];
                 for (int l = 0; l < 3; ++l) grad[3 * (size_t)(m - 1) + l] += wm * gdir[l] * (-1.0 / om) * nm / c;
                 for (int k = 0; k < nk; ++k) {
                     double acc[4] = {0, 0, 0, 0};
                     for (int b = 0; b < gblk; ++b)
-                        for (int q = 0; q < 4; ++q) acc[q] += hg[((size_t)k * gblk + b) * 4 + q];
+                        for (int x = 0; x < 4; ++x) acc[x] += hg[q * ng + ((size_t)k * gblk + b) * 4 + x];
                     const double ilh = lamc[LAM_N * k + 2];
                     for (int l = 0; l < 3; ++l)
                         grad[3 * (size_t)(m - 1) + l] += ilh * (acc[l] / c + am[l] / (c * c) * acc[3]);
                 }
             }
         }
+        {
+            // the dipole increment from the currents of the forward pass
+            std::vector<double> hj(3 * (size_t)nsteps);
+            CK(cudaMemcpy(hj.data(), jdev, hj.size() * sizeof(double), cudaMemcpyDeviceToHost));
+            double dmu[3] = {0, 0, 0}, jprev[3] = {saved.jind_prev[0], saved.jind_prev[1], saved.jind_prev[2]};
+            for (int m = 0; m < nsteps; ++m)
+                for (int l = 0; l < 3; ++l) {
+                    const double jind = -hj[3 * (size_t)m + l] / om - saved.j_gs[l];
+                    dmu[l] += om * dt * 0.5 * (jprev[l] + jind);
+                    jprev[l] = jind;
+                }
+            if (dmu_out)
+                for (int l = 0; l < 3; ++l) dmu_out[l] = dmu[l];
+        }
+        sync_and_check(ctx);  // a wait that ran out in a series
         // ---- restore
         for (int k = 0; k < nk; ++k)
             CK(cudaMemcpy(ctx->hkd[k].theta, theta_saved[k], vs * sizeof(zd), cudaMemcpyDeviceToDevice));
         CK(cudaMemcpy(ctx->d_st, &saved, sizeof(DevState), cudaMemcpyHostToDevice));
         restore = false;
-        for (void* q : tmp) dfree(ctx, q);
+        drop();
         return RTTDDFT_OK;
     } catch (Fail& f) {
         if (restore) {
@@ -2450,7 +2489,7 @@ int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const
                            cudaMemcpyDeviceToDevice);
             cudaMemcpy(ctx->d_st, &saved, sizeof(DevState), cudaMemcpyHostToDevice);
         }
-        for (void* q : tmp) dfree(ctx, q);
+        drop();
         return f.code;
     }
 }

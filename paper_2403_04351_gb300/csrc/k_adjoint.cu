@@ -176,6 +176,25 @@ __global__ void __launch_bounds__(256) k_adj_jterm(StepArgs a, zd* __restrict__ 
     if (lane == 0) nrm[(size_t)k * n + i] = nr;
 }
 
+// sum_k w_k of the rows' shares of J_sub (k_post, k_jrho), in the order of (k, row)
+__global__ void __launch_bounds__(256) k_adj_current(StepArgs a, double* __restrict__ out) {
+    __shared__ double sh[8][3];
+    double v[3] = {0.0, 0.0, 0.0};
+    for (int e = threadIdx.x; e < a.nk * a.naux; e += 256)
+        for (int l = 0; l < 3; ++l) v[l] += a.wk[e / a.naux] * a.part_post[(size_t)e * POST_STRIDE + 1 + l];
+    for (int l = 0; l < 3; ++l) {
+        v[l] = warp_sum(v[l]);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][l] = v[l];
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += sh[w][threadIdx.x];
+        out[threadIdx.x] = t;
+    }
+}
+
+void launch_adj_current(const StepArgs& a, double* out, cudaStream_t s) { k_adj_current<<<1, 256, 0, s>>>(a, out); }
 void launch_adj_fwd_term(const StepArgs& a, zd* Yh, int nterm, int nt, cudaStream_t s) {
     k_adj_fwd_term<<<dim3(a.naux, 1, a.nk), 128, 0, s>>>(a, Yh, nterm, nt);
 }

@@ -286,9 +286,11 @@ __device__ __forceinline__ int4 cs_hentry(const StepArgs& a, const KDev& K, cons
 
 // NT columns (N_s <= NT), JU entries of the row per thread.  The thread's entries of
 // y_(n-1) come into its part of shared memory all at once (cp.async: no registers
-// for loads in flight).
-template <int NT, int JU>
-__global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepArgs a, ChebSync* sy) {
+// for loads in flight).  MODE 0: the series of theta.  The adjoint's forms: MODE 1
+// also keeps y_0 .. y_(N - 2) in hist ([k][N][N_s][N_aux]), MODE 2 runs the reversed
+// recurrence from vec (see k_adjoint.cu), keeps every ybar_n and leaves ybar_0 in vec.
+template <int NT, int JU, int MODE>
+__global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepArgs a, ChebSync* sy, zd* hist, zd* vec) {
     constexpr int CW = NT < 4 ? NT : 4;  // columns at a time (registers)
     constexpr int V = 2 * NT;
     extern __shared__ int4 ysm[];  // [N_s][N_aux]
@@ -296,11 +298,13 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
     __shared__ i64 cf[CS_MAXC][2];
     __shared__ int smx[CS_THREADS / 32][NT];
     __shared__ float snm[CS_THREADS / 32][NT];
+    __shared__ int smg;
     const int n = a.naux, ns = a.ns;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const size_t vs = (size_t)n * ns;
     const int k = blockIdx.x / n, i = blockIdx.x % n;
     const KDev& K = a.kd[k];
+    const zd* th = MODE == 2 ? vec + (size_t)k * vs : K.theta;
     int2 hr[JU], hi[JU];
     {
         // row i of HH(t_k) (Eq. auxiliary_hamiltonian_with_parts)
@@ -318,9 +322,29 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
             __threadfence();
         }
     }
-    for (int t = tid; t < min(a.nterms, CS_MAXC); t += CS_THREADS) {
-        cf[t][0] = __double2ll_rn(K.coef[t].x * 4611686018427387904.0);
-        cf[t][1] = __double2ll_rn(K.coef[t].y * 4611686018427387904.0);
+    auto coef = [&](int t0) {  // c_n, or conj(beta c_(N - 1 - n)) of the reverse sweep, in units 2^-62
+        for (int t = tid; t < min(a.nterms - t0, CS_MAXC); t += CS_THREADS) {
+            zd c = K.coef[MODE == 2 ? a.nterms - 1 - t0 - t : t0 + t];
+            if (MODE == 2) {
+                if (a.prop == 0) c = zmul(zmk(K.lam[3], K.lam[4]), c);
+                c.y = -c.y;
+            }
+            cf[t][0] = __double2ll_rn(c.x * 4611686018427387904.0);
+            cf[t][1] = __double2ll_rn(c.y * 4611686018427387904.0);
+        }
+    };
+    coef(0);
+    int margin = 0;
+    if (MODE == 2) {
+        // |ybar_n| <= sum_m (m + 1) |c_m| |o|: the power of two above the sum widens the scale
+        if (warp == 0) {
+            float q = 0.f;
+            for (int t = lane; t < a.nterms; t += 32) q += (float)(t + 1) * ((float)fabs(K.coef[t].x) + (float)fabs(K.coef[t].y));
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            if (lane == 0) smg = max(0, ((__float_as_int(q) >> 23) & 255) - 126);
+        }
+        __syncthreads();
+        margin = smg;
     }
     // the scale of every column of theta: the power of two above its 2-norm
     int e[NT];
@@ -334,7 +358,7 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
 #pragma unroll
             for (int c = 0; c < NT; ++c) {
                 if (j >= n || c >= ns) continue;
-                const zd t = K.theta[j + (size_t)c * n];
+                const zd t = th[j + (size_t)c * n];
                 mx[c] = max(mx[c], max(__double2hiint(t.x) & 0x7fffffff, __double2hiint(t.y) & 0x7fffffff));
             }
         }
@@ -359,7 +383,7 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
 #pragma unroll
             for (int c = 0; c < NT; ++c) {
                 if (j >= n || c >= ns) continue;
-                const zd t = K.theta[j + (size_t)c * n];
+                const zd t = th[j + (size_t)c * n];
                 const float x = cs_small(t.x, e[c]), y = cs_small(t.y, e[c]);
                 q[c] += x * x + y * y;
             }
@@ -376,7 +400,7 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
 #pragma unroll
             for (int w = 0; w < CS_THREADS / 32; ++w) t += snm[w][c];
             // a column that is not finite: e = 1024 and more, answered with NaN at the end
-            if (e[c] < 1024) e[c] += ((__float_as_int(sqrtf(t) * 1.00001f) >> 23) & 255) - 126;
+            if (e[c] < 1024) e[c] += ((__float_as_int(sqrtf(t) * 1.00001f) >> 23) & 255) - 126 + margin;
         }
     }
     // the block's own entries of the recurrence: thread c of the first warp
@@ -388,13 +412,30 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
         if (oc == c) eo = e[c];
     const size_t oe = i + (size_t)oc * n;
     i64 y1r = 0, y1i = 0, y2r = 0, y2i = 0, sr = 0, si = 0;
+    i64 orr = 0, oi = 0;  // the source's entry (reverse sweep)
     if (own && eo < 1024) {
-        const zd t = K.theta[oe];
+        const zd t = th[oe];
         y1r = cs_fix(t.x, eo, 59);
         y1i = cs_fix(t.y, eo, 59);
         sr = cs_mul62(cf[0][0], y1r) - cs_mul62(cf[0][1], y1i);
         si = cs_mul62(cf[0][0], y1i) + cs_mul62(cf[0][1], y1r);
+        if (MODE == 2) {
+            orr = y1r;
+            oi = y1i;
+            y1r = sr;
+            y1i = si;
+        }
     }
+    // y_n as doubles (the adjoint's history)
+    const int hs = min(eo, 1024) - 59;
+    const double hp1 = cs_pow2(hs / 2), hp2 = cs_pow2(hs - hs / 2);
+    auto keep = [&](int t, i64 yr, i64 yi) {
+        zd v = zmk(((double)yr * hp1) * hp2, ((double)yi * hp1) * hp2);
+        if (eo >= 1024 || *(volatile unsigned*)&sy->bad != 0u) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+        hist[((size_t)k * a.nterms + t) * vs + oe] = v;
+        return v;
+    };
+    if (MODE != 0 && own) keep(MODE == 1 ? 0 : a.nterms - 1, y1r, y1i);
     unsigned mycnt = 0;  // blocks that arrive at the counter this lane polls
     if (lane < CS_CNT) mycnt = (gridDim.x - lane + CS_CNT - 1) / CS_CNT;
     int4* ring = (int4*)K.ring;
@@ -404,10 +445,7 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
         const int4* yin = ring + ((nt - 1) & 1) * vs;
         if (nt >= CS_MAXC && nt % CS_MAXC == 0) {
             __syncthreads();
-            for (int t = tid; t < min(a.nterms - nt, CS_MAXC); t += CS_THREADS) {
-                cf[t][0] = __double2ll_rn(K.coef[nt + t].x * 4611686018427387904.0);
-                cf[t][1] = __double2ll_rn(K.coef[nt + t].y * 4611686018427387904.0);
-            }
+            coef(nt);
             __syncthreads();
         }
 #pragma unroll
@@ -424,8 +462,13 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
                 } else {
                     *d = make_int4(0, 0, 0, 0);
                     if (e[c] < 1024) {
-                        const zd t = K.theta[j + (size_t)c * n];
-                        const int2 p = cs_split(cs_fix(t.x, e[c], 57)), r = cs_split(cs_fix(t.y, e[c], 57));
+                        const zd t = th[j + (size_t)c * n];
+                        int2 p = cs_split(cs_fix(t.x, e[c], 57)), r = cs_split(cs_fix(t.y, e[c], 57));
+                        if (MODE == 2) {
+                            const i64 x = cs_fix(t.x, e[c], 59), y = cs_fix(t.y, e[c], 59);
+                            p = cs_split((cs_mul62(cf[0][0], x) - cs_mul62(cf[0][1], y) + 2) >> 2);
+                            r = cs_split((cs_mul62(cf[0][0], y) + cs_mul62(cf[0][1], x) + 2) >> 2);
+                        }
                         *d = make_int4(p.x, p.y, r.x, r.y);
                     }
                 }
@@ -460,7 +503,12 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
                     yr += red[w][2 * tid];
                     yi += red[w][2 * tid + 1];
                 }
-                if (nt > 1) {
+                const i64 cr = cf[nt % CS_MAXC][0], ci = cf[nt % CS_MAXC][1];
+                if (MODE == 2) {
+                    // ybar_m = conj(beta c_m) o + 2 H~ ybar_(m + 1) - ybar_(m + 2), once H~ for m = 0
+                    yr = (last ? yr : 2 * yr) - y2r + cs_mul62(cr, orr) - cs_mul62(ci, oi);
+                    yi = (last ? yi : 2 * yi) - y2i + cs_mul62(cr, oi) + cs_mul62(ci, orr);
+                } else if (nt > 1) {
                     yr = 2 * yr - y2r;
                     yi = 2 * yi - y2i;
                 }
@@ -481,9 +529,16 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
                                  : "memory");
             }
             if (own) {
-                const i64 cr = cf[nt % CS_MAXC][0], ci = cf[nt % CS_MAXC][1];
-                sr += cs_mul62(cr, yr) - cs_mul62(ci, yi);
-                si += cs_mul62(cr, yi) + cs_mul62(ci, yr);
+                if (MODE != 2) {
+                    const i64 cr = cf[nt % CS_MAXC][0], ci = cf[nt % CS_MAXC][1];
+                    sr += cs_mul62(cr, yr) - cs_mul62(ci, yi);
+                    si += cs_mul62(cr, yi) + cs_mul62(ci, yr);
+                }
+                if (MODE == 1 && !last) keep(nt, y1r, y1i);
+                if (MODE == 2) {
+                    const zd v = keep(a.nterms - 1 - nt, y1r, y1i);
+                    if (last) vec[(size_t)k * vs + oe] = v;  // theta-bar
+                }
             }
             if (!last) {
                 const unsigned want = mycnt * (unsigned)nt;
@@ -506,7 +561,7 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
     }
     if (!ok && tid == 0) atomicOr(a.flag, 4);
     // (every block read theta before it wrote its y_1, so theta may be written now)
-    if (ok && own) {
+    if (MODE != 2 && ok && own) {
         K.theta[oe] = cs_result(a, K, sr, si, eo, *(volatile unsigned*)&sy->bad != 0u);
     }
     __syncthreads();
@@ -2060,11 +2115,12 @@ void launch_phase_fix(const KDev* kd, int nk, int naux, zd* const* extra, const 
 }
 
 // ------------------------------------------------------------ orchestration
+template <int MODE>
 static const void* cheb_coop_fn(const StepArgs& a) {
     const bool two = a.naux <= 2 * CS_THREADS;
-    if (a.ns <= 2) return two ? (const void*)k_cheb_coop<2, 2> : (const void*)k_cheb_coop<2, 4>;
-    if (a.ns <= 4) return two ? (const void*)k_cheb_coop<4, 2> : (const void*)k_cheb_coop<4, 4>;
-    return two ? (const void*)k_cheb_coop<8, 2> : (const void*)k_cheb_coop<8, 4>;
+    if (a.ns <= 2) return two ? (const void*)k_cheb_coop<2, 2, MODE> : (const void*)k_cheb_coop<2, 4, MODE>;
+    if (a.ns <= 4) return two ? (const void*)k_cheb_coop<4, 2, MODE> : (const void*)k_cheb_coop<4, 4, MODE>;
+    return two ? (const void*)k_cheb_coop<8, 2, MODE> : (const void*)k_cheb_coop<8, 4, MODE>;
 }
 static const void* cheb_cl_fn(const StepArgs& a) {
     return a.ns <= 2 ? (const void*)k_cheb_cl<2> : (a.ns <= 4 ? (const void*)k_cheb_cl<4> : (const void*)k_cheb_cl<8>);
@@ -2072,33 +2128,41 @@ static const void* cheb_cl_fn(const StepArgs& a) {
 // the cluster's shared memory: two slots of y and the coefficients
 static size_t cheb_cl_smem(const StepArgs& a, int nterms) { return ((size_t)2 * a.naux * a.ns + nterms) * sizeof(int4); }
 static size_t cheb_coop_smem(const StepArgs& a) { return (size_t)a.naux * a.ns * sizeof(int4); }
+template <int MODE>
+static cudaError_t launch_cheb_grid(const StepArgs& a, void* sync, zd* hist, zd* vec, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(a.nk * a.naux);
+    cfg.blockDim = dim3(CS_THREADS);
+    cfg.dynamicSmemBytes = cheb_coop_smem(a);
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    StepArgs arg = a;
+    ChebSync* sy = (ChebSync*)sync;
+    void* args[4] = {&arg, &sy, &hist, &vec};
+    return cudaLaunchKernelExC(&cfg, cheb_coop_fn<MODE>(a), args);
+}
 static cudaError_t launch_cheb_coop_raw(const StepArgs& a, cudaStream_t s) {
+    if (!a.cheb_cl) return launch_cheb_grid<0>(a, a.cheb_sync, nullptr, nullptr, s);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     StepArgs arg = a;
-    if (a.cheb_cl) {
-        int* rowbad = (int*)a.cheb_sync;
-        k_cs_rows<<<dim3(a.naux, a.nk), 128, 0, s>>>(a, rowbad);
-        cfg.gridDim = dim3(CL_N * a.nk);
-        cfg.blockDim = dim3(CL_THREADS);
-        cfg.dynamicSmemBytes = cheb_cl_smem(a, a.nterms);
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = CL_N;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        void* args[2] = {&arg, &rowbad};
-        return cudaLaunchKernelExC(&cfg, cheb_cl_fn(a), args);
-    }
-    cfg.gridDim = dim3(a.nk * a.naux);
-    cfg.blockDim = dim3(CS_THREADS);
-    cfg.dynamicSmemBytes = cheb_coop_smem(a);
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    ChebSync* sy = (ChebSync*)a.cheb_sync;
-    void* args[2] = {&arg, &sy};
-    return cudaLaunchKernelExC(&cfg, cheb_coop_fn(a), args);
+    int* rowbad = (int*)a.cheb_sync;
+    k_cs_rows<<<dim3(a.naux, a.nk), 128, 0, s>>>(a, rowbad);
+    cfg.gridDim = dim3(CL_N * a.nk);
+    cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = cheb_cl_smem(a, a.nterms);
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL_N;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    void* args[2] = {&arg, &rowbad};
+    return cudaLaunchKernelExC(&cfg, cheb_cl_fn(a), args);
 }
 int launch_cheb_coop(const StepArgs& a, cudaStream_t s) {
     launch_cheb_coop_raw(a, s);
@@ -2113,6 +2177,18 @@ static cudaError_t grow_smem(const void* f, size_t bytes) {  // the attribute is
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// whether all blocks of the grid form are resident at once
+static bool grid_fits(const void* f, const StepArgs& a, int nsm) {
+    int per_sm = 0;
+    cudaError_t e = grow_smem(f, cheb_coop_smem(a));
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, CS_THREADS, cheb_coop_smem(a));
+    if (e != cudaSuccess || (long long)a.nk * a.naux > (long long)per_sm * nsm) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
 // Blocks of the one-launch series for at most eight states, or 0; *cl: 1 for the
 // cluster form.  16 SMs take 1.4 cycles per product of a row's entry and a
 // column, so the cluster form is the faster one only while N_aux^2 N_s / 16 is
@@ -2122,7 +2198,7 @@ static cudaError_t grow_smem(const void* f, size_t bytes) {  // the attribute is
 // capturable in a graph on this driver.
 #define CL_WORK 2000
 int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s, int* cl) {
-    int dev = 0, coop = 0, nsm = 0, per_sm = 0;
+    int dev = 0, coop = 0, nsm = 0;
     *cl = 0;
     if (a0.ns > 8 || a0.naux > 4 * CS_THREADS) return 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -2152,14 +2228,7 @@ int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s, int* cl) {
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (!coop || nsm <= 0) return 0;
-    const long long grid = (long long)a.nk * a.naux;
-    cudaError_t e = grow_smem(cheb_coop_fn(a), cheb_coop_smem(a));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cheb_coop_fn(a), CS_THREADS, cheb_coop_smem(a));
-    if (e != cudaSuccess || per_sm <= 0 || grid > (long long)per_sm * nsm) {
-        cudaGetLastError();
-        return 0;
-    }
+    if (!grid_fits(cheb_coop_fn<0>(a), a, nsm)) return 0;
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
@@ -2175,7 +2244,21 @@ int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s, int* cl) {
     }
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
-    return ok ? (int)grid : 0;
+    return ok ? a.nk * a.naux : 0;
+}
+
+// the grid form's launches of the adjoint (not captured): whether they can run
+bool adj_series_fits(const StepArgs& a) {
+    int dev = 0, coop = 0, nsm = 0;
+    if (a.ns > 8 || a.naux > 4 * CS_THREADS || cudaGetDevice(&dev) != cudaSuccess) return false;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return coop && grid_fits(cheb_coop_fn<1>(a), a, nsm) && grid_fits(cheb_coop_fn<2>(a), a, nsm);
+}
+size_t adj_sync_bytes() { return sizeof(ChebSync); }
+void launch_adj_series(const StepArgs& a, void* sync, zd* hist, zd* vec, cudaStream_t s) {
+    if (vec) launch_cheb_grid<2>(a, sync, hist, vec, s);
+    else launch_cheb_grid<1>(a, sync, hist, vec, s);
 }
 
 void launch_set_cur(const StepArgs& a, cudaStream_t s) { k_set_cur<<<1, 1, 0, s>>>(a); }
@@ -2591,32 +2674,40 @@ void launch_check_samples(const double* a, int na, double amax, const double* s,
 __global__ void k_set_cstep(DevState* st, int c) { st->cstep = c; }
 
 // The subspace part of a step only (HH(t_k) and its Chebyshev series, one
-// launch per term): what the adjoint recomputes.  cstep selects the sample.
-void launch_propagate_only(const StepArgs& a, const StepPlan& p, int cstep, cudaStream_t s) {
+// launch per term): what the adjoint recomputes.  cstep selects the sample; with
+// hist the series keeps its y_n there.
+void launch_propagate_only(const StepArgs& a, const StepPlan& p, int cstep, void* sync, zd* hist, cudaStream_t s) {
     k_set_cstep<<<1, 1, 0, s>>>(a.st, cstep);
     if (a.dv_on) {
         k_set_cur<<<1, 1, 0, s>>>(a);
         k_vstep<<<(a.nvt + 255) / 256, 256, 0, s>>>(a);
         launch_dv_rebuild(a, p, s, nullptr);
     }
-    k_hsub<<<dim3((a.naux * a.naux + 255) / 256, 1, a.nk), 256, 0, s>>>(a);
-    dim3 g(a.naux, 1, a.nk);
-    for (int t = 1; t < a.nterms; ++t) {
-        const int last = (t == a.nterms - 1);
-        if (a.ns <= 2) k_cheb<2><<<g, 128, 0, s>>>(a, t, last);
-        else if (a.ns <= 4) k_cheb<4><<<g, 128, 0, s>>>(a, t, last);
-        else k_cheb<8><<<g, 128, 0, s>>>(a, t, last);
+    if (hist) {
+        launch_adj_series(a, sync, hist, nullptr, s);
+    } else if (p.series) {
+        launch_dg_series(p.series, a, s);
+    } else if (a.coop_grid > 0) {
+        launch_cheb_coop(a, s);
+    } else {
+        k_hsub<<<dim3((a.naux * a.naux + 255) / 256, 1, a.nk), 256, 0, s>>>(a);
+        dim3 g(a.naux, 1, a.nk);
+        for (int t = 1; t < a.nterms; ++t) {
+            const int last = (t == a.nterms - 1);
+            if (a.ns <= 2) k_cheb<2><<<g, 128, 0, s>>>(a, t, last);
+            else if (a.ns <= 4) k_cheb<4><<<g, 128, 0, s>>>(a, t, last);
+            else k_cheb<8><<<g, 128, 0, s>>>(a, t, last);
+        }
     }
 }
-
 // HH(t_k) only (the adjoint's reverse sweep needs the matrix of step cstep)
-void launch_hsub_only(const StepArgs& a, const StepPlan& p, int cstep, cudaStream_t s) {
+void launch_hsub_only(const StepArgs& a, const StepPlan& p, int cstep, bool form, cudaStream_t s) {
     k_set_cstep<<<1, 1, 0, s>>>(a.st, cstep);
     if (a.dv_on) {
         k_set_cur<<<1, 1, 0, s>>>(a);
         launch_dv_rebuild(a, p, s, nullptr);
     }
-    k_hsub<<<dim3((a.naux * a.naux + 255) / 256, 1, a.nk), 256, 0, s>>>(a);
+    if (form) k_hsub<<<dim3((a.naux * a.naux + 255) / 256, 1, a.nk), 256, 0, s>>>(a);
 }
 
 // J contributions of the current theta (rows into part_post[.][1..3])

@@ -258,8 +258,12 @@ void launch_scale_cols(zd* const* mats, const double* const* vals, int nbatch, i
                        cudaStream_t s);
 
 // ---- adjoint (k_step.cu, k_adjoint.cu)
-void launch_propagate_only(const StepArgs& a, const StepPlan& p, int cstep, cudaStream_t s);
-void launch_hsub_only(const StepArgs& a, const StepPlan& p, int cstep, cudaStream_t s);
+void launch_propagate_only(const StepArgs& a, const StepPlan& p, int cstep, void* sync, zd* hist, cudaStream_t s);
+void launch_hsub_only(const StepArgs& a, const StepPlan& p, int cstep, bool form, cudaStream_t s);
+bool adj_series_fits(const StepArgs& a);
+size_t adj_sync_bytes();
+void launch_adj_series(const StepArgs& a, void* sync, zd* hist, zd* vec, cudaStream_t s);
+void launch_adj_current(const StepArgs& a, double* out, cudaStream_t s);
 void launch_subspace_j(const StepArgs& a, cudaStream_t s);
 // muffin-tin density matrices of theta: the reference n0 (set-up) or dh = U (n - n0) and its bound term
 int launch_mt_feedback(const StepArgs& a, const StepPlan& p, int reference, double* l1, cudaStream_t s);
