@@ -93,6 +93,7 @@ struct rttddft_ctx {
     DgGemm *dg_expand = nullptr, *dg_fwd = nullptr, *dg_back = nullptr, *dg_proj = nullptr;
     DgLeft *dgl_mt = nullptr, *dgl_dh = nullptr, *dgl_lh = nullptr;  // muffin-tin stacks, dh, L^H
     DgGemm *dg_mt = nullptr, *dg_mtd = nullptr, *dg_dvw = nullptr, *dg_dvg = nullptr, *dg_dvi = nullptr;
+    DgToep* dg_toep = nullptr;                  // interstitial sum (direct, FP64 form)
     zd* d_mtd = nullptr;
     int mtd_stride = 0;
     std::vector<zd*> dv_t, dv_w;                // per k T = dV~ * CC_G and W = dh L of the rebuild
@@ -283,7 +284,7 @@ static StepArgs make_args(rttddft_ctx* ctx, int dv_on) {
     a.tc_st = tc_table_scale(ctx->tc);
     a.at_n = ctx->at.n;
     a.at_maxm = ctx->maxm;
-    a.ith = (ctx->opt.precision >= RTTDDFT_PREC_BF16X3 || ctx->fft || ctx->toep_global) ? 1 : 0;
+    a.ith = (ctx->opt.precision >= RTTDDFT_PREC_BF16X3 || ctx->fft || ctx->toep_global || ctx->dg_toep) ? 1 : 0;
     a.toep_global = ctx->toep_global;
     a.hartree = ctx->opt.hartree;
     a.mtg = ctx->d_mtg;
@@ -339,6 +340,7 @@ static StepPlan make_plan(rttddft_ctx* ctx) {
     p.dg_back = ctx->dg_back;
     p.dg_proj = ctx->dg_proj;
     p.dg_mt = ctx->dg_mt;
+    p.dg_toep = ctx->dg_toep;
     p.dg_mtd = ctx->dg_mtd;
     p.dgl_dh = ctx->dgl_dh;
     p.dg_dvw = ctx->dg_dvw;
@@ -618,6 +620,8 @@ static void validate(const rttddft_system* s, const rttddft_options* o) {
 }
 
 static void drop_dg(rttddft_ctx* ctx) {
+    dg_toep_destroy(ctx->dg_toep);
+    ctx->dg_toep = nullptr;
     for (DgGemm** g : {&ctx->dg_expand, &ctx->dg_fwd, &ctx->dg_back, &ctx->dg_proj, &ctx->dg_mt, &ctx->dg_mtd, &ctx->dg_dvw,
                        &ctx->dg_dvg, &ctx->dg_dvi}) {
         dg_gemm_destroy(*g);
@@ -695,6 +699,21 @@ static bool build_dg(rttddft_ctx* ctx) {
              (ctx->dg_mt = dg_gemm_create(ctx->dgl_mt, nk * at.n, rm.data(), ns, ctx->d_flag, at.n));
         CK(cudaStreamSynchronize(ctx->stream));
         dfree(ctx, stk);
+    }
+    if (ok && ctx->opt.interstitial == RTTDDFT_INTERSTITIAL_TOEPLITZ) {
+        std::vector<DgRight> rt(nk);
+        std::vector<const int*> gl(nk);
+        for (int k = 0; k < nk; ++k) {
+            KDev& K = ctx->hkd[k];
+            if (!K.th) K.th = dalloc<zd>(ctx, (size_t)K.ng * ns);
+            rt[k] = DgRight{K.C, K.nb, K.ng, K.th, K.ng};
+            gl[k] = K.glin;
+        }
+        ok = (ctx->dg_toep = dg_toep_create(nk, rt.data(), gl.data(), ns, ctx->dg_fwd, ctx->nvt, ctx->vt_center, ctx->d_flag));
+        if (ok) {
+            launch_dg_table(ctx->dg_toep, 0, ctx->d_vtab, ctx->stream);
+            KCHECK();
+        }
     }
     if (!ok) drop_dg(ctx);
     return ok;
@@ -2637,7 +2656,8 @@ extern "C" int rttddft_apply_noalloc(rttddft_ctx* ctx, int k, int ncols, const d
         p.side = nullptr;
         p.tile_cnt = nullptr;  // the context's counters may be in use on another stream
         p.gd_mt1 = nullptr;
-        p.dg_fwd = p.dg_back = p.dg_mt = p.dg_mtd = nullptr;  // their digit buffers belong to the context
+        p.dg_fwd = p.dg_back = p.dg_mt = p.dg_mtd = nullptr;
+        p.dg_toep = nullptr;  // their digit buffers belong to the context
         p.gd_fwd = (const GemmDesc*)(base + o_gd);
         p.maxng = ng;
         p.part = (zd*)(base + o_part);

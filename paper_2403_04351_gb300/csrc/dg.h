@@ -31,6 +31,14 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
 void dg_gemm_destroy(DgGemm* g);
 int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s, bool packed = false);  // returns its launches
 
+// the interstitial sum with the left operand generated from the table
+struct DgToep;
+DgToep* dg_toep_create(int nk, const DgRight* r, const int* const* glin, int ncol, const DgGemm* x, int nvt, int center, int* flag);
+void dg_toep_destroy(DgToep* t);
+// which: 0 V~, 1 the step's V~ + s dV~
+int launch_dg_table(const DgToep* t, int which, const zd* tab, cudaStream_t s);
+int launch_dg_toep(const DgToep* t, int which, int kofs, int nk, cudaStream_t s);
+
 struct StepArgs;
 DgSeries* dg_series_create(int nk, int n, int ns);
 void dg_series_destroy(DgSeries* g);

@@ -36,6 +36,9 @@ namespace cg = cooperative_groups;
 #define DG_S0 4             // smallest i + j kept
 #define DG_G 7              // groups kept, s = DG_S0 + g, NT columns of tensor memory each
 #define DG_THREADS 320      // 8 read-out warps, one product warp, one copy warp
+// and 256 (16 columns) or 128 threads that generate the left operand (GEN): with more columns the
+// read-out's integers need the registers
+__host__ __device__ constexpr int dg_gen(int NT) { return NT == 16 ? 256 : 128; }
 #define DG_A_PL (DG_BM * 64)
 
 // slices of 64 reals that a group collects before it is read out
@@ -141,6 +144,7 @@ struct DgOut {
     const int* ec;      // column exponents of X
     zd* C;
     const double* scale;  // factor on the product, or null
+    const int* glin;    // GEN: table offsets of the G set
     int tile0;          // first tile in the split buffers
 };
 struct DgCheb {
@@ -158,6 +162,10 @@ struct DgArgs {
     i64* part;
     unsigned* cnt;
     int* flag;
+    const uint4* tab4;   // GEN: digits 0 .. 3 of every table entry, (re, im) pairs,
+    const uint2* tab2;   // digits 4 and 5,
+    const int* tabe;     // and the exponent of the table
+    int center;
 };
 
 __device__ __forceinline__ uint64_t dg_desc(uint32_t saddr) {  // K-major, 64-byte swizzle, 8-row atoms of 512 B
@@ -202,9 +210,12 @@ __device__ __forceinline__ i64 dg_mul62(i64 a, i64 b) {
 // and forth by a pair of mbarriers.  The K slices of a tile meet in the
 // distributed shared memory of a cluster, further clusters of the tile in
 // global memory, where the last one finishes it.
-// MODE 0: C (+)= the product, scaled back.  MODE 1: a Chebyshev term.
-template <int NT, int MODE>
-__global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
+// MODE 0: C (+)= the product, scaled back.  MODE 1: a Chebyshev term.  GEN: the left
+// operand is V~_(G - G') of the table (Eq. v_interstitial): eight more warps write
+// a stage's planes from the table's digits, 24 bytes an entry through L1, loaded
+// before the wait for the stage's slot.
+template <int NT, int MODE, bool GEN>
+__global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(const DgArgs g) {
     extern __shared__ unsigned char dgsm[];
     constexpr int STAGES = NT == 16 ? 4 : 3;
     constexpr int B_PL = NT * 64;
@@ -212,7 +223,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
     constexpr int CP = NT / 2;  // columns per read-out thread
     constexpr uint32_t NCOLS = DG_G * NT <= 128 ? 128 : (DG_G * NT <= 256 ? 256 : 512);
     unsigned char* smem = dgsm + ((1024u - (smem_u32(dgsm) & 1023u)) & 1023u);
-    __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], gfull[DG_G], gfree[DG_G], done;
+    constexpr int THREADS = DG_THREADS + (GEN ? dg_gen(NT) : 0);
+    __shared__ __align__(8) uint64_t full[STAGES], fullA[STAGES], empty[STAGES], gfull[DG_G], gfree[DG_G], done;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
     __shared__ int is_last;
@@ -229,6 +241,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
+            mbar_init(&fullA[s], dg_gen(NT) / 32);
             mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < DG_G; ++s) {
@@ -267,8 +280,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
                 }
                 if (abort_flag) break;
                 unsigned char* sa = smem + s * STAGE;
-                mbar_expect_tx(&full[s], STAGE);
-                dg_copy(sa, ga + (size_t)t * (DG_P * DG_A_PL), DG_P * DG_A_PL, &full[s]);
+                mbar_expect_tx(&full[s], GEN ? DG_P * B_PL : STAGE);
+                if (!GEN) dg_copy(sa, ga + (size_t)t * (DG_P * DG_A_PL), DG_P * DG_A_PL, &full[s]);
                 dg_copy(sa + DG_P * DG_A_PL, gb + (size_t)t * (DG_P * B_PL), DG_P * B_PL, &full[s]);
                 issued = t + 1;
             }
@@ -284,7 +297,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
             bool ok = true;
             for (int t = 0; t < nk && ok; ++t) {
                 const int s = t % STAGES;
-                if (!mbar_wait(&full[s], (uint32_t)((t / STAGES) & 1))) {
+                if (!mbar_wait(&full[s], (uint32_t)((t / STAGES) & 1)) ||
+                    (GEN && !mbar_wait(&fullA[s], (uint32_t)((t / STAGES) & 1)))) {
                     ok = false;
                     break;
                 }
@@ -343,6 +357,77 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
                 abort_flag = 1;
                 atomicOr(g.flag, 8);
             }
+        }
+    } else if (GEN && warp >= 10) {
+        // row r, PER of a stage's 16 k in batches of QB; for 16 columns the next batch's entries are on
+        // their way while one is written (203 us at N_G 5900, 2 columns, 212 without; 512 threads with
+        // fewer registers: 361.  Loads and stores of a stage take 1700 cycles of the L1 pipe, the products
+        // 600; the FP64 pipe took 697 us)
+        constexpr int PER = 16 * DG_BM / dg_gen(NT), QB = 4, NB = PER / QB;
+        constexpr bool AHEAD = NT == 16;
+        const int r = (tid - DG_THREADS) & (DG_BM - 1), h = (tid - DG_THREADS) / DG_BM;
+        const int row = m0 + r;
+        const bool act = row < o.M;
+        const int lrow = act ? o.glin[row] + g.center : 0;
+        uint4 a4[QB], b4[QB];
+        uint2 a2[QB], b2[QB];
+        auto load = [&](int t, int b) {
+            const int k0 = (st0 + t) * 16 + h * PER + b * QB;
+#pragma unroll
+            for (int q = 0; q < QB; ++q) {
+                b4[q] = make_uint4(0u, 0u, 0u, 0u);
+                b2[q] = make_uint2(0u, 0u);
+                if (act && k0 + q < o.M) {
+                    const int d = lrow - __ldg(o.glin + k0 + q);
+                    b4[q] = __ldg(g.tab4 + d);
+                    b2[q] = __ldg(g.tab2 + d);
+                }
+            }
+        };
+        if (AHEAD && nk > 0) load(0, 0);
+        bool ok = true;
+        for (int t = 0; t < nk && ok; ++t) {
+            const int s = t % STAGES;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                if (!AHEAD) load(t, b);
+#pragma unroll
+                for (int q = 0; q < QB; ++q) {
+                    a4[q] = b4[q];
+                    a2[q] = b2[q];
+                }
+                if (AHEAD) {
+                    if (b + 1 < NB) load(t, b + 1);
+                    else if (t + 1 < nk) load(t + 1, 0);
+                }
+                if (b == 0 && t >= STAGES && !mbar_wait(&empty[s], (uint32_t)((t / STAGES - 1) & 1))) {
+                    abort_flag = 1;
+                    if (lane == 0) atomicOr(g.flag, 8);
+                }
+                if (abort_flag) {
+                    ok = false;
+                    break;
+                }
+                unsigned char* d = smem + s * STAGE + r * 64;
+#pragma unroll
+                for (int c = 0; c < QB / 4; ++c) {
+                    const int ch = (h * PER + b * QB) / 4 + c;  // the row's 16-byte chunk
+                    unsigned char* p = d + ((ch ^ ((r >> 1) & 3)) << 4);
+                    const uint4* w = a4 + 4 * c;
+                    const uint2* v = a2 + 4 * c;
+                    *(uint4*)(p + 0 * DG_A_PL) = make_uint4(w[0].x, w[1].x, w[2].x, w[3].x);
+                    *(uint4*)(p + 1 * DG_A_PL) = make_uint4(w[0].y, w[1].y, w[2].y, w[3].y);
+                    *(uint4*)(p + 2 * DG_A_PL) = make_uint4(w[0].z, w[1].z, w[2].z, w[3].z);
+                    *(uint4*)(p + 3 * DG_A_PL) = make_uint4(w[0].w, w[1].w, w[2].w, w[3].w);
+                    *(uint4*)(p + 4 * DG_A_PL) = make_uint4(v[0].x, v[1].x, v[2].x, v[3].x);
+                    *(uint4*)(p + 5 * DG_A_PL) = make_uint4(v[0].y, v[1].y, v[2].y, v[3].y);
+                }
+            }
+            if (!ok) break;
+            // the planes are read by the products' proxy
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&fullA[s])) : "memory");
         }
     } else {
         const int nsl = (nk + 1) >> 1;
@@ -411,7 +496,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
     if (g.gs > 1) {
         const int tile = (o.tile0 + m_i * g.ntn + nt_i) * g.cs + rank;
         unsigned long long* P = (unsigned long long*)g.part + (size_t)tile * share * 2 * DG_BM;
-        for (int it = tid; it < 2 * items; it += DG_THREADS) {
+        for (int it = tid; it < 2 * items; it += THREADS) {
             i64 v = 0;
             for (int q = 0; q < g.cs; ++q) v += (g.cs > 1 ? cl.map_shared_rank(S, q) : S)[(size_t)2 * c0 * DG_BM + it];
             atomicAdd(P + it, (unsigned long long)v);
@@ -426,7 +511,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
         mine = is_last != 0;
         if (mine) {
             __threadfence();
-            for (int it = tid; it < 2 * items; it += DG_THREADS) {
+            for (int it = tid; it < 2 * items; it += THREADS) {
                 T0[it] = (i64)__ldcg(P + it);
                 __stcg(P + it, 0ull);  // ready for the next launch
             }
@@ -434,7 +519,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
         }
     }
     if (mine) {
-        for (int it = tid; it < items / 2; it += DG_THREADS) {
+        for (int it = tid; it < items / 2; it += THREADS) {
             const int rl = it & (DG_BM - 1), row = m0 + rl, c = (it / DG_BM) * 2, n = (n0 + c0 + c) >> 1;
             if (row >= o.M || n >= g.ncol) continue;
             i64 hv[2], lv[2];
@@ -455,7 +540,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dg(const DgArgs g) {
                 }
             }
             if constexpr (MODE == 0) {
-                const int er = o.er[row], ec = o.ec[n];
+                const int er = GEN ? *g.tabe : o.er[row], ec = o.ec[n];
                 zd v;
                 if (ec >= 2048 || er >= 2048) {
                     v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
@@ -664,24 +749,27 @@ template <int NT>
 static constexpr int dg_smem() {
     return (NT == 16 ? 4 : 3) * DG_P * (DG_A_PL + NT * 64) + 1024;
 }
-template <int MODE>
+template <int MODE, bool GEN>
 static const void* dg_fn(int NT, int* smem) {
     *smem = NT == 16 ? dg_smem<16>() : (NT == 32 ? dg_smem<32>() : dg_smem<64>());
-    return NT == 16 ? (const void*)k_dg<16, MODE> : (NT == 32 ? (const void*)k_dg<32, MODE> : (const void*)k_dg<64, MODE>);
+    if constexpr (GEN) return NT == 16 ? (const void*)k_dg<16, MODE, true> : (const void*)k_dg<32, MODE, true>;
+    else
+        return NT == 16 ? (const void*)k_dg<16, MODE, false>
+                        : (NT == 32 ? (const void*)k_dg<32, MODE, false> : (const void*)k_dg<64, MODE, false>);
 }
-template <int MODE>
+template <int MODE, bool GEN>
 static cudaError_t dg_attr(int NT) {
     int sm;
-    const void* f = dg_fn<MODE>(NT, &sm);
+    const void* f = dg_fn<MODE, GEN>(NT, &sm);
     return raise_smem(f, sm);
 }
-template <int MODE>
+template <int MODE, bool GEN>
 static void dg_launch(int NT, int mt, int nk, DgArgs a, cudaStream_t s) {
     int sm;
-    const void* f = dg_fn<MODE>(NT, &sm);
+    const void* f = dg_fn<MODE, GEN>(NT, &sm);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.cs * a.ntn * a.gs, mt, nk);
-    cfg.blockDim = dim3(DG_THREADS);
+    cfg.blockDim = dim3(DG_THREADS + (GEN ? dg_gen(NT) : 0));
     cfg.dynamicSmemBytes = sm;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -724,6 +812,7 @@ struct DgGemm {
     int nk = 0, ncol = 0, NT = 0, ntn = 0, mt = 0, cs = 1, gs = 1;
     DgOut* out = nullptr;
     DgPackB* pb = nullptr;
+    std::vector<DgPackB> host;
     i64* part = nullptr;
     unsigned* cnt = nullptr;
     int* flag = nullptr;
@@ -781,16 +870,19 @@ DgLeft* dg_left_create(int nk, const DgMat* m, cudaStream_t s) {
 // device bytes of dg_left_create
 size_t dg_left_bytes(int M, int K) { return dg_bytes(dg_up(M, DG_BM), K); }
 
-DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag, int lmod) {
+// x: a product whose right operands (the same ones) are taken; glin: the left operand is generated
+static DgGemm* dg_gemm_build(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag, int lmod, const DgGemm* x,
+                             const int* const* glin) {
     DgGemm* g = new DgGemm();
     g->nk = nk;
     g->ncol = ncol;
-    g->NT = dg_nt(ncol);
+    g->NT = glin ? std::min(32, dg_nt(ncol)) : dg_nt(ncol);
     g->ntn = (2 * ncol + g->NT - 1) / g->NT;
     g->flag = flag;
     const int np = g->ntn * g->NT;
     std::vector<DgOut> out(nk);
-    std::vector<DgPackB> pb(nk);
+    g->host.resize(nk);
+    std::vector<DgPackB>& pb = g->host;
     int tiles = 0, nst = 1;
     for (int k = 0; k < nk; ++k) {
         const DgSrc& d = l->src[lmod > 0 ? k % lmod : k];
@@ -802,8 +894,8 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
         pb[k].K = r[k].K;
         pb[k].NT = g->NT;
         pb[k].nst = dg_nst(r[k].K);
-        pb[k].dst = (uint32_t*)g->pool.get(dg_bytes(np, r[k].K), true);
-        pb[k].ec = (int*)g->pool.get(ncol * sizeof(int), true);
+        pb[k].dst = x ? x->host[k].dst : (uint32_t*)g->pool.get(dg_bytes(np, r[k].K), true);
+        pb[k].ec = x ? x->host[k].ec : (int*)g->pool.get(ncol * sizeof(int), true);
         out[k].A = (const unsigned char*)d.dst;
         out[k].B = (const unsigned char*)pb[k].dst;
         out[k].M = d.M;
@@ -814,6 +906,7 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
         out[k].ec = pb[k].ec;
         out[k].C = r[k].C;
         out[k].scale = r[k].scale;
+        out[k].glin = glin ? glin[k] : nullptr;
         out[k].tile0 = tiles;
         const int mt = (d.M + DG_BM - 1) / DG_BM;
         g->mt = std::max(g->mt, mt);
@@ -829,16 +922,18 @@ DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int*
         g->out = g->pool.up(out);
         g->pb = g->pool.up(pb);
     }
-    if (!g->pool.ok || dg_attr<0>(g->NT) != cudaSuccess) {
+    if (!g->pool.ok || dg_attr<0, false>(g->NT) != cudaSuccess) {
         dg_gemm_destroy(g);
         return nullptr;
     }
     return g;
 }
 
-// C (+)= A X for entries kofs .. kofs + nk - 1; packed: X's digits are those of the last call
-int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s, bool packed) {
-    if (!packed) k_dg_pack_b<<<dim3(8 * g->ncol, 1, nk), DG_PB_T, 0, s>>>(g->pb, kofs);
+DgGemm* dg_gemm_create(const DgLeft* l, int nk, const DgRight* r, int ncol, int* flag, int lmod) {
+    return dg_gemm_build(l, nk, r, ncol, flag, lmod, nullptr, nullptr);
+}
+
+static DgArgs dg_args(const DgGemm* g, int kofs, int beta) {
     DgArgs a{};
     a.out = g->out;
     a.kofs = kofs;
@@ -850,8 +945,101 @@ int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s, 
     a.part = g->part;
     a.cnt = g->cnt;
     a.flag = g->flag;
-    dg_launch<0>(g->NT, g->mt, nk, a, s);
+    return a;
+}
+
+// C (+)= A X for entries kofs .. kofs + nk - 1; packed: X's digits are those of the last call
+int launch_dg_gemm(const DgGemm* g, int kofs, int nk, int beta, cudaStream_t s, bool packed) {
+    if (!packed) k_dg_pack_b<<<dim3(8 * g->ncol, 1, nk), DG_PB_T, 0, s>>>(g->pb, kofs);
+    dg_launch<0, false>(g->NT, g->mt, nk, dg_args(g, kofs, beta), s);
     return packed ? 1 : 2;
+}
+
+// ------------------------------------------------------------ interstitial sum
+struct DgToep {
+    DgPool pool;
+    DgGemm* g = nullptr;  // shapes, right operand and split buffers
+    bool own = false;     // it packs the right operand itself
+    // of V~ (0) and of the step's V~ + s dV~ (1):
+    uint4* tab4[2] = {nullptr, nullptr};
+    uint2* tab2[2] = {nullptr, nullptr};
+    int* hw = nullptr;    // high words of the tables' largest entries
+    int* e = nullptr;     // their exponents
+    int nvt = 0, center = 0;
+};
+__global__ void __launch_bounds__(256) k_dg_tab_max(const zd* __restrict__ tab, int n, int* hw) {
+    int m = 0;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) m = max(m, max(dg_hw(tab[i].x), dg_hw(tab[i].y)));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(hw, m);
+}
+__global__ void __launch_bounds__(256) k_dg_tab_cut(const zd* __restrict__ tab, int n, const int* hw, int* eo, uint4* t4, uint2* t2) {
+    const int i = blockIdx.x * 256 + threadIdx.x, e = dg_exp(*hw);
+    if (i == 0) *eo = e;
+    if (i >= n) return;
+    const DgScale sc = dg_scale(e >= 2048 ? 0 : e);
+    uint32_t dr[DG_P], di[DG_P], p[DG_P];
+    dg_cut(e >= 2048 ? 0 : dg_int(tab[i].x, sc), dr);
+    dg_cut(e >= 2048 ? 0 : dg_int(tab[i].y, sc), di);
+#pragma unroll
+    for (int q = 0; q < DG_P; ++q) p[q] = dg_pair(dr[q], di[q]);
+    t4[i] = make_uint4(p[0], p[1], p[2], p[3]);
+    t2[i] = make_uint2(p[4], p[5]);
+}
+
+void dg_toep_destroy(DgToep* t) {
+    if (!t) return;
+    dg_gemm_destroy(t->g);
+    t->pool.drop();
+    delete t;
+}
+
+// T = V~ * C_G per k-point (r: C_G and T).  x: a product with the same right
+// operands, whose digits are then taken, or null.
+DgToep* dg_toep_create(int nk, const DgRight* r, const int* const* glin, int ncol, const DgGemm* x, int nvt, int center, int* flag) {
+    DgToep* t = new DgToep();
+    if (x && x->NT > 32) x = nullptr;
+    t->nvt = nvt;
+    t->center = center;
+    t->own = !x;
+    for (int q = 0; q < 2; ++q) {
+        t->tab4[q] = (uint4*)t->pool.get((size_t)nvt * sizeof(uint4), false);
+        t->tab2[q] = (uint2*)t->pool.get((size_t)nvt * sizeof(uint2), false);
+    }
+    t->hw = (int*)t->pool.get(2 * sizeof(int), true);
+    t->e = (int*)t->pool.get(2 * sizeof(int), true);
+    DgLeft l;  // shapes only
+    l.src.resize(nk);
+    for (int k = 0; k < nk; ++k) {
+        l.src[k] = DgSrc{};
+        l.src[k].M = l.src[k].K = r[k].K;
+        l.src[k].nst = dg_nst(r[k].K);
+    }
+    if (t->pool.ok) t->g = dg_gemm_build(&l, nk, r, ncol, flag, 0, x, glin);
+    if (!t->g || dg_attr<0, true>(t->g->NT) != cudaSuccess) {
+        dg_toep_destroy(t);
+        return nullptr;
+    }
+    return t;
+}
+
+// cut a table; which: 0 V~, 1 the step's
+int launch_dg_table(const DgToep* t, int which, const zd* tab, cudaStream_t s) {
+    cudaMemsetAsync(t->hw + which, 0, sizeof(int), s);
+    k_dg_tab_max<<<std::min(304, (t->nvt + 255) / 256), 256, 0, s>>>(tab, t->nvt, t->hw + which);
+    k_dg_tab_cut<<<(t->nvt + 255) / 256, 256, 0, s>>>(tab, t->nvt, t->hw + which, t->e + which, t->tab4[which], t->tab2[which]);
+    return 2;
+}
+int launch_dg_toep(const DgToep* t, int which, int kofs, int nk, cudaStream_t s) {
+    const DgGemm* g = t->g;
+    if (t->own) k_dg_pack_b<<<dim3(8 * g->ncol, 1, nk), DG_PB_T, 0, s>>>(g->pb, kofs);
+    DgArgs a = dg_args(g, kofs, 0);
+    a.tab4 = t->tab4[which];
+    a.tab2 = t->tab2[which];
+    a.tabe = t->e + which;
+    a.center = t->center;
+    dg_launch<0, true>(g->NT, g->mt, nk, a, s);
+    return t->own ? 2 : 1;
 }
 
 // ------------------------------------------------------------ Chebyshev series
@@ -1053,7 +1241,7 @@ DgSeries* dg_series_create(int nk, int n, int ns) {
         g->ch = g->pool.up(ch);
         g->sk = g->pool.up(sk);
     }
-    if (!g->pool.ok || dg_attr<1>(g->NT) != cudaSuccess) {
+    if (!g->pool.ok || dg_attr<1, false>(g->NT) != cudaSuccess) {
         dg_series_destroy(g);
         return nullptr;
     }
@@ -1076,7 +1264,7 @@ int launch_dg_series(const DgSeries* g, const StepArgs& a, cudaStream_t s) {
     for (int t = 1; t < a.nterms; ++t) {
         d.term = t;
         d.last = t == a.nterms - 1;
-        dg_launch<1>(g->NT, g->mt, g->nk, d, s);
+        dg_launch<1, false>(g->NT, g->mt, g->nk, d, s);
     }
     k_dg_theta<<<dim3(g->ns, 1, g->nk), 128, 0, s>>>(a, g->sk, g->ch);
     return a.nterms + 2;

@@ -2389,7 +2389,7 @@ int launch_operator_pass(const StepArgs& a, const StepPlan& p, cudaStream_t s, T
         mark(tr, "tc_reduce", s);
         nl += 2;
     } else {
-        if (a.toep_global && !p.fft) {
+        if (a.toep_global && !p.fft && !p.dg_toep) {
             // a table window too large for shared memory: V~ * C_G (V~ + s dV~ when the
             // change is on) with the table gathered through L1/L2, FP64, into K.th
             launch_toeplitz(a.kd, p.td_op + a.kofs, a.nk, p.maxng, a.ns, a.dv_on ? a.vstep : a.vtab, a.vt_center, 0,
@@ -2412,6 +2412,13 @@ int launch_operator_pass(const StepArgs& a, const StepPlan& p, cudaStream_t s, T
                 ++nl;
             }
         }
+    }
+    if (p.dg_toep) {
+        // V~ * C_G (V~ + s dV~, cut anew, when the change is on); after the matching rows, whose digits
+        // of C_G it takes
+        if (a.dv_on) nl += launch_dg_table(p.dg_toep, 1, a.vstep, s);
+        nl += launch_dg_toep(p.dg_toep, a.dv_on ? 1 : 0, a.kofs, a.nk, s);
+        mark(tr, "toeplitz", s);
     }
     if (a.lrows > 0 && ((f32 && p.gd_mt1 && a.mtg) || mt_digits(a, p))) {
         nl += launch_mt_gemm(a, p, s);

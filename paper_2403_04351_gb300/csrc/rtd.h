@@ -216,6 +216,7 @@ struct StepPlan {
     const struct TcMT* tcmt;  // tensor-core muffin-tin blocks (split-BF16 form, many states) or null
     const struct DgGemm *dg_expand, *dg_fwd, *dg_back, *dg_proj;  // FP64 products on the tensor cores, or null
     const struct DgGemm *dg_mt, *dg_mtd;        // FP64 muffin-tin stacks, and dh, times [Q; C_lo]
+    const struct DgToep* dg_toep;               // FP64 interstitial sum, or null
     const struct DgLeft* dgl_dh;                // dh of every atom
     const struct DgGemm *dg_dvw, *dg_dvg, *dg_dvi;  // potential change: dh L, L^H W, CC_G^H T (all forms)
     const struct DgSeries* series;  // Chebyshev series as digit products (many states) or null
