@@ -57,6 +57,7 @@ struct FftArgs {
     int F1, F2, F3;
     int nst[3];
     int rad[3][FFT_MAX_ST];
+    unsigned mg[3][2 * FFT_MAX_ST];  // per stage: multipliers that divide by its butterflies per line and its stride
     int lpb[3];             // lines per block of the passes along each axis
     const void* w[3];       // twiddles e^{-2 pi i m / F_a}, m < F_a (FP64 or FP32 complex)
     const FftK* fk;         // per k-point of the launch
@@ -131,9 +132,13 @@ template <typename C> __device__ __forceinline__ C cwt(const C* W, int i, bool i
     return w;
 }
 __device__ __forceinline__ zd cvt(zd a, zd) { return a; }
-__device__ __forceinline__ zf cvt(zd a, zf) { return make_float2((float)a.x, (float)a.y); }
+__device__ __forceinline__ zf cvt(zd a, zf) { return tof(a); }
 __device__ __forceinline__ zd todz(zd a) { return a; }
-__device__ __forceinline__ zd todz(zf a) { return zmk(a.x, a.y); }
+__device__ __forceinline__ zd todz(zf a) { return tod(a); }
+
+// floor(n / d) for n d < 2^32 by the multiplier ceil(2^32 / d) (0: d = 1)
+__host__ __device__ __forceinline__ unsigned fft_magic(int d) { return d == 1 ? 0u : 0xffffffffu / (unsigned)d + 1u; }
+__device__ __forceinline__ int fft_div(int n, unsigned mg) { return mg ? (int)__umulhi((unsigned)n, mg) : n; }
 
 // Stockham autosort, decimation in frequency: nl lines of length L stored
 // line by line in x (y is scratch of the same size).  A stage of radix R on
@@ -142,65 +147,83 @@ __device__ __forceinline__ zd todz(zf a) { return zmk(a.x, a.y); }
 // m = n/R, p < m, q < s; after the last stage the transform is in natural
 // order.  inv selects e^{+}.  Element j of line l sits at l ls + j es (in x and
 // y alike).  Returns the buffer holding the result.
-template <typename C>
-__device__ C* fft_lines_s(C* x, C* y, int nl, int L, int ls, int es, const int* rad, int nst, const C* W,
-                          bool inv) {
+// LF: neighbouring threads take the same butterfly of neighbouring lines (lines
+// stored side by side, ls = 1: no bank conflicts); otherwise neighbouring
+// butterflies of a line.  Indices are divided by multiplication (mg, fft_div) and
+// the last stage, whose twiddles are all 1, multiplies by none: an integer
+// division costs as much as a radix-4 butterfly in FP32, a twiddle four of the
+// slow FP64 instructions.
+template <bool LF, bool LAST, typename C>
+__device__ __forceinline__ void fft_stage(const C* x, C* y, int R, int m, int s0, unsigned mgl, unsigned mgs, int nl, int L,
+                                          int ls, int es, const C* W, bool inv) {
     typedef typename Rt<C>::R R_;
     const R_ sg = inv ? R_(1) : R_(-1);  // sign of i in w_4 = e^{-+ i pi/2}
+    const int nb = m * s0;               // butterflies per line
+    const int tot = nl * nb;
+    for (int b = threadIdx.x; b < tot; b += blockDim.x) {
+        const int o = fft_div(b, mgl);  // LF: the butterfly, else the line
+        const int l = LF ? b - o * nl : o;
+        const int bb = LF ? o : b - o * nb;
+        const int p = fft_div(bb, mgs);
+        const int q = bb - p * s0;
+        auto tw = [&](C v, int t) {
+            if constexpr (LAST) return v;
+            else return cml(v, cwt(W, t * p * s0, inv));
+        };
+        const C* xi = x + l * ls + (q + s0 * p) * es;
+        C* yo = y + l * ls + (q + s0 * R * p) * es;
+        const int ms = m * s0 * es;  // input stride between the radix points
+        const int os = s0 * es;      // output stride between the radix points
+        if (R == 2) {
+            const C a0 = xi[0], a1 = xi[ms];
+            yo[0] = cad(a0, a1);
+            yo[os] = tw(csb(a0, a1), 1);
+        } else if (R == 4) {
+            const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms], a3 = xi[3 * ms];
+            const C s02 = cad(a0, a2), d02 = csb(a0, a2), s13 = cad(a1, a3), d13 = csb(a1, a3);
+            // w_4 = -i (forward): b1 = d02 - i d13, b3 = d02 + i d13
+            const C id13 = cis(d13, sg);
+            yo[0] = cad(s02, s13);
+            yo[os] = tw(cad(d02, id13), 1);
+            yo[2 * os] = tw(csb(s02, s13), 2);
+            yo[3 * os] = tw(csb(d02, id13), 3);
+        } else if (R == 3) {
+            const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms];
+            const C w = cwt(W, L / 3, inv);  // w_3
+            const C sm = cad(a1, a2), df = csb(a1, a2);
+            const C t = cmk<C>(a0.x + w.x * sm.x, a0.y + w.x * sm.y);
+            const C u = cis(df, w.y);  // i Im(w_3) (a1 - a2)
+            yo[0] = cad(a0, sm);
+            yo[os] = tw(cad(t, u), 1);
+            yo[2 * os] = tw(csb(t, u), 2);
+        } else {  // R == 5
+            const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms], a3 = xi[3 * ms], a4 = xi[4 * ms];
+            const C w1 = cwt(W, L / 5, inv), w2 = cwt(W, 2 * (L / 5), inv);  // w_5, w_5^2
+            const C s1 = cad(a1, a4), d1 = csb(a1, a4), s2 = cad(a2, a3), d2 = csb(a2, a3);
+            const C ta = cmk<C>(a0.x + w1.x * s1.x + w2.x * s2.x, a0.y + w1.x * s1.y + w2.x * s2.y);
+            const C tb = cmk<C>(a0.x + w2.x * s1.x + w1.x * s2.x, a0.y + w2.x * s1.y + w1.x * s2.y);
+            // i (Im w1 d1 + Im w2 d2) and i (Im w2 d1 - Im w1 d2)
+            const C ua = cmk<C>(-(w1.y * d1.y + w2.y * d2.y), w1.y * d1.x + w2.y * d2.x);
+            const C ub = cmk<C>(-(w2.y * d1.y - w1.y * d2.y), w2.y * d1.x - w1.y * d2.x);
+            yo[0] = cad(a0, cad(s1, s2));
+            yo[os] = tw(cad(ta, ua), 1);
+            yo[2 * os] = tw(cad(tb, ub), 2);
+            yo[3 * os] = tw(csb(tb, ub), 3);
+            yo[4 * os] = tw(csb(ta, ua), 4);
+        }
+    }
+}
+template <bool LF, typename C>
+__device__ C* fft_lines_s(C* x, C* y, int nl, int L, int ls, int es, const int* rad, const unsigned* mg, int nst,
+                          const C* W, bool inv) {
     int s0 = 1;
+    const unsigned mnl = LF ? fft_magic(nl) : 0u;
     for (int st = 0; st < nst; ++st) {
         const int R = rad[st];
         const int m = L / (s0 * R);
-        const int nb = m * s0;  // butterflies per line
-        const int tot = nl * nb;
-        for (int b = threadIdx.x; b < tot; b += blockDim.x) {
-            const int l = b / nb;
-            const int bb = b - l * nb;
-            const int p = bb / s0;
-            const int q = bb - p * s0;
-            const C* xi = x + l * ls + (q + s0 * p) * es;
-            C* yo = y + l * ls + (q + s0 * R * p) * es;
-            const int tws = p * s0;      // twiddle index step: w_n^{p t} = W[p s t]
-            const int ms = m * s0 * es;  // input stride between the radix points
-            const int os = s0 * es;      // output stride between the radix points
-            if (R == 2) {
-                const C a0 = xi[0], a1 = xi[ms];
-                yo[0] = cad(a0, a1);
-                yo[os] = cml(csb(a0, a1), cwt(W, tws, inv));
-            } else if (R == 4) {
-                const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms], a3 = xi[3 * ms];
-                const C s02 = cad(a0, a2), d02 = csb(a0, a2), s13 = cad(a1, a3), d13 = csb(a1, a3);
-                // w_4 = -i (forward): b1 = d02 - i d13, b3 = d02 + i d13
-                const C id13 = cis(d13, sg);
-                yo[0] = cad(s02, s13);
-                yo[os] = cml(cad(d02, id13), cwt(W, tws, inv));
-                yo[2 * os] = cml(csb(s02, s13), cwt(W, 2 * tws, inv));
-                yo[3 * os] = cml(csb(d02, id13), cwt(W, 3 * tws, inv));
-            } else if (R == 3) {
-                const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms];
-                const C w = cwt(W, L / 3, inv);  // w_3
-                const C sm = cad(a1, a2), df = csb(a1, a2);
-                const C t = cmk<C>(a0.x + w.x * sm.x, a0.y + w.x * sm.y);
-                const C u = cis(df, w.y);  // i Im(w_3) (a1 - a2)
-                yo[0] = cad(a0, sm);
-                yo[os] = cml(cad(t, u), cwt(W, tws, inv));
-                yo[2 * os] = cml(csb(t, u), cwt(W, 2 * tws, inv));
-            } else {  // R == 5
-                const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms], a3 = xi[3 * ms], a4 = xi[4 * ms];
-                const C w1 = cwt(W, L / 5, inv), w2 = cwt(W, 2 * (L / 5), inv);  // w_5, w_5^2
-                const C s1 = cad(a1, a4), d1 = csb(a1, a4), s2 = cad(a2, a3), d2 = csb(a2, a3);
-                const C ta = cmk<C>(a0.x + w1.x * s1.x + w2.x * s2.x, a0.y + w1.x * s1.y + w2.x * s2.y);
-                const C tb = cmk<C>(a0.x + w2.x * s1.x + w1.x * s2.x, a0.y + w2.x * s1.y + w1.x * s2.y);
-                // i (Im w1 d1 + Im w2 d2) and i (Im w2 d1 - Im w1 d2)
-                const C ua = cmk<C>(-(w1.y * d1.y + w2.y * d2.y), w1.y * d1.x + w2.y * d2.x);
-                const C ub = cmk<C>(-(w2.y * d1.y - w1.y * d2.y), w2.y * d1.x - w1.y * d2.x);
-                yo[0] = cad(a0, cad(s1, s2));
-                yo[os] = cml(cad(ta, ua), cwt(W, tws, inv));
-                yo[2 * os] = cml(cad(tb, ub), cwt(W, 2 * tws, inv));
-                yo[3 * os] = cml(csb(tb, ub), cwt(W, 3 * tws, inv));
-                yo[4 * os] = cml(csb(ta, ua), cwt(W, 4 * tws, inv));
-            }
-        }
+        const unsigned mgl = LF ? mnl : mg[2 * st], mgs = mg[2 * st + 1];
+        if (st + 1 < nst) fft_stage<LF, false>(x, y, R, m, s0, mgl, mgs, nl, L, ls, es, W, inv);
+        else fft_stage<LF, true>(x, y, R, m, s0, mgl, mgs, nl, L, ls, es, W, inv);
         __syncthreads();
         C* t = x;
         x = y;
@@ -211,8 +234,13 @@ __device__ C* fft_lines_s(C* x, C* y, int nl, int L, int ls, int es, const int* 
 }
 
 template <typename C>
-__device__ __forceinline__ C* fft_lines(C* x, C* y, int nl, int L, const int* rad, int nst, const C* W, bool inv) {
-    return fft_lines_s(x, y, nl, L, L, 1, rad, nst, W, inv);
+__device__ __forceinline__ C* fft_lines(C* x, C* y, int nl, int L, const FftArgs& f, int ax, const C* W, bool inv) {
+    return fft_lines_s<false>(x, y, nl, L, L, 1, f.rad[ax], f.mg[ax], f.nst[ax], W, inv);
+}
+// lines side by side: element j of line l at j nl + l
+template <typename C>
+__device__ __forceinline__ C* fft_cols(C* x, C* y, int nl, int L, const FftArgs& f, int ax, const C* W, bool inv) {
+    return fft_lines_s<true>(x, y, nl, L, 1, nl, f.rad[ax], f.mg[ax], f.nst[ax], W, inv);
 }
 
 template <typename C>
@@ -243,7 +271,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_a(FftArgs f) {
     for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x)
         x[K.lpos[j] - base] = cvt(td.X[K.gperm[j] + (size_t)c * td.ldx], C());
     __syncthreads();
-    const C* r = fft_lines(x, y, nl, F3, f.rad[2], f.nst[2], W, true);
+    const C* r = fft_lines(x, y, nl, F3, f, 2, W, true);
     C* out = (C*)f.b3 + ((size_t)k * f.ncol + c) * f.b3_col + (size_t)base;
     for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) out[i] = r[i];
 }
@@ -267,8 +295,9 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_bd(FftArgs f, int fwd) {
     C* b3 = (C*)f.b3 + ((size_t)k * f.ncol + c) * f.b3_col;
     C* b2 = (C*)f.b2 + ((size_t)k * f.ncol + c) * f.b2_col + (size_t)p * F2 * F3;
     const int* lo = K.line_of + (size_t)p * F2;
+    const unsigned mnl = fft_magic(nl);
     for (int i = threadIdx.x; i < F2 * nl; i += blockDim.x) {
-        const int r2 = i / nl, l = i - r2 * nl;
+        const int r2 = fft_div(i, mnl), l = i - r2 * nl;
         C v = cmk<C>(0, 0);
         if (fwd) {
             v = b2[(size_t)r2 * F3 + i30 + l];
@@ -276,17 +305,17 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_bd(FftArgs f, int fwd) {
             const int id = lo[r2];
             if (id >= 0) v = b3[(size_t)id * F3 + i30 + l];
         }
-        x[l * F2 + r2] = v;
+        x[i] = v;
     }
     __syncthreads();
-    const C* r = fft_lines(x, y, nl, F2, f.rad[1], f.nst[1], W, !fwd);
+    const C* r = fft_cols(x, y, nl, F2, f, 1, W, !fwd);
     for (int i = threadIdx.x; i < F2 * nl; i += blockDim.x) {
-        const int r2 = i / nl, l = i - r2 * nl;
+        const int r2 = fft_div(i, mnl), l = i - r2 * nl;
         if (fwd) {
             const int id = lo[r2];
-            if (id >= 0) b3[(size_t)id * F3 + i30 + l] = r[l * F2 + r2];
+            if (id >= 0) b3[(size_t)id * F3 + i30 + l] = r[i];
         } else {
-            b2[(size_t)r2 * F3 + i30 + l] = r[l * F2 + r2];
+            b2[(size_t)r2 * F3 + i30 + l] = r[i];
         }
     }
 }
@@ -308,11 +337,12 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_c(FftArgs f) {
     load_tw(W, f.w[0], F1);
     C* b2 = (C*)f.b2 + ((size_t)k * f.ncol + c) * f.b2_col;
     const size_t pst = (size_t)F2 * F3;
+    const unsigned mnl = fft_magic(nl);
     const size_t off = (size_t)r2 * F3 + i30;
     for (int i = threadIdx.x; i < F1 * nl; i += blockDim.x) {
-        const int r1 = i / nl, l = i - r1 * nl;
+        const int r1 = fft_div(i, mnl), l = i - r1 * nl;
         const int p = K.plane_of[r1];
-        x[l * F1 + r1] = (p >= 0) ? b2[(size_t)p * pst + off + l] : cmk<C>(0, 0);
+        x[i] = (p >= 0) ? b2[(size_t)p * pst + off + l] : cmk<C>(0, 0);
     }
     // the potential of this block's points, loaded (coalesced along r3) before
     // the inverse transform so that the loads overlap it
@@ -328,7 +358,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_c(FftArgs f) {
             const int i = threadIdx.x + u * FFT_THREADS;
             pv[u] = cmk<C>(0, 0);
             if (i < F1 * nl) {
-                const int r1 = i / nl, l = i - r1 * nl;
+                const int r1 = fft_div(i, mnl), l = i - r1 * nl;
                 const size_t gi = (size_t)r1 * pst + off + l;
                 if (f.vmode == 0) {
                     pv[u] = v[gi];
@@ -344,21 +374,20 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_c(FftArgs f) {
         }
     }
     __syncthreads();
-    C* r = fft_lines(x, y, nl, F1, f.rad[0], f.nst[0], W, true);
+    C* r = fft_cols(x, y, nl, F1, f, 0, W, true);
 #pragma unroll
     for (int u = 0; u < PV; ++u) {
         const int i = threadIdx.x + u * FFT_THREADS;
         if (i < F1 * nl) {
-            const int r1 = i / nl, l = i - r1 * nl;
-            r[l * F1 + r1] = cml(r[l * F1 + r1], pv[u]);
+            r[i] = cml(r[i], pv[u]);
         }
     }
     __syncthreads();
-    const C* o = fft_lines(r, r == x ? y : x, nl, F1, f.rad[0], f.nst[0], W, false);
+    const C* o = fft_cols(r, r == x ? y : x, nl, F1, f, 0, W, false);
     for (int i = threadIdx.x; i < F1 * nl; i += blockDim.x) {
-        const int r1 = i / nl, l = i - r1 * nl;
+        const int r1 = fft_div(i, mnl), l = i - r1 * nl;
         const int p = K.plane_of[r1];
-        if (p >= 0) b2[(size_t)p * pst + off + l] = o[l * F1 + r1];
+        if (p >= 0) b2[(size_t)p * pst + off + l] = o[i];
     }
 }
 
@@ -380,7 +409,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_e(FftArgs f) {
     const C* in = (const C*)f.b3 + ((size_t)k * f.ncol + c) * f.b3_col + (size_t)base;
     for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) x[i] = in[i];
     __syncthreads();
-    const C* r = fft_lines(x, y, nl, F3, f.rad[2], f.nst[2], W, false);
+    const C* r = fft_lines(x, y, nl, F3, f, 2, W, false);
     const ToepDesc td = f.td[k];
     const int j0 = K.lg0[l0], j1 = K.lg0[l0 + nl];
     for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x)
@@ -403,6 +432,7 @@ __global__ void __launch_bounds__(FFT_PTHREADS) k_fft_plane(FftArgs f, int fwd) 
     if (p >= K.nplane) return;
     load_tw(W2, f.w[1], F2);
     load_tw(W3, f.w[2], F3);
+    const unsigned m3 = fft_magic(F3);
     const int l0 = K.pl0[p], nl = K.pl0[p + 1] - l0;
     const int base = l0 * F3;
     C* b2 = (C*)f.b2 + ((size_t)k * f.ncol + c) * f.b2_col + (size_t)p * n2;
@@ -414,28 +444,28 @@ __global__ void __launch_bounds__(FFT_PTHREADS) k_fft_plane(FftArgs f, int fwd) 
         for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x)
             A[K.lpos[j] - base] = cvt(td.X[K.gperm[j] + (size_t)c * td.ldx], C());
         __syncthreads();
-        C* r = fft_lines(A, B, nl, F3, f.rad[2], f.nst[2], W3, true);
+        C* r = fft_lines(A, B, nl, F3, f, 2, W3, true);
         C* P = (r == A) ? B : A;
         for (int i = threadIdx.x; i < n2; i += blockDim.x) P[i] = cmk<C>(0, 0);
         __syncthreads();
         for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) {
-            const int l = i / F3, r3 = i - l * F3;
+            const int l = fft_div(i, m3), r3 = i - l * F3;
             P[K.lr2[l0 + l] * F3 + r3] = r[i];
         }
         __syncthreads();
-        const C* q = fft_lines_s(P, r, F3, F2, 1, F3, f.rad[1], f.nst[1], W2, true);
+        const C* q = fft_cols(P, r, F3, F2, f, 1, W2, true);
         for (int i = threadIdx.x; i < n2; i += blockDim.x) b2[i] = q[i];
     } else {
         for (int i = threadIdx.x; i < n2; i += blockDim.x) A[i] = b2[i];
         __syncthreads();
-        C* q = fft_lines_s(A, B, F3, F2, 1, F3, f.rad[1], f.nst[1], W2, false);
+        C* q = fft_cols(A, B, F3, F2, f, 1, W2, false);
         C* o = (q == A) ? B : A;
         for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) {
-            const int l = i / F3, r3 = i - l * F3;
+            const int l = fft_div(i, m3), r3 = i - l * F3;
             o[i] = q[K.lr2[l0 + l] * F3 + r3];
         }
         __syncthreads();
-        const C* r = fft_lines(o, q, nl, F3, f.rad[2], f.nst[2], W3, false);
+        const C* r = fft_lines(o, q, nl, F3, f, 2, W3, false);
         for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x)
             td.Y[K.gperm[j] + (size_t)c * td.ldy] = todz(r[K.lpos[j] - base]);
     }
@@ -470,17 +500,16 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_density(FftArgs f, int nk, 
             for (int i = threadIdx.x; i < F1 * nl; i += blockDim.x) {
                 const int r1 = i / nl, l = i - r1 * nl;
                 const int p = K.plane_of[r1];
-                x[l * F1 + r1] = (p >= 0) ? b2[(size_t)p * pst + off + l] : cmk<C>(0, 0);
+                x[i] = (p >= 0) ? b2[(size_t)p * pst + off + l] : cmk<C>(0, 0);
             }
             __syncthreads();
-            const C* r = fft_lines(x, y, nl, F1, f.rad[0], f.nst[0], W, true);
+            const C* r = fft_cols(x, y, nl, F1, f, 0, W, true);
             const double wf = wk[k] * occ[c];
 #pragma unroll
             for (int u = 0; u < PV; ++u) {
                 const int i = threadIdx.x + u * FFT_THREADS;
                 if (i < F1 * nl) {
-                    const int r1 = i / nl, l = i - r1 * nl;
-                    const C v = r[l * F1 + r1];
+                    const C v = r[i];
                     acc[u] += wf * ((double)v.x * v.x + (double)v.y * v.y);
                 }
             }
@@ -537,7 +566,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_full(FftArgs f, C* buf, int
         x[l * L + j] = buf[base + l * ls + j * es];
     }
     __syncthreads();
-    const C* r = fft_lines(x, y, nl, L, f.rad[axis], f.nst[axis], W, inv != 0);
+    const C* r = fft_lines(x, y, nl, L, f, axis, W, inv != 0);
     for (int i = threadIdx.x; i < nl * L; i += blockDim.x) {
         int l, j;
         if (axis == 2) {
@@ -902,6 +931,17 @@ void fft_plan_info(const FftPlan* pl, int F[3], int* fused) {
     if (fused) *fused = pl ? pl->fused : 0;
 }
 
+static void fft_stages(FftArgs& f, const FftPlan* pl, int a) {
+    int s0 = 1;
+    for (int i = 0; i < FFT_MAX_ST; ++i) {
+        f.rad[a][i] = pl->rad[a][i];
+        if (i >= pl->nst[a]) continue;
+        f.mg[a][2 * i] = fft_magic(pl->F[a] / pl->rad[a][i]);
+        f.mg[a][2 * i + 1] = fft_magic(s0);
+        s0 *= pl->rad[a][i];
+    }
+}
+
 // The convolution for k-points kofs .. kofs + nk - 1 (descriptors td[kofs ..])
 // over ncol columns; vmode 0 multiplies by v (+ s vd when
 // use_vd), vmode 1 by s vd alone.  Five launches.
@@ -913,7 +953,7 @@ static int launch_fft_any(const FftPlan* pl, int fused, const ToepDesc* td, int 
     f.F3 = pl->F[2];
     for (int a = 0; a < 3; ++a) {
         f.nst[a] = pl->nst[a];
-        for (int i = 0; i < FFT_MAX_ST; ++i) f.rad[a][i] = pl->rad[a][i];
+        fft_stages(f, pl, a);
         f.lpb[a] = fft_lpb(pl->F[a]);
         f.w[a] = pl->prec == 0 ? (const void*)pl->w64[a] : (const void*)pl->w32[a];
     }
@@ -1017,7 +1057,7 @@ static FftArgs fft_args64(const FftPlan* pl, const ToepDesc* td, int kofs, int n
     f.F3 = pl->F[2];
     for (int a = 0; a < 3; ++a) {
         f.nst[a] = pl->nst[a];
-        for (int i = 0; i < FFT_MAX_ST; ++i) f.rad[a][i] = pl->rad[a][i];
+        fft_stages(f, pl, a);
         f.lpb[a] = fft_lpb(pl->F[a]);
         f.w[a] = (const void*)pl->w64[a];
     }
