@@ -96,6 +96,9 @@ struct rttddft_ctx {
     DgToep* dg_toep = nullptr;                  // interstitial sum (direct, FP64 form)
     zd* d_mtd = nullptr;
     int mtd_stride = 0;
+    DgLeft* dgl_pp = nullptr;                   // many states: [PP_x; PP_y; PP_z] and its product with theta
+    DgGemm* dg_j = nullptr;
+    zd* d_jw = nullptr;
     std::vector<zd*> dv_t, dv_w;                // per k T = dV~ * CC_G and W = dh L of the rebuild
     zd* d_proj = nullptr;                       // CC^H S C of every k-point (one slice)
     DgSeries* series = nullptr;                 // Chebyshev series as digit products (many states)
@@ -295,6 +298,8 @@ static StepArgs make_args(rttddft_ctx* ctx, int dv_on) {
     a.mtd = ctx->d_mtd;
     a.mtd_stride = ctx->mtd_stride;
     a.mt64 = ctx->dg_mt ? 1 : 0;
+    a.dg_j = ctx->dg_j;
+    a.jw = ctx->d_jw;
     return a;
 }
 
@@ -820,6 +825,8 @@ void rttddft_destroy(rttddft_ctx* ctx) {
     tc_mt_destroy(ctx->tcmt);
     dg_series_destroy(ctx->series);
     drop_dg(ctx);
+    dg_gemm_destroy(ctx->dg_j);
+    dg_left_destroy(ctx->dgl_pp);
     fft_plan_destroy(ctx->fft);
     for (void* p : ctx->allocs) cudaFree(p);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
@@ -1459,6 +1466,8 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
                 std::string why;
                 const int e = tc_mt_create(&ctx->tcmt, nk, at.n, ctx->maxm, ns, ctx->d_flag, ctx->stream, &why);
                 if (e) fail(ctx, e, why);
+                launch_tc_mt_static(ctx->tcmt, make_args(ctx, 0), ctx->stream);
+                KCHECK();
             }
         }
         {
@@ -1470,6 +1479,19 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
             // many states or rows: digit products; without the memory for the digits one launch
             // per term
             if (o->propagator != RTTDDFT_PROP_EIG && ctx->coop_grid == 0) ctx->series = dg_series_create(nk, naux, ns);
+        }
+        if (ns > JRHO_MIN_NS) {
+            // the subspace current of many states: PP theta on the tensor cores
+            std::vector<DgMat> pm(nk);
+            std::vector<DgRight> pr(nk);
+            ctx->d_jw = dalloc<zd>(ctx, (size_t)nk * 3 * naux * ns);
+            for (int k = 0; k < nk; ++k) {
+                KDev& K = ctx->hkd[k];
+                pm[k] = DgMat{K.psub, (size_t)naux, 1, 1, 3 * naux, naux};  // PP is Hermitian: rows from the stored columns
+                pr[k] = DgRight{K.theta, naux, naux, ctx->d_jw + (size_t)k * 3 * naux * ns, 3 * naux};
+            }
+            ctx->dgl_pp = dg_left_create(nk, pm.data(), ctx->stream);
+            if (ctx->dgl_pp) ctx->dg_j = dg_gemm_create(ctx->dgl_pp, nk, pr.data(), ns, ctx->d_flag);
         }
         // ---- theta(0)
         if (s->c0) {

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(256) k_gemm_cn32(const GemmDesc* __restrict__ 
             const int q = e / NT, j = e % NT;
             const int m = m0 + q, n = n0 + j;
             if (m >= d.M || n >= N) continue;
-            const zd val = zscale(zmk((double)red[warp][2 * e], (double)red[warp][2 * e + 1]), sc);
+            const zd val = zscale(zmk(f2d(red[warp][2 * e]), f2d(red[warp][2 * e + 1])), sc);
             if (part) {
                 part[d.part_off + ((size_t)blockIdx.y * N + n) * d.M + m] = val;
             } else {

@@ -940,36 +940,38 @@ __global__ void __launch_bounds__(32) k_local(StepArgs a) {
         for (int e = 10 * NT; e < VP; ++e) v[e] = (R)0;
         warp_sum_store<R, VP>(v, lane, red);
         __syncwarp();
-        if (lane == 0) {
-            for (int j = 0; j < NT; ++j) {
-                const int c = n0 + j;
-                if (c >= ns) break;
-                const zd zh = zmk((double)red[10 * j], (double)red[10 * j + 1]);
-                const zd zs = zmk((double)red[10 * j + 2], (double)red[10 * j + 3]);
-                const zd q0 = zmk((double)red[10 * j + 4], (double)red[10 * j + 5]);
-                const zd q1 = zmk((double)red[10 * j + 6], (double)red[10 * j + 7]);
-                const zd q2 = zmk((double)red[10 * j + 8], (double)red[10 * j + 9]);
-                zd xi;
-                const double f = a.occ[c];
-                if (i < na) {
-                    K.Z[aoff + i + (size_t)c * ma] = zh;
-                    K.Z[aoff + i + (size_t)(ns + c) * ma] = zs;
-                    xi = K.Q[aoff + i + (size_t)c * ma];
-                } else {
-                    const int r = lo0 + (i - na);
-                    K.Y[r + (size_t)c * nb] = zh;
-                    K.Y[r + (size_t)(ns + c) * nb] = zs;
-                    xi = K.C[r + (size_t)c * nb];
-                    jc[3] += f * (xi.x * zh.x + xi.y * zh.y);
-                    jc[4] += f * (xi.x * zs.x + xi.y * zs.y);
-                }
-                jc[0] += f * (xi.x * q0.x + xi.y * q0.y);
-                jc[1] += f * (xi.x * q1.x + xi.y * q1.y);
-                jc[2] += f * (xi.x * q2.x + xi.y * q2.y);
+        // lane j finishes column n0 + j (one lane after the other took 10 us at four columns)
+        if (lane < NT && n0 + lane < ns) {
+            const int j = lane, c = n0 + j;
+            const zd zh = zmk((double)red[10 * j], (double)red[10 * j + 1]);
+            const zd zs = zmk((double)red[10 * j + 2], (double)red[10 * j + 3]);
+            const zd q0 = zmk((double)red[10 * j + 4], (double)red[10 * j + 5]);
+            const zd q1 = zmk((double)red[10 * j + 6], (double)red[10 * j + 7]);
+            const zd q2 = zmk((double)red[10 * j + 8], (double)red[10 * j + 9]);
+            zd xi;
+            const double f = a.occ[c];
+            if (i < na) {
+                K.Z[aoff + i + (size_t)c * ma] = zh;
+                K.Z[aoff + i + (size_t)(ns + c) * ma] = zs;
+                xi = zscale(K.Q[aoff + i + (size_t)c * ma], f);
+            } else {
+                const int r = lo0 + (i - na);
+                K.Y[r + (size_t)c * nb] = zh;
+                K.Y[r + (size_t)(ns + c) * nb] = zs;
+                xi = zscale(K.C[r + (size_t)c * nb], f);
+                jc[3] += xi.x * zh.x + xi.y * zh.y;
+                jc[4] += xi.x * zs.x + xi.y * zs.y;
             }
+            jc[0] += xi.x * q0.x + xi.y * q0.y;
+            jc[1] += xi.x * q1.x + xi.y * q1.y;
+            jc[2] += xi.x * q2.x + xi.y * q2.y;
         }
         __syncwarp();
     }
+#pragma unroll
+    for (int o = 1; o < NT; o <<= 1)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) jc[q] += __shfl_xor_sync(0xffffffffu, jc[q], o);
     if (lane == 0) {
         double* pj = a.part_jmt + ((size_t)k * at.lrows + row) * 5;
 #pragma unroll
@@ -1341,16 +1343,18 @@ __global__ void __launch_bounds__(BT) k_toep_seg(StepArgs a, int n0, int slot0) 
 // Re c^H HC, Re c^H SC and sum (G+k)|c|^2 into its slot of part_full.
 template <int NT>
 // Columns n0 .. n1-1: at most NT when the slot partials are read; all
-// columns in one launch when both parts arrive whole (K.th and K.tb).
-__global__ void __launch_bounds__(BKB) k_back(StepArgs a, int n0, int n1) {
-    __shared__ double rs[8];
+// columns in one launch when both parts arrive whole (K.th and K.tb).  A warp
+// takes every (number of warps)-th column of the block's 32 rows: a row's FP64
+// chain over all of them took 75 us at N_s 60 whatever the number of rows.
+__global__ void __launch_bounds__(256) k_back(StepArgs a, int n0, int n1) {
+    __shared__ double rs[8][8];
     const int k = blockIdx.z;
     const KDev& K = a.kd[k];
     const int ng = K.ng;
     const int g0 = blockIdx.x * BKB;
     if (g0 >= ng) return;
-    const int tid = threadIdx.x;
-    const int g = g0 + tid;
+    const int lane = threadIdx.x & 31, cg = threadIdx.x >> 5, ncg = blockDim.x >> 5;
+    const int g = g0 + lane;
     const bool act = g < ng;
     const int ns = a.ns, nb = K.nb;
     const zd* __restrict__ X = K.C;
@@ -1362,7 +1366,8 @@ __global__ void __launch_bounds__(BKB) k_back(StepArgs a, int n0, int n1) {
         const double* q = K.gk + 3 * (size_t)g;
         const double dg = 0.5 * (dsq(q[0] + st->cur_a[0] * a.inv_c) + dsq(q[1] + st->cur_a[1] * a.inv_c) +
                                  dsq(q[2] + st->cur_a[2] * a.inv_c));
-        for (int cc = n0; cc < n1; ++cc) {
+        double wsum = 0.0;
+        for (int cc = n0 + cg; cc < n1; cc += ncg) {
             const int c = cc - n0;  // column within the slot partials
             zd th = zmk(0.0, 0.0), ts = zmk(0.0, 0.0);
             // slot partials, loads issued four slots at a time (in slot order)
@@ -1394,23 +1399,24 @@ __global__ void __launch_bounds__(BKB) k_back(StepArgs a, int n0, int n1) {
             const zd sv = zadd(ts, x);
             K.Y[g + (size_t)(n0 + c) * nb] = hv;
             K.Y[g + (size_t)(ns + n0 + c) * nb] = sv;
-            const double f = a.occ[n0 + c];
-            const double w = f * (x.x * x.x + x.y * x.y);
-            red[0] += f * (x.x * hv.x + x.y * hv.y);
-            red[1] += f * (x.x * sv.x + x.y * sv.y);
-            red[2] += q[0] * w;
-            red[3] += q[1] * w;
-            red[4] += q[2] * w;
+            const zd fx = zscale(x, a.occ[n0 + c]);
+            red[0] += fx.x * hv.x + fx.y * hv.y;
+            red[1] += fx.x * sv.x + fx.y * sv.y;
+            wsum += fx.x * x.x + fx.y * x.y;
         }
+        red[2] = q[0] * wsum;
+        red[3] = q[1] * wsum;
+        red[4] = q[2] * wsum;
     }
-    // one warp: halving sum of the five shares
-    const int lane = tid & 31;
+    // halving sums of the five shares, then the warps' sums in order
     double v[8] = {red[0], red[1], red[2], red[3], red[4], 0.0, 0.0, 0.0};
-    warp_sum_store<double, 8>(v, lane, rs);
-    __syncwarp();
-    if (tid < 5) {
-        double* pf = a.part_full + ((size_t)k * a.max_nback + blockIdx.x) * 5 + tid;
-        *pf = (n0 == 0) ? rs[tid] : *pf + rs[tid];
+    warp_sum_store<double, 8>(v, lane, rs[cg]);
+    __syncthreads();
+    if (threadIdx.x < 5) {
+        double t = rs[0][threadIdx.x];
+        for (int w = 1; w < ncg; ++w) t += rs[w][threadIdx.x];
+        double* pf = a.part_full + ((size_t)k * a.max_nback + blockIdx.x) * 5 + threadIdx.x;
+        *pf = (n0 == 0) ? t : *pf + t;
     }
 }
 
@@ -1440,11 +1446,12 @@ __device__ double block_max(double v, double* sh) {
 // theta~ = CC^H S C from the split-K partials (l == 0: its deviation from
 // theta and, for N_s <= 4, the row's share of theta^H theta~), and the
 // row's share of J_sub,l = sum_n f_n Re theta_in^* ((PP_l + A_l/c) theta)_in.
-__device__ void post_body(const StepArgs& a, int do_theta, int do_j);
+// The rows of theta~ and of the current are warps of their own (in one warp
+// after the other a row took the sum of both), and the four columns of a step
+// are finished by four lanes: 44 -> 30 us at N_aux 240, N_s 7.
 // (the step's finalize stays a launch of its own: run by the last post block
 // it measured slower, 30 against 25 us at h2_6000, with fewer threads)
-__global__ void __launch_bounds__(128) k_post(StepArgs a, int do_theta, int do_j) { post_body(a, do_theta, do_j); }
-__device__ void post_body(const StepArgs& a, int do_theta, int do_j) {
+__global__ void __launch_bounds__(128) k_post(StepArgs a, int do_theta, int do_j) {
     // halving warp sums over up to 4 columns at a time (each warp-wide FP64 add
     // is costly on GB300); per-warp scratch for the sums
     __shared__ double ws[4][8];
@@ -1452,80 +1459,137 @@ __device__ void post_body(const StepArgs& a, int do_theta, int do_j) {
     const KDev& K = a.kd[k];
     const int n = a.naux, ns = a.ns;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int w = blockIdx.x * 4 + warp;
-    if (w >= 3 * n) return;
-    const int i = w / 3, l = w % 3;
-    double* prow = a.part_post + ((size_t)k * n + i) * POST_STRIDE;
-    if (do_theta && l == 0) {
-        const GemmDesc d = a.gd_proj[k];
-        const int nsp = (d.K + a.kc_proj - 1) / a.kc_proj;
-        double res = 0.0;
-        zd mine = zmk(0.0, 0.0);
-        for (int c0 = 0; c0 < ns; c0 += 4) {
-            double v[8];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                zd t = zmk(0.0, 0.0);
-                if (c0 + q < ns)
-                    for (int sp = lane; sp < nsp; sp += 32)
-                        t = zadd(t, a.part_proj[d.part_off + ((size_t)sp * ns + c0 + q) * n + i]);
-                v[2 * q] = t.x;
-                v[2 * q + 1] = t.y;
-            }
-            warp_sum_store<double, 8>(v, lane, ws[warp]);
-            __syncwarp();
-            for (int q = 0; q < 4 && c0 + q < ns; ++q) {
-                const int c = c0 + q;
-                const zd t = zmk(ws[warp][2 * q], ws[warp][2 * q + 1]);
-                if (lane == 0) K.theta_t[i + (size_t)c * n] = t;
-                const zd dd = zsub(t, K.theta[i + (size_t)c * n]);
-                res = fmax(res, dd.x * dd.x + dd.y * dd.y);
-                if (lane == c) mine = t;
-            }
-            __syncwarp();
-        }
-        res = sqrt(res);
-        if (ns <= 4) {
-            // row i's share of theta^H theta~ (= C^H S C for C = CC theta)
-            const int pq = lane, pp = pq % ns, qq = pq / ns;
-            const double tx = __shfl_sync(0xffffffffu, mine.x, qq < 32 ? qq : 0);
-            const double ty = __shfl_sync(0xffffffffu, mine.y, qq < 32 ? qq : 0);
-            if (pq < ns * ns) {
-                const zd tp = K.theta[i + (size_t)pp * n];
-                prow[4 + 2 * pq] = tp.x * tx + tp.y * ty;
-                prow[4 + 2 * pq + 1] = tp.x * ty - tp.y * tx;
-            }
-        }
-        if (lane == 0) prow[0] = res;
-    }
-    if (do_j) {
+    int w = blockIdx.x * 4 + warp;
+    if (do_j && w < 3 * n) {
+        const int i = w / 3, l = w % 3;
         const zd* __restrict__ P = K.psub + (size_t)l * n * n + (size_t)i * n;
         const double al = a.st->cur_a[l] * a.inv_c;
         double jl = 0.0;
         for (int c0 = 0; c0 < ns; c0 += 4) {
+            zd t[4] = {zmk(0.0, 0.0), zmk(0.0, 0.0), zmk(0.0, 0.0), zmk(0.0, 0.0)};
+            const zd* th = K.theta + (size_t)c0 * n;
+            const int nc = min(4, ns - c0);
+            for (int j = lane; j < n; j += 32) {
+                const zd p = P[j];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q < nc) zfmac(t[q], p, th[(size_t)q * n + j]);
+            }
             double v[8];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                zd t = zmk(0.0, 0.0);
-                if (c0 + q < ns) {
-                    const zd* th = K.theta + (size_t)(c0 + q) * n;
-                    for (int j = lane; j < n; j += 32) zfmac(t, P[j], th[j]);
-                }
-                v[2 * q] = t.x;
-                v[2 * q + 1] = t.y;
+                v[2 * q] = t[q].x;
+                v[2 * q + 1] = t[q].y;
             }
             warp_sum_store<double, 8>(v, lane, ws[warp]);
             __syncwarp();
-            if (lane == 0) {
-                for (int q = 0; q < 4 && c0 + q < ns; ++q) {
-                    const int c = c0 + q;
-                    const zd ti = K.theta[i + (size_t)c * n];
-                    jl += a.occ[c] * (ti.x * (ws[warp][2 * q] + al * ti.x) + ti.y * (ws[warp][2 * q + 1] + al * ti.y));
-                }
+            if (lane < nc) {
+                const zd ti = th[(size_t)lane * n + i];
+                jl += a.occ[c0 + lane] * (ti.x * (ws[warp][2 * lane] + al * ti.x) + ti.y * (ws[warp][2 * lane + 1] + al * ti.y));
             }
             __syncwarp();
         }
-        if (lane == 0) prow[1 + l] = jl;
+        jl += __shfl_xor_sync(0xffffffffu, jl, 1);
+        jl += __shfl_xor_sync(0xffffffffu, jl, 2);
+        if (lane == 0) a.part_post[((size_t)k * n + i) * POST_STRIDE + 1 + l] = jl;
+        return;
+    }
+    if (do_j) w -= 3 * n;
+    if (!do_theta || w >= n) return;
+    const int i = w;
+    double* prow = a.part_post + ((size_t)k * n + i) * POST_STRIDE;
+    const GemmDesc d = a.gd_proj[k];
+    const int nsp = (d.K + a.kc_proj - 1) / a.kc_proj;
+    double res = 0.0;
+    zd mine = zmk(0.0, 0.0);  // N_s <= 4: lane c holds column c
+    for (int c0 = 0; c0 < ns; c0 += 4) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            zd t = zmk(0.0, 0.0);
+            if (c0 + q < ns)
+                for (int sp = lane; sp < nsp; sp += 32)
+                    t = zadd(t, a.part_proj[d.part_off + ((size_t)sp * ns + c0 + q) * n + i]);
+            v[2 * q] = t.x;
+            v[2 * q + 1] = t.y;
+        }
+        warp_sum_store<double, 8>(v, lane, ws[warp]);
+        __syncwarp();
+        if (lane < 4 && c0 + lane < ns) {
+            const zd t = zmk(ws[warp][2 * lane], ws[warp][2 * lane + 1]);
+            const size_t e = i + (size_t)(c0 + lane) * n;
+            K.theta_t[e] = t;
+            const zd dd = zsub(t, K.theta[e]);
+            res = fmax(res, dd.x * dd.x + dd.y * dd.y);
+            mine = t;
+        }
+        __syncwarp();
+    }
+    res = fmax(res, __shfl_xor_sync(0xffffffffu, res, 1));
+    res = fmax(res, __shfl_xor_sync(0xffffffffu, res, 2));
+    if (ns <= 4) {
+        // row i's share of theta^H theta~ (= C^H S C for C = CC theta)
+        const int pq = lane, pp = pq % ns, qq = pq / ns;
+        const double tx = __shfl_sync(0xffffffffu, mine.x, qq < 32 ? qq : 0);
+        const double ty = __shfl_sync(0xffffffffu, mine.y, qq < 32 ? qq : 0);
+        if (pq < ns * ns) {
+            const zd tp = K.theta[i + (size_t)pp * n];
+            prow[4 + 2 * pq] = tp.x * tx + tp.y * ty;
+            prow[4 + 2 * pq + 1] = tp.x * ty - tp.y * tx;
+        }
+    }
+    if (lane == 0) prow[0] = sqrt(res);
+}
+// theta~ and its deviation from theta for many states: 32 rows x 8 column groups
+__global__ void __launch_bounds__(256) k_post_theta(StepArgs a) {
+    __shared__ double red[8][32];
+    const int k = blockIdx.z;
+    const KDev& K = a.kd[k];
+    const int n = a.naux, ns = a.ns;
+    const int lane = threadIdx.x & 31, cg = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    const GemmDesc d = a.gd_proj[k];
+    const int nsp = (d.K + a.kc_proj - 1) / a.kc_proj;
+    double res = 0.0;
+    if (i < n)
+        for (int c = cg; c < ns; c += 8) {
+            zd t = zmk(0.0, 0.0);
+            for (int sp = 0; sp < nsp; ++sp) t = zadd(t, a.part_proj[d.part_off + ((size_t)sp * ns + c) * n + i]);
+            const size_t e = i + (size_t)c * n;
+            K.theta_t[e] = t;
+            const zd dd = zsub(t, K.theta[e]);
+            res = fmax(res, dd.x * dd.x + dd.y * dd.y);
+        }
+    red[cg][lane] = res;
+    __syncthreads();
+    if (cg == 0 && i < n) {
+        for (int w = 1; w < 8; ++w) res = fmax(res, red[w][lane]);
+        a.part_post[((size_t)k * n + i) * POST_STRIDE] = sqrt(res);
+    }
+}
+// Rows' shares of the current from W = [PP_x; PP_y; PP_z] theta (digit products):
+// sum_n f_n Re theta_in^* (W_(l,i)n + (A_l/c) theta_in); 32 rows x 8 column groups
+__global__ void __launch_bounds__(256) k_jw(StepArgs a) {
+    __shared__ double red[8][32];
+    const int k = blockIdx.z, l = blockIdx.y;
+    const KDev& K = a.kd[k];
+    const int n = a.naux, ns = a.ns;
+    const int lane = threadIdx.x & 31, cg = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    const zd* W = a.jw + (size_t)k * 3 * n * ns + (size_t)l * n;
+    const double al = a.st->cur_a[l] * a.inv_c;
+    double v = 0.0, q = 0.0;
+    if (i < n)
+        for (int c = cg; c < ns; c += 8) {
+            const zd t = K.theta[i + (size_t)c * n], w = W[i + (size_t)c * 3 * n];
+            const zd ft = zscale(t, a.occ[c]);
+            v += ft.x * w.x + ft.y * w.y;
+            q += ft.x * t.x + ft.y * t.y;
+        }
+    red[cg][lane] = v + al * q;
+    __syncthreads();
+    if (cg == 0 && i < n) {
+        v = red[0][lane];
+        for (int w = 1; w < 8; ++w) v += red[w][lane];
+        a.part_post[((size_t)k * n + i) * POST_STRIDE + 1 + l] = v;
     }
 }
 
@@ -1611,18 +1675,31 @@ __global__ void __launch_bounds__(256) k_jrho(StepArgs a) {
 }
 
 // The post-projection launch(es): theta~ and its residual per row (do_theta),
-// and the subspace current (do_j), by rows for few states and through the
-// density matrix for many.
-void launch_post(const StepArgs& a, int do_theta, int do_j, cudaStream_t s) {
-    const bool rho = do_j && a.ns > JRHO_MIN_NS;
-    if (do_theta || !rho) {
-        dim3 g((3 * a.naux + 3) / 4, 1, a.nk);
-        k_post<<<g, 128, 0, s>>>(a, do_theta, rho ? 0 : do_j);
+// and the subspace current (do_j): by rows for few states, for many from PP theta
+// as digit products (without the memory for PP's digits through the density
+// matrix).  N_aux 300, N_s 60, 2 k: theta~ and J together 146 us with the density
+// matrix in FP64, 54 us with the digits.  Returns the launches.
+int launch_post(const StepArgs& a, int do_theta, int do_j, cudaStream_t s) {
+    if (a.ns <= JRHO_MIN_NS) {
+        const int rows = (do_j ? 3 * a.naux : 0) + (do_theta ? a.naux : 0);
+        k_post<<<dim3((rows + 3) / 4, 1, a.nk), 128, 0, s>>>(a, do_theta, do_j);
+        return 1;
     }
-    if (rho) {
+    const dim3 g((a.naux + 31) / 32, 1, a.nk);
+    int nl = 0;
+    if (do_theta) {
+        k_post_theta<<<g, 256, 0, s>>>(a);
+        ++nl;
+    }
+    if (do_j && a.dg_j) {
+        nl += launch_dg_gemm(a.dg_j, 0, a.nk, 0, s) + 1;
+        k_jw<<<dim3(g.x, 3, a.nk), 256, 0, s>>>(a);
+    } else if (do_j) {
         const int nt = (a.naux + JRHO_T - 1) / JRHO_T;
         k_jrho<<<dim3(nt * (nt + 1) / 2, 1, a.nk), 256, 0, s>>>(a);
+        ++nl;
     }
+    return nl;
 }
 
 // theta <- theta~ (3 I - theta~^H theta~) / 2: one Newton-Schulz step of the
@@ -1755,27 +1832,53 @@ __global__ void __launch_bounds__(256) k_fin_part(StepArgs a, int set_gs) {
 // |C^H S C - I| for many states: column j of the gram theta^H theta~ per block
 // (one warp per row i, lanes over the subspace rows), its largest deviation
 // from the identity into gdev[k][j] (FP64).
-__global__ void __launch_bounds__(256) k_gram_dev(StepArgs a) {
-    __shared__ double wm[8];
+#define GRAM_W 16
+__host__ __device__ constexpr int gram_per_warp(int ns) { return ns > GRAM_W ? 4 : 1; }
+__global__ void __launch_bounds__(32 * GRAM_W) k_gram_dev(StepArgs a) {
+    __shared__ double wm[GRAM_W], ws[GRAM_W][8];
     const int k = blockIdx.y, j = blockIdx.x;
     const KDev& K = a.kd[k];
     const int n = a.naux, ns = a.ns;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const zd* tt = K.theta_t + (size_t)j * n;
     double dev = 0.0;
-    for (int i = warp; i < ns; i += 8) {
-        const zd* th = K.theta + (size_t)i * n;
-        zd g = zmk(0.0, 0.0);
-        for (int r = lane; r < n; r += 32) zfmac(g, th[r], tt[r]);
-        g = warp_zsum(g);
-        if (i == j) g.x -= 1.0;
-        dev = fmax(dev, hypot(g.x, g.y));
+    // many states: four of a warp at a time, one halving sum, four lanes' deviations
+    const int pq = gram_per_warp(ns);
+    for (int i0 = warp * pq; i0 < ns; i0 += (int)(blockDim.x >> 5) * pq) {
+        if (pq == 1) {
+            zd g = zmk(0.0, 0.0);
+            for (int r = lane; r < n; r += 32) zfmac(g, K.theta[(size_t)i0 * n + r], tt[r]);
+            g = warp_zsum(g);
+            if (i0 == j) g.x -= 1.0;
+            dev = fmax(dev, hypot(g.x, g.y));
+            continue;
+        }
+        zd g[4] = {zmk(0.0, 0.0), zmk(0.0, 0.0), zmk(0.0, 0.0), zmk(0.0, 0.0)};
+        const int nc = min(pq, ns - i0);
+        for (int r = lane; r < n; r += 32) {
+            const zd t = tt[r];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (q < nc) zfmac(g[q], K.theta[(size_t)(i0 + q) * n + r], t);
+        }
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[2 * q] = g[q].x;
+            v[2 * q + 1] = g[q].y;
+        }
+        warp_sum_store<double, 8>(v, lane, ws[warp]);
+        __syncwarp();
+        if (lane < nc) dev = fmax(dev, hypot(ws[warp][2 * lane] - (i0 + lane == j ? 1.0 : 0.0), ws[warp][2 * lane + 1]));
+        __syncwarp();
     }
+    dev = fmax(dev, __shfl_xor_sync(0xffffffffu, dev, 1));
+    dev = fmax(dev, __shfl_xor_sync(0xffffffffu, dev, 2));
     if (lane == 0) wm[warp] = dev;
     __syncthreads();
     if (threadIdx.x == 0) {
         double m = wm[0];
-        for (int w = 1; w < 8; ++w) m = fmax(m, wm[w]);
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wm[w]);
         a.gdev[(size_t)k * ns + j] = m;
     }
 }
@@ -2300,7 +2403,7 @@ static int back_launch(const StepArgs& a, int maxng, cudaStream_t s, TraceHook* 
     if (gt.y == 0) {
         // both parts arrive whole (K.th and K.tb): every column in one launch
         if (join) cudaStreamWaitEvent(s, join, 0);
-        k_back<NT><<<gb, BKB, 0, s>>>(a, 0, a.ns);
+        k_back<NT><<<gb, 32 * std::min(8, a.ns), 0, s>>>(a, 0, a.ns);
         mark(tr, "back_finish", s);
         return 1;
     }
@@ -2309,7 +2412,7 @@ static int back_launch(const StepArgs& a, int maxng, cudaStream_t s, TraceHook* 
         k_toep_seg<TA, TT, TC, NT><<<gt, BT, sm, s>>>(a, n0, slot0);
         mark(tr, slot0 ? "backprojection" : "toeplitz_and_backprojection", s);
         if (join && n0 == 0) cudaStreamWaitEvent(s, join, 0);  // the interstitial rows of the side stream
-        k_back<NT><<<gb, BKB, 0, s>>>(a, n0, std::min(n0 + NT, a.ns));
+        k_back<NT><<<gb, 32 * std::min(8, std::min(NT, a.ns - n0)), 0, s>>>(a, n0, std::min(n0 + NT, a.ns));
         mark(tr, "back_finish", s);
         ++nl;
     }
@@ -2625,11 +2728,11 @@ void launch_step(const StepArgs& a, const StepPlan& p, cudaStream_t s, int* nlau
     else if (p.dg_proj) nl += launch_dg_gemm(p.dg_proj, 0, a.nk, 0, s) - 1;
     else launch_gemm_cn(p.gd_proj, a.nk, a.naux, p.maxnb, a.ns, p.kc_proj, p.part, 0, f32, nullptr, s);
     mark(tr, "gemm_project", s);
-    launch_post(a, 1, a.reproject ? 0 : 1, s);
+    nl += launch_post(a, 1, a.reproject ? 0 : 1, s) - 1;
     mark(tr, "project_finish_current", s);
-    if (!a.reproject && a.ns > JRHO_MIN_NS) ++nl;
     if (a.ns > 4) {
-        k_gram_dev<<<dim3(a.ns, a.nk), 256, 0, s>>>(a);
+        k_gram_dev<<<dim3(a.ns, a.nk), 32 * std::min(GRAM_W, (a.ns + gram_per_warp(a.ns) - 1) / gram_per_warp(a.ns)), 0,
+                     s>>>(a);
         mark(tr, "gram", s);
         ++nl;
     }

@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(128, 1)
 // the same split in FP64 arithmetic ran on the 1/64-rate pipe, 40 us of a
 // 9917 x 300 operand
 __device__ __forceinline__ void split_bf16(double v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
-    const float w = (float)v;
+    const float w = d2f(v);
     hi = __float2bfloat16_rn(w);
     lo = __float2bfloat16_rn(w - __bfloat162float(hi));
 }
@@ -227,8 +227,8 @@ __global__ void __launch_bounds__(256) k_tc_combine(const float* __restrict__ D,
         double re = 0.0, im = 0.0;
         for (int s = 0; s < splits; ++s) {
             const float* d = D + ((size_t)s * M + m) * Dn;
-            re += (double)d[n];
-            im += (double)d[Nc + n];
+            re += f2d(d[n]);
+            im += f2d(d[Nc + n]);
         }
         t[q][x] = zmk(re, im);
     }
@@ -1026,7 +1026,7 @@ struct Sum2f {
         e += (s - (t - bp)) + (x - bp);
         s = t;
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+    __device__ __forceinline__ double value() const { return f2d(s) + f2d(e); }
 };
 // A tile of TC_RT output rows of one product: the FP32 slice partials
 // D[s][row][Dn] (real columns c < nc: Re, nc + c: Im) summed over the nsp
@@ -1034,13 +1034,14 @@ struct Sum2f {
 // shared memory so that the loads run along the rows of D and the stores
 // along the columns of the column-major output out[row + c ld].
 #define TC_RT 16
+template <int RT>
 __device__ void tc_red_tile(const float* __restrict__ D, size_t sstride, int nsp, int Dn, int nc, int row0,
                             int nrow, double scale, zd* __restrict__ out, size_t ld, double (*tile)[257]) {
     const int n2 = 2 * nc;
     if ((n2 & 3) == 0 && (Dn & 3) == 0 && (sstride & 3) == 0 && ((uintptr_t)D & 15) == 0) {
         // four adjacent columns per thread (16-byte loads), the same slice order
         const int q4 = n2 >> 2;
-        for (int e = threadIdx.x; e < TC_RT * q4; e += blockDim.x) {
+        for (int e = threadIdx.x; e < RT * q4; e += blockDim.x) {
             const int r = e / q4, c = (e % q4) * 4, row = row0 + r;
             Sum2f v0, v1, v2, v3;
             if (row < nrow) {
@@ -1066,7 +1067,7 @@ __device__ void tc_red_tile(const float* __restrict__ D, size_t sstride, int nsp
             tile[r][c + 3] = v3.value();
         }
     } else {
-        for (int e = threadIdx.x; e < TC_RT * n2; e += blockDim.x) {
+        for (int e = threadIdx.x; e < RT * n2; e += blockDim.x) {
             const int r = e / n2, c = e % n2, row = row0 + r;
             Sum2f v;
             if (row < nrow) {
@@ -1083,9 +1084,10 @@ __device__ void tc_red_tile(const float* __restrict__ D, size_t sstride, int nsp
         }
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < TC_RT * nc; e += blockDim.x) {
-        const int r = e % TC_RT, c = e / TC_RT, row = row0 + r;
-        if (row < nrow) out[row + (size_t)c * ld] = zmk(tile[r][c] * scale, tile[r][nc + c] * scale);
+    for (int e = threadIdx.x; e < RT * nc; e += blockDim.x) {
+        const int r = e % RT, c = e / RT, row = row0 + r;
+        const zd v = zmk(tile[r][c], tile[r][nc + c]);
+        if (row < nrow) out[row + (size_t)c * ld] = scale == 1.0 ? v : zscale(v, scale);
     }
 }
 
@@ -1103,7 +1105,7 @@ __global__ void __launch_bounds__(256) k_tc_opred(TcRedParams p) {
         const int nsp = min(p.splits_b, (p.nkb_b + p.kbps_b - 1) / p.kbps_b);
         const int row0 = blockIdx.x * TC_RT;
         if (row0 >= ng) return;
-        tc_red_tile(p.Db + (size_t)k * p.splits_b * p.Rb * p.Dnb, (size_t)p.Rb * p.Dnb, nsp, p.Dnb, 2 * ns, row0, ng,
+        tc_red_tile<TC_RT>(p.Db + (size_t)k * p.splits_b * p.Rb * p.Dnb, (size_t)p.Rb * p.Dnb, nsp, p.Dnb, 2 * ns, row0, ng,
                     p.inv_b, K.tb, ng, tile);
         return;
     }
@@ -1112,13 +1114,13 @@ __global__ void __launch_bounds__(256) k_tc_opred(TcRedParams p) {
         const int row0 = blockIdx.x * TC_RT;
         if (row0 >= ng) return;
         const int nsp = min(p.splits_t, (nkb + p.kbps_t - 1) / p.kbps_t);
-        tc_red_tile(p.Dt + (size_t)k * p.splits_t * p.Rt * p.Dn, (size_t)p.Rt * p.Dn, nsp, p.Dn, ns, row0, ng, p.inv_t,
+        tc_red_tile<TC_RT>(p.Dt + (size_t)k * p.splits_t * p.Rt * p.Dn, (size_t)p.Rt * p.Dn, nsp, p.Dn, ns, row0, ng, p.inv_t,
                     K.th, ng, tile);
     } else if (p.part != 1) {
         const int row0 = (blockIdx.x - tiles_t) * TC_RT;
         if (row0 >= p.ma) return;
         const int nsp = min(p.splits_a, (nkb + p.kbps_a - 1) / p.kbps_a);
-        tc_red_tile(p.Da + (size_t)k * p.splits_a * p.Ra * p.Dn, (size_t)p.Ra * p.Dn, nsp, p.Dn, ns, row0, p.ma,
+        tc_red_tile<TC_RT>(p.Da + (size_t)k * p.splits_a * p.Ra * p.Dn, (size_t)p.Ra * p.Dn, nsp, p.Dn, ns, row0, p.ma,
                     p.inv_a, K.Q, p.ma, tile);
     }
 }
@@ -1995,7 +1997,7 @@ __global__ void __launch_bounds__(256) k_tc_dvred(TcDvRedParams p) {
     const int row0 = blockIdx.x * TC_RT;
     if (row0 >= ng) return;
     const int nsp = min(p.splits, (nkb + p.kbps - 1) / p.kbps);
-    tc_red_tile(p.D + (size_t)k * p.splits * p.Rt * TC_DV_NT, (size_t)p.Rt * TC_DV_NT, nsp, TC_DV_NT, p.h, row0, ng,
+    tc_red_tile<TC_RT>(p.D + (size_t)k * p.splits * p.Rt * TC_DV_NT, (size_t)p.Rt * TC_DV_NT, nsp, TC_DV_NT, p.h, row0, ng,
                 p.st->cur_s * p.inv, p.td[k].Y + (size_t)p.c0 * ng, ng, tile);
 }
 
@@ -2178,17 +2180,20 @@ struct TcCCRed {
     const float* D;
     zd* part;
 };
+// RT rows per block: the projection has only N_aux rows and many slices (16 a
+// block were 19 blocks at N_aux 300, 50 us)
+template <int RT>
 __global__ void __launch_bounds__(256) k_tc_ccred(TcCCRed p) {
-    __shared__ double tile[TC_RT][257];
+    __shared__ double tile[RT][257];
     const int k = blockIdx.z;
     const KDev& K = p.kd[k];
-    const int row0 = blockIdx.x * TC_RT;
+    const int row0 = blockIdx.x * RT;
     const int nrow = p.mode ? p.naux : K.nb;
     if (row0 >= nrow) return;
     const int nsp = p.mode ? min(p.splits, (((K.nb + 31) >> 5) + p.kbps - 1) / p.kbps) : 1;
     zd* out = p.mode ? p.part + (size_t)k * p.naux * p.ns : K.C;
-    tc_red_tile(p.D + (size_t)k * p.splits * p.R * p.Dn, (size_t)p.R * p.Dn, nsp, p.Dn, p.ns, row0, nrow, 1.0, out,
-                p.mode ? p.naux : K.nb, tile);
+    tc_red_tile<RT>(p.D + (size_t)k * p.splits * p.R * p.Dn, (size_t)p.R * p.Dn, nsp, p.Dn, p.ns, row0, nrow, 1.0, out,
+                    p.mode ? p.naux : K.nb, tile);
 }
 
 int tc_cc_create(TcCC** out, int nk, int naux, int ns, const int* nb, const zd* const* cc_dev, int* flag,
@@ -2327,7 +2332,7 @@ int launch_tcc_expand(const TcCC* t, const StepArgs& a, cudaStream_t s) {
                                                                                 t->Kp_e, t->NT, t->beh, t->bel, a.flag);
     tcc_product(t, 0, a.kd, a.nk, a.flag, s);
     TcCCRed r{0, t->ns, t->naux, t->Dn, t->Mp_e, 1, t->nkb_e, a.kd, t->De, nullptr};
-    k_tc_ccred<<<dim3((t->maxnb + TC_RT - 1) / TC_RT, 1, a.nk), 256, 0, s>>>(r);
+    k_tc_ccred<TC_RT><<<dim3((t->maxnb + TC_RT - 1) / TC_RT, 1, a.nk), 256, 0, s>>>(r);
     return 3;
 }
 // theta~ partials = CC^H (S C) into part (one slice per k-point, k * naux * ns apart)
@@ -2336,7 +2341,7 @@ int launch_tcc_project(const TcCC* t, const StepArgs& a, zd* part, cudaStream_t 
                                                                                  t->Kp_p, t->NT, t->bph, t->bpl, a.flag);
     tcc_product(t, 1, a.kd, a.nk, a.flag, s);
     TcCCRed r{1, t->ns, t->naux, t->Dn, t->Mp_p, t->splits_p, t->kbps_p, a.kd, t->Dp, part};
-    k_tc_ccred<<<dim3((t->naux + TC_RT - 1) / TC_RT, 1, a.nk), 256, 0, s>>>(r);
+    k_tc_ccred<2><<<dim3((t->naux + 1) / 2, 1, a.nk), 64, 0, s>>>(r);
     return 3;
 }
 
@@ -2433,35 +2438,54 @@ int tc_mt_create(TcMT** out, int nk, int nat, int maxm, int ns, int* flag, cudaS
 // left operand of a step: per atom the rows of [h_eff; o; p_x; p_y; p_z] with K
 // over the columns j of the m x m blocks (row r of the stack: [Re G(r, .) | Im
 // G(r, .)] per K block of 32), one thread per (i, j) of the atom's blocks
-__global__ void k_tc_mt_pack_a(StepArgs a, int Mp, int Kp, unsigned short* __restrict__ ah,
-                               unsigned short* __restrict__ al) {
+// q0 .. q1 - 1 of the stack's blocks: h_eff (0) changes every step, o and p do
+// not.  32 x 32 tiles turned through shared memory: read along the blocks'
+// columns, written along K.  Packing only h_eff, by tiles, took the muffin-tin
+// slot of 22 atoms, 60 states and 2 k from 220 to 126 us a step (all five blocks
+// written along the rows were 2 bytes per 32-byte sector).
+__global__ void __launch_bounds__(256) k_tc_mt_pack_a(StepArgs a, int Mp, int Kp, int q0, int q1, unsigned short* __restrict__ ah,
+                                                      unsigned short* __restrict__ al) {
+    __shared__ zd t[32][33];
     const AtomTab& at = *a.at;
-    const int atom = blockIdx.y;
-    if (atom >= at.n) return;
-    const int m = at.m[atom];
+    const int atom = blockIdx.z;
+    const int m = at.m[atom], i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+    if (i0 >= m || j0 >= m) return;
     const size_t mm = (size_t)m * m, bo = at.boff[atom];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
     const DevState* st = a.st;
     const double fx = st->cur_a[0] * a.inv_c, fy = st->cur_a[1] * a.inv_c, fz = st->cur_a[2] * a.inv_c;
     const double fa = st->cur_aa, sdv = st->cur_s;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < mm; e += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e % m), j = (int)(e / m);
-        const zd hv = a.h[bo + e], ov = a.o[bo + e];
-        const zd px = a.p[3 * bo + e], py = a.p[3 * bo + mm + e], pz = a.p[3 * bo + 2 * mm + e];
-        zd he = zmk(hv.x + fx * px.x + fy * py.x + fz * pz.x + fa * ov.x,
-                    hv.y + fx * px.y + fy * py.y + fz * pz.y + fa * ov.y);
-        if (a.dh && sdv != 0.0) {
-            const zd d = a.dh[bo + e];
-            he.x += sdv * d.x;
-            he.y += sdv * d.y;
+    for (int q = q0; q < q1; ++q) {
+        const zd* __restrict__ src = q == 1 ? a.o + bo : a.p + 3 * bo + (size_t)(q - 2) * mm;
+        for (int r = y; r < 32; r += 8) {
+            const int i = i0 + x, j = j0 + r;
+            if (i >= m || j >= m) continue;
+            const size_t e = i + (size_t)j * m;
+            zd v;
+            if (q == 0) {
+                const zd hv = a.h[bo + e], ov = a.o[bo + e];
+                const zd px = a.p[3 * bo + e], py = a.p[3 * bo + mm + e], pz = a.p[3 * bo + 2 * mm + e];
+                v = zmk(hv.x + fx * px.x + fy * py.x + fz * pz.x + fa * ov.x,
+                        hv.y + fx * px.y + fy * py.y + fz * pz.y + fa * ov.y);
+                if (a.dh && sdv != 0.0) {
+                    const zd d = a.dh[bo + e];
+                    v.x += sdv * d.x;
+                    v.y += sdv * d.y;
+                }
+            } else {
+                v = src[e];
+            }
+            t[x][r] = v;
         }
-        const zd blk[5] = {he, ov, px, py, pz};
-        const size_t col = (size_t)(j >> 5) * 64 + (j & 31);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            const size_t row = ((size_t)atom * Mp + q * m + i) * Kp + col;
-            put16(blk[q].x, 1, 1.0, ah, al, row, a.flag);
-            put16(blk[q].y, 1, 1.0, ah, al, row + 32, a.flag);
+        __syncthreads();
+        for (int r = y; r < 32; r += 8) {
+            const int i = i0 + r, j = j0 + x;
+            if (i >= m || j >= m) continue;
+            const size_t row = ((size_t)atom * Mp + q * m + i) * Kp + (size_t)(j >> 5) * 64 + (j & 31);
+            put16(t[r][x].x, 1, 1.0, ah, al, row, a.flag);
+            put16(t[r][x].y, 1, 1.0, ah, al, row + 32, a.flag);
         }
+        __syncthreads();
     }
 }
 // right operand of a step from the gathered V = [Q; C_lo] of every (k, atom) of
@@ -2498,13 +2522,19 @@ __global__ void k_tc_mt_w(StepArgs a, const float* __restrict__ D, int Mp, int D
     const float* d = D + z * Mp * Dn;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m5 * ns; e += gridDim.x * blockDim.x) {
         const int r = e % m5, c = e / m5;
-        W[e] = zmk((double)d[(size_t)r * Dn + c], (double)d[(size_t)r * Dn + ns + c]);
+        W[e] = zmk(f2d(d[(size_t)r * Dn + c]), f2d(d[(size_t)r * Dn + ns + c]));
     }
 }
 
+// the blocks that no step changes, once at set-up
+void launch_tc_mt_static(const TcMT* t, const StepArgs& a, cudaStream_t s) {
+    const int mtl = (t->maxm + 31) / 32;
+    k_tc_mt_pack_a<<<dim3(mtl, mtl, t->nat), 256, 0, s>>>(a, t->Mp, t->Kp, 1, 5, t->ah, t->al);
+}
 int launch_tc_mt(const TcMT* t, const StepArgs& a, cudaStream_t s) {
     const int nat = t->nat;
-    k_tc_mt_pack_a<<<dim3(64, nat), 256, 0, s>>>(a, t->Mp, t->Kp, t->ah, t->al);
+    const int mtl = (t->maxm + 31) / 32;
+    k_tc_mt_pack_a<<<dim3(mtl, mtl, nat), 256, 0, s>>>(a, t->Mp, t->Kp, 0, 1, t->ah, t->al);
     k_tc_mt_pack_b<<<dim3((t->maxm * t->ns + 255) / 256, nat, a.nk), 256, 0, s>>>(a, t->NT, t->Kp, t->bh, t->bl);
     TcOpParams p{};
     p.nk = a.nk * nat;

@@ -164,6 +164,8 @@ struct StepArgs {
     zd* mtv;                  //   per (k, atom) the gathered [Q; C_lo] (m x N_s, stride mtv_stride)
     int mtw_stride, mtv_stride;
     zd* mtd;                  //   FP64 form: its product with dh (m x N_s, stride mtd_stride)
+    const struct DgGemm* dg_j; // many states: PP theta as digit products into jw ([k][3 naux][ns]), or null
+    zd* jw;
     int mtd_stride, mt64;     //   mt64: mtw holds [h; o; p] [Q; C_lo], h_eff is combined by k_mt_epi
 };
 #define ZT_MIN_N 16           // columns from which the FP32 contractions take the 64 x 64 tiled kernel
@@ -332,6 +334,7 @@ int launch_tcc_project(const TcCC* t, const StepArgs& a, zd* part, cudaStream_t 
 struct TcMT;
 int tc_mt_create(TcMT** out, int nk, int nat, int maxm, int ns, int* flag, cudaStream_t s, std::string* why);
 void tc_mt_destroy(TcMT* t);
+void launch_tc_mt_static(const TcMT* t, const StepArgs& a, cudaStream_t s);
 int launch_tc_mt(const TcMT* t, const StepArgs& a, cudaStream_t s);
 // ---- tensor-core split-BF16 complex GEMM (k_tc.cu); returns an RTTDDFT_* code
 int tc_zgemm(int opA, int M, int N, int K, const zd* A, int lda, const zd* X, int ldx, zd* C, int ldc,
