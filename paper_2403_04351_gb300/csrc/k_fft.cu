@@ -71,6 +71,14 @@ struct FftArgs {
     const void* v;          // potential on the grid (complex, FP64 or FP32)
     const void* vd;
     const double* s;        // scale of vd (device)
+    // fixed-point form: the potential's image and its exponents per (r2, chunk
+    // of axis 1's blocks); exponents of the stored values per (line, chunk),
+    // (plane, chunk) and (r2, chunk) of each column
+    const struct zq* vq;
+    const int* vqe;
+    int2 *ma, *mb, *mc;
+    int lines_max, planes_max;
+    int qb[3];              // bits that an axis' transform may start with
 };
 
 struct FftPlan {
@@ -92,6 +100,13 @@ struct FftPlan {
     FftK* d_fk = nullptr;
     void* b3 = nullptr;
     void* b2 = nullptr;
+    // fixed-point form (FP64 plans, axes of at most FX_MAX_N points): twiddles,
+    // images of v and of a call's v + s vd with their exponents, exponents of b3 and b2
+    int fx = 0;
+    struct zq* wq[3] = {nullptr, nullptr, nullptr};
+    struct zq* vq[2] = {nullptr, nullptr};
+    int* vqe[2] = {nullptr, nullptr};
+    int2 *ma = nullptr, *mb = nullptr, *mc = nullptr;
     std::vector<void*> tables;  // per-k index arrays
     // Hartree feedback: density grid (forward transformed), its value at the
     // start, the box extents, the reciprocal vectors, the l1 accumulator
@@ -131,6 +146,47 @@ template <typename C> __device__ __forceinline__ C cwt(const C* W, int i, bool i
     if (inv) w.y = -w.y;
     return w;
 }
+// a +- i b by the direction's sign; a + w b, i w z, i (w1 d1 + w2 d2) for real w
+template <typename C> __device__ __forceinline__ C cisg(C z, bool inv) {
+    return inv ? cmk<C>(-z.y, z.x) : cmk<C>(z.y, -z.x);
+}
+template <typename C> __device__ __forceinline__ C cma(C a, typename Rt<C>::R w, C b) {
+    return cmk<C>(a.x + w * b.x, a.y + w * b.y);
+}
+template <typename C> __device__ __forceinline__ C ci2(typename Rt<C>::R w1, C d1, typename Rt<C>::R w2, C d2) {
+    return cmk<C>(-(w1 * d1.y + w2 * d2.y), w1 * d1.x + w2 * d2.x);
+}
+
+// Fixed point: 64-bit integers of at most 2^61 with a power-of-two scale per
+// block, twiddles with 62 binary places.  A product keeps the three largest of
+// its four 32-bit partial products; the low words are signed (balanced), so what
+// is dropped averages to zero and stays below one unit.
+struct __align__(16) zq {
+    long long x, y;
+};
+template <> struct Rt<zq> { typedef long long R; };
+__device__ __forceinline__ int qhi(long long a) { return (int)((a + 0x80000000LL) >> 32); }
+__device__ __forceinline__ long long qml(long long a, long long w) {
+    const int ah = qhi(a), al = (int)a, wh = qhi(w), wl = (int)w;
+    return (((long long)ah * wh) << 2) + (((long long)ah * wl + (long long)al * wh + (1LL << 29)) >> 30);
+}
+__device__ __forceinline__ zq cml(zq a, zq w) {
+    const int ah = qhi(a.x), al = (int)a.x, bh = qhi(a.y), bl = (int)a.y;
+    const int ch = qhi(w.x), cl = (int)w.x, dh = qhi(w.y), dl = (int)w.y;
+    const long long h0 = (long long)ah * ch - (long long)bh * dh;
+    const long long m0 = (long long)ah * cl + (long long)al * ch - (long long)bh * dl - (long long)bl * dh;
+    const long long h1 = (long long)ah * dh + (long long)bh * ch;
+    const long long m1 = (long long)ah * dl + (long long)al * dh + (long long)bh * cl + (long long)bl * ch;
+    zq r;
+    r.x = (h0 << 2) + ((m0 + (1LL << 29)) >> 30);
+    r.y = (h1 << 2) + ((m1 + (1LL << 29)) >> 30);
+    return r;
+}
+__device__ __forceinline__ zq cis(zq z, long long w) { return cmk<zq>(-qml(z.y, w), qml(z.x, w)); }
+__device__ __forceinline__ zq cma(zq a, long long w, zq b) { return cmk<zq>(a.x + qml(b.x, w), a.y + qml(b.y, w)); }
+__device__ __forceinline__ zq ci2(long long w1, zq d1, long long w2, zq d2) {
+    return cmk<zq>(-(qml(d1.y, w1) + qml(d2.y, w2)), qml(d1.x, w1) + qml(d2.x, w2));
+}
 __device__ __forceinline__ zd cvt(zd a, zd) { return a; }
 __device__ __forceinline__ zf cvt(zd a, zf) { return tof(a); }
 __device__ __forceinline__ zd todz(zd a) { return a; }
@@ -156,8 +212,6 @@ __device__ __forceinline__ int fft_div(int n, unsigned mg) { return mg ? (int)__
 template <bool LF, bool LAST, typename C>
 __device__ __forceinline__ void fft_stage(const C* x, C* y, int R, int m, int s0, unsigned mgl, unsigned mgs, int nl, int L,
                                           int ls, int es, const C* W, bool inv) {
-    typedef typename Rt<C>::R R_;
-    const R_ sg = inv ? R_(1) : R_(-1);  // sign of i in w_4 = e^{-+ i pi/2}
     const int nb = m * s0;               // butterflies per line
     const int tot = nl * nb;
     for (int b = threadIdx.x; b < tot; b += blockDim.x) {
@@ -182,7 +236,7 @@ __device__ __forceinline__ void fft_stage(const C* x, C* y, int R, int m, int s0
             const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms], a3 = xi[3 * ms];
             const C s02 = cad(a0, a2), d02 = csb(a0, a2), s13 = cad(a1, a3), d13 = csb(a1, a3);
             // w_4 = -i (forward): b1 = d02 - i d13, b3 = d02 + i d13
-            const C id13 = cis(d13, sg);
+            const C id13 = cisg(d13, inv);
             yo[0] = cad(s02, s13);
             yo[os] = tw(cad(d02, id13), 1);
             yo[2 * os] = tw(csb(s02, s13), 2);
@@ -191,7 +245,7 @@ __device__ __forceinline__ void fft_stage(const C* x, C* y, int R, int m, int s0
             const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms];
             const C w = cwt(W, L / 3, inv);  // w_3
             const C sm = cad(a1, a2), df = csb(a1, a2);
-            const C t = cmk<C>(a0.x + w.x * sm.x, a0.y + w.x * sm.y);
+            const C t = cma(a0, w.x, sm);
             const C u = cis(df, w.y);  // i Im(w_3) (a1 - a2)
             yo[0] = cad(a0, sm);
             yo[os] = tw(cad(t, u), 1);
@@ -200,11 +254,11 @@ __device__ __forceinline__ void fft_stage(const C* x, C* y, int R, int m, int s0
             const C a0 = xi[0], a1 = xi[ms], a2 = xi[2 * ms], a3 = xi[3 * ms], a4 = xi[4 * ms];
             const C w1 = cwt(W, L / 5, inv), w2 = cwt(W, 2 * (L / 5), inv);  // w_5, w_5^2
             const C s1 = cad(a1, a4), d1 = csb(a1, a4), s2 = cad(a2, a3), d2 = csb(a2, a3);
-            const C ta = cmk<C>(a0.x + w1.x * s1.x + w2.x * s2.x, a0.y + w1.x * s1.y + w2.x * s2.y);
-            const C tb = cmk<C>(a0.x + w2.x * s1.x + w1.x * s2.x, a0.y + w2.x * s1.y + w1.x * s2.y);
+            const C ta = cma(cma(a0, w1.x, s1), w2.x, s2);
+            const C tb = cma(cma(a0, w2.x, s1), w1.x, s2);
             // i (Im w1 d1 + Im w2 d2) and i (Im w2 d1 - Im w1 d2)
-            const C ua = cmk<C>(-(w1.y * d1.y + w2.y * d2.y), w1.y * d1.x + w2.y * d2.x);
-            const C ub = cmk<C>(-(w2.y * d1.y - w1.y * d2.y), w2.y * d1.x - w1.y * d2.x);
+            const C ua = ci2(w1.y, d1, w2.y, d2);
+            const C ub = ci2(w2.y, d1, -w1.y, d2);
             yo[0] = cad(a0, cad(s1, s2));
             yo[os] = tw(cad(ta, ua), 1);
             yo[2 * os] = tw(cad(tb, ub), 2);
@@ -471,6 +525,433 @@ __global__ void __launch_bounds__(FFT_PTHREADS) k_fft_plane(FftArgs f, int fwd) 
     }
 }
 
+// ---------------------------------------------------------------- fixed point
+// The FP64 form's convolution on the integer pipe.  FP64 instructions (2 lanes
+// per clock and SM) bound its transforms: a radix-4 butterfly has 28 of them,
+// 14 clocks a lane; in 64-bit integers its 16 additions are 2 instructions each
+// at 64 or more lanes per clock and a twiddle 12 wide products at about 16.
+// Values are q 2^e with one exponent per block of a pass: a block takes the
+// largest magnitude of the blocks that it reads, aligned so that its transform
+// of L points cannot pass 2^61 (the terms of any partial sum are at most
+// sqrt(2) L times the largest part), and stores the bit length of its results.
+// So 53 bits or more lie below the largest value of a block at each pass (the
+// reason for FX_MAX_N), and what a pass rounds is below what FP64 rounds in it.
+// A block that reads an infinity or a NaN makes the column NaN, as the sums did.
+// 200 columns on 48^3 points 3273 -> 1367 us, 60 columns of the interface 1414 ->
+// 613 us, 7 columns of 25527 plane waves 524 -> 245 us (FP64 transforms before).
+// Exponent entries: x = e, y = top, the values are below 2^top.
+#define FX_MAX_N 181              // 60.5 - log2(181) = 53 bits
+#define FX_ZERO (-(1 << 28))      // top of a block of zeros (its values are not stored)
+#define FX_NAN (1 << 28)          // top of a block that met a non-finite value (nor are these)
+
+// bits that the values of a transform of L points may start with: floor(60.5 - log2 L)
+static int fx_bits(int L) {
+    int b = 60;
+    while ((double)L * (double)(1LL << b) > 1630477228166597777.0) --b;
+    return b;
+}
+__device__ __forceinline__ long long fx_sh1(long long v, int s) {
+    if (s >= 0) return v << s;
+    const int n = -s;
+    return n > 62 ? 0 : (v + (1LL << (n - 1))) >> n;
+}
+__device__ __forceinline__ zq fx_sh(zq v, int s) { return cmk<zq>(fx_sh1(v.x, s), fx_sh1(v.y, s)); }
+__device__ __forceinline__ unsigned long long fx_mag(zq v) {
+    return (unsigned long long)((v.x ^ (v.x >> 63)) | (v.y ^ (v.y >> 63)));
+}
+// largest m of the block (two barriers)
+__device__ __forceinline__ int fx_bmax(int m, int* red) {
+    m = __reduce_max_sync(0xffffffffu, m);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, red[w]);
+    return m;
+}
+// bit length of the block's largest magnitude (0: all zero)
+__device__ __forceinline__ int fx_bbits(unsigned long long o, int* red) {
+    const unsigned h = __reduce_or_sync(0xffffffffu, (unsigned)(o >> 32));
+    const unsigned l = __reduce_or_sync(0xffffffffu, (unsigned)o);
+    return fx_bmax(h ? 64 - __clz(h) : 32 - __clz(l), red);
+}
+// exponent field of the larger part (subnormals as 1, zero 0, non-finite 2047)
+__device__ __forceinline__ int fx_ex1(double v) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+    return u == 0 ? 0 : max((int)(u >> 52), 1);
+}
+__device__ __forceinline__ int fx_ex(zd v) { return max(fx_ex1(v.x), fx_ex1(v.y)); }
+// v 2^-e for a finite v, rounded to an integer (below 2^62)
+__device__ __forceinline__ long long fx_from1(double v, int e) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    const int ex = (int)(u >> 52) & 2047;
+    const long long m = (long long)(u & 0xfffffffffffffULL) | (ex ? 1LL << 52 : 0LL);
+    const long long q = fx_sh1(m, max(ex, 1) - 1075 - e);
+    return v < 0.0 ? -q : q;
+}
+__device__ __forceinline__ zq fx_from(zd v, int e) { return cmk<zq>(fx_from1(v.x, e), fx_from1(v.y, e)); }
+// the exponent entry of results below 2^bits with exponent e
+__device__ __forceinline__ int2 fx_entry(int e, int bits) { return make_int2(e, bits ? e + bits : FX_ZERO); }
+// the value of an entry's block aligned to exponent e
+__device__ __forceinline__ zq fx_get(const zq* p, int2 m, int e) {
+    return m.y == FX_ZERO ? cmk<zq>(0, 0) : fx_sh(*p, m.x - e);
+}
+
+// The potential of a call, v + s vd, v or s vd, in fixed point: values below
+// 2^61 of 2^62, an exponent per block of pass C (its (r2, chunk))
+__global__ void __launch_bounds__(FFT_THREADS) k_fx_v(FftArgs f, zq* __restrict__ vq, int* __restrict__ vqe) {
+    __shared__ int red[8];
+    const int F1 = f.F1, F3 = f.F3, LPB = f.lpb[0];
+    const int nch = (F3 + LPB - 1) / LPB;
+    const int r2 = blockIdx.x / nch, i30 = (blockIdx.x - r2 * nch) * LPB;
+    const int nl = min(LPB, F3 - i30);
+    const unsigned mnl = fft_magic(nl);
+    const size_t pst = (size_t)f.F2 * F3, off = (size_t)r2 * F3 + i30;
+    const zd* v = (const zd*)f.v;
+    const zd* vd = (const zd*)f.vd;
+    const double sc = f.vmode != 0 || f.use_vd ? *f.s : 0.0;
+    zd pv[FFT_PV];  // F1 nl <= FFT_BLK_PTS
+    int m = 0;
+#pragma unroll
+    for (int u = 0; u < FFT_PV; ++u) {
+        const int i = threadIdx.x + u * FFT_THREADS;
+        pv[u] = zmk(0.0, 0.0);
+        if (i < F1 * nl) {
+            const int r1 = fft_div(i, mnl), l = i - r1 * nl;
+            const size_t gi = (size_t)r1 * pst + off + l;
+            if (f.vmode == 0) pv[u] = v[gi];
+            if (f.vmode != 0 || f.use_vd) {
+                const zd d = vd[gi];
+                pv[u] = f.vmode == 0 ? zmk(pv[u].x + sc * d.x, pv[u].y + sc * d.y) : zmk(sc * d.x, sc * d.y);
+            }
+        }
+        m = max(m, fx_ex(pv[u]));
+    }
+    m = fx_bmax(m, red);
+    // below 2^(m - 1022): e = that - 61 leaves |v| < 2^61
+    const int e = m - 1022 - 61;
+    if (threadIdx.x == 0) vqe[blockIdx.x] = m == 0 ? FX_ZERO : m == 2047 ? FX_NAN : e + 62;
+    if (m == 0 || m == 2047) return;
+#pragma unroll
+    for (int u = 0; u < FFT_PV; ++u) {
+        const int i = threadIdx.x + u * FFT_THREADS;
+        if (i < F1 * nl) {
+            const int r1 = fft_div(i, mnl), l = i - r1 * nl;
+            vq[(size_t)r1 * pst + off + l] = fx_from(pv[u], e);
+        }
+    }
+}
+
+// Passes A to E as above
+__global__ void __launch_bounds__(FFT_THREADS) k_fx_a(FftArgs f) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    __shared__ int red[8];
+    const int F3 = f.F3, LPB = f.lpb[2];
+    zq* W = (zq*)fsm;
+    zq* x = W + F3;
+    zq* y = x + LPB * F3;
+    const int k = blockIdx.z, c = blockIdx.y;
+    const FftK K = f.fk[k];
+    const int l0 = blockIdx.x * LPB;
+    if (l0 >= K.nline) return;
+    const int nl = min(LPB, K.nline - l0);
+    load_tw(W, f.w[2], F3);
+    for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) x[i] = cmk<zq>(0, 0);
+    const ToepDesc td = f.td[k];
+    const zd* X = td.X + (size_t)c * td.ldx;
+    const int j0 = K.lg0[l0], j1 = K.lg0[l0 + nl];
+    const int base = l0 * F3;
+    int m = 0;
+    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) m = max(m, fx_ex(X[K.gperm[j]]));
+    m = fx_bmax(m, red);
+    const size_t kc = (size_t)k * f.ncol + c;
+    const int ch1 = (F3 + f.lpb[1] - 1) / f.lpb[1];
+    int2 mt = make_int2(0, m == 0 ? FX_ZERO : FX_NAN);
+    if (m != 0 && m != 2047) {
+        const int e = m - 1022 - f.qb[2];
+        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) x[K.lpos[j] - base] = fx_from(X[K.gperm[j]], e);
+        __syncthreads();
+        const zq* r = fft_lines(x, y, nl, F3, f, 2, W, true);
+        zq* out = (zq*)f.b3 + kc * f.b3_col + (size_t)base;
+        unsigned long long o = 0;
+        for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) {
+            out[i] = r[i];
+            o |= fx_mag(r[i]);
+        }
+        mt = fx_entry(e, fx_bbits(o, red));
+    }
+    int2* ma = f.ma + (kc * f.lines_max + l0) * ch1;
+    for (int i = threadIdx.x; i < nl * ch1; i += blockDim.x) ma[i] = mt;
+}
+
+__global__ void __launch_bounds__(FFT_THREADS) k_fx_bd(FftArgs f, int fwd) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    __shared__ int red[8];
+    const int F2 = f.F2, F3 = f.F3, LPB = f.lpb[1];
+    zq* W = (zq*)fsm;
+    zq* x = W + F2;
+    zq* y = x + LPB * F2;
+    const int k = blockIdx.z, c = blockIdx.y;
+    const FftK K = f.fk[k];
+    const int ch1 = (F3 + LPB - 1) / LPB, ch0 = (F3 + f.lpb[0] - 1) / f.lpb[0];
+    const int p = blockIdx.x / ch1, ch = blockIdx.x - p * ch1, i30 = ch * LPB;
+    if (p >= K.nplane) return;
+    const int nl = min(LPB, F3 - i30);
+    load_tw(W, f.w[1], F2);
+    const size_t kc = (size_t)k * f.ncol + c;
+    zq* b3 = (zq*)f.b3 + kc * f.b3_col;
+    zq* b2 = (zq*)f.b2 + kc * f.b2_col + (size_t)p * F2 * F3;
+    int2* ma = f.ma + kc * f.lines_max * ch1;
+    int2* mb = f.mb + (kc * f.planes_max + p) * ch1;
+    const int2* mc = f.mc + kc * F2 * ch0;
+    const int* lo = K.line_of + (size_t)p * F2;
+    const unsigned mnl = fft_magic(nl), m0 = fft_magic(f.lpb[0]);
+    int t = FX_ZERO;
+    if (fwd) {
+        const int c0 = fft_div(i30, m0), nc = fft_div(i30 + nl - 1, m0) - c0 + 1;
+        for (int i = threadIdx.x; i < F2 * nc; i += blockDim.x) t = max(t, mc[(i / nc) * ch0 + c0 + i % nc].y);
+    } else {
+        for (int r2 = threadIdx.x; r2 < F2; r2 += blockDim.x)
+            if (lo[r2] >= 0) t = max(t, ma[lo[r2] * ch1 + ch].y);
+    }
+    t = fx_bmax(t, red);
+    int2 mt = make_int2(0, t);
+    if (t != FX_ZERO && t != FX_NAN) {
+        const int e = t - f.qb[1];
+        for (int i = threadIdx.x; i < F2 * nl; i += blockDim.x) {
+            const int r2 = fft_div(i, mnl), l = i - r2 * nl;
+            zq v = cmk<zq>(0, 0);
+            if (fwd) {
+                v = fx_get(b2 + (size_t)r2 * F3 + i30 + l, mc[r2 * ch0 + fft_div(i30 + l, m0)], e);
+            } else {
+                const int id = lo[r2];
+                if (id >= 0) v = fx_get(b3 + (size_t)id * F3 + i30 + l, ma[id * ch1 + ch], e);
+            }
+            x[i] = v;
+        }
+        __syncthreads();
+        const zq* r = fft_cols(x, y, nl, F2, f, 1, W, !fwd);
+        unsigned long long o = 0;
+        for (int i = threadIdx.x; i < F2 * nl; i += blockDim.x) {
+            const int r2 = fft_div(i, mnl), l = i - r2 * nl;
+            if (fwd) {
+                const int id = lo[r2];
+                if (id >= 0) {
+                    b3[(size_t)id * F3 + i30 + l] = r[i];
+                    o |= fx_mag(r[i]);
+                }
+            } else {
+                b2[(size_t)r2 * F3 + i30 + l] = r[i];
+                o |= fx_mag(r[i]);
+            }
+        }
+        mt = fx_entry(e, fx_bbits(o, red));
+    }
+    if (fwd) {
+        for (int l = K.pl0[p] + threadIdx.x; l < K.pl0[p + 1]; l += blockDim.x) ma[l * ch1 + ch] = mt;
+    } else if (threadIdx.x == 0) {
+        mb[ch] = mt;
+    }
+}
+
+__global__ void __launch_bounds__(FFT_THREADS) k_fx_c(FftArgs f) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    __shared__ int red[8];
+    const int F1 = f.F1, F2 = f.F2, F3 = f.F3, LPB = f.lpb[0];
+    zq* W = (zq*)fsm;
+    zq* x = W + F1;
+    zq* y = x + LPB * F1;
+    const int k = blockIdx.z, c = blockIdx.y;
+    const FftK K = f.fk[k];
+    const int ch0 = (F3 + LPB - 1) / LPB, ch1 = (F3 + f.lpb[1] - 1) / f.lpb[1];
+    const int r2 = blockIdx.x / ch0, i30 = (blockIdx.x - r2 * ch0) * LPB;
+    const int nl = min(LPB, F3 - i30);
+    load_tw(W, f.w[0], F1);
+    const size_t kc = (size_t)k * f.ncol + c;
+    zq* b2 = (zq*)f.b2 + kc * f.b2_col;
+    const int2* mb = f.mb + kc * f.planes_max * ch1;
+    const size_t pst = (size_t)F2 * F3, off = (size_t)r2 * F3 + i30;
+    const unsigned mnl = fft_magic(nl), m1 = fft_magic(f.lpb[1]);
+    int t = FX_ZERO;
+    {
+        const int c1 = fft_div(i30, m1), nc = fft_div(i30 + nl - 1, m1) - c1 + 1;
+        for (int i = threadIdx.x; i < K.nplane * nc; i += blockDim.x) t = max(t, mb[(i / nc) * ch1 + c1 + i % nc].y);
+    }
+    const int ve = f.vqe[blockIdx.x];
+    t = fx_bmax(t, red);
+    int2 mt = make_int2(0, t == FX_NAN || ve == FX_NAN ? FX_NAN : FX_ZERO);
+    if (t != FX_ZERO && t != FX_NAN && ve != FX_ZERO && ve != FX_NAN) {
+        const int b = f.qb[0];
+        int e = t - b;
+        for (int i = threadIdx.x; i < F1 * nl; i += blockDim.x) {
+            const int r1 = fft_div(i, mnl), l = i - r1 * nl;
+            const int p = K.plane_of[r1];
+            x[i] = p >= 0 ? fx_get(b2 + (size_t)p * pst + off + l, mb[p * ch1 + fft_div(i30 + l, m1)], e) : cmk<zq>(0, 0);
+        }
+        __syncthreads();
+        zq* r = fft_cols(x, y, nl, F1, f, 0, W, true);
+        // times v (its own exponent), and aligned again
+        unsigned long long o = 0;
+        for (int i = threadIdx.x; i < F1 * nl; i += blockDim.x) {
+            const int r1 = fft_div(i, mnl), l = i - r1 * nl;
+            const zq w = cml(r[i], f.vq[(size_t)r1 * pst + off + l]);
+            r[i] = w;
+            o |= fx_mag(w);
+        }
+        const int bits = fx_bbits(o, red), sh = b - bits;
+        e += ve - sh;
+        for (int i = threadIdx.x; i < F1 * nl; i += blockDim.x) r[i] = fx_sh(r[i], sh);
+        __syncthreads();
+        const zq* q = fft_cols(r, r == x ? y : x, nl, F1, f, 0, W, false);
+        o = 0;
+        for (int i = threadIdx.x; i < F1 * nl; i += blockDim.x) {
+            const int r1 = fft_div(i, mnl), l = i - r1 * nl;
+            const int p = K.plane_of[r1];
+            if (p >= 0) {
+                b2[(size_t)p * pst + off + l] = q[i];
+                o |= fx_mag(q[i]);
+            }
+        }
+        mt = fx_entry(e, fx_bbits(o, red));
+    }
+    if (threadIdx.x == 0) f.mc[kc * F2 * ch0 + blockIdx.x] = mt;
+}
+
+// q 2^e in FP64: one product by a power of two where that is a normal number
+__device__ __forceinline__ zd fx_out(zq v, int e) {
+    if (e > -960 && e < 960) {
+        const double f = __longlong_as_double((long long)(e + 1023) << 52);
+        return zmk((double)v.x * f, (double)v.y * f);
+    }
+    return zmk(scalbn((double)v.x, e), scalbn((double)v.y, e));
+}
+
+__global__ void __launch_bounds__(FFT_THREADS) k_fx_e(FftArgs f) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    __shared__ int red[8];
+    const int F3 = f.F3, LPB = f.lpb[2];
+    zq* W = (zq*)fsm;
+    zq* x = W + F3;
+    zq* y = x + LPB * F3;
+    const int k = blockIdx.z, c = blockIdx.y;
+    const FftK K = f.fk[k];
+    const int l0 = blockIdx.x * LPB;
+    if (l0 >= K.nline) return;
+    const int nl = min(LPB, K.nline - l0);
+    load_tw(W, f.w[2], F3);
+    const int base = l0 * F3;
+    const size_t kc = (size_t)k * f.ncol + c;
+    const int ch1 = (F3 + f.lpb[1] - 1) / f.lpb[1];
+    const unsigned m1 = fft_magic(f.lpb[1]), m3 = fft_magic(F3);
+    const int2* ma = f.ma + (kc * f.lines_max + l0) * ch1;
+    const zq* in = (const zq*)f.b3 + kc * f.b3_col + (size_t)base;
+    int t = FX_ZERO;
+    for (int i = threadIdx.x; i < nl * ch1; i += blockDim.x) t = max(t, ma[i].y);
+    t = fx_bmax(t, red);
+    const ToepDesc td = f.td[k];
+    zd* Y = td.Y + (size_t)c * td.ldy;
+    const int j0 = K.lg0[l0], j1 = K.lg0[l0 + nl];
+    if (t == FX_ZERO || t == FX_NAN) {
+        const double v = t == FX_NAN ? nan("") : 0.0;
+        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) Y[K.gperm[j]] = zmk(v, v);
+        return;
+    }
+    const int e = t - f.qb[2];
+    for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) {
+        const int l = fft_div(i, m3);
+        x[i] = fx_get(in + i, ma[l * ch1 + fft_div(i - l * F3, m1)], e);
+    }
+    __syncthreads();
+    const zq* r = fft_lines(x, y, nl, F3, f, 2, W, false);
+    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) Y[K.gperm[j]] = fx_out(r[K.lpos[j] - base], e);
+}
+
+// A+B (fwd = 0) and D+E (fwd = 1) of one plane, aligned again between the axes
+__global__ void __launch_bounds__(FFT_PTHREADS) k_fx_plane(FftArgs f, int fwd) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    __shared__ int red[8];
+    const int F2 = f.F2, F3 = f.F3, n2 = F2 * F3;
+    zq* W2 = (zq*)fsm;
+    zq* W3 = W2 + F2;
+    zq* A = W3 + F3;
+    zq* B = A + n2;
+    const int k = blockIdx.z, c = blockIdx.y, p = blockIdx.x;
+    const FftK K = f.fk[k];
+    if (p >= K.nplane) return;
+    load_tw(W2, f.w[1], F2);
+    load_tw(W3, f.w[2], F3);
+    const unsigned m3 = fft_magic(F3), m0 = fft_magic(f.lpb[0]);
+    const int l0 = K.pl0[p], nl = K.pl0[p + 1] - l0;
+    const int base = l0 * F3;
+    const size_t kc = (size_t)k * f.ncol + c;
+    const int ch1 = (F3 + f.lpb[1] - 1) / f.lpb[1], ch0 = (F3 + f.lpb[0] - 1) / f.lpb[0];
+    zq* b2 = (zq*)f.b2 + kc * f.b2_col + (size_t)p * n2;
+    const ToepDesc td = f.td[k];
+    const int j0 = K.lg0[l0], j1 = K.lg0[l0 + nl];
+    unsigned long long o = 0;
+    if (!fwd) {
+        const zd* X = td.X + (size_t)c * td.ldx;
+        int m = 0;
+        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) m = max(m, fx_ex(X[K.gperm[j]]));
+        for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) A[i] = cmk<zq>(0, 0);
+        m = fx_bmax(m, red);
+        int2 mt = make_int2(0, m == 0 ? FX_ZERO : FX_NAN);
+        if (m != 0 && m != 2047) {
+            int e = m - 1022 - f.qb[2];
+            for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) A[K.lpos[j] - base] = fx_from(X[K.gperm[j]], e);
+            __syncthreads();
+            zq* r = fft_lines(A, B, nl, F3, f, 2, W3, true);
+            zq* P = (r == A) ? B : A;
+            for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) o |= fx_mag(r[i]);
+            for (int i = threadIdx.x; i < n2; i += blockDim.x) P[i] = cmk<zq>(0, 0);
+            const int sh = f.qb[1] - fx_bbits(o, red);
+            e -= sh;
+            for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) {
+                const int l = fft_div(i, m3), r3 = i - l * F3;
+                P[K.lr2[l0 + l] * F3 + r3] = fx_sh(r[i], sh);
+            }
+            __syncthreads();
+            const zq* q = fft_cols(P, r, F3, F2, f, 1, W2, true);
+            o = 0;
+            for (int i = threadIdx.x; i < n2; i += blockDim.x) {
+                b2[i] = q[i];
+                o |= fx_mag(q[i]);
+            }
+            mt = fx_entry(e, fx_bbits(o, red));
+        }
+        for (int i = threadIdx.x; i < ch1; i += blockDim.x) f.mb[(kc * f.planes_max + p) * ch1 + i] = mt;
+    } else {
+        const int2* mc = f.mc + kc * F2 * ch0;
+        int t = FX_ZERO;
+        for (int i = threadIdx.x; i < F2 * ch0; i += blockDim.x) t = max(t, mc[i].y);
+        t = fx_bmax(t, red);
+        zd* Y = td.Y + (size_t)c * td.ldy;
+        if (t == FX_ZERO || t == FX_NAN) {
+            const double v = t == FX_NAN ? nan("") : 0.0;
+            for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) Y[K.gperm[j]] = zmk(v, v);
+            return;
+        }
+        int e = t - f.qb[1];
+        for (int i = threadIdx.x; i < n2; i += blockDim.x) {
+            const int r2 = fft_div(i, m3);
+            A[i] = fx_get(b2 + i, mc[r2 * ch0 + fft_div(i - r2 * F3, m0)], e);
+        }
+        __syncthreads();
+        zq* q = fft_cols(A, B, F3, F2, f, 1, W2, false);
+        zq* u = (q == A) ? B : A;
+        for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) {
+            const int l = fft_div(i, m3), r3 = i - l * F3;
+            u[i] = q[K.lr2[l0 + l] * F3 + r3];
+            o |= fx_mag(u[i]);
+        }
+        const int sh = f.qb[2] - fx_bbits(o, red);
+        e -= sh;
+        for (int i = threadIdx.x; i < nl * F3; i += blockDim.x) u[i] = fx_sh(u[i], sh);
+        __syncthreads();
+        const zq* r = fft_lines(u, q, nl, F3, f, 2, W3, false);
+        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) Y[K.gperm[j]] = fx_out(r[K.lpos[j] - base], e);
+    }
+}
+
 // Interstitial density of the propagated states on the grid: for every
 // (r2, r3) line of axis 1 the inverse transform of each (k, state) column
 // (planes from the plane pass), |psi|^2 summed with the weights w_k f_j in
@@ -697,6 +1178,8 @@ static int smooth_at_least(int n) {
 static size_t fft_smem(int L, int elt) { return (size_t)(L + 2 * fft_lpb(L) * L) * elt; }
 static size_t fft_plane_smem(int F2, int F3, int elt) { return (size_t)(F2 + F3 + 2 * F2 * F3) * elt; }
 #define FFT_PLANE_SMEM_MAX (200 * 1024)
+// blocks of a line pass over one row of axis 3
+static inline int fft_chunks(int F3, int L) { return (F3 + fft_lpb(L) - 1) / fft_lpb(L); }
 
 template <typename T> static T* fdalloc(size_t n, std::string* why, bool* ok) {
     void* p = nullptr;
@@ -742,12 +1225,24 @@ static bool fft_alloc_buffers(FftPlan* pl, int ncol, std::string* why) {
     const size_t c2 = (size_t)pl->max_planes * pl->F[1] * pl->F[2];
     void* b3 = nullptr;
     void* b2 = nullptr;
+    // exponents of the fixed-point form: per (line, chunk), (plane, chunk), (r2, chunk)
+    const size_t nm = pl->fx ? (size_t)pl->nk * ncol : 0;
+    const size_t ch1 = fft_chunks(pl->F[2], pl->F[1]), ch0 = fft_chunks(pl->F[2], pl->F[0]);
+    const size_t na = nm * pl->max_lines * ch1, nb = nm * pl->max_planes * ch1, nc = nm * pl->F[1] * ch0;
+    int2* mm = nullptr;
     if (cudaMalloc(&b3, std::max<size_t>((size_t)pl->nk * ncol * c3 * elt, 16)) != cudaSuccess ||
-        cudaMalloc(&b2, std::max<size_t>((size_t)pl->nk * ncol * c2 * elt, 16)) != cudaSuccess) {
+        cudaMalloc(&b2, std::max<size_t>((size_t)pl->nk * ncol * c2 * elt, 16)) != cudaSuccess ||
+        (nm && cudaMalloc((void**)&mm, (na + nb + nc) * sizeof(int2)) != cudaSuccess)) {
         if (b3) cudaFree(b3);
+        if (b2) cudaFree(b2);
+        cudaGetLastError();
         if (why) *why = "FFT route: device allocation of the transform buffers failed";
         return false;
     }
+    if (pl->ma) cudaFree(pl->ma);
+    pl->ma = mm;
+    pl->mb = mm + na;
+    pl->mc = mm + na + nb;
     if (pl->b3) cudaFree(pl->b3);
     if (pl->b2) cudaFree(pl->b2);
     pl->b3 = b3;
@@ -848,6 +1343,23 @@ int fft_plan_create(FftPlan** out, int nk, const int* ng, const int* const* gint
         if (ok) cudaMemcpy(pl->d_fk, hk.data(), nk * sizeof(FftK), cudaMemcpyHostToDevice);
     }
     const size_t n3 = (size_t)F1 * F2 * F3;
+    pl->fx = prec == 0 && std::max(F1, std::max(F2, F3)) <= FX_MAX_N;
+    const int nvb = F2 * fft_chunks(F3, F1);
+    for (int a = 0; a < 3 && pl->fx; ++a) {
+        const int L = pl->F[a];
+        std::vector<zq> w(L);
+        for (int m = 0; m < L; ++m) {
+            const long double th = 2.0L * 3.14159265358979323846264338327950288L * m / L;
+            w[m].x = llroundl(cosl(th) * 4611686018427387904.0L);
+            w[m].y = -llroundl(sinl(th) * 4611686018427387904.0L);
+        }
+        pl->wq[a] = fdalloc<zq>(L, why, &ok);
+        if (ok) cudaMemcpy(pl->wq[a], w.data(), L * sizeof(zq), cudaMemcpyHostToDevice);
+    }
+    for (int i = 0; i < 2 && pl->fx; ++i) {
+        pl->vq[i] = fdalloc<zq>(n3, why, &ok);
+        pl->vqe[i] = fdalloc<int>(nvb, why, &ok);
+    }
     if (ok) pl->v64 = fdalloc<zd>(n3, why, &ok);
     if (ok && prec != 0) pl->v32 = fdalloc<zf>(n3, why, &ok);
     if (ok) ok = fft_alloc_buffers(pl, ncol, why);
@@ -861,8 +1373,20 @@ int fft_plan_create(FftPlan** out, int nk, const int* ng, const int* const* gint
         const int mx = (int)fft_smem(std::max(F1, std::max(F2, F3)), elt);
         const size_t psm = fft_plane_smem(F2, F3, elt);
         if (psm <= FFT_PLANE_SMEM_MAX) {
+            if (pl->fx) cudaFuncSetAttribute(k_fx_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
             if (prec == 0) cudaFuncSetAttribute(k_fft_plane<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
             else cudaFuncSetAttribute(k_fft_plane<zf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
+        }
+        if (pl->fx) {
+            cudaFuncSetAttribute(k_fx_a, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+            cudaFuncSetAttribute(k_fx_bd, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+            cudaFuncSetAttribute(k_fx_c, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+            cudaFuncSetAttribute(k_fx_e, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+            FftArgs f = {};
+            f.F1 = F1, f.F2 = F2, f.F3 = F3;
+            f.lpb[0] = fft_lpb(F1);
+            f.v = pl->v64;
+            k_fx_v<<<nvb, FFT_THREADS, 0, st>>>(f, pl->vq[0], pl->vqe[0]);
         }
         if (prec == 0) {
             cudaFuncSetAttribute(k_fft_a<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
@@ -918,7 +1442,13 @@ void fft_plan_destroy(FftPlan* pl) {
     for (int a = 0; a < 3; ++a) {
         if (pl->w64[a]) cudaFree(pl->w64[a]);
         if (pl->w32[a]) cudaFree(pl->w32[a]);
+        if (pl->wq[a]) cudaFree(pl->wq[a]);
     }
+    for (int i = 0; i < 2; ++i) {
+        if (pl->vq[i]) cudaFree(pl->vq[i]);
+        if (pl->vqe[i]) cudaFree(pl->vqe[i]);
+    }
+    if (pl->ma) cudaFree(pl->ma);
     for (void* p : {(void*)pl->v64, (void*)pl->v32, (void*)pl->vd64, (void*)pl->vd32, (void*)pl->d_fk, pl->b3, pl->b2,
                     (void*)pl->rho, (void*)pl->rho0, (void*)pl->l1, (void*)pl->b3d, (void*)pl->b2d})
         if (p) cudaFree(p);
@@ -947,7 +1477,7 @@ static void fft_stages(FftArgs& f, const FftPlan* pl, int a) {
 // use_vd), vmode 1 by s vd alone.  Five launches.
 static int launch_fft_any(const FftPlan* pl, int fused, const ToepDesc* td, int kofs, int nk, int ncol, int vmode,
                           int use_vd, const double* s, cudaStream_t st) {
-    FftArgs f;
+    FftArgs f = {};
     f.F1 = pl->F[0];
     f.F2 = pl->F[1];
     f.F3 = pl->F[2];
@@ -955,7 +1485,7 @@ static int launch_fft_any(const FftPlan* pl, int fused, const ToepDesc* td, int 
         f.nst[a] = pl->nst[a];
         fft_stages(f, pl, a);
         f.lpb[a] = fft_lpb(pl->F[a]);
-        f.w[a] = pl->prec == 0 ? (const void*)pl->w64[a] : (const void*)pl->w32[a];
+        f.w[a] = pl->fx ? (const void*)pl->wq[a] : pl->prec == 0 ? (const void*)pl->w64[a] : (const void*)pl->w32[a];
     }
     f.fk = pl->d_fk + kofs;
     f.td = td + kofs;
@@ -973,6 +1503,32 @@ static int launch_fft_any(const FftPlan* pl, int fused, const ToepDesc* td, int 
     const dim3 ga((pl->max_lines + f.lpb[2] - 1) / f.lpb[2], ncol, nk);
     const dim3 gb(pl->max_planes * ch1, ncol, nk);
     const dim3 gc(f.F2 * ch0, ncol, nk);
+    if (pl->fx) {
+        const int own = vmode != 0 || use_vd;
+        if (own) k_fx_v<<<f.F2 * ch0, FFT_THREADS, 0, st>>>(f, pl->vq[1], pl->vqe[1]);
+        f.vq = pl->vq[own];
+        f.vqe = pl->vqe[own];
+        f.ma = pl->ma;
+        f.mb = pl->mb;
+        f.mc = pl->mc;
+        f.lines_max = pl->max_lines;
+        f.planes_max = pl->max_planes;
+        for (int a = 0; a < 3; ++a) f.qb[a] = fx_bits(pl->F[a]);
+        if (fused) {
+            const dim3 gp(pl->max_planes, ncol, nk);
+            const size_t psm = fft_plane_smem(f.F2, f.F3, sizeof(zq));
+            k_fx_plane<<<gp, FFT_PTHREADS, psm, st>>>(f, 0);
+            k_fx_c<<<gc, FFT_THREADS, fft_smem(f.F1, sizeof(zq)), st>>>(f);
+            k_fx_plane<<<gp, FFT_PTHREADS, psm, st>>>(f, 1);
+            return 3 + own;
+        }
+        k_fx_a<<<ga, FFT_THREADS, fft_smem(f.F3, sizeof(zq)), st>>>(f);
+        k_fx_bd<<<gb, FFT_THREADS, fft_smem(f.F2, sizeof(zq)), st>>>(f, 0);
+        k_fx_c<<<gc, FFT_THREADS, fft_smem(f.F1, sizeof(zq)), st>>>(f);
+        k_fx_bd<<<gb, FFT_THREADS, fft_smem(f.F2, sizeof(zq)), st>>>(f, 1);
+        k_fx_e<<<ga, FFT_THREADS, fft_smem(f.F3, sizeof(zq)), st>>>(f);
+        return 5 + own;
+    }
     if (fused) {
         const dim3 gp(pl->max_planes, ncol, nk);
         if (pl->prec == 0) {
