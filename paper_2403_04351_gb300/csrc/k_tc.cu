@@ -319,13 +319,16 @@ int tc_zgemm(int opA, int M, int N, int K, const zd* A, int lda, const zd* X, in
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     // K slices: one block runs per SM, so the blocks come in waves of nsm; a block costs its K
-    // blocks and about ten more for its start, its read-out and its share of D.  A slice's FP32
-    // sum is kept to 32 K blocks (2048 reals) where more slices than that cost nothing.
+    // blocks and about ten more for its start, its read-out and its share of D.  At least the
+    // slices of two blocks per SM: an FP32 sum over fewer, longer ones is further off
+    // (9917 x 300 by 61: 5.3e-6 in two slices, 4.4e-6 in four); beyond that a slice is kept to 32
+    // K blocks (2048 reals) where more slices cost nothing.
     int splits = 1;
     {
         double best = 1e30;
         const int smax = std::max(1, std::min(total / 4, (4 * nsm + mt * ntile - 1) / (mt * ntile)));
-        for (int sp = 1; sp <= smax; ++sp) {
+        const int smin = std::max(1, std::min(total / 4, (2 * nsm + mt * ntile - 1) / (mt * ntile)));
+        for (int sp = smin; sp <= std::max(smin, smax); ++sp) {
             const int kbs = (total + sp - 1) / sp;
             const double t = (double)((mt * ntile * sp + nsm - 1) / nsm) * (kbs + 10.0) * (kbs > 32 && sp < smax ? 4.0 : 1.0);
             if (t < best) {
