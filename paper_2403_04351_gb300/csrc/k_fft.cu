@@ -74,7 +74,7 @@ struct FftArgs {
     // fixed-point form: the potential's image and its exponents per (r2, chunk
     // of axis 1's blocks); exponents of the stored values per (line, chunk),
     // (plane, chunk) and (r2, chunk) of each column
-    const struct zq* vq;
+    const struct tq* vq;
     const int* vqe;
     int2 *ma, *mb, *mc;
     int lines_max, planes_max;
@@ -104,8 +104,8 @@ struct FftPlan {
     // fixed-point form (FP64 plans, axes of at most FX_MAX_N points): twiddles,
     // images of v and of a call's v + s vd with their exponents, exponents of b3 and b2
     int fx = 0;
-    struct zq* wq[3] = {nullptr, nullptr, nullptr};
-    struct zq* vq[2] = {nullptr, nullptr};
+    struct tq* wq[3] = {nullptr, nullptr, nullptr};
+    struct tq* vq[2] = {nullptr, nullptr};
     int* vqe[2] = {nullptr, nullptr};
     int2 *ma = nullptr, *mb = nullptr, *mc = nullptr;
     std::vector<void*> tables;  // per-k index arrays
@@ -154,40 +154,76 @@ template <typename C> __device__ __forceinline__ C cisg(C z, bool inv) {
 template <typename C> __device__ __forceinline__ C cma(C a, typename Rt<C>::R w, C b) {
     return cmk<C>(a.x + w * b.x, a.y + w * b.y);
 }
+template <typename C> __device__ __forceinline__ C cma2(C a, typename Rt<C>::R w, C b, typename Rt<C>::R v, C d) {
+    return cma(cma(a, w, b), v, d);
+}
 template <typename C> __device__ __forceinline__ C ci2(typename Rt<C>::R w1, C d1, typename Rt<C>::R w2, C d2) {
     return cmk<C>(-(w1 * d1.y + w2 * d2.y), w1 * d1.x + w2 * d2.x);
 }
 
-// Fixed point: 64-bit integers of at most 2^61 with a power-of-two scale per
-// block, twiddles with 62 binary places.  A product keeps the three largest of
-// its four 32-bit partial products; the low words are signed (balanced), so what
-// is dropped averages to zero and stays below one unit.
+// Fixed point: 64-bit integers below 2^61 with a power-of-two scale per block,
+// factors (twiddles, potential) with 62 binary places.  A product keeps the three
+// largest of its four 32-bit partial products; the low words are signed
+// (balanced), so what is dropped averages to zero and stays below one unit.
+// Factors are stored split; their low word is never -2^31, so that it can change
+// its sign.
 struct __align__(16) zq {
     long long x, y;
 };
+struct rq {
+    int h, l;
+};
+struct __align__(16) tq {
+    rq x, y;
+};
 template <> struct Rt<zq> { typedef long long R; };
-__device__ __forceinline__ int qhi(long long a) { return (int)((a + 0x80000000LL) >> 32); }
-__device__ __forceinline__ long long qml(long long a, long long w) {
-    const int ah = qhi(a), al = (int)a, wh = qhi(w), wl = (int)w;
-    return (((long long)ah * wh) << 2) + (((long long)ah * wl + (long long)al * wh + (1LL << 29)) >> 30);
-}
-__device__ __forceinline__ zq cml(zq a, zq w) {
-    const int ah = qhi(a.x), al = (int)a.x, bh = qhi(a.y), bl = (int)a.y;
-    const int ch = qhi(w.x), cl = (int)w.x, dh = qhi(w.y), dl = (int)w.y;
-    const long long h0 = (long long)ah * ch - (long long)bh * dh;
-    const long long m0 = (long long)ah * cl + (long long)al * ch - (long long)bh * dl - (long long)bl * dh;
-    const long long h1 = (long long)ah * dh + (long long)bh * ch;
-    const long long m1 = (long long)ah * dl + (long long)al * dh + (long long)bh * cl + (long long)bl * ch;
-    zq r;
-    r.x = (h0 << 2) + ((m0 + (1LL << 29)) >> 30);
-    r.y = (h1 << 2) + ((m1 + (1LL << 29)) >> 30);
+__host__ __device__ __forceinline__ rq qsplit(long long w) {
+    rq r;
+    r.l = (int)w;
+    if (r.l == (int)0x80000000) r.l += 1, w += 1;
+    r.h = (int)((w - r.l) >> 32);
     return r;
 }
-__device__ __forceinline__ zq cis(zq z, long long w) { return cmk<zq>(-qml(z.y, w), qml(z.x, w)); }
-__device__ __forceinline__ zq cma(zq a, long long w, zq b) { return cmk<zq>(a.x + qml(b.x, w), a.y + qml(b.y, w)); }
-__device__ __forceinline__ zq ci2(long long w1, zq d1, long long w2, zq d2) {
-    return cmk<zq>(-(qml(d1.y, w1) + qml(d2.y, w2)), qml(d1.x, w1) + qml(d2.x, w2));
+__device__ __forceinline__ rq qneg(rq w) {
+    w.h = -w.h;
+    w.l = -w.l;
+    return w;
 }
+__device__ __forceinline__ int qhi(long long a) { return (int)((a + 0x80000000LL) >> 32); }
+// a w and a w + b v
+__device__ __forceinline__ long long qml(long long a, rq w) {
+    const int ah = qhi(a), al = (int)a;
+    return (((long long)ah * w.h) << 2) + ((((long long)ah * w.l + (1LL << 29)) + (long long)al * w.h) >> 30);
+}
+__device__ __forceinline__ long long qml2(long long a, rq w, long long b, rq v) {
+    const int ah = qhi(a), al = (int)a, bh = qhi(b), bl = (int)b;
+    const long long h = (long long)ah * w.h + (long long)bh * v.h;
+    const long long m =
+        ((((long long)ah * w.l + (1LL << 29)) + (long long)al * w.h) + (long long)bh * v.l) + (long long)bl * v.h;
+    return (h << 2) + (m >> 30);
+}
+__device__ __forceinline__ zq cml(zq a, tq w) {
+    return cmk<zq>(qml2(a.x, w.x, a.y, qneg(w.y)), qml2(a.x, w.y, a.y, w.x));
+}
+__device__ __forceinline__ zq cis(zq z, rq w) { return cmk<zq>(qml(z.y, qneg(w)), qml(z.x, w)); }
+__device__ __forceinline__ zq cma(zq a, rq w, zq b) { return cmk<zq>(a.x + qml(b.x, w), a.y + qml(b.y, w)); }
+__device__ __forceinline__ zq cma2(zq a, rq w, zq b, rq v, zq d) {
+    return cmk<zq>(a.x + qml2(b.x, w, d.x, v), a.y + qml2(b.y, w, d.y, v));
+}
+__device__ __forceinline__ zq ci2(rq w1, zq d1, rq w2, zq d2) {
+    return cmk<zq>(qml2(d1.y, qneg(w1), d2.y, qneg(w2)), qml2(d1.x, w1, d2.x, w2));
+}
+// the table's entries and their parts
+template <typename C> struct Tw { typedef C T; };
+template <> struct Tw<zq> { typedef tq T; };
+__device__ __forceinline__ tq cwt(const tq* W, int i, bool inv) {
+    tq w = W[i];
+    if (inv) w.y = qneg(w.y);
+    return w;
+}
+__device__ __forceinline__ double rneg(double w) { return -w; }
+__device__ __forceinline__ float rneg(float w) { return -w; }
+__device__ __forceinline__ rq rneg(rq w) { return qneg(w); }
 __device__ __forceinline__ zd cvt(zd a, zd) { return a; }
 __device__ __forceinline__ zf cvt(zd a, zf) { return tof(a); }
 __device__ __forceinline__ zd todz(zd a) { return a; }
@@ -216,7 +252,7 @@ __device__ __forceinline__ int fft_div(int n, unsigned mg) { return mg ? (int)__
 // 676 us at 240 columns in FP32: a block has half the butterflies, fewer than it
 // has threads, and the registers halve the blocks per SM.)
 template <int R, typename C>
-__device__ __forceinline__ void fft_bfly(C* a, const C* W, int L, bool inv) {
+__device__ __forceinline__ void fft_bfly(C* a, const typename Tw<C>::T* W, int L, bool inv) {
     if constexpr (R == 2) {
         const C t = a[0];
         a[0] = cad(t, a[1]);
@@ -230,7 +266,7 @@ __device__ __forceinline__ void fft_bfly(C* a, const C* W, int L, bool inv) {
         a[2] = csb(s02, s13);
         a[3] = csb(d02, id13);
     } else if constexpr (R == 3) {
-        const C w = cwt(W, L / 3, inv);  // w_3
+        const auto w = cwt(W, L / 3, inv);  // w_3
         const C sm = cad(a[1], a[2]), df = csb(a[1], a[2]);
         const C t = cma(a[0], w.x, sm);
         const C u = cis(df, w.y);  // i Im(w_3) (a1 - a2)
@@ -238,13 +274,13 @@ __device__ __forceinline__ void fft_bfly(C* a, const C* W, int L, bool inv) {
         a[1] = cad(t, u);
         a[2] = csb(t, u);
     } else {
-        const C w1 = cwt(W, L / 5, inv), w2 = cwt(W, 2 * (L / 5), inv);  // w_5, w_5^2
+        const auto w1 = cwt(W, L / 5, inv), w2 = cwt(W, 2 * (L / 5), inv);  // w_5, w_5^2
         const C s1 = cad(a[1], a[4]), d1 = csb(a[1], a[4]), s2 = cad(a[2], a[3]), d2 = csb(a[2], a[3]);
-        const C ta = cma(cma(a[0], w1.x, s1), w2.x, s2);
-        const C tb = cma(cma(a[0], w2.x, s1), w1.x, s2);
+        const C ta = cma2(a[0], w1.x, s1, w2.x, s2);
+        const C tb = cma2(a[0], w2.x, s1, w1.x, s2);
         // i (Im w1 d1 + Im w2 d2) and i (Im w2 d1 - Im w1 d2)
         const C ua = ci2(w1.y, d1, w2.y, d2);
-        const C ub = ci2(w2.y, d1, -w1.y, d2);
+        const C ub = ci2(w2.y, d1, rneg(w1.y), d2);
         a[0] = cad(a[0], cad(s1, s2));
         a[1] = cad(ta, ua);
         a[2] = cad(tb, ub);
@@ -255,7 +291,7 @@ __device__ __forceinline__ void fft_bfly(C* a, const C* W, int L, bool inv) {
 
 template <int R, bool LF, bool LAST, typename C>
 __device__ __forceinline__ void fft_stage_r(const C* x, C* y, int m, int s0, unsigned mgl, unsigned mgs, int nl, int L,
-                                            int ls, int es, const C* W, bool inv) {
+                                            int ls, int es, const typename Tw<C>::T* W, bool inv) {
     const int nb = m * s0;  // butterflies per line
     const int tot = nl * nb;
     const int ms = nb * es, os = s0 * es;  // strides between the points of a butterfly: input, output
@@ -283,7 +319,7 @@ __device__ __forceinline__ void fft_stage_r(const C* x, C* y, int m, int s0, uns
 
 template <bool LF, bool LAST, typename C>
 __device__ __forceinline__ void fft_stage(const C* x, C* y, int R, int m, int s0, unsigned mgl, unsigned mgs, int nl, int L,
-                                          int ls, int es, const C* W, bool inv) {
+                                          int ls, int es, const typename Tw<C>::T* W, bool inv) {
     switch (R) {
 #define FFT_R(r) \
     case r: fft_stage_r<r, LF, LAST>(x, y, m, s0, mgl, mgs, nl, L, ls, es, W, inv); break;
@@ -293,7 +329,7 @@ __device__ __forceinline__ void fft_stage(const C* x, C* y, int R, int m, int s0
 }
 template <bool LF, typename C>
 __device__ C* fft_lines_s(C* x, C* y, int nl, int L, int ls, int es, const int* rad, const unsigned* mg, int nst,
-                          const C* W, bool inv) {
+                          const typename Tw<C>::T* W, bool inv) {
     int s0 = 1;
     const unsigned mnl = LF ? fft_magic(nl) : 0u;
     for (int st = 0; st < nst; ++st) {
@@ -312,12 +348,14 @@ __device__ C* fft_lines_s(C* x, C* y, int nl, int L, int ls, int es, const int* 
 }
 
 template <typename C>
-__device__ __forceinline__ C* fft_lines(C* x, C* y, int nl, int L, const FftArgs& f, int ax, const C* W, bool inv) {
+__device__ __forceinline__ C* fft_lines(C* x, C* y, int nl, int L, const FftArgs& f, int ax,
+                                       const typename Tw<C>::T* W, bool inv) {
     return fft_lines_s<false>(x, y, nl, L, L, 1, f.rad[ax], f.mg[ax], f.nst[ax], W, inv);
 }
 // lines side by side: element j of line l at j nl + l
 template <typename C>
-__device__ __forceinline__ C* fft_cols(C* x, C* y, int nl, int L, const FftArgs& f, int ax, const C* W, bool inv) {
+__device__ __forceinline__ C* fft_cols(C* x, C* y, int nl, int L, const FftArgs& f, int ax,
+                                       const typename Tw<C>::T* W, bool inv) {
     return fft_lines_s<true>(x, y, nl, L, 1, nl, f.rad[ax], f.mg[ax], f.nst[ax], W, inv);
 }
 
@@ -622,7 +660,7 @@ __device__ __forceinline__ zq fx_get(const zq* p, int2 m, int e) {
 
 // The potential of a call, v + s vd, v or s vd, in fixed point: values below
 // 2^61 of 2^62, an exponent per block of pass C (its (r2, chunk))
-__global__ void __launch_bounds__(FFT_THREADS) k_fx_v(FftArgs f, zq* __restrict__ vq, int* __restrict__ vqe) {
+__global__ void __launch_bounds__(FFT_THREADS) k_fx_v(FftArgs f, tq* __restrict__ vq, int* __restrict__ vqe) {
     __shared__ int red[8];
     const int F1 = f.F1, F3 = f.F3, LPB = f.lpb[0];
     const int nch = (F3 + LPB - 1) / LPB;
@@ -660,7 +698,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fx_v(FftArgs f, zq* __restrict_
         const int i = threadIdx.x + u * FFT_THREADS;
         if (i < F1 * nl) {
             const int r1 = fft_div(i, mnl), l = i - r1 * nl;
-            vq[(size_t)r1 * pst + off + l] = fx_from(pv[u], e);
+            const zq q = fx_from(pv[u], e);
+            vq[(size_t)r1 * pst + off + l] = tq{qsplit(q.x), qsplit(q.y)};
         }
     }
 }
@@ -670,8 +709,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fx_a(FftArgs f) {
     extern __shared__ __align__(16) unsigned char fsm[];
     __shared__ int red[8];
     const int F3 = f.F3, LPB = f.lpb[2];
-    zq* W = (zq*)fsm;
-    zq* x = W + F3;
+    tq* W = (tq*)fsm;
+    zq* x = (zq*)W + F3;
     zq* y = x + LPB * F3;
     const int k = blockIdx.z, c = blockIdx.y;
     const FftK K = f.fk[k];
@@ -711,8 +750,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fx_bd(FftArgs f, int fwd) {
     extern __shared__ __align__(16) unsigned char fsm[];
     __shared__ int red[8];
     const int F2 = f.F2, F3 = f.F3, LPB = f.lpb[1];
-    zq* W = (zq*)fsm;
-    zq* x = W + F2;
+    tq* W = (tq*)fsm;
+    zq* x = (zq*)W + F2;
     zq* y = x + LPB * F2;
     const int k = blockIdx.z, c = blockIdx.y;
     const FftK K = f.fk[k];
@@ -781,8 +820,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fx_c(FftArgs f) {
     extern __shared__ __align__(16) unsigned char fsm[];
     __shared__ int red[8];
     const int F1 = f.F1, F2 = f.F2, F3 = f.F3, LPB = f.lpb[0];
-    zq* W = (zq*)fsm;
-    zq* x = W + F1;
+    tq* W = (tq*)fsm;
+    zq* x = (zq*)W + F1;
     zq* y = x + LPB * F1;
     const int k = blockIdx.z, c = blockIdx.y;
     const FftK K = f.fk[k];
@@ -853,8 +892,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fx_e(FftArgs f) {
     extern __shared__ __align__(16) unsigned char fsm[];
     __shared__ int red[8];
     const int F3 = f.F3, LPB = f.lpb[2];
-    zq* W = (zq*)fsm;
-    zq* x = W + F3;
+    tq* W = (tq*)fsm;
+    zq* x = (zq*)W + F3;
     zq* y = x + LPB * F3;
     const int k = blockIdx.z, c = blockIdx.y;
     const FftK K = f.fk[k];
@@ -894,9 +933,9 @@ __global__ void __launch_bounds__(FFT_PTHREADS) k_fx_plane(FftArgs f, int fwd) {
     extern __shared__ __align__(16) unsigned char fsm[];
     __shared__ int red[8];
     const int F2 = f.F2, F3 = f.F3, n2 = F2 * F3;
-    zq* W2 = (zq*)fsm;
-    zq* W3 = W2 + F2;
-    zq* A = W3 + F3;
+    tq* W2 = (tq*)fsm;
+    tq* W3 = W2 + F2;
+    zq* A = (zq*)W3 + F3;
     zq* B = A + n2;
     const int k = blockIdx.z, c = blockIdx.y, p = blockIdx.x;
     const FftK K = f.fk[k];
@@ -1371,17 +1410,17 @@ int fft_plan_create(FftPlan** out, int nk, const int* ng, const int* const* gint
     const int nvb = F2 * fft_chunks(F3, F1);
     for (int a = 0; a < 3 && pl->fx; ++a) {
         const int L = pl->F[a];
-        std::vector<zq> w(L);
+        std::vector<tq> w(L);
         for (int m = 0; m < L; ++m) {
             const long double th = 2.0L * 3.14159265358979323846264338327950288L * m / L;
-            w[m].x = llroundl(cosl(th) * 4611686018427387904.0L);
-            w[m].y = -llroundl(sinl(th) * 4611686018427387904.0L);
+            w[m].x = qsplit(llroundl(cosl(th) * 4611686018427387904.0L));
+            w[m].y = qsplit(-llroundl(sinl(th) * 4611686018427387904.0L));
         }
-        pl->wq[a] = fdalloc<zq>(L, why, &ok);
-        if (ok) cudaMemcpy(pl->wq[a], w.data(), L * sizeof(zq), cudaMemcpyHostToDevice);
+        pl->wq[a] = fdalloc<tq>(L, why, &ok);
+        if (ok) cudaMemcpy(pl->wq[a], w.data(), L * sizeof(tq), cudaMemcpyHostToDevice);
     }
     for (int i = 0; i < 2 && pl->fx; ++i) {
-        pl->vq[i] = fdalloc<zq>(n3, why, &ok);
+        pl->vq[i] = fdalloc<tq>(n3, why, &ok);
         pl->vqe[i] = fdalloc<int>(nvb, why, &ok);
     }
     if (ok) pl->v64 = fdalloc<zd>(n3, why, &ok);
