@@ -235,6 +235,7 @@ static StepArgs make_args(rttddft_ctx* ctx, int dv_on) {
     a.inv_c = 1.0 / ctx->c;
     a.half_inv_c2 = 0.5 / (ctx->c * ctx->c);
     a.omega = ctx->omega;
+    a.neg_inv_omega = -1.0 / ctx->omega;
     a.kd = ctx->d_kd;
     a.occ = ctx->d_occ;
     a.wk = ctx->d_wk;

@@ -99,13 +99,14 @@ struct DevState {
     double cur_aa;      // |A|^2 / (2 c^2)
     int err;            // nonzero: a device iteration limit ran out
     unsigned bar;       // arrival counter of the grid barrier (zeroed by k_hsub and k_finalize)
+    unsigned fin;       // arrival counter of k_finalize's blocks (wraps to zero)
 };
 
 // Everything the step kernels need, passed by value
 struct StepArgs {
     int nk, ns, naux, prop, prec, reproject, nterms, dv_on;
     int vt_center, nvt, lrows, ma, rec_cap, pad;
-    double dt, c, omega;
+    double dt, c, omega, neg_inv_omega;
     double inv_c, half_inv_c2;  // 1/c and 1/(2 c^2): GB300 FP64 division is slow, multiply instead
     const KDev* kd;
     const double* occ;   // ns
