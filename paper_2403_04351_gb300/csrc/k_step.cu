@@ -984,7 +984,6 @@ __global__ void __launch_bounds__(32) k_local(StepArgs a) {
 // staged once in shared memory as FP32, lanes own columns (CPL per lane) and
 // a warp walks one local row at a time, reading the row of h, o, p (FP32
 // copies, broadcast) once for all columns.  Outputs as k_local.
-#define LOCW_MIN_NS 16  // above this many states the columns-per-lane kernel wins
 template <int CPL>
 __global__ void __launch_bounds__(128) k_local_wide(StepArgs a, int rowchunks) {
     extern __shared__ zf xs[];  // [m][ns]

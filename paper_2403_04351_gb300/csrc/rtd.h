@@ -171,6 +171,7 @@ struct StepArgs {
 };
 #define ZT_MIN_N 16           // columns from which the FP32 contractions take the 64 x 64 tiled kernel
 #define JRHO_MIN_NS 8         // above this many states the subspace current goes through rho = theta F theta^H
+#define LOCW_MIN_NS 16  // above this many states the columns-per-lane muffin-tin kernel wins (FP32 forms)
 #define FIN_CH 8              // row chunks per k-point of the first reduction phase
 #define FIN_STRIDE 16
 #define POST_STRIDE 36        // part_post row: residual, J_sub (3), then theta^H theta~ (ns <= 4)

@@ -73,3 +73,22 @@ def test_non_finite_columns_stay_their_own(bad, launches, monkeypatch):
     assert np.array_equal(got[:, [0, 2]], want[:, [0, 2]])
     assert not np.any(np.isfinite(got[:, 1]))
     ctx.close()
+
+
+@pytest.mark.parametrize("route", ["toeplitz", "fft"])
+@pytest.mark.parametrize("n_s,n_cols", [(7, 9), (7, 17), (16, 19), (17, 18)])
+def test_last_columns_of_an_fp32_block(n_s, n_cols, route):
+    """Blocks that the states do not divide: the last columns alone (16 states and
+    fewer) or padded, at the FP32 form's 1e-5 (|H||x|)."""
+    s = make_system(tiny_config(n_g=150, n_atoms=2, lmax=2, n_lo_per_atom=3, n_s=n_s, n_aux=24))
+    rng = np.random.default_rng(n_cols)
+    nb = int(s["n_g"][0]) + int(np.sum(s["n_lo"]))
+    x = rng.standard_normal((nb, n_cols)) + 1j * rng.standard_normal((nb, n_cols))
+    a_vec = np.array([3.0, -1.0, 2.0])
+    ctx = Context(s, precision="fp32", interstitial=route)
+    hx, sx = ctx.apply(0, x, a_vec, 0.0)
+    ops = explicit_operators(s, 0)
+    h = hamiltonian(ops, a_vec, s["c_light"])
+    assert np.max(np.abs(hx - h @ x) / (np.abs(h) @ np.abs(x))) < 1e-5
+    assert np.max(np.abs(sx - ops["S"] @ x) / (np.abs(ops["S"]) @ np.abs(x))) < 1e-5
+    ctx.close()
