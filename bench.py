@@ -56,16 +56,13 @@ SM_COUNT, SM_MAX_MHZ, FP32_LANES = 152, 2070.0, 128
 
 # dram bytes (read + write) per launch from ncu captures, keyed by kernel slot,
 # form and workload; valid only while the kernel source hashes match.
-TRAFFIC = {
-    # dram__bytes_read.sum + dram__bytes_write.sum per launch, keyed by the kernel
-    # sources they were taken on.  mos2_16k: an ncu capture of the DRAM counters on two
-    # of its k-points (--k-subset 0,1), scaled to all 16: the series by the
-    # k-points (8x, every k-point has the same N_aux), the interstitial and matching-
-    # row products by sum_k N_G (6.833x; their streams are the matching coefficients
-    # and the packed C_G, both proportional to N_G).
-    ("chebyshev_series", "bf16x3", "mos2_16k", "7a742d39b168f133"): 27926528.0,
-    ("tc_interstitial_and_forward", "bf16x3", "mos2_16k", "7a742d39b168f133"): 4533407514.0,
-}
+# (slot, form, workload, source hash): bytes.  None is held for the present sources.
+TRAFFIC = {}
+
+# 16-bit products of one FP64 multiply-add in the exact digit products (k_dg.cu):
+# six digits a factor, the 26 pairs that reach the result
+DIGIT_PAIRS = 26
+DIGIT_SERIES_MIN_NS = 9  # states from which the Chebyshev series runs as digit products
 
 
 def _peaks():
@@ -308,10 +305,16 @@ def roofline_of(name, tr, s, prec, nterms):
         ach = fl / dur / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak, "peak_source": src + " (cuBLAS bf16 burst)"}
+    elif (name == "chebyshev_series" and int(s["n_s"]) >= DIGIT_SERIES_MIN_NS) or \
+            (prec == "fp64" and name in ("gemm_expand", "gemm_project", "gemm_forward")):
+        peak, src = _bf16_peak()
+        ach = DIGIT_PAIRS * fl / dur / 1e12
+        roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+                "frac": ach / peak, "peak_source": src + " (cuBLAS bf16 burst; 26 16-bit products per FP64 one)"}
     else:
         if prec == "fp64" or name in ("chebyshev_term", "chebyshev_series"):
             peak = FP64_PEAK_TFLOPS
-            src = "recipe FP64 nominal"
+            src = "FP64 nominal (the series and the FP64 transforms run in 64-bit integers)"
         else:
             peak = SM_COUNT * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12
             src = "152 SM x 128 FP32 lanes x 2 x 2070 MHz"

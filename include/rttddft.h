@@ -68,7 +68,9 @@ extern "C" {
 #define RTTDDFT_PROP_CN 2        /* Crank-Nicolson (I + i dt/2 HH)^{-1} (I - i dt/2 HH), by its Chebyshev series */
 
 /* precision of the full-basis contractions (expand, operator, project);
- * the subspace propagation and every reduction stay FP64 */
+ * the subspace propagation and every reduction stay FP64, or exact digit
+ * products and 64-bit fixed point of that accuracy, as do the contractions and
+ * transforms of the FP64 form */
 #define RTTDDFT_PREC_FP64 0
 #define RTTDDFT_PREC_FP32 1
 /* split-BF16 on the tensor cores: the interstitial convolution and the
@@ -366,9 +368,10 @@ RTTDDFT_API int rttddft_polarizability(int n_t, double t0, double dt, const doub
  * of K, the slices summed in FP64.  Error per element: a few 2^-16 of
  * sum_k |a||x| (the dropped lo.lo term and the rounding of lo).
  * a, x, c: device pointers, complex, column-major, lda >= rows of A,
- * ldx >= k, ldc >= m.  stream: a cudaStream_t or NULL.  The call allocates
- * and frees its own workspace (about (m + 2n) x 8k bytes) and synchronizes
- * the stream before it returns.  m, n or k = 0 is allowed (C unchanged for
+ * ldx >= k, ldc >= m.  stream: a cudaStream_t or NULL.  The call takes its
+ * workspace (about (m + 2n) x 8k bytes) in stream order from a pool of the
+ * library, one per device, which keeps up to 128 MiB between calls, and
+ * synchronizes the stream before it returns.  m, n or k = 0 is allowed (C unchanged for
  * k = 0 with beta_add = 1, zero otherwise).
  * Errors: ERR_ARG (sizes, leading dimensions, NULL), ERR_OOM, ERR_CUDA,
  * ERR_TIMEOUT (a bounded wait of the copy/product pipeline ran out),
