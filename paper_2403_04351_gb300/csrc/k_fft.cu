@@ -161,7 +161,8 @@ template <typename C> __device__ __forceinline__ C ci2(typename Rt<C>::R w1, C d
     return cmk<C>(-(w1 * d1.y + w2 * d2.y), w1 * d1.x + w2 * d2.x);
 }
 
-// Fixed point: 64-bit integers below 2^61 with a power-of-two scale per block,
+// Fixed point: 64-bit integers, complex values below 2^62 in modulus (so the middle
+// sums of a product stay below 2 sqrt(2) 2^61), a power-of-two scale per block,
 // factors (twiddles, potential) with 62 binary places.  A product keeps the three
 // largest of its four 32-bit partial products; the low words are signed
 // (balanced), so what is dropped averages to zero and stays below one unit.
@@ -594,22 +595,22 @@ __global__ void __launch_bounds__(FFT_PTHREADS) k_fft_plane(FftArgs f, int fwd) 
 // at 64 or more lanes per clock and a twiddle 12 wide products at about 16.
 // Values are q 2^e with one exponent per block of a pass: a block takes the
 // largest magnitude of the blocks that it reads, aligned so that its transform
-// of L points cannot pass 2^61 (the terms of any partial sum are at most
+// of L points cannot pass 2^62 (the terms of any partial sum are at most
 // sqrt(2) L times the largest part), and stores the bit length of its results.
-// So 53 bits or more lie below the largest value of a block at each pass (the
+// So 54 bits or more lie below the largest value of a block at each pass (the
 // reason for FX_MAX_N), and what a pass rounds is below what FP64 rounds in it.
 // A block that reads an infinity or a NaN makes the column NaN, as the sums did.
 // 200 columns on 48^3 points 3273 -> 1367 us, 60 columns of the interface 1414 ->
 // 613 us, 7 columns of 25527 plane waves 524 -> 245 us (FP64 transforms before).
 // Exponent entries: x = e, y = top, the values are below 2^top.
-#define FX_MAX_N 181              // 60.5 - log2(181) = 53 bits
+#define FX_MAX_N 181              // 61.5 - log2(181) = 54 bits
 #define FX_ZERO (-(1 << 28))      // top of a block of zeros (its values are not stored)
 #define FX_NAN (1 << 28)          // top of a block that met a non-finite value (nor are these)
 
-// bits that the values of a transform of L points may start with: floor(60.5 - log2 L)
+// bits that the values of a transform of L points may start with: floor(61.5 - log2 L)
 static int fx_bits(int L) {
-    int b = 60;
-    while ((double)L * (double)(1LL << b) > 1630477228166597777.0) --b;
+    int b = 61;
+    while ((double)L * (double)(1LL << b) > 3260954456333195553.0) --b;
     return b;
 }
 __device__ __forceinline__ long long fx_sh1(long long v, int s) {
