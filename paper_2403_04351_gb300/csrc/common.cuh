@@ -81,6 +81,7 @@ template <> struct Cx<zd> {
     static __device__ __forceinline__ zd zero() { return zmk(0.0, 0.0); }
     static __device__ __forceinline__ zd from(zd a) { return a; }
     static __device__ __forceinline__ zd from(zf a) { return tod(a); }
+    static __device__ __forceinline__ zd ld(zd a) { return a; }
     static __device__ __forceinline__ void fma(zd& c, zd a, zd b) { zfma(c, a, b); }
     static __device__ __forceinline__ void fmac(zd& c, zd a, zd b) { zfmac(c, a, b); }
     static __device__ __forceinline__ zd todbl(zd a) { return a; }
@@ -89,6 +90,8 @@ template <> struct Cx<zf> {
     static __device__ __forceinline__ zf zero() { return make_float2(0.f, 0.f); }
     static __device__ __forceinline__ zf from(zd a) { return tof(a); }
     static __device__ __forceinline__ zf from(zf a) { return a; }
+    // by the conversion instruction: no branches between the loads of a batch
+    static __device__ __forceinline__ zf ld(zd a) { return make_float2(__double2float_rn(a.x), __double2float_rn(a.y)); }
     static __device__ __forceinline__ void fma(zf& c, zf a, zf b) { cfma(c, a, b); }
     static __device__ __forceinline__ void fmac(zf& c, zf a, zf b) { cfmac(c, a, b); }
     static __device__ __forceinline__ zd todbl(zf a) { return tod(a); }

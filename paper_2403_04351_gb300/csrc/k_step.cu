@@ -1280,7 +1280,7 @@ __global__ void __launch_bounds__(BT) k_toep_seg(StepArgs a, int n0, int slot0) 
                 ls[tid] = glin[c0 + tid];
 #pragma unroll
                 for (int c = 0; c < NT; ++c)
-                    xs[tid * NT + c] = (c < nc) ? Cx<TC>::from(X[(c0 + tid) + (size_t)(n0 + c) * nb]) : Cx<TC>::zero();
+                    xs[tid * NT + c] = (c < nc) ? Cx<TC>::ld(X[(c0 + tid) + (size_t)(n0 + c) * nb]) : Cx<TC>::zero();
             }
             for (int e = tid; e < wn; e += BT) ws[e] = tab[wlo + e];
             __syncthreads();
@@ -1306,8 +1306,8 @@ __global__ void __launch_bounds__(BT) k_toep_seg(StepArgs a, int n0, int slot0) 
             const int q = r - r_lo;
 #pragma unroll
             for (int c = 0; c < NT; ++c) {
-                zs[q * 2 * NT + c] = (c < nc) ? Cx<TC>::from(Z[r + (size_t)(n0 + c) * ma]) : Cx<TC>::zero();
-                zs[q * 2 * NT + NT + c] = (c < nc) ? Cx<TC>::from(Z[r + (size_t)(ns + n0 + c) * ma]) : Cx<TC>::zero();
+                zs[q * 2 * NT + c] = (c < nc) ? Cx<TC>::ld(Z[r + (size_t)(n0 + c) * ma]) : Cx<TC>::zero();
+                zs[q * 2 * NT + NT + c] = (c < nc) ? Cx<TC>::ld(Z[r + (size_t)(ns + n0 + c) * ma]) : Cx<TC>::zero();
             }
         }
         __syncthreads();
