@@ -94,7 +94,7 @@ template <> struct Cx<zf> {
     static __device__ __forceinline__ zf ld(zd a) { return make_float2(__double2float_rn(a.x), __double2float_rn(a.y)); }
     static __device__ __forceinline__ void fma(zf& c, zf a, zf b) { cfma(c, a, b); }
     static __device__ __forceinline__ void fmac(zf& c, zf a, zf b) { cfmac(c, a, b); }
-    static __device__ __forceinline__ zd todbl(zf a) { return tod(a); }
+    static __device__ __forceinline__ zd todbl(zf a) { return zmk((double)a.x, (double)a.y); }
 };
 
 // 16-bit split w = v * scale = hi + lo (each rounded to nearest): fmt 1 bf16,
