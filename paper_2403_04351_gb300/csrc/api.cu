@@ -786,6 +786,36 @@ static void build_dv_dg(rttddft_ctx* ctx) {
     for (DgGemm* g : {gi, gw, gg, gd}) dg_gemm_destroy(g);
 }
 
+// Undo a first rttddft_set_dv that failed: whatever it allocated (the allocations
+// past `mark`) and built goes, so that the next call starts from nothing.
+static void drop_dv(rttddft_ctx* ctx, size_t mark) {
+    cudaStreamSynchronize(ctx->stream);
+    for (DgGemm** g : {&ctx->dg_dvw, &ctx->dg_dvg, &ctx->dg_dvi, &ctx->dg_mtd}) {
+        dg_gemm_destroy(*g);
+        *g = nullptr;
+    }
+    for (DgLeft** l : {&ctx->dgl_dh, &ctx->dgl_lh}) {
+        dg_left_destroy(*l);
+        *l = nullptr;
+    }
+    if (!ctx->dg_proj) {  // CC^H's digits, unless the operator's
+        dg_left_destroy(ctx->dgl_cch);
+        ctx->dgl_cch = nullptr;
+    }
+    while (ctx->allocs.size() > mark) {
+        cudaFree(ctx->allocs.back());
+        ctx->allocs.pop_back();
+    }
+    ctx->dv_t.clear();
+    ctx->dv_w.clear();
+    ctx->d_dh = ctx->d_dvtab = ctx->d_vstep = ctx->d_mtd = ctx->d_part_dv = nullptr;
+    ctx->d_dh32 = ctx->d_vstep32 = nullptr;
+    ctx->d_vsteps = nullptr;
+    ctx->gd_dvi = ctx->gd_dvw = ctx->gd_dvg = ctx->gd_dvi32 = ctx->gd_dvw32 = ctx->gd_dvg32 = nullptr;
+    ctx->td_dv = nullptr;
+    for (KDev& K : ctx->hkd) K.dvsub = nullptr;
+}
+
 // ------------------------------------------------------------ ABI
 extern "C" {
 
@@ -2058,6 +2088,7 @@ extern "C" {
 
 int rttddft_set_dv(rttddft_ctx* ctx, const double* dh, const double* dvtab) {
     if (!ctx) return RTTDDFT_ERR_ARG;
+    const size_t mark = ctx->allocs.size();
     try {
         if (ctx->opt.hartree) fail(ctx, RTTDDFT_ERR_ARG, "with the Hartree feedback the potential change comes from the density");
         const AtomTab& at = ctx->at;
@@ -2181,6 +2212,7 @@ int rttddft_set_dv(rttddft_ctx* ctx, const double* dh, const double* dvtab) {
         }
         return RTTDDFT_OK;
     } catch (Fail& f) {
+        if (!ctx->dv_set && ctx->allocs.size() > mark) drop_dv(ctx, mark);
         return f.code;
     }
 }

@@ -2032,6 +2032,10 @@ int tc_dv_prepare(TcPlan* tp, const zd* const* caux_dev, const int* nb, const in
         cudaMalloc(&tp->dvtabs, (size_t)std::max(1, nvt) * sizeof(uint2)) != cudaSuccess ||
         cudaMalloc(&tp->Dd, nd * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
+        for (void* q : {(void*)tp->cch, (void*)tp->ccl, (void*)tp->dvtabs, (void*)tp->Dd}) cudaFree(q);
+        tp->cch = tp->ccl = nullptr;
+        tp->dvtabs = nullptr;
+        tp->Dd = nullptr;
         *why = "out of device memory for the potential-change operands";
         return RTTDDFT_ERR_OOM;
     }

@@ -1,0 +1,69 @@
+"""Calls made while the device memory is nearly full: what a call that ran out
+of it leaves behind, and what runs without the memory for the digits."""
+import numpy as np
+import pytest
+
+from paper_2403_04351_gb300 import Context, RttddftError
+from synth import make_dv, make_system, pulse_samples, dv_scale_samples, tiny_config
+
+pytestmark = pytest.mark.gpu
+
+MIB = 1 << 20
+
+
+class Full:
+    """All of the device memory taken but `left` bytes (to the driver's granularity)."""
+
+    def __init__(self, left):
+        import torch
+        torch.cuda.empty_cache()
+        torch.cuda.synchronize()
+        self.hold = []
+        for part in (4096 * MIB, 256 * MIB, 32 * MIB, 4 * MIB):
+            while torch.cuda.mem_get_info()[0] > left + part:
+                try:
+                    n = (torch.cuda.mem_get_info()[0] - left) // part
+                    self.hold.append(torch.empty(int(n) * part, dtype=torch.uint8, device="cuda"))
+                except torch.OutOfMemoryError:  # not in one piece
+                    try:
+                        self.hold.append(torch.empty(part, dtype=torch.uint8, device="cuda"))
+                    except torch.OutOfMemoryError:
+                        break
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *_):
+        import torch
+        self.hold.clear()
+        torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_set_dv_after_one_that_ran_out_of_memory(prec):
+    """The first call fails in the transform's columns, the last buffers it
+    takes.  The same call with the memory free again gives the dVV of a context
+    that never failed: the states bit for bit, since both run the same launches."""
+    s = make_system(tiny_config(n_g=2500, n_atoms=2, lmax=3, n_lo_per_atom=4, n_s=3, n_aux=200))
+    dv = make_dv(s, amp=0.3)
+    a, sc = pulse_samples(s, n_steps=3, a0=5.0), dv_scale_samples(3, s["dt"], freq=3.0)
+
+    def steps(ctx):
+        ctx.step(a, sc)
+        return ctx.get_state(0), ctx.observables()["energy"]
+
+    ctx = Context(s, precision=prec, interstitial="fft", graph_steps=3)
+    ctx.set_dv(dv)
+    want = steps(ctx)
+    ctx.close()
+    ctx = Context(s, precision=prec, interstitial="fft", graph_steps=3)
+    for _ in range(2):
+        with Full(48 * MIB):
+            with pytest.raises(RttddftError) as e:
+                ctx.set_dv(dv)
+        assert e.value.code == -6
+    ctx.set_dv(dv)
+    got = steps(ctx)
+    ctx.close()
+    assert np.array_equal(got[0], want[0])
+    assert np.array_equal(got[1], want[1])
