@@ -2247,6 +2247,8 @@ int rttddft_apply(rttddft_ctx* ctx, int k, int ncols, const double* x, const dou
         if (p.gd_mt1) p.gd_mt1 = ctx->gd_mt1 + (size_t)k * ctx->at.n;
         p.maxng = K.ng;
         if (dv_on && !ctx->opt.hartree) launch_vstep(a, ctx->stream);
+        // density feedback: the last step's dh came after its rebuild had cut the digits
+        if (dv_on && ctx->opt.hartree && p.dg_mtd) launch_dg_left(ctx->dgl_dh, ctx->stream);
         const zd* xz = (const zd*)x;
         zd* hz = (zd*)hx;
         zd* sz = (zd*)sx;

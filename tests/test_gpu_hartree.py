@@ -179,3 +179,38 @@ def test_hartree_bound_is_enforced_and_other_calls_refused(tiny):
         ctx.adjoint(a, np.array([0.0, 0.0, 1.0]))
     assert e.value.code == -9
     ctx.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-11), ("fp32", 1e-5)])
+def test_operator_carries_the_present_density(tiny, prec, tol):
+    """rttddft_apply with the feedback on, after no step, one and several: H with the
+    Hartree matrix and the muffin-tin blocks of the present density, entrywise on the
+    scale of |H||x|.  The operator's own bound is 1e-12 (1e-5 in FP32), the states
+    behind the two densities agree to about as much."""
+    from oracle import hamiltonian, interstitial_density, mt_density
+    a = pulse_samples(tiny, n_steps=4, a0=20.0)
+    o = Oracle(tiny)
+    th0 = [kp["theta0"].copy() for kp in o.kp]
+    cs0 = [kp["caux"] @ t for kp, t in zip(o.kp, th0)]
+    n0 = interstitial_density(tiny, cs0, o.occ, o.wk, o.omega)
+    mt0 = mt_density(tiny, cs0, o.occ, o.wk)
+    rng = np.random.default_rng(2)
+    nb = o.kp[0]["caux"].shape[0]
+    x = rng.standard_normal((nb, 5)) + 1j * rng.standard_normal((nb, 5))
+    a_vec = np.array([0.4, -0.9, 1.3])
+    h0 = hamiltonian(o.kp[0]["ops"], a_vec, o.c)
+    ctx = Context(tiny, precision=prec, interstitial="fft", hartree=True, hartree_mt_u=0.5)
+    done = 0
+    for n in (0, 1, 4):
+        th = Oracle(tiny).run(a[:n], tiny["dt"], hartree=True, mt_u=0.5)["theta"] if n else th0
+        if n:
+            ctx.step(a[done:n])
+            done = n
+        full, part = o.hartree_matrices(th, n0, mt0, 0.5)[0][0], o.hartree_matrices(th, n0)[0][0]
+        h = h0 + full
+        size = np.abs(h) @ np.abs(x)
+        # the blocks alone are far above FP64's bound
+        assert n == 0 or np.max(np.abs((full - part) @ x) / size) > 1e-8
+        hx, _ = ctx.apply(0, x, a_vec, 1.0)
+        assert np.max(np.abs(hx - h @ x) / size) < tol, n
+    ctx.close()
