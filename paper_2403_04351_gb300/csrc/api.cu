@@ -1509,7 +1509,11 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
             ctx->coop_grid = prepare_cheb_coop(a, ctx->stream, &ctx->cheb_cl);
             // many states or rows: digit products; without the memory for the digits one launch
             // per term
-            if (o->propagator != RTTDDFT_PROP_EIG && ctx->coop_grid == 0) ctx->series = dg_series_create(nk, naux, ns);
+            if (o->propagator != RTTDDFT_PROP_EIG && ctx->coop_grid == 0) {
+                std::vector<const zd*> cf(nk);
+                for (int k = 0; k < nk; ++k) cf[k] = ctx->hkd[k].coef;
+                ctx->series = dg_series_create(nk, naux, ns, cf.data());
+            }
         }
         if (ns > JRHO_MIN_NS) {
             // the subspace current of many states: PP theta on the tensor cores

@@ -63,6 +63,19 @@ __device__ __forceinline__ double f2d(float v) {
 __device__ __forceinline__ zf tof(zd a) { return make_float2(d2f(a.x), d2f(a.y)); }
 __device__ __forceinline__ zd tod(zf a) { return zmk(f2d(a.x), f2d(a.y)); }
 
+// x 2^(f - e) rounded to an integer, f <= 62, with integer arithmetic; |x| < 2^e, what
+// lies beyond (and NaN) taken as 2^e at most
+__device__ __forceinline__ long long fix64(double x, int e, int f) {
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)(b >> 52) & 2047;
+    if (ex == 0) return 0;  // zero, or below 2^-1022: nothing of it is left at this scale
+    long long m = (b & ((1ll << 52) - 1)) | (1ll << 52);
+    const int sh = ex - 1075 + f - e;
+    if (sh > f - 53) m = 1ll << f;
+    else m = sh >= 0 ? m << sh : (sh < -54 ? 0 : (m + (1ll << (-sh - 1))) >> -sh);
+    return b < 0 ? -m : m;
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -40,6 +40,6 @@ int launch_dg_table(const DgToep* t, int which, const zd* tab, cudaStream_t s);
 int launch_dg_toep(const DgToep* t, int which, int kofs, int nk, cudaStream_t s);
 
 struct StepArgs;
-DgSeries* dg_series_create(int nk, int n, int ns);
+DgSeries* dg_series_create(int nk, int n, int ns, const zd* const* coef);  // coef: the c_n of every k-point (device)
 void dg_series_destroy(DgSeries* g);
 int launch_dg_series(const DgSeries* g, const StepArgs& a, cudaStream_t s);       // returns its launches

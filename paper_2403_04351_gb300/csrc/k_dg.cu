@@ -149,11 +149,12 @@ struct DgOut {
 };
 struct DgCheb {
     int n;              // N_aux
-    i64 *y0, *y1;       // y of even and of odd terms, units 2^-62 of the column's scale: [2 ns][n]
-    i64* acc;           // sum_n c_n y_n
+    zd *y0, *y1;        // y of even and of odd terms: [ns][n]
+    zd* acc;            // sum_n c_n y_n
+    const double* diag; // of H~
     uint32_t* Bn[2];    // digit operands of even and odd terms
     int nst;
-    i64* coef;          // c_n in units 2^-62
+    const zd* coef;     // c_n
 };
 struct DgArgs {
     const DgOut* out;
@@ -193,11 +194,6 @@ __device__ __forceinline__ void dg_ld(uint32_t taddr, uint32_t* r) {
             : "r"(taddr));
     }
 }
-// a b 2^-62 of two integers in units 2^-62
-__device__ __forceinline__ i64 dg_mul62(i64 a, i64 b) {
-    return (i64)(((unsigned long long)__mul64hi(a, b) << 2) | (((unsigned long long)a * (unsigned long long)b) >> 62));
-}
-
 // One 128-row x NT-column tile of D = A^ B^^T over this split's K stages (NT
 // real columns: Re and Im of NT / 2 complex ones).  The copy warp brings the
 // six digit planes of both operands of a stage with one bulk copy each.  A group has
@@ -553,24 +549,24 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                 if (g.beta) v = zadd(*p, v);
                 *p = v;
             } else {
+                // H~ y: its diagonal in FP64, the rest as digits; the recurrence and the sum in FP64
                 const DgCheb& ch = g.ch[z];
-                i64* yb = (g.term & 1) ? ch.y1 : ch.y0;
-                i64 y[2];
-                const size_t e = (size_t)(2 * n) * ch.n + row;
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    // H~ y in units 2^-62: hi has 2^-43, lo has 2^-70
-                    i64 w = (i64)((unsigned long long)hv[q] << 19) + ((lv[q] + 128) >> 8);
-                    if (g.term > 1) w = (i64)(2ull * (unsigned long long)w - (unsigned long long)yb[e + (size_t)q * ch.n]);
-                    y[q] = w;
+                zd* yb = (g.term & 1) ? ch.y1 : ch.y0;
+                const size_t e = (size_t)n * ch.n + row;
+                const int er = o.er[row], ec = o.ec[n];
+                const zd yp = ((g.term & 1) ? ch.y0 : ch.y1)[e];
+                const double d = ch.diag[row];
+                zd y = zmk(fma(d, yp.x, dg_double(hv[0], lv[0], er + ec - 70)), fma(d, yp.y, dg_double(hv[1], lv[1], er + ec - 70)));
+                if (g.term > 1) {
+                    const zd y2 = yb[e];
+                    y = zmk(fma(2.0, y.x, -y2.x), fma(2.0, y.y, -y2.y));
                 }
-                const i64 cr = ch.coef[2 * g.term], ci = ch.coef[2 * g.term + 1];
-                ch.acc[e] += dg_mul62(cr, y[0]) - dg_mul62(ci, y[1]);
-                ch.acc[e + ch.n] += dg_mul62(cr, y[1]) + dg_mul62(ci, y[0]);
+                zd sm = ch.acc[e];
+                zfma(sm, ch.coef[g.term], y);
+                ch.acc[e] = sm;
                 if (!g.last) {
-                    yb[e] = y[0];
-                    yb[e + ch.n] = y[1];
-                    dg_put_col(ch.Bn[g.term & 1], NT, ch.nst, n, row, (y[0] + 256) >> 9, (y[1] + 256) >> 9);
+                    yb[e] = y;
+                    dg_put_col(ch.Bn[g.term & 1], NT, ch.nst, n, row, fix64(y.x, ec, 53), fix64(y.y, ec, 53));
                 }
             }
         }
@@ -1046,16 +1042,22 @@ int launch_dg_toep(const DgToep* t, int which, int kofs, int nk, cudaStream_t s)
 // The series with H~ y_{n-1} as digit products, one launch per term, for more
 // states or rows than k_cheb_coop takes.  In FP64 its rate was the FP64 pipe's (16
 // k-points of N_aux 300, N_s 60: 9.0 GFLOP in 8.3 ms; 2 k-points 1.91 ms); here the
-// 2 k-points take 0.27 ms, bound by the 14 launches of a few stages each.
-// H~ = (HH - lam_c) / lam_h has norm <= 1, so its entries take the scale
-// 1; a column of theta takes the power of two above its 2-norm, which bounds
-// every y_n.  y_n, the recurrence and the sum are integers in units of 2^-62
-// of that scale: nothing is rounded between the terms but the digits' cut.
+// 2 k-points take 0.26 ms, bound by the 14 launches of a few stages each.
+// H~ = (HH - lam_c) / lam_h is its diagonal, which multiplies y in FP64, and the
+// rest as digits, a power of two above the largest entry for each row; a column of
+// y takes the power of two above theta's 2-norm, which bounds every y_n (H~ has
+// norm <= 1).  The recurrence and the sum are FP64.  So the cut is 2^-54 of what
+// couples an amplitude to the others, and an amplitude that a weak field feeds
+// keeps FP64's relative accuracy (with the diagonal among the digits and y_n in
+// integers it kept 2^-54 of the column's norm: 1e-8 of the excited amplitudes at
+// A = 1e-4).
 struct DgSeriesK {
-    uint32_t* A;     // digits of H~, tiles of 128 rows
+    uint32_t* A;     // digits of H~ off its diagonal, tiles of 128 rows
     int nst, NT;
+    int* er;         // their row exponents
+    double* diag;
     int* bad;        // per row: HH not finite
-    int* ec;
+    int* ec;         // column exponents of y; 2048: theta not finite
 };
 struct DgSeries {
     DgPool pool;
@@ -1067,9 +1069,12 @@ struct DgSeries {
     unsigned* cnt = nullptr;
 };
 
-// digits of row i of H~ (HH as in k_hsub; HH is Hermitian, so row i is read
-// as the conjugate of the contiguous column i)
+// digits of row i of H~ off its diagonal (HH as in k_hsub; HH is Hermitian, so
+// row i is read as the conjugate of the contiguous column i).  A thread holds
+// its first DG_HS_E entries from the search for the largest one to the cut.
+#define DG_HS_E 4
 __global__ void __launch_bounds__(128) k_dg_hsub(StepArgs a, const DgSeriesK* sk) {
+    __shared__ int smx[4];
     const DgSeriesK& S = sk[blockIdx.z];
     const KDev& K = a.kd[blockIdx.z];
     const int n = a.naux, i = blockIdx.x;
@@ -1089,9 +1094,7 @@ __global__ void __launch_bounds__(128) k_dg_hsub(StepArgs a, const DgSeriesK* sk
     const double lc = K.lam[0], ilh = K.lam[2];
     const double al[3] = {ax * a.inv_c, ay * a.inv_c, az * a.inv_c};
     const size_t nn = (size_t)n * n;
-    const DgScale sc = dg_scale(0);
-    int bad = 0;
-    for (int j = threadIdx.x; j < n; j += 128) {
+    auto entry = [&](int j) {
         const size_t e = (size_t)i * n + j;
         zd v = zmk(0.0, 0.0);
 #pragma unroll
@@ -1100,23 +1103,61 @@ __global__ void __launch_bounds__(128) k_dg_hsub(StepArgs a, const DgSeriesK* sk
         if (i == j) v.x += K.eps[i] + aa;
         if (a.dv_on) v = zadd(v, K.dvsub[e]);
         if (i == j) v.x -= lc;
-        v = zscale(v, ilh);
-        if (dg_hw(v.x) >= 0x7ff00000 || dg_hw(v.y) >= 0x7ff00000) bad = 1;
-        // |H~_ij| <= 1; a step beyond its bounds (reported by its flag) stays in range
-        v.x = fmin(fmax(v.x, -1.0), 1.0);
-        v.y = fmin(fmax(v.y, -1.0), 1.0);
+        return zscale(v, ilh);
+    };
+    int bad = 0, hm = 0;
+    auto look = [&](int j, zd& v) {  // the diagonal entry's real part goes to S.diag
+        const int hx = dg_hw(v.x), hy = dg_hw(v.y);
+        if (hx >= 0x7ff00000 || hy >= 0x7ff00000) bad = 1;
+        if (j == i) {
+            S.diag[i] = v.x;
+            v.x = 0.0;
+            hm = max(hm, hy);
+        } else {
+            hm = max(hm, max(hx, hy));
+        }
+    };
+    zd h[DG_HS_E];
+#pragma unroll
+    for (int u = 0; u < DG_HS_E; ++u) {
+        const int j = threadIdx.x + u * 128;
+        if (j >= n) continue;
+        h[u] = entry(j);
+        look(j, h[u]);
+    }
+    for (int j = threadIdx.x + DG_HS_E * 128; j < n; j += 128) {
+        zd v = entry(j);
+        look(j, v);
+    }
+    hm = __reduce_max_sync(0xffffffffu, hm);
+    if ((threadIdx.x & 31) == 0) smx[threadIdx.x >> 5] = hm;
+    bad = __syncthreads_or(bad);
+    const int e = bad ? 0 : dg_exp(max(max(smx[0], smx[1]), max(smx[2], smx[3])));
+    if (threadIdx.x == 0) {
+        S.bad[i] = bad;
+        S.er[i] = e;
+    }
+    auto put = [&](int j, zd v) {
         uint32_t dr[DG_P], di[DG_P];
-        dg_cut(dg_int(v.x, sc), dr);
-        dg_cut(dg_int(-v.y, sc), di);
+        dg_cut(fix64(v.x, e, 53), dr);
+        dg_cut(-fix64(v.y, e, 53), di);
 #pragma unroll
         for (int q = 0; q < DG_P; ++q)
             S.A[dg_word(i, j, DG_BM, S.nst) + (size_t)q * DG_BM * 16] = dg_pair(dr[q], di[q]);
+    };
+#pragma unroll
+    for (int u = 0; u < DG_HS_E; ++u) {
+        const int j = threadIdx.x + u * 128;
+        if (j < n) put(j, h[u]);
     }
-    bad = __syncthreads_or(bad);
-    if (threadIdx.x == 0) S.bad[i] = bad;
+    for (int j = threadIdx.x + DG_HS_E * 128; j < n; j += 128) {
+        zd v = entry(j);
+        if (j == i) v.x = 0.0;
+        put(j, v);
+    }
 }
 
-// y_0 = theta in units of its column's scale, its digits, and c_0 y_0
+// y_0 = theta, its digits, and c_0 y_0
 __global__ void __launch_bounds__(128) k_dg_y0(StepArgs a, const DgSeriesK* sk, const DgCheb* chs) {
     __shared__ double sh[4];
     const DgSeriesK& S = sk[blockIdx.z];
@@ -1145,28 +1186,17 @@ __global__ void __launch_bounds__(128) k_dg_y0(StepArgs a, const DgSeriesK* sk, 
     if ((tid & 31) == 0) sh[tid >> 5] = q;
     __syncthreads();
     q = sqrt(sh[0] + sh[1] + sh[2] + sh[3]);
-    // the power of two above the norm, less a rounding error's room at exact powers
-    const int en = q > 0.0 ? dg_exp(dg_hw(q * (1.0 - 1e-12))) : 53;
+    // the power of two above the norm, with room for the rounding of the terms
+    const int en = q > 0.0 ? dg_exp(dg_hw(q * (1.0 + 1e-9))) : 53;
     e += en - 53;
     if (tid == 0) S.ec[c] = bad ? 2048 : e;
-    const int s = 62 - e, h = s / 2;
-    const double p1 = dg_pow2(max(-1000, min(1000, h))), p2 = dg_pow2(max(-1000, min(1000, s - h)));
-    // the coefficients in units 2^-62 (|c_n| < 2), once per k-point and by every block for c_0
-    const double one62 = 4611686018427387904.0;
-    const i64 cr = __double2ll_rn(K.coef[0].x * one62), ci = __double2ll_rn(K.coef[0].y * one62);
-    if (c == 0)
-        for (int i = tid; i < a.nterms; i += 128) {
-            ch.coef[2 * i] = __double2ll_rn(K.coef[i].x * one62);
-            ch.coef[2 * i + 1] = __double2ll_rn(K.coef[i].y * one62);
-        }
+    const zd c0 = K.coef[0];
     for (int i = tid; i < n; i += 128) {
-        const i64 yr = bad ? 0 : __double2ll_rn((th[i].x * p1) * p2), yi = bad ? 0 : __double2ll_rn((th[i].y * p1) * p2);
-        const size_t x = (size_t)(2 * c) * n + i;
-        ch.y0[x] = yr;
-        ch.y0[x + n] = yi;
-        ch.acc[x] = dg_mul62(cr, yr) - dg_mul62(ci, yi);
-        ch.acc[x + n] = dg_mul62(cr, yi) + dg_mul62(ci, yr);
-        dg_put_col(ch.Bn[0], S.NT, ch.nst, c, i, (yr + 256) >> 9, (yi + 256) >> 9);
+        const zd y = bad ? zmk(0.0, 0.0) : th[i];
+        const size_t x = (size_t)c * n + i;
+        ch.y0[x] = y;
+        ch.acc[x] = zmul(c0, y);
+        dg_put_col(ch.Bn[0], S.NT, ch.nst, c, i, fix64(y.x, e, 53), fix64(y.y, e, 53));
     }
 }
 
@@ -1176,17 +1206,12 @@ __global__ void __launch_bounds__(128) k_dg_theta(StepArgs a, const DgSeriesK* s
     const DgCheb& ch = chs[blockIdx.z];
     const KDev& K = a.kd[blockIdx.z];
     const int n = a.naux, c = blockIdx.x, tid = threadIdx.x;
-    const int e = S.ec[c];
-    int bad = e >= 2048;
+    int bad = S.ec[c] >= 2048;
     for (int i = tid; i < n; i += 128) bad |= S.bad[i];
     bad = __syncthreads_or(bad);
     const zd ph = (a.prop == 0) ? zmk(K.lam[3], K.lam[4]) : zmk(1.0, 0.0);
-    const int s = bad ? 0 : e - 62, h = s / 2;
-    const double p1 = dg_pow2(max(-1000, min(1000, h))), p2 = dg_pow2(max(-1000, min(1000, s - h)));
     for (int i = tid; i < n; i += 128) {
-        const size_t x = (size_t)(2 * c) * n + i;
-        zd v = zmul(ph, zmk((double)ch.acc[x], (double)ch.acc[x + n]));
-        v = zmk((v.x * p1) * p2, (v.y * p1) * p2);
+        zd v = zmul(ph, ch.acc[(size_t)c * n + i]);
         if (bad) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
         K.theta[i + (size_t)c * n] = v;
     }
@@ -1198,7 +1223,7 @@ void dg_series_destroy(DgSeries* g) {
     delete g;
 }
 
-DgSeries* dg_series_create(int nk, int n, int ns) {
+DgSeries* dg_series_create(int nk, int n, int ns, const zd* const* coef) {
     DgSeries* g = new DgSeries();
     g->nk = nk;
     g->n = n;
@@ -1218,14 +1243,19 @@ DgSeries* dg_series_create(int nk, int n, int ns) {
         sk[k].ec = (int*)g->pool.get(ns * sizeof(int), true);
         DgCheb& c = ch[k];
         c.n = n;
-        c.y0 = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
-        c.y1 = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
-        c.acc = (i64*)g->pool.get((size_t)2 * ns * n * sizeof(i64), true);
+        sk[k].er = (int*)g->pool.get(n * sizeof(int), true);
+        sk[k].diag = (double*)g->pool.get(n * sizeof(double), true);
+        c.y0 = (zd*)g->pool.get((size_t)ns * n * sizeof(zd), true);
+        c.y1 = (zd*)g->pool.get((size_t)ns * n * sizeof(zd), true);
+        c.acc = (zd*)g->pool.get((size_t)ns * n * sizeof(zd), true);
+        c.diag = sk[k].diag;
         for (int q = 0; q < 2; ++q) c.Bn[q] = (uint32_t*)g->pool.get(dg_bytes(np, n), true);
         c.nst = nst;
-        c.coef = (i64*)g->pool.get((size_t)2 * RTD_MAX_TERMS * sizeof(i64), true);
+        c.coef = coef[k];
         out[k] = DgOut{};
         out[k].A = (const unsigned char*)sk[k].A;
+        out[k].er = sk[k].er;
+        out[k].ec = sk[k].ec;
         out[k].M = n;
         out[k].nst = out[k].nsta = nst;
         out[k].tile0 = k * g->mt * g->ntn;
