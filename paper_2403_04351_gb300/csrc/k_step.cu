@@ -152,13 +152,18 @@ __global__ void __launch_bounds__(128) k_cheb(StepArgs a, int nt, int last) {
 // The whole series of few states in one cooperative launch, one block per row
 // (k, i) of HH.  An FP64 instruction of a warp holds its sub-partition for 64
 // cycles on GB300 whatever the number of active lanes, so a term's dot product,
-// sums and update took 3 us; here they run on the integer pipe (a series of N_aux
-// 200, N_s 2: 82 -> 48 us; N_aux 240, N_s 7: 111 -> 73 us).  H~ = (HH - lam_c) / lam_h has norm <= 1 and takes units of 2^-58, a
-// column of theta the power of two above its 2-norm (which bounds every y_n),
-// y_n units of 2^-57 of it.  An operand is held as hi 2^28 + lo; a product keeps
-// hi hi and hi lo + lo hi (the dropped lo lo is below 2^-61), summed exactly in
-// 64 bits, so a term's error is the cut of its operands, 2^-58 of the norm, below
-// FP64's own.  The recurrence and sum_n c_n y_n are integers in units of 2^-59.
+// sums and update took 3 us; here the dot products run on the integer pipe, and
+// the N_s entries of a row have their diagonal, recurrence and sum in FP64 (a
+// series of N_aux 200, N_s 2: 82 -> 50 us; N_aux 240, N_s 7: 111 -> 75 us).
+// H~ = (HH - lam_c) / lam_h is its diagonal plus the rest of the row in units of
+// 2^-59 of a power of two above the row's 2-norm; y_n goes into the products in
+// units of 2^-57 of the power of two above its column's 2-norm (which bounds every
+// y_n).  An operand is held as hi 2^28 + lo; a product keeps hi hi and hi lo + lo
+// hi (the dropped lo lo is below 2^-60), summed exactly in 64 bits.  So what a term
+// loses is 2^-54 of the largest off-diagonal entry of its row: an amplitude that a
+// weak field feeds keeps FP64's relative accuracy, as small as it is (with the
+// diagonal in the same units, and the recurrence in them, it kept 2^-58 of the
+// column's norm: 5e-10 of the excited amplitudes at A = 1e-4).
 //
 // Per term y_n goes around through L2 (two slots of 16 bytes per entry) and a
 // grid barrier follows.  The barrier has CS_CNT arrival counters on lines of
@@ -169,7 +174,6 @@ __global__ void __launch_bounds__(128) k_cheb(StepArgs a, int nt, int last) {
 // (reported as ERR_TIMEOUT).  The last block to leave sets the counters back.
 #define CS_THREADS 128
 #define CS_CNT 16
-#define CS_MAXC 128  // coefficients kept in shared memory at a time
 struct ChebSync {
     unsigned cnt[CS_CNT][32];
     unsigned left;
@@ -182,16 +186,6 @@ __device__ __forceinline__ int2 cs_split(i64 q) {  // q = hi 2^28 + lo
     return make_int2((int)((q - lo) >> 28), lo);
 }
 __device__ __forceinline__ double cs_pow2(int n) { return __hiloint2double((n + 1023) << 20, 0); }
-// x 2^(f - e) rounded to an integer, |x| < 2^e, f <= 62, with integer arithmetic
-__device__ __forceinline__ i64 cs_fix(double x, int e, int f) {
-    const i64 b = __double_as_longlong(x);
-    const int ex = (int)(b >> 52) & 2047;
-    if (ex == 0) return 0;  // zero, or below 2^-1022: nothing of it is left at this scale
-    i64 m = (b & ((1ll << 52) - 1)) | (1ll << 52);
-    const int sh = ex - 1075 + f - e;
-    m = sh >= 0 ? m << sh : (sh < -54 ? 0 : (m + (1ll << (-sh - 1))) >> -sh);
-    return b < 0 ? -m : m;
-}
 // |x| 2^-e for the norm's estimate, from the high word (relative error 2^-20, small values 0)
 __device__ __forceinline__ float cs_small(double x, int e) {
     const int hw = __double2hiint(x) & 0x7fffffff;
@@ -219,13 +213,16 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     return v;
 }
 
-// phase x sum of c_n y_n (units 2^-59 of the column's scale 2^e) as theta
-__device__ __forceinline__ zd cs_result(const StepArgs& a, const KDev& K, i64 sr, i64 si, int e, bool bad) {
+// t 2^e, the power of two applied in two halves so that neither leaves FP64's range
+__device__ __forceinline__ zd cs_scale(zd t, int e) {
+    const int h = e / 2;
+    const double p1 = cs_pow2(h), p2 = cs_pow2(e - h);
+    return zmk((t.x * p1) * p2, (t.y * p1) * p2);
+}
+// phase x sum of c_n y_n (in units of the column's scale 2^e) as theta
+__device__ __forceinline__ zd cs_result(const StepArgs& a, const KDev& K, zd s, int e, bool bad) {
     const zd ph = (a.prop == 0) ? zmk(K.lam[3], K.lam[4]) : zmk(1.0, 0.0);
-    zd t = zmul(ph, zmk((double)sr, (double)si));
-    const int s = min(e, 1024) - 59, h = s / 2;
-    const double p1 = cs_pow2(h), p2 = cs_pow2(s - h);
-    t = zmk((t.x * p1) * p2, (t.y * p1) * p2);
+    zd t = cs_scale(zmul(ph, s), min(e, 1024));
     if (e >= 1024 || bad) t.x = t.y = __longlong_as_double(0x7ff8000000000000ll);
     return t;
 }
@@ -261,9 +258,8 @@ __device__ __forceinline__ CsPulse cs_pulse(const StepArgs& a, const KDev& K, bo
     p.diag = aa - K.lam[0];
     return p;
 }
-// the stored column i, entry j, of H~ cut into (re hi, re lo, im hi, im lo); it is
-// the conjugate of row i (HH is Hermitian)
-__device__ __forceinline__ int4 cs_hentry(const StepArgs& a, const KDev& K, const CsPulse& p, int i, int j, bool& bad) {
+// the stored column i, entry j, of H~; it is the conjugate of row i (HH is Hermitian)
+__device__ __forceinline__ zd cs_hentry(const StepArgs& a, const KDev& K, const CsPulse& p, int i, int j) {
     const int n = a.naux;
     const size_t nn = (size_t)n * n, e = (size_t)i * n + j;
     zd v = zmk(0.0, 0.0);
@@ -276,12 +272,23 @@ __device__ __forceinline__ int4 cs_hentry(const StepArgs& a, const KDev& K, cons
             v.y = fma(q.y, p.al[l], v.y);
         }
     if (i == j) v.x += (K.eps[i] + p.diag) * p.ilh;
-    const int hx = __double2hiint(v.x) & 0x7fffffff, hy = __double2hiint(v.y) & 0x7fffffff;
-    bad |= hx >= 0x7ff00000 || hy >= 0x7ff00000;
-    // |H~_ij| <= 1; a step beyond its bounds (reported by its flag) stays in range
-    const int2 r = cs_split(hx >= 0x40000000 ? 1ll << 58 : cs_fix(v.x, 0, 58));
-    const int2 m = cs_split(hy >= 0x40000000 ? 1ll << 58 : cs_fix(v.y, 0, 58));
+    return v;
+}
+// the power of two above the 2-norm of a row of n entries whose parts' largest high word is hw
+__device__ __forceinline__ int cs_rowexp(int hw, int n) {
+    int h = 1;
+    while ((1 << (2 * h)) < 2 * n) ++h;  // 2^h >= sqrt(2 n)
+    return max((hw >> 20) - 1022 + h, -900);
+}
+// an entry cut at 2^-59 of 2^e: (re hi, re lo, im hi, im lo)
+__device__ __forceinline__ int4 cs_hcut(zd v, int e) {
+    const int2 r = cs_split(fix64(v.x, e, 59)), m = cs_split(fix64(v.y, e, 59));
     return make_int4(r.x, r.y, m.x, m.y);
+}
+#define CS_WEXP 60  // the products of a row are in units of 2^(e - 60) and the column's scale
+// v 2^s rounded to an integer
+__device__ __forceinline__ i64 cs_shift(i64 v, int s) {
+    return s >= 0 ? v << min(s, 8) : (s < -62 ? 0 : (v + (1ll << (-s - 1))) >> -s);
 }
 
 // NT columns (N_s <= NT), JU entries of the row per thread.  The thread's entries of
@@ -290,13 +297,14 @@ __device__ __forceinline__ int4 cs_hentry(const StepArgs& a, const KDev& K, cons
 // also keeps y_0 .. y_(N - 2) in hist ([k][N][N_s][N_aux]), MODE 2 runs the reversed
 // recurrence from vec (see k_adjoint.cu), keeps every ybar_n and leaves ybar_0 in vec.
 template <int NT, int JU, int MODE>
-__global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepArgs a, ChebSync* sy, zd* hist, zd* vec) {
+__global__ void __launch_bounds__(CS_THREADS, (JU == 2 ? 4 : 3) + (NT == 2 ? 1 : 0)) k_cheb_coop(StepArgs a, ChebSync* sy, zd* hist, zd* vec) {
     constexpr int CW = NT < 4 ? NT : 4;  // columns at a time (registers)
     constexpr int V = 2 * NT;
     extern __shared__ int4 ysm[];  // [N_s][N_aux]
     __shared__ i64 red[CS_THREADS / 32][V];
-    __shared__ i64 cf[CS_MAXC][2];
-    __shared__ int smx[CS_THREADS / 32][NT];
+    __shared__ i64 sti[2][NT][2];  // what a term's products are added to, units 2^-57 (even and odd terms)
+    __shared__ int smx[CS_THREADS / 32][NT + 1];
+    __shared__ double sdg;
     __shared__ float snm[CS_THREADS / 32][NT];
     __shared__ int smg;
     const int n = a.naux, ns = a.ns;
@@ -305,7 +313,8 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
     const int k = blockIdx.x / n, i = blockIdx.x % n;
     const KDev& K = a.kd[k];
     const zd* th = MODE == 2 ? vec + (size_t)k * vs : K.theta;
-    int2 hr[JU], hi[JU];
+    zd hv[JU];
+    int hm = 0;  // largest high word of the row's entries off the diagonal
     {
         // row i of HH(t_k) (Eq. auxiliary_hamiltonian_with_parts)
         const CsPulse pu = cs_pulse(a, K, blockIdx.x == 0 && tid == 0);
@@ -313,27 +322,31 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
 #pragma unroll
         for (int u = 0; u < JU; ++u) {
             const int j = tid + u * CS_THREADS;
-            const int4 h = j < n ? cs_hentry(a, K, pu, i, j, bad) : make_int4(0, 0, 0, 0);
-            hr[u] = make_int2(h.x, h.y);
-            hi[u] = make_int2(h.z, h.w);
+            hv[u] = j < n ? cs_hentry(a, K, pu, i, j) : zmk(0.0, 0.0);
+            const int hx = __double2hiint(hv[u].x) & 0x7fffffff, hy = __double2hiint(hv[u].y) & 0x7fffffff;
+            bad |= hx >= 0x7ff00000 || hy >= 0x7ff00000;
+            if (j == i) {
+                sdg = hv[u].x;  // read after the barriers below
+                hv[u].x = 0.0;
+                hm = max(hm, hy);
+            } else {
+                hm = max(hm, max(hx, hy));
+            }
         }
         if (bad) {
             atomicOr(&sy->bad, 1u);
             __threadfence();
         }
     }
-    auto coef = [&](int t0) {  // c_n, or conj(beta c_(N - 1 - n)) of the reverse sweep, in units 2^-62
-        for (int t = tid; t < min(a.nterms - t0, CS_MAXC); t += CS_THREADS) {
-            zd c = K.coef[MODE == 2 ? a.nterms - 1 - t0 - t : t0 + t];
-            if (MODE == 2) {
-                if (a.prop == 0) c = zmul(zmk(K.lam[3], K.lam[4]), c);
-                c.y = -c.y;
-            }
-            cf[t][0] = __double2ll_rn(c.x * 4611686018427387904.0);
-            cf[t][1] = __double2ll_rn(c.y * 4611686018427387904.0);
+    auto coef = [&](int t) {  // c_n, or conj(beta c_(N - 1 - n)) of the reverse sweep
+        zd c = K.coef[MODE == 2 ? a.nterms - 1 - t : t];
+        if (MODE == 2) {
+            if (a.prop == 0) c = zmul(zmk(K.lam[3], K.lam[4]), c);
+            c.y = -c.y;
         }
+        return c;
     };
-    coef(0);
+    const zd c0 = coef(0);
     int margin = 0;
     if (MODE == 2) {
         // |ybar_n| <= sum_m (m + 1) |c_m| |o|: the power of two above the sum widens the scale
@@ -367,6 +380,8 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
             mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
             if (lane == 0) smx[warp][c] = mx[c];
         }
+        hm = __reduce_max_sync(0xffffffffu, hm);
+        if (lane == 0) smx[warp][NT] = hm;
         __syncthreads();
         float q[NT];
 #pragma unroll
@@ -403,39 +418,79 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
             if (e[c] < 1024) e[c] += ((__float_as_int(sqrtf(t) * 1.00001f) >> 23) & 255) - 126 + margin;
         }
     }
-    // the block's own entries of the recurrence: thread c of the first warp
-    const int oc = tid;
-    const bool own = tid < NT && oc < ns;
+    hm = 0;
+#pragma unroll
+    for (int w = 0; w < CS_THREADS / 32; ++w) hm = max(hm, smx[w][NT]);
+    const int eh = cs_rowexp(hm, n);
+    int2 hr[JU], hi[JU];
+#pragma unroll
+    for (int u = 0; u < JU; ++u) {
+        const int4 h = cs_hcut(hv[u], eh);
+        hr[u] = make_int2(h.x, h.y);
+        hi[u] = make_int2(h.z, h.w);
+        // as 32-bit values and no more: seen as parts of a 64-bit one, their products below
+        // became 64-bit multiplications (86 against 75 us a series of N_aux 240, N_s 7)
+        asm volatile("" : "+r"(hr[u].x), "+r"(hr[u].y), "+r"(hi[u].x), "+r"(hi[u].y));
+    }
+    // The block's own entries of the recurrence, a lane per column: FP64 in units of the
+    // column's scale in the second warp, while the first one sends y_n out and polls.  It
+    // leaves, for the next term, what that term's products are added to (H~'s diagonal
+    // among it) as integers, so that y_n goes out as a sum of integers, rounded twice at
+    // 2^-57, and no FP64 instruction lies on the way from one term to the next.
+    const bool own = warp == 1 && lane < NT && lane < ns;
     int eo = 0;
 #pragma unroll
     for (int c = 0; c < NT; ++c)
-        if (oc == c) eo = e[c];
-    const size_t oe = i + (size_t)oc * n;
-    i64 y1r = 0, y1i = 0, y2r = 0, y2i = 0, sr = 0, si = 0;
-    i64 orr = 0, oi = 0;  // the source's entry (reverse sweep)
+        if (lane == c) eo = e[c];
+    const size_t oe = i + (size_t)lane * n;
+    const double hd1 = sdg, hd2 = 2.0 * hd1, hp1 = cs_pow2(eh - CS_WEXP), hp2 = 2.0 * hp1;
+    // y_n, the term after it but for its products, the sum; src: the source's entry (reverse sweep)
+    zd y1 = zmk(0.0, 0.0), t = y1, sum = y1, src = y1;
     if (own && eo < 1024) {
-        const zd t = th[oe];
-        y1r = cs_fix(t.x, eo, 59);
-        y1i = cs_fix(t.y, eo, 59);
-        sr = cs_mul62(cf[0][0], y1r) - cs_mul62(cf[0][1], y1i);
-        si = cs_mul62(cf[0][0], y1i) + cs_mul62(cf[0][1], y1r);
+        y1 = cs_scale(th[oe], -eo);
+        sum = zmul(c0, y1);
         if (MODE == 2) {
-            orr = y1r;
-            oi = y1i;
-            y1r = sr;
-            y1i = si;
+            src = y1;
+            y1 = sum;
         }
     }
-    // y_n as doubles (the adjoint's history)
-    const int hs = min(eo, 1024) - 59;
-    const double hp1 = cs_pow2(hs / 2), hp2 = cs_pow2(hs - hs / 2);
-    auto keep = [&](int t, i64 yr, i64 yi) {
-        zd v = zmk(((double)yr * hp1) * hp2, ((double)yi * hp1) * hp2);
+    // ybar_m = conj(beta c_m) o + 2 H~ ybar_(m + 1) - ybar_(m + 2), once H~ for m = 0 (MODE 2)
+    auto once = [&](int nt) { return MODE == 2 ? nt == a.nterms - 1 : nt == 1; };
+    auto ahead = [&](int nt) {
+        if (MODE == 2) zfma(t, coef(nt), src);
+        sti[nt & 1][lane][0] = fix64(t.x, 3, 60);
+        sti[nt & 1][lane][1] = fix64(t.y, 3, 60);
+    };
+    if (own) {
+        const double h = once(1) ? hd1 : hd2;
+        t = zmk(h * y1.x, h * y1.y);
+        ahead(1);
+    }
+    // y_n as the adjoint's history takes it
+    auto keep = [&](int t, zd y) {
+        zd v = cs_scale(y, min(eo, 1024));
         if (eo >= 1024 || *(volatile unsigned*)&sy->bad != 0u) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
         hist[((size_t)k * a.nterms + t) * vs + oe] = v;
         return v;
     };
-    if (MODE != 0 && own) keep(MODE == 1 ? 0 : a.nterms - 1, y1r, y1i);
+    if (MODE != 0 && own) keep(MODE == 1 ? 0 : a.nterms - 1, y1);
+    // the thread's entries of y_0
+#pragma unroll 1
+    for (int j = tid; j < n; j += CS_THREADS) {
+#pragma unroll
+        for (int c = 0; c < NT; ++c) {
+            if (c >= ns) continue;
+            const zd v = e[c] < 1024 ? th[j + (size_t)c * n] : zmk(0.0, 0.0);
+            int2 p = cs_split(fix64(v.x, e[c], 57)), r = cs_split(fix64(v.y, e[c], 57));
+            if (MODE == 2) {
+                const i64 x = fix64(v.x, e[c], 59), y = fix64(v.y, e[c], 59);
+                const i64 cr = fix64(c0.x, 0, 62), ci = fix64(c0.y, 0, 62);
+                p = cs_split((cs_mul62(cr, x) - cs_mul62(ci, y) + 2) >> 2);
+                r = cs_split((cs_mul62(cr, y) + cs_mul62(ci, x) + 2) >> 2);
+            }
+            ysm[j + (size_t)c * n] = make_int4(p.x, p.y, r.x, r.y);
+        }
+    }
     unsigned mycnt = 0;  // blocks that arrive at the counter this lane polls
     if (lane < CS_CNT) mycnt = (gridDim.x - lane + CS_CNT - 1) / CS_CNT;
     int4* ring = (int4*)K.ring;
@@ -443,35 +498,18 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
     for (int nt = 1; nt < a.nterms; ++nt) {
         const bool last = nt == a.nterms - 1;
         const int4* yin = ring + ((nt - 1) & 1) * vs;
-        if (nt >= CS_MAXC && nt % CS_MAXC == 0) {
-            __syncthreads();
-            coef(nt);
-            __syncthreads();
-        }
+        zd cn = zmk(0.0, 0.0);
+        if (MODE != 2 && own) cn = coef(nt);
 #pragma unroll
         for (int u = 0; u < JU; ++u) {
             const int j = tid + u * CS_THREADS;
 #pragma unroll
             for (int c = 0; c < NT; ++c) {
-                if (j >= n || c >= ns) continue;
-                int4* d = ysm + j + (size_t)c * n;
-                if (nt > 1) {
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(d)),
-                                 "l"(yin + j + (size_t)c * n)
-                                 : "memory");
-                } else {
-                    *d = make_int4(0, 0, 0, 0);
-                    if (e[c] < 1024) {
-                        const zd t = th[j + (size_t)c * n];
-                        int2 p = cs_split(cs_fix(t.x, e[c], 57)), r = cs_split(cs_fix(t.y, e[c], 57));
-                        if (MODE == 2) {
-                            const i64 x = cs_fix(t.x, e[c], 59), y = cs_fix(t.y, e[c], 59);
-                            p = cs_split((cs_mul62(cf[0][0], x) - cs_mul62(cf[0][1], y) + 2) >> 2);
-                            r = cs_split((cs_mul62(cf[0][0], y) + cs_mul62(cf[0][1], x) + 2) >> 2);
-                        }
-                        *d = make_int4(p.x, p.y, r.x, r.y);
-                    }
-                }
+                if (j >= n || c >= ns || nt == 1) continue;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                 (unsigned)__cvta_generic_to_shared(ysm + j + (size_t)c * n)),
+                             "l"(yin + j + (size_t)c * n)
+                             : "memory");
             }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
@@ -489,58 +527,33 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
                     if (h + q < ns) cs_mac(A + 2 * q, B + 2 * q, hr[u], hi[u], ysm[j + (size_t)(h + q) * n]);
             }
 #pragma unroll
-            for (int v = 0; v < 2 * CW; ++v) A[v] += (B[v] + (1ll << 27)) >> 28;  // units 2^-59
+            for (int v = 0; v < 2 * CW; ++v) A[v] += (B[v] + (1ll << 27)) >> 28;  // units 2^-CS_WEXP
             warp_sum_store<i64, 2 * CW>(A, lane, &red[warp][2 * h]);
         }
         __syncthreads();
-        if (warp == 0) {
-            i64 yr = 0, yi = 0;
-            if (own) {
-                yr = red[0][2 * tid];
-                yi = red[0][2 * tid + 1];
+        if (warp < 2) {
+            i64 wr = 0, wi = 0;
+            if (lane < NT && lane < ns) {
+                wr = red[0][2 * lane];
+                wi = red[0][2 * lane + 1];
 #pragma unroll
                 for (int w = 1; w < CS_THREADS / 32; ++w) {
-                    yr += red[w][2 * tid];
-                    yi += red[w][2 * tid + 1];
+                    wr += red[w][2 * lane];
+                    wi += red[w][2 * lane + 1];
                 }
-                const i64 cr = cf[nt % CS_MAXC][0], ci = cf[nt % CS_MAXC][1];
-                if (MODE == 2) {
-                    // ybar_m = conj(beta c_m) o + 2 H~ ybar_(m + 1) - ybar_(m + 2), once H~ for m = 0
-                    yr = (last ? yr : 2 * yr) - y2r + cs_mul62(cr, orr) - cs_mul62(ci, oi);
-                    yi = (last ? yi : 2 * yi) - y2i + cs_mul62(cr, oi) + cs_mul62(ci, orr);
-                } else if (nt > 1) {
-                    yr = 2 * yr - y2r;
-                    yi = 2 * yi - y2i;
-                }
-                y2r = y1r;
-                y2i = y1i;
-                y1r = yr;
-                y1i = yi;
-                if (!last) {
-                    const int2 p = cs_split((yr + 2) >> 2), q = cs_split((yi + 2) >> 2);
+                if (warp == 0 && !last) {
+                    const int s = eh + 57 - CS_WEXP + (once(nt) ? 0 : 1);
+                    const int2 p = cs_split(sti[nt & 1][lane][0] + cs_shift(wr, s));
+                    const int2 q = cs_split(sti[nt & 1][lane][1] + cs_shift(wi, s));
                     __stcg(ring + (nt & 1) * vs + oe, make_int4(p.x, p.y, q.x, q.y));
                 }
             }
-            if (!last) {
+            if (warp == 0 && !last) {
                 // release: the warp's stores become visible to every block that acquires the count
                 __syncwarp();
                 if (lane == 0)
                     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&sy->cnt[blockIdx.x % CS_CNT][0]), "r"(1u)
                                  : "memory");
-            }
-            if (own) {
-                if (MODE != 2) {
-                    const i64 cr = cf[nt % CS_MAXC][0], ci = cf[nt % CS_MAXC][1];
-                    sr += cs_mul62(cr, yr) - cs_mul62(ci, yi);
-                    si += cs_mul62(cr, yi) + cs_mul62(ci, yr);
-                }
-                if (MODE == 1 && !last) keep(nt, y1r, y1i);
-                if (MODE == 2) {
-                    const zd v = keep(a.nterms - 1 - nt, y1r, y1i);
-                    if (last) vec[(size_t)k * vs + oe] = v;  // theta-bar
-                }
-            }
-            if (!last) {
                 const unsigned want = mycnt * (unsigned)nt;
                 bool there = lane >= CS_CNT;
                 unsigned it = 0;
@@ -553,6 +566,19 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
                     }
                 }
             }
+            if (own) {
+                const double g = once(nt) ? hp1 : hp2, h = once(nt + 1) ? hd1 : hd2;
+                const zd y = zmk(fma((double)wr, g, t.x), fma((double)wi, g, t.y));
+                t = zmk(fma(h, y.x, -y1.x), fma(h, y.y, -y1.y));
+                y1 = y;
+                if (!last) ahead(nt + 1);
+                if (MODE != 2) zfma(sum, cn, y1);
+                if (MODE == 1 && !last) keep(nt, y1);
+                if (MODE == 2) {
+                    const zd v = keep(a.nterms - 1 - nt, y1);
+                    if (last) vec[(size_t)k * vs + oe] = v;  // theta-bar
+                }
+            }
         }
         if (!last) {
             ok = !__syncthreads_or(!ok);
@@ -562,7 +588,7 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
     if (!ok && tid == 0) atomicOr(a.flag, 4);
     // (every block read theta before it wrote its y_1, so theta may be written now)
     if (MODE != 2 && ok && own) {
-        K.theta[oe] = cs_result(a, K, sr, si, eo, *(volatile unsigned*)&sy->bad != 0u);
+        K.theta[oe] = cs_result(a, K, sum, eo, *(volatile unsigned*)&sy->bad != 0u);
     }
     __syncthreads();
     if (tid == 0) {
@@ -587,14 +613,45 @@ __global__ void __launch_bounds__(CS_THREADS, JU == 2 ? 4 : 3) k_cheb_coop(StepA
 #define CL_N 16
 #define CL_MAXN 256
 #define CL_THREADS 512
-__global__ void __launch_bounds__(128) k_cs_rows(StepArgs a, int* rowbad) {
+struct CsRow {
+    double diag;  // of H~
+    int e;        // the row's exponent (cs_rowexp)
+    int bad;      // not finite
+};
+__global__ void __launch_bounds__(128) k_cs_rows(StepArgs a, CsRow* rows) {
+    __shared__ double sdg;
+    __shared__ int smx[4];
     const int k = blockIdx.y, i = blockIdx.x, n = a.naux;
     const KDev& K = a.kd[k];
     const CsPulse pu = cs_pulse(a, K, i == 0 && k == 0 && threadIdx.x == 0);
+    zd v[CL_MAXN / 128];
+    int hm = 0;
     bool bad = false;
-    for (int j = threadIdx.x; j < n; j += 128) ((int4*)K.hsub)[(size_t)i * n + j] = cs_hentry(a, K, pu, i, j, bad);
+#pragma unroll
+    for (int u = 0; u < CL_MAXN / 128; ++u) {
+        const int j = threadIdx.x + u * 128;
+        v[u] = j < n ? cs_hentry(a, K, pu, i, j) : zmk(0.0, 0.0);
+        const int hx = __double2hiint(v[u].x) & 0x7fffffff, hy = __double2hiint(v[u].y) & 0x7fffffff;
+        bad |= hx >= 0x7ff00000 || hy >= 0x7ff00000;
+        if (j == i) {
+            sdg = v[u].x;
+            v[u].x = 0.0;
+            hm = max(hm, hy);
+        } else {
+            hm = max(hm, max(hx, hy));
+        }
+    }
+    hm = __reduce_max_sync(0xffffffffu, hm);
+    if ((threadIdx.x & 31) == 0) smx[threadIdx.x >> 5] = hm;
     const int any = __syncthreads_or(bad);
-    if (threadIdx.x == 0) rowbad[(size_t)k * n + i] = any;
+    hm = max(max(smx[0], smx[1]), max(smx[2], smx[3]));
+    const int e = cs_rowexp(hm, n);
+#pragma unroll
+    for (int u = 0; u < CL_MAXN / 128; ++u) {
+        const int j = threadIdx.x + u * 128;
+        if (j < n) ((int4*)K.hsub)[(size_t)i * n + j] = cs_hcut(v[u], e);
+    }
+    if (threadIdx.x == 0) rows[(size_t)k * n + i] = CsRow{sdg, e, any};
 }
 __device__ __forceinline__ bool cl_wait(uint64_t* b, unsigned parity) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(b);
@@ -611,7 +668,7 @@ __device__ __forceinline__ bool cl_wait(uint64_t* b, unsigned parity) {
     }
 }
 template <int NT>
-__global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int* rowbad) {
+__global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const CsRow* rows) {
     constexpr int CW = NT < 4 ? NT : 4, JU = CL_MAXN / 32;
     extern __shared__ int4 csm[];  // [2][N_s][N_aux] y, then the coefficients
     __shared__ __align__(8) uint64_t bar[2];
@@ -625,7 +682,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int
     const int i = warp * CL_N + rank;
     const bool act = i < n;
     const size_t vs = (size_t)n * ns;
-    i64* cf = (i64*)(csm + 2 * vs);
+    double* cf = (double*)(csm + 2 * vs);
     const unsigned bytes = (unsigned)(vs * sizeof(int4));
     if (tid == 0) {
         for (int q = 0; q < 2; ++q) {
@@ -644,8 +701,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int
         hi[u] = make_int2(h.z, h.w);
     }
     for (int t = tid; t < a.nterms; t += CL_THREADS) {
-        cf[2 * t] = __double2ll_rn(K.coef[t].x * 4611686018427387904.0);
-        cf[2 * t + 1] = __double2ll_rn(K.coef[t].y * 4611686018427387904.0);
+        cf[2 * t] = K.coef[t].x;
+        cf[2 * t + 1] = K.coef[t].y;
     }
     if (warp < ns) {  // a warp per column: the power of two above its 2-norm
         const zd* th = K.theta + (size_t)warp * n;
@@ -663,28 +720,27 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int
         if (lane == 0) es[warp] = e;
     }
     bool bad = false;
-    for (int j = tid; j < n; j += CL_THREADS) bad |= rowbad[(size_t)k * n + j] != 0;
+    for (int j = tid; j < n; j += CL_THREADS) bad |= rows[(size_t)k * n + j].bad != 0;
     bad = __syncthreads_or(bad);
     for (int t = tid; t < (int)vs; t += CL_THREADS) {
         const int c = t / n, e = es[c];
         const zd v = K.theta[t];
         int2 p = make_int2(0, 0), q = make_int2(0, 0);
         if (e < 1024) {
-            p = cs_split(cs_fix(v.x, e, 57));
-            q = cs_split(cs_fix(v.y, e, 57));
+            p = cs_split(fix64(v.x, e, 57));
+            q = cs_split(fix64(v.y, e, 57));
         }
         csm[t] = make_int4(p.x, p.y, q.x, q.y);
     }
     const bool own = act && lane < ns;
     const int eo = lane < ns ? es[lane] : 0;
     const size_t oe = i + (size_t)lane * n;
-    i64 y1r = 0, y1i = 0, y2r = 0, y2i = 0, sr = 0, si = 0;
+    const CsRow row = act ? rows[(size_t)k * n + i] : CsRow{0.0, 0, 0};
+    const double hd1 = row.diag, hd2 = 2.0 * hd1, hp1 = cs_pow2(row.e - CS_WEXP), hp2 = 2.0 * hp1;
+    zd y1 = zmk(0.0, 0.0), y2 = y1, sum = y1;
     if (own && eo < 1024) {
-        const zd t = K.theta[oe];
-        y1r = cs_fix(t.x, eo, 59);
-        y1i = cs_fix(t.y, eo, 59);
-        sr = cs_mul62(cf[0], y1r) - cs_mul62(cf[1], y1i);
-        si = cs_mul62(cf[0], y1i) + cs_mul62(cf[1], y1r);
+        y1 = cs_scale(K.theta[oe], -eo);
+        sum = zmul(zmk(cf[0], cf[1]), y1);
     }
     // every block's mbarriers stand before anything is sent
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -694,6 +750,10 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int
         for (int nt = 1; nt < a.nterms; ++nt) {
             const bool last = nt == a.nterms - 1;
             const int4* y = csm + ((nt - 1) & 1) * vs;
+            // as in the grid form: the diagonal's part while y_(n-1) comes in, y_n out as integers
+            const double g = nt == 1 ? hd1 : hd2, gp = nt == 1 ? hp1 : hp2;
+            const zd t = zmk(fma(g, y1.x, -y2.x), fma(g, y1.y, -y2.y));
+            const i64 tr = fix64(t.x, 3, 60), ti = fix64(t.y, 3, 60);
             if (nt > 1) {
                 const int m = nt - 1;  // y_m
                 if (!cl_wait(&bar[m & 1], (unsigned)((m - 1) >> 1 & 1))) {
@@ -721,23 +781,16 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int
                         if (h + q < ns) cs_mac(A + 2 * q, B + 2 * q, hr[u], hi[u], y[j + (size_t)(h + q) * n]);
                 }
 #pragma unroll
-                for (int v = 0; v < 2 * CW; ++v) A[v] += (B[v] + (1ll << 27)) >> 28;  // units 2^-59
+                for (int v = 0; v < 2 * CW; ++v) A[v] += (B[v] + (1ll << 27)) >> 28;  // units 2^-CS_WEXP
                 warp_sum_store<i64, 2 * CW>(A, lane, &red[warp][2 * h]);
             }
             __syncwarp();
-            i64 yr = 0, yi = 0;
+            i64 wr = 0, wi = 0;
             if (own) {
-                yr = red[warp][2 * lane];
-                yi = red[warp][2 * lane + 1];
-                if (nt > 1) {
-                    yr = 2 * yr - y2r;
-                    yi = 2 * yi - y2i;
-                }
-                y2r = y1r;
-                y2i = y1i;
-                y1r = yr;
-                y1i = yi;
-                const int2 p = cs_split((yr + 2) >> 2), q = cs_split((yi + 2) >> 2);
+                wr = red[warp][2 * lane];
+                wi = red[warp][2 * lane + 1];
+                const int s = row.e + 57 - CS_WEXP + (nt > 1 ? 1 : 0);
+                const int2 p = cs_split(tr + cs_shift(wr, s)), q = cs_split(ti + cs_shift(wi, s));
                 snd[warp][lane] = make_int4(p.x, p.y, q.x, q.y);
             }
             __syncwarp();
@@ -755,14 +808,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1) k_cheb_cl(StepArgs a, const int
                                  : "memory");
                 }
             }
-            if (own) {
-                const i64 cr = cf[2 * nt], ci = cf[2 * nt + 1];
-                sr += cs_mul62(cr, yr) - cs_mul62(ci, yi);
-                si += cs_mul62(cr, yi) + cs_mul62(ci, yr);
-            }
+            y2 = y1;
+            y1 = zmk(fma((double)wr, gp, t.x), fma((double)wi, gp, t.y));
+            zfma(sum, zmk(cf[2 * nt], cf[2 * nt + 1]), y1);
         }
         if (!ok && lane == 0) atomicOr(a.flag, 4);
-        if (ok && own) K.theta[oe] = cs_result(a, K, sr, si, eo, bad);
+        if (ok && own) K.theta[oe] = cs_result(a, K, sum, eo, bad);
     }
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -2269,22 +2320,22 @@ static cudaError_t launch_cheb_coop_raw(const StepArgs& a, cudaStream_t s) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     StepArgs arg = a;
-    int* rowbad = (int*)a.cheb_sync;
-    k_cs_rows<<<dim3(a.naux, a.nk), 128, 0, s>>>(a, rowbad);
+    CsRow* rows = (CsRow*)a.cheb_sync;
+    k_cs_rows<<<dim3(a.naux, a.nk), 128, 0, s>>>(a, rows);
     cfg.gridDim = dim3(CL_N * a.nk);
     cfg.blockDim = dim3(CL_THREADS);
     cfg.dynamicSmemBytes = cheb_cl_smem(a, a.nterms);
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = CL_N;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    void* args[2] = {&arg, &rowbad};
+    void* args[2] = {&arg, &rows};
     return cudaLaunchKernelExC(&cfg, cheb_cl_fn(a), args);
 }
 int launch_cheb_coop(const StepArgs& a, cudaStream_t s) {
     launch_cheb_coop_raw(a, s);
     return a.cheb_cl ? 2 : 1;
 }
-size_t cheb_sync_bytes(int nk, int naux) { return std::max(sizeof(ChebSync), (size_t)nk * naux * sizeof(int)); }
+size_t cheb_sync_bytes(int nk, int naux) { return std::max(sizeof(ChebSync), (size_t)nk * naux * sizeof(CsRow)); }
 
 static cudaError_t grow_smem(const void* f, size_t bytes) {  // the attribute is shared by every context: never lowered
     cudaFuncAttributes fa{};
