@@ -2447,7 +2447,7 @@ int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const
             gpart = (double*)take((size_t)K * ng * sizeof(double));
             nrm = (double*)take((size_t)K * nn * sizeof(double));
             jdev = (double*)take(3 * (size_t)nsteps * sizeof(double));
-            sync = take(adj_sync_bytes());
+            sync = take(adj_sync_bytes(nk));
             if (pass) break;
             if (off > ctx->adj_cap) {
                 dfree(ctx, ctx->adj_ws);
@@ -2458,7 +2458,7 @@ int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const
             }
             ws = ctx->adj_ws;
         }
-        CK(cudaMemsetAsync(sync, 0, adj_sync_bytes(), st));
+        CK(cudaMemsetAsync(sync, 0, adj_sync_bytes(nk), st));
         for (int k = 0; k < nk; ++k) {
             theta_saved.push_back(th0 + (size_t)k * vs);
             CK(cudaMemcpyAsync(theta_saved[k], ctx->hkd[k].theta, vs * sizeof(zd), cudaMemcpyDeviceToDevice, st));

@@ -177,9 +177,10 @@ __global__ void __launch_bounds__(128) k_cheb(StepArgs a, int nt, int last) {
 struct ChebSync {
     unsigned cnt[CS_CNT][32];
     unsigned left;
-    unsigned bad;  // HH of some k-point is not finite (a NaN or infinite pulse or change)
-    unsigned pad[30];
+    unsigned pad[31];
 };
+// after it, per k-point: HH is not finite (a NaN or infinite pulse or change)
+__host__ __device__ __forceinline__ unsigned* cs_bad(ChebSync* sy) { return (unsigned*)(sy + 1); }
 typedef long long i64;
 __device__ __forceinline__ int2 cs_split(i64 q) {  // q = hi 2^28 + lo
     const int lo = (int)(q << 36 >> 36);
@@ -312,6 +313,7 @@ __global__ void __launch_bounds__(CS_THREADS, (JU == 2 ? 4 : 3) + (NT == 2 ? 1 :
     const size_t vs = (size_t)n * ns;
     const int k = blockIdx.x / n, i = blockIdx.x % n;
     const KDev& K = a.kd[k];
+    unsigned* bad_k = cs_bad(sy) + k;
     const zd* th = MODE == 2 ? vec + (size_t)k * vs : K.theta;
     zd hv[JU];
     int hm = 0;  // largest high word of the row's entries off the diagonal
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(CS_THREADS, (JU == 2 ? 4 : 3) + (NT == 2 ? 1 :
             }
         }
         if (bad) {
-            atomicOr(&sy->bad, 1u);
+            atomicOr(bad_k, 1u);
             __threadfence();
         }
     }
@@ -469,7 +471,7 @@ __global__ void __launch_bounds__(CS_THREADS, (JU == 2 ? 4 : 3) + (NT == 2 ? 1 :
     // y_n as the adjoint's history takes it
     auto keep = [&](int t, zd y) {
         zd v = cs_scale(y, min(eo, 1024));
-        if (eo >= 1024 || *(volatile unsigned*)&sy->bad != 0u) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+        if (eo >= 1024 || *(volatile unsigned*)bad_k != 0u) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
         hist[((size_t)k * a.nterms + t) * vs + oe] = v;
         return v;
     };
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(CS_THREADS, (JU == 2 ? 4 : 3) + (NT == 2 ? 1 :
     if (!ok && tid == 0) atomicOr(a.flag, 4);
     // (every block read theta before it wrote its y_1, so theta may be written now)
     if (MODE != 2 && ok && own) {
-        K.theta[oe] = cs_result(a, K, sum, eo, *(volatile unsigned*)&sy->bad != 0u);
+        K.theta[oe] = cs_result(a, K, sum, eo, *(volatile unsigned*)bad_k != 0u);
     }
     __syncthreads();
     if (tid == 0) {
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(CS_THREADS, (JU == 2 ? 4 : 3) + (NT == 2 ? 1 :
         if (atomicAdd(&sy->left, 1u) == gridDim.x - 1) {
             // every block has read what it needs
             for (int c = 0; c < CS_CNT; ++c) sy->cnt[c][0] = 0u;
-            sy->bad = 0u;
+            for (int q = 0; q < a.nk; ++q) cs_bad(sy)[q] = 0u;
             sy->left = 0u;
         }
     }
@@ -2335,7 +2337,8 @@ int launch_cheb_coop(const StepArgs& a, cudaStream_t s) {
     launch_cheb_coop_raw(a, s);
     return a.cheb_cl ? 2 : 1;
 }
-size_t cheb_sync_bytes(int nk, int naux) { return std::max(sizeof(ChebSync), (size_t)nk * naux * sizeof(CsRow)); }
+size_t adj_sync_bytes(int nk) { return sizeof(ChebSync) + (size_t)nk * sizeof(unsigned); }
+size_t cheb_sync_bytes(int nk, int naux) { return std::max(adj_sync_bytes(nk), (size_t)nk * naux * sizeof(CsRow)); }
 
 static cudaError_t grow_smem(const void* f, size_t bytes) {  // the attribute is shared by every context: never lowered
     cudaFuncAttributes fa{};
@@ -2422,7 +2425,6 @@ bool adj_series_fits(const StepArgs& a) {
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     return coop && grid_fits(cheb_coop_fn<1>(a), a, nsm) && grid_fits(cheb_coop_fn<2>(a), a, nsm);
 }
-size_t adj_sync_bytes() { return sizeof(ChebSync); }
 void launch_adj_series(const StepArgs& a, void* sync, zd* hist, zd* vec, cudaStream_t s) {
     if (vec) launch_cheb_grid<2>(a, sync, hist, vec, s);
     else launch_cheb_grid<1>(a, sync, hist, vec, s);

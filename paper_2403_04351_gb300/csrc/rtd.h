@@ -266,7 +266,7 @@ void launch_scale_cols(zd* const* mats, const double* const* vals, int nbatch, i
 void launch_propagate_only(const StepArgs& a, const StepPlan& p, int cstep, void* sync, zd* hist, cudaStream_t s);
 void launch_hsub_only(const StepArgs& a, const StepPlan& p, int cstep, bool form, cudaStream_t s);
 bool adj_series_fits(const StepArgs& a);
-size_t adj_sync_bytes();
+size_t adj_sync_bytes(int nk);
 void launch_adj_series(const StepArgs& a, void* sync, zd* hist, zd* vec, cudaStream_t s);
 void launch_adj_current(const StepArgs& a, double* out, cudaStream_t s);
 void launch_subspace_j(const StepArgs& a, cudaStream_t s);

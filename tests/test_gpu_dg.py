@@ -6,7 +6,7 @@ import pytest
 import scipy.linalg as sla
 
 from paper_2403_04351_gb300 import Context
-from synth import make_system, tiny_config
+from synth import make_dv, make_system, tiny_config
 
 pytestmark = pytest.mark.gpu
 
@@ -146,4 +146,32 @@ def test_series_of_few_states(n_aux, n_s, n_k, prop):
         assert np.all(got[:, size == 0.0] == 0.0)
         size[size == 0.0] = 1.0
         assert np.max(np.linalg.norm((got - want[k]) / size, axis=0) / np.maximum(np.linalg.norm(want[k] / size, axis=0), 1.0)) < 4e-14
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_aux,n_s", [(130, 3), (33, 4), (60, 12)])
+def test_a_k_point_that_is_not_finite_stays_alone(n_aux, n_s):
+    """A potential change whose norm leaves FP64's range for one k-point only, at scale
+    0: that k-point's interval is not a number, the other's steps are those without
+    the change (the same operator; the rounding of a different interval, 1e-12)."""
+    from oracle import explicit_dv
+    s = make_system(tiny_config(n_g=max(n_aux, 60), n_s=n_s, n_aux=n_aux, n_k=2, kgrid=(2, 1, 1)))
+    a = np.random.default_rng(5).standard_normal((3, 3))
+    plain = Context(s, graph_steps=1)
+    plain.step(a)
+    want = [plain.get_state(k) for k in range(2)]
+    dv = make_dv(s, amp=0.3)
+    norm = []
+    for k in range(2):
+        cc = plain.get_aux(k)[0]
+        norm.append(np.linalg.norm(cc.conj().T @ explicit_dv(s, k, dv) @ cc))
+    plain.close()
+    assert abs(norm[0] / norm[1] - 1.0) > 1e-6
+    big = np.sqrt(np.finfo(float).max / (norm[0] * norm[1]))
+    keep = int(np.argmin(norm))
+    ctx = Context(s, graph_steps=1)
+    ctx.set_dv(dict(dh=[d * big for d in dv["dh"]], dvtab=dv["dvtab"] * big))
+    ctx.step(a, np.zeros(3))
+    assert np.linalg.norm(ctx.get_state(keep) - want[keep]) < 1e-12 * np.sqrt(n_s)
+    assert np.all(np.isnan(ctx.get_state(1 - keep)))
     ctx.close()
