@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                     abort_flag = 1;
                     if (lane == 0) atomicOr(g.flag, 8);
                 }
-                if (abort_flag) {
+                if (__any_sync(0xffffffffu, abort_flag)) {  // the warp's lanes leave together
                     ok = false;
                     break;
                 }
@@ -433,7 +433,8 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
 #pragma unroll
             for (int gi = DG_G - 1; gi >= 0; --gi) {
                 if (sl != nsl - 1 && (sl & (dg_run(gi) - 1)) != dg_run(gi) - 1) continue;
-                if (!mbar_wait(&gfull[gi], (uint32_t)((sl / dg_run(gi)) & 1)) || abort_flag) {
+                // the warp's lanes leave together: the loads below take all of them
+                if (__any_sync(0xffffffffu, !mbar_wait(&gfull[gi], (uint32_t)((sl / dg_run(gi)) & 1)) || abort_flag)) {
                     ok = false;
                     break;
                 }
