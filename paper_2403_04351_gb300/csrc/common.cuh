@@ -63,6 +63,16 @@ __device__ __forceinline__ double f2d(float v) {
 __device__ __forceinline__ zf tof(zd a) { return make_float2(d2f(a.x), d2f(a.y)); }
 __device__ __forceinline__ zd tod(zf a) { return zmk(f2d(a.x), f2d(a.y)); }
 
+// The dynamic shared-memory attribute is global per kernel and shared by every
+// context of the process: raise it to `bytes`, never lower it.
+static inline cudaError_t raise_smem(const void* f, int bytes) {
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaFuncGetAttributes(&fa, f);
+    if (e != cudaSuccess) return e;
+    if (fa.maxDynamicSharedSizeBytes >= bytes) return cudaSuccess;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 // x 2^(f - e) rounded to an integer, f <= 62, with integer arithmetic; |x| < 2^e, what
 // lies beyond (and NaN) taken as 2^e at most
 __device__ __forceinline__ long long fix64(double x, int e, int f) {

@@ -1437,15 +1437,15 @@ int fft_plan_create(FftPlan** out, int nk, const int* ng, const int* const* gint
         const int mx = (int)fft_smem(std::max(F1, std::max(F2, F3)), elt);
         const size_t psm = fft_plane_smem(F2, F3, elt);
         if (psm <= FFT_PLANE_SMEM_MAX) {
-            if (pl->fx) cudaFuncSetAttribute(k_fx_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
-            if (prec == 0) cudaFuncSetAttribute(k_fft_plane<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
-            else cudaFuncSetAttribute(k_fft_plane<zf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
+            if (pl->fx) raise_smem((const void*)k_fx_plane, (int)psm);
+            if (prec == 0) raise_smem((const void*)k_fft_plane<zd>, (int)psm);
+            else raise_smem((const void*)k_fft_plane<zf>, (int)psm);
         }
         if (pl->fx) {
-            cudaFuncSetAttribute(k_fx_a, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fx_bd, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fx_c, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fx_e, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+            raise_smem((const void*)k_fx_a, mx);
+            raise_smem((const void*)k_fx_bd, mx);
+            raise_smem((const void*)k_fx_c, mx);
+            raise_smem((const void*)k_fx_e, mx);
             FftArgs f = {};
             f.F1 = F1, f.F2 = F2, f.F3 = F3;
             f.lpb[0] = fft_lpb(F1);
@@ -1453,15 +1453,15 @@ int fft_plan_create(FftPlan** out, int nk, const int* ng, const int* const* gint
             k_fx_v<<<nvb, FFT_THREADS, 0, st>>>(f, pl->vq[0], pl->vqe[0]);
         }
         if (prec == 0) {
-            cudaFuncSetAttribute(k_fft_a<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fft_bd<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fft_c<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fft_e<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+            raise_smem((const void*)k_fft_a<zd>, mx);
+            raise_smem((const void*)k_fft_bd<zd>, mx);
+            raise_smem((const void*)k_fft_c<zd>, mx);
+            raise_smem((const void*)k_fft_e<zd>, mx);
         } else {
-            cudaFuncSetAttribute(k_fft_a<zf>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fft_bd<zf>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fft_c<zf>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-            cudaFuncSetAttribute(k_fft_e<zf>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+            raise_smem((const void*)k_fft_a<zf>, mx);
+            raise_smem((const void*)k_fft_bd<zf>, mx);
+            raise_smem((const void*)k_fft_c<zf>, mx);
+            raise_smem((const void*)k_fft_e<zf>, mx);
         }
         if (cudaGetLastError() != cudaSuccess) {
             ok = false;
@@ -1730,11 +1730,11 @@ int fft_hartree_init(FftPlan* pl, const double recip[9], const int vt_dim[3], do
     pl->bound = bound;
     pl->hartree = 1;
     const int mx = (int)fft_smem(std::max(pl->F[0], std::max(pl->F[1], pl->F[2])), (int)sizeof(zd));
-    cudaFuncSetAttribute(k_fft_density<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(k_fft_full<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(k_fft_a<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(k_fft_bd<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (pl->fused_d) cudaFuncSetAttribute(k_fft_plane<zd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
+    raise_smem((const void*)k_fft_density<zd>, mx);
+    raise_smem((const void*)k_fft_full<zd>, mx);
+    raise_smem((const void*)k_fft_a<zd>, mx);
+    raise_smem((const void*)k_fft_bd<zd>, mx);
+    if (pl->fused_d) raise_smem((const void*)k_fft_plane<zd>, (int)psm);
     if (cudaGetLastError() != cudaSuccess) {
         if (why) *why = "Hartree feedback: set-up failed";
         return RTTDDFT_ERR_CUDA;

@@ -2340,17 +2340,10 @@ int launch_cheb_coop(const StepArgs& a, cudaStream_t s) {
 size_t adj_sync_bytes(int nk) { return sizeof(ChebSync) + (size_t)nk * sizeof(unsigned); }
 size_t cheb_sync_bytes(int nk, int naux) { return std::max(adj_sync_bytes(nk), (size_t)nk * naux * sizeof(CsRow)); }
 
-static cudaError_t grow_smem(const void* f, size_t bytes) {  // the attribute is shared by every context: never lowered
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, f);
-    if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // whether all blocks of the grid form are resident at once
 static bool grid_fits(const void* f, const StepArgs& a, int nsm) {
     int per_sm = 0;
-    cudaError_t e = grow_smem(f, cheb_coop_smem(a));
+    cudaError_t e = raise_smem(f, (int)cheb_coop_smem(a));
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, CS_THREADS, cheb_coop_smem(a));
     if (e != cudaSuccess || (long long)a.nk * a.naux > (long long)per_sm * nsm) {
         cudaGetLastError();
@@ -2388,7 +2381,7 @@ int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s, int* cl) {
         cfg.numAttrs = 1;
         int ncl = 0;
         if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            grow_smem(f, sm) == cudaSuccess && cudaOccupancyMaxActiveClusters(&ncl, f, &cfg) == cudaSuccess && ncl > 0) {
+            raise_smem(f, (int)sm) == cudaSuccess && cudaOccupancyMaxActiveClusters(&ncl, f, &cfg) == cudaSuccess && ncl > 0) {
             *cl = 1;
             return CL_N * a.nk;
         }

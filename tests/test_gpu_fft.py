@@ -262,3 +262,21 @@ def test_split_forms_by_fft_over_200_steps(prec):
     assert rel(obs["j_full"], r["J_full"]) < 1e-3
     assert np.max(obs["norm_dev"]) < 1e-4
     ctx.close()
+
+
+@pytest.mark.parametrize("launches", ["5", "3"])
+def test_a_smaller_grid_leaves_the_larger_one_its_shared_memory(launches, monkeypatch):
+    """The limit of a kernel's dynamic shared memory belongs to the process: a second
+    context's smaller grid does not lower it under the first one's launches."""
+    monkeypatch.setenv("RTTDDFT_FFT_LAUNCHES", launches)
+    large, small = [make_system(tiny_config(n_g=n, n_atoms=1, lmax=1, n_lo_per_atom=1, n_s=2, n_aux=4)) for n in (11000, 5500)]
+    one = Context(large, interstitial="fft")
+    rng = np.random.default_rng(0)
+    nb = int(large["n_g"][0]) + int(np.sum(large["n_lo"]))
+    x = rng.standard_normal((nb, 2)) + 1j * rng.standard_normal((nb, 2))
+    want = one.apply(0, x)[0]
+    two = Context(small, interstitial="fft")
+    assert max(two.info()["fft_grid"]) < max(one.info()["fft_grid"])
+    assert np.array_equal(one.apply(0, x)[0], want)
+    two.close()
+    one.close()
