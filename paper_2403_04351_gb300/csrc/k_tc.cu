@@ -173,7 +173,8 @@ __device__ __forceinline__ void split_bf16(double v, __nv_bfloat16& hi, __nv_bfl
 __global__ void __launch_bounds__(256) k_tc_pack_a(const zd* __restrict__ A, int ld, int R, int K, int Kp, int mode,
                                                    __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
     __shared__ zd t[32][33];
-    const int k0 = blockIdx.y * 32, r0 = blockIdx.x * 32;
+    const unsigned mt = (R + 31) / 32, kt = blockIdx.x / mt;  // one index: a grid's y ends at 65535
+    const int k0 = (int)kt * 32, r0 = (int)(blockIdx.x - kt * mt) * 32;
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
     for (int q = y; q < 32; q += 8) {
         const int r = mode == 0 ? r0 + x : r0 + q, k = mode == 0 ? k0 + q : k0 + x;
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(256) k_tc_pack_a(const zd* __restrict__ A, int
             split_bf16(t[q][x].x, hi[row + k], lo[row + k]);
             split_bf16(t[q][x].y, hi[row + K + k], lo[row + K + k]);
         }
-        if (blockIdx.y == 0)
+        if (kt == 0)
             for (int kp = 2 * K + x; kp < Kp; kp += 32) hi[row + kp] = lo[row + kp] = __float2bfloat16_rn(0.f);
     }
 }
@@ -200,7 +201,8 @@ __global__ void __launch_bounds__(256) k_tc_pack_a(const zd* __restrict__ A, int
 // n' < N: [Re X_n | -Im X_n], N <= n' < 2N: [Im X_n | Re X_n], else 0.
 __global__ void k_tc_pack_b(const zd* __restrict__ X, int ldx, int K, int N, int Kp, int Rp,
                             __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
-    const int kp = blockIdx.y * 256 + threadIdx.x, r = blockIdx.x;
+    const unsigned kt = blockIdx.x / (unsigned)Rp;
+    const int kp = (int)kt * 256 + threadIdx.x, r = (int)(blockIdx.x - kt * Rp);
     if (kp >= Kp) return;
     const size_t e = (size_t)r * Kp + kp;
     double v = 0.0;
@@ -219,7 +221,8 @@ __global__ void k_tc_pack_b(const zd* __restrict__ X, int ldx, int K, int N, int
 __global__ void __launch_bounds__(256) k_tc_combine(const float* __restrict__ D, int splits, int M, int Nc, int Dn,
                                                     zd* __restrict__ C, int ldc, int beta_add) {
     __shared__ zd t[32][33];
-    const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+    const unsigned mt = (M + 31) / 32, nt = blockIdx.x / mt;
+    const int m0 = (int)(blockIdx.x - nt * mt) * 32, n0 = (int)nt * 32;
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
     for (int q = y; q < 32; q += 8) {
         const int m = m0 + q, n = n0 + x;
@@ -355,8 +358,8 @@ int tc_zgemm(int opA, int M, int N, int K, const zd* A, int lda, const zd* X, in
     int* flag = (int*)(ws + 2 * up(na) + 2 * up(nb) + up(nd));
     int rc = RTTDDFT_OK;
     cudaMemsetAsync(flag, 0, sizeof(int), s);
-    k_tc_pack_a<<<dim3((M + 31) / 32, (K + 31) / 32), 256, 0, s>>>(A, lda, M, K, Kp, opA, ah, al);
-    k_tc_pack_b<<<dim3(Rp, (Kp + 255) / 256), 256, 0, s>>>(X, ldx, K, N, Kp, Rp, bh, bl);
+    k_tc_pack_a<<<(unsigned)((M + 31) / 32) * (unsigned)((K + 31) / 32), 256, 0, s>>>(A, lda, M, K, Kp, opA, ah, al);
+    k_tc_pack_b<<<(unsigned)Rp * (unsigned)((Kp + 255) / 256), 256, 0, s>>>(X, ldx, K, N, Kp, Rp, bh, bl);
     CUtensorMap tah, tal, tbh, tbl;
     if (tc_tmap(&tah, ah, Kp, mrows, Kp, TC_BM) || tc_tmap(&tal, al, Kp, mrows, Kp, TC_BM) ||
         tc_tmap(&tbh, bh, Kp, Rp, Kp, NT) || tc_tmap(&tbl, bl, Kp, Rp, Kp, NT)) {
@@ -373,7 +376,7 @@ int tc_zgemm(int opA, int M, int N, int K, const zd* A, int lda, const zd* X, in
             default: lr = -1;
         }
         if (lr) rc = RTTDDFT_ERR_CUDA;
-        else k_tc_combine<<<dim3((M + 31) / 32, (N + 31) / 32), 256, 0, s>>>(D, splits, M, N, Dn, C, ldc, beta_add);
+        else k_tc_combine<<<(unsigned)((M + 31) / 32) * (unsigned)((N + 31) / 32), 256, 0, s>>>(D, splits, M, N, Dn, C, ldc, beta_add);
     }
     int hflag = 0;
     if (cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = RTTDDFT_ERR_CUDA;

@@ -112,3 +112,19 @@ def test_degenerate_sizes_and_bad_arguments():
         R.rttddft_zgemm_bf16x3(0, 4, 2, 1, h, 4, c, 1, c, 4, 0)  # host pointer
     assert e.value.code == -1
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("trans,m,n,k", [(0, 3, 2, 2_200_001), (1, 3, 2, 2_200_001), (0, 2, 2_200_001, 3)])
+def test_sizes_beyond_a_grid_s_second_index(trans, m, n, k):
+    """More than 65535 tiles of 32 along K or N; integers, so the result is exact."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(k + n)
+
+    def ints(rows, cols):  # column-major: a contiguous (cols, rows) tensor; the sums stay below 2^24
+        return torch.complex(*[torch.randint(-1, 2, (cols, rows), generator=g, device="cuda").double() for _ in range(2)])
+
+    a, x = ints(k, m) if trans else ints(m, k), ints(k, n)
+    c = torch.zeros((n, m), dtype=torch.complex128, device="cuda")
+    R.rttddft_zgemm_bf16x3(trans, m, n, k, a, k if trans else m, x, k, c, m)
+    want = x @ (a.conj().T if trans else a)
+    assert torch.equal(c, want)
