@@ -2568,6 +2568,7 @@ int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const
         drop();
         return RTTDDFT_OK;
     } catch (Fail& f) {
+        cudaStreamSynchronize(ctx->stream);  // steps still queued write the state and the workspace
         if (restore) {
             for (size_t k = 0; k < theta_saved.size(); ++k)
                 cudaMemcpy(ctx->hkd[k].theta, theta_saved[k], (size_t)ctx->naux * ctx->ns * sizeof(zd),
