@@ -152,6 +152,17 @@ static T* dalloc(rttddft_ctx* ctx, size_t n) {
     ctx->allocs.push_back(p);
     return (T*)p;
 }
+// null where the memory does not suffice
+template <typename T>
+static T* dtry(rttddft_ctx* ctx, size_t n) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    ctx->allocs.push_back(p);
+    return (T*)p;
+}
 template <typename T>
 static T* dupload(rttddft_ctx* ctx, const T* h, size_t n) {
     T* d = dalloc<T>(ctx, n);
@@ -737,7 +748,8 @@ static void build_dv_dg(rttddft_ctx* ctx) {
         need += dg_left_bytes(naux, ctx->nb[k]) + dg_left_bytes(2 * naux, ctx->ng[k]) + 3 * dg_left_bytes(2 * naux, at.lrows + 1);
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || need > fr / 2) return;
     bool ok = true;
-    if (!ctx->dgl_cch) {
+    const bool own_cch = !ctx->dgl_cch;
+    if (own_cch) {
         std::vector<DgMat> cch(nk);
         for (int k = 0; k < nk; ++k)
             cch[k] = DgMat{ctx->hkd[k].caux, (size_t)ctx->nb[k], 1, 1, naux, ctx->nb[k]};
@@ -750,7 +762,7 @@ static void build_dv_dg(rttddft_ctx* ctx) {
         std::vector<DgMat> dh, lh(nk);
         std::vector<DgRight> rw, rg(nk), rd;
         ctx->mtd_stride = ctx->maxm * ns;
-        if (ctx->dg_mt) ctx->d_mtd = dalloc<zd>(ctx, (size_t)nk * at.n * ctx->mtd_stride);
+        if (ctx->dg_mt) ok = ok && (ctx->d_mtd = dtry<zd>(ctx, (size_t)nk * at.n * ctx->mtd_stride));
         for (int al = 0; al < at.n; ++al)
             dh.push_back(DgMat{ctx->d_dh + at.boff[al], 1, (size_t)at.m[al], 0, at.m[al], at.m[al]});
         for (int k = 0; k < nk; ++k) {
@@ -767,7 +779,7 @@ static void build_dv_dg(rttddft_ctx* ctx) {
             rg[k] = DgRight{ctx->dv_w[k], at.lrows, at.lrows, K.dvsub, naux};
             rg[k].scale = &ctx->d_st->cur_s;
         }
-        ok = (ctx->dgl_dh = dg_left_create(at.n, dh.data(), ctx->stream)) &&
+        ok = ok && (ctx->dgl_dh = dg_left_create(at.n, dh.data(), ctx->stream)) &&
              (ctx->dgl_lh = dg_left_create(nk, lh.data(), ctx->stream)) &&
              (gw = dg_gemm_create(ctx->dgl_dh, nk * at.n, rw.data(), naux, ctx->d_flag, at.n)) &&
              (gg = dg_gemm_create(ctx->dgl_lh, nk, rg.data(), naux, ctx->d_flag)) &&
@@ -783,7 +795,15 @@ static void build_dv_dg(rttddft_ctx* ctx) {
         CK(cudaStreamSynchronize(ctx->stream));
         return;
     }
+    // nothing stays of what does not fit: the products of the form without digits run
     for (DgGemm* g : {gi, gw, gg, gd}) dg_gemm_destroy(g);
+    for (DgLeft** l : {&ctx->dgl_dh, &ctx->dgl_lh, own_cch ? &ctx->dgl_cch : nullptr}) {
+        if (!l) continue;
+        dg_left_destroy(*l);
+        *l = nullptr;
+    }
+    dfree(ctx, ctx->d_mtd);
+    ctx->d_mtd = nullptr;
 }
 
 // Undo a first rttddft_set_dv that failed: whatever it allocated (the allocations
@@ -2173,8 +2193,6 @@ int rttddft_set_dv(rttddft_ctx* ctx, const double* dh, const double* dvtab) {
         }
         if (at.n > 0) CK(cudaMemcpy(ctx->d_dh, dh, nblk * sizeof(zd), cudaMemcpyHostToDevice));
         if (ctx->d_dh32) launch_convert_f32(ctx->d_dh, ctx->d_dh32, nblk, ctx->stream);
-        if (!ctx->dv_set) build_dv_dg(ctx);
-        else if (ctx->dgl_dh) launch_dg_left(ctx->dgl_dh, ctx->stream);
         CK(cudaMemcpy(ctx->d_dvtab, dvtab, ctx->nvt * sizeof(zd), cudaMemcpyHostToDevice));
         if (ctx->tc && !ctx->fft) {
             double vmax = 0.0;
@@ -2187,6 +2205,9 @@ int rttddft_set_dv(rttddft_ctx* ctx, const double* dh, const double* dvtab) {
             if (e) fail(ctx, e, why);
             KCHECK();
         }
+        // the digits take of the memory what the buffers that the change needs have left
+        if (!ctx->dv_set) build_dv_dg(ctx);
+        else if (ctx->dgl_dh) launch_dg_left(ctx->dgl_dh, ctx->stream);
         ctx->dv_set = true;
         // bound || CC^H dV_1 CC ||_F for the Chebyshev scaling (one evaluation with s = 1)
         {

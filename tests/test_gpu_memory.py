@@ -67,3 +67,25 @@ def test_set_dv_after_one_that_ran_out_of_memory(prec):
     ctx.close()
     assert np.array_equal(got[0], want[0])
     assert np.array_equal(got[1], want[1])
+
+
+def test_set_dv_fits_where_its_buffers_do():
+    """The digits of the rebuild are optional: they come after the buffers that the call
+    cannot do without (the transform's 97 MiB among 112), not before them.  Same states
+    with and without them, to FP64's 1e-11 over three steps."""
+    s = make_system(tiny_config(n_g=2500, n_atoms=2, lmax=3, n_lo_per_atom=4, n_s=3, n_aux=200))
+    dv = make_dv(s, amp=0.3)
+    a, sc = pulse_samples(s, n_steps=3, a0=5.0), dv_scale_samples(3, s["dt"], freq=3.0)
+    want = None
+    for left in (None, 200, 128):
+        ctx = Context(s, interstitial="fft", graph_steps=3)
+        if left is None:
+            ctx.set_dv(dv)
+        else:
+            with Full(left * MIB):
+                ctx.set_dv(dv)
+        ctx.step(a, sc)
+        th = ctx.get_state(0)
+        ctx.close()
+        want = th if want is None else want
+        assert np.linalg.norm(th - want) < 1e-11 * np.linalg.norm(want)
