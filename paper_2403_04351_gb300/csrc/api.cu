@@ -650,23 +650,54 @@ static void drop_dg(rttddft_ctx* ctx) {
     }
 }
 
+// Device bytes that this context may still ask for after build_dg: the split-K
+// partials of set-up (bounded by C in every slice of the narrowest chunk) and
+// what a potential change needs, N_aux columns of the transforms among it.
+static size_t later_bytes(const rttddft_ctx* ctx) {
+    const AtomTab& at = ctx->at;
+    const size_t nk = ctx->nk, ns = ctx->ns, naux = ctx->naux;
+    size_t n = 16 * ctx->nvt * 3 + 16 * (6 * ctx->nblk + nk * at.lrows * ns);
+    for (int k = 0; k < ctx->nk; ++k)
+        n += 16 * (naux * (ctx->ng[k] + at.lrows + naux) + 16 * ns * (size_t)ctx->nb[k] + 4 * naux * ns);
+    return n + fft_change_bytes(ctx->fft, ctx->naux) + ((size_t)16 << 20);
+}
+
 // FP64 form: digits of CC (rows; and CC^H) and of the matching coefficients (A
 // and A^H), 12 bytes per real against 8, and the products they serve.  Returns
-// false, with nothing built, where they would take more than half of the free
-// device memory: the FP64 kernels run instead.
+// false, with nothing built, where they would take more than half of the device
+// memory that later_bytes leaves, or where an allocation fails: the FP64 kernels
+// run instead.
 static bool build_dg(rttddft_ctx* ctx) {
     const int nk = ctx->nk, ns = ctx->ns, naux = ctx->naux, ma = ctx->at.ma;
+    const size_t mark = ctx->allocs.size();
+    const std::vector<KDev> was = ctx->hkd;  // th and tb as they are without the digits
+    auto give_up = [&] {
+        cudaStreamSynchronize(ctx->stream);
+        cudaGetLastError();
+        drop_dg(ctx);
+        while (ctx->allocs.size() > mark) {
+            cudaFree(ctx->allocs.back());
+            ctx->allocs.pop_back();
+        }
+        ctx->hkd = was;
+        ctx->d_proj = ctx->d_mtw = nullptr;
+        ctx->mtw_stride = 0;
+        return false;
+    };
+    const size_t later = later_bytes(ctx);
     size_t need = 0, fr = 0, tot = 0;
     for (int k = 0; k < nk; ++k)
         need += dg_left_bytes(ctx->nb[k], naux) + dg_left_bytes(naux, ctx->nb[k]) + dg_left_bytes(ma, ctx->ng[k]) +
                 dg_left_bytes(ctx->ng[k], ma) + 2 * dg_left_bytes(2 * ns, ctx->nb[k]) + dg_left_bytes(4 * ns, ma);
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || need > fr / 2) return false;
+    for (int al = 0; al < ctx->at.n; ++al)
+        need += dg_left_bytes(5 * ctx->at.m[al], ctx->at.m[al]) + nk * (dg_left_bytes(2 * ns, ctx->at.m[al]) + (size_t)80 * ctx->maxm * ns);
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || fr < later || need > (fr - later) / 2) return false;
     std::vector<DgMat> cc(nk), cch(nk), am(nk), ah(nk);
     std::vector<DgRight> re(nk), rf(nk), rb(nk), rp(nk);
-    ctx->d_proj = dalloc<zd>(ctx, (size_t)nk * ns * naux);
+    if (!(ctx->d_proj = dtry<zd>(ctx, (size_t)nk * ns * naux))) return give_up();
     for (int k = 0; k < nk; ++k) {
         KDev& K = ctx->hkd[k];
-        if (ma > 0 && !K.tb) K.tb = dalloc<zd>(ctx, (size_t)K.ng * 2 * ns);
+        if (ma > 0 && !K.tb && !(K.tb = dtry<zd>(ctx, (size_t)K.ng * 2 * ns))) return give_up();
         cc[k] = DgMat{K.caux, 1, (size_t)K.nb, 0, K.nb, naux};
         cch[k] = DgMat{K.caux, (size_t)K.nb, 1, 1, naux, K.nb};
         am[k] = DgMat{K.at, (size_t)K.ng, 1, 1, ma, K.ng};
@@ -688,9 +719,10 @@ static bool build_dg(rttddft_ctx* ctx) {
     const AtomTab& at = ctx->at;
     if (ok && at.n > 0 && (long long)nk * at.n <= 65535) {
         // the muffin-tin stacks [h; o; p_x; p_y; p_z] of every atom, static; their products per (k, atom)
-        zd* stk = dalloc<zd>(ctx, 5 * ctx->nblk);
+        zd* stk = dtry<zd>(ctx, 5 * ctx->nblk);
         ctx->mtw_stride = 5 * ctx->maxm * ns;
-        ctx->d_mtw = dalloc<zd>(ctx, (size_t)nk * at.n * ctx->mtw_stride);
+        ctx->d_mtw = dtry<zd>(ctx, (size_t)nk * at.n * ctx->mtw_stride);
+        if (!stk || !ctx->d_mtw) return give_up();
         std::vector<DgMat> mm;
         std::vector<DgRight> rm;
         for (int al = 0; al < at.n; ++al) {
@@ -722,7 +754,7 @@ static bool build_dg(rttddft_ctx* ctx) {
         std::vector<const int*> gl(nk);
         for (int k = 0; k < nk; ++k) {
             KDev& K = ctx->hkd[k];
-            if (!K.th) K.th = dalloc<zd>(ctx, (size_t)K.ng * ns);
+            if (!K.th && !(K.th = dtry<zd>(ctx, (size_t)K.ng * ns))) return give_up();
             rt[k] = DgRight{K.C, K.nb, K.ng, K.th, K.ng};
             gl[k] = K.glin;
         }
@@ -732,8 +764,7 @@ static bool build_dg(rttddft_ctx* ctx) {
             KCHECK();
         }
     }
-    if (!ok) drop_dg(ctx);
-    return ok;
+    return ok || give_up();
 }
 
 // The potential-change rebuild (dh L, L^H W, CC_G^H T) as digit products, in

@@ -1283,6 +1283,15 @@ static bool potential_on_grid(const FftPlan* pl, const zd* tab, const int vt_dim
     return ok;
 }
 
+// device bytes that a potential change over ncol columns asks for: the grids of the
+// change and of the density, and the transform buffers
+size_t fft_change_bytes(const FftPlan* pl, int ncol) {
+    if (!pl) return 0;
+    const size_t elt = pl->prec == 0 ? sizeof(zd) : sizeof(zf), L = pl->max_lines, P = pl->max_planes;
+    const size_t ch1 = fft_chunks(pl->F[2], pl->F[1]), ch0 = fft_chunks(pl->F[2], pl->F[0]);
+    return (size_t)pl->F[0] * pl->F[1] * pl->F[2] * (3 * sizeof(zd) + sizeof(zf)) + (size_t)pl->nk * ncol *
+           ((L + P * pl->F[1]) * pl->F[2] * elt + (pl->fx ? ((L + P) * ch1 + pl->F[1] * ch0) * sizeof(int2) : 0));
+}
 static bool fft_alloc_buffers(FftPlan* pl, int ncol, std::string* why) {
     const size_t elt = pl->prec == 0 ? sizeof(zd) : sizeof(zf);
     const size_t c3 = (size_t)pl->max_lines * pl->F[2];

@@ -294,6 +294,7 @@ int fft_set_dv(FftPlan* pl, const zd* dvtab_dev, const int vt_dim[3], int ncol, 
 void fft_plan_destroy(FftPlan* pl);
 void fft_plan_info(const FftPlan* pl, int F[3], int* fused);
 int fft_tune(FftPlan* pl, const ToepDesc* td, int ncol, cudaStream_t st);
+size_t fft_change_bytes(const FftPlan* pl, int ncol);
 int fft_reserve_columns(FftPlan* pl, int ncol, cudaStream_t st, std::string* why);
 int fft_hartree_init(FftPlan* pl, const double recip[9], const int vt_dim[3], double omega, double bound, int ns,
                      cudaStream_t st, std::string* why);

@@ -89,3 +89,39 @@ def test_set_dv_fits_where_its_buffers_do():
         ctx.close()
         want = th if want is None else want
         assert np.linalg.norm(th - want) < 1e-11 * np.linalg.norm(want)
+
+
+def _names(ctx, a, sc=None):
+    return {n for n, _ in ctx.trace(a, sc)}
+
+
+@pytest.mark.parametrize("route", ["toeplitz", "fft"])
+@pytest.mark.parametrize("n_s", [3, 12])
+def test_fp64_form_without_the_memory_for_its_digits(route, n_s):
+    """Set-up and a potential change in memory that the digits do not fit into: the FP64
+    kernels run, with the record and the states of the digit products to their
+    common rounding (1e-11 of E and of the states' norm over four steps, the bound
+    that both have against the oracle)."""
+    s = make_system(tiny_config(n_g=2500, n_atoms=2, lmax=3, n_lo_per_atom=4, n_s=n_s, n_aux=200))
+    dv = make_dv(s, amp=0.3)
+    a, sc = pulse_samples(s, n_steps=4, a0=5.0), dv_scale_samples(4, s["dt"], freq=3.0)
+
+    def run(ctx):
+        ctx.set_dv(dv)
+        ctx.step(a, sc)
+        hx, sx = ctx.apply(0, x, np.array([1.0, -2.0, 3.0]), 0.7)
+        names = _names(ctx, a[:1], sc[:1])
+        out = ctx.observables()["energy"], ctx.get_state(0), hx, sx
+        ctx.close()
+        return names, out
+
+    rng = np.random.default_rng(1)
+    nb = int(s["n_g"][0]) + int(np.sum(s["n_lo"]))
+    x = rng.standard_normal((nb, n_s + 2)) + 1j * rng.standard_normal((nb, n_s + 2))
+    names, want = run(Context(s, interstitial=route, graph_steps=2))
+    assert "split_reduce_forward" not in names and "gemm_forward" in names
+    with Full((230 if route == "fft" else 110) * MIB):
+        names, got = run(Context(s, interstitial=route, graph_steps=2))
+    assert "split_reduce_forward" in names or "tc_backprojection" not in names
+    for g, w in zip(got, want):
+        assert np.max(np.abs(g - w)) < 1e-11 * np.linalg.norm(w)
