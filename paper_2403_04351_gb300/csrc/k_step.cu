@@ -613,8 +613,9 @@ __global__ void __launch_bounds__(CS_THREADS, (JU == 2 ? 4 : 3) + (NT == 2 ? 1 :
 // warp sends y_(n+2) after all of y_(n+1) has arrived, and every warp sends its
 // entries of y_(n+1) after it has read y_n.  Waits are bounded as elsewhere.
 #define CL_N 16
-#define CL_MAXN 256
-#define CL_THREADS 512
+#define CL_MAXN 64
+#define CL_MAXS 2
+#define CL_THREADS (32 * CL_MAXN / CL_N)
 struct CsRow {
     double diag;  // of H~
     int e;        // the row's exponent (cs_rowexp)
@@ -626,11 +627,11 @@ __global__ void __launch_bounds__(128) k_cs_rows(StepArgs a, CsRow* rows) {
     const int k = blockIdx.y, i = blockIdx.x, n = a.naux;
     const KDev& K = a.kd[k];
     const CsPulse pu = cs_pulse(a, K, i == 0 && k == 0 && threadIdx.x == 0);
-    zd v[CL_MAXN / 128];
+    zd v[(CL_MAXN + 127) / 128];
     int hm = 0;
     bool bad = false;
 #pragma unroll
-    for (int u = 0; u < CL_MAXN / 128; ++u) {
+    for (int u = 0; u < (CL_MAXN + 127) / 128; ++u) {
         const int j = threadIdx.x + u * 128;
         v[u] = j < n ? cs_hentry(a, K, pu, i, j) : zmk(0.0, 0.0);
         const int hx = __double2hiint(v[u].x) & 0x7fffffff, hy = __double2hiint(v[u].y) & 0x7fffffff;
@@ -649,7 +650,7 @@ __global__ void __launch_bounds__(128) k_cs_rows(StepArgs a, CsRow* rows) {
     hm = max(max(smx[0], smx[1]), max(smx[2], smx[3]));
     const int e = cs_rowexp(hm, n);
 #pragma unroll
-    for (int u = 0; u < CL_MAXN / 128; ++u) {
+    for (int u = 0; u < (CL_MAXN + 127) / 128; ++u) {
         const int j = threadIdx.x + u * 128;
         if (j < n) ((int4*)K.hsub)[(size_t)i * n + j] = cs_hcut(v[u], e);
     }
@@ -2291,9 +2292,7 @@ static const void* cheb_coop_fn(const StepArgs& a) {
     if (a.ns <= 4) return two ? (const void*)k_cheb_coop<4, 2, MODE> : (const void*)k_cheb_coop<4, 4, MODE>;
     return two ? (const void*)k_cheb_coop<8, 2, MODE> : (const void*)k_cheb_coop<8, 4, MODE>;
 }
-static const void* cheb_cl_fn(const StepArgs& a) {
-    return a.ns <= 2 ? (const void*)k_cheb_cl<2> : (a.ns <= 4 ? (const void*)k_cheb_cl<4> : (const void*)k_cheb_cl<8>);
-}
+static const void* cheb_cl_fn() { return (const void*)k_cheb_cl<CL_MAXS>; }
 // the cluster's shared memory: two slots of y and the coefficients
 static size_t cheb_cl_smem(const StepArgs& a, int nterms) { return ((size_t)2 * a.naux * a.ns + nterms) * sizeof(int4); }
 static size_t cheb_coop_smem(const StepArgs& a) { return (size_t)a.naux * a.ns * sizeof(int4); }
@@ -2331,7 +2330,7 @@ static cudaError_t launch_cheb_coop_raw(const StepArgs& a, cudaStream_t s) {
     at[0].val.clusterDim.x = CL_N;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     void* args[2] = {&arg, &rows};
-    return cudaLaunchKernelExC(&cfg, cheb_cl_fn(a), args);
+    return cudaLaunchKernelExC(&cfg, cheb_cl_fn(), args);
 }
 int launch_cheb_coop(const StepArgs& a, cudaStream_t s) {
     launch_cheb_coop_raw(a, s);
@@ -2354,20 +2353,22 @@ static bool grid_fits(const void* f, const StepArgs& a, int nsm) {
 
 // Blocks of the one-launch series for at most eight states, or 0; *cl: 1 for the
 // cluster form.  16 SMs take 1.4 cycles per product of a row's entry and a
-// column, so the cluster form is the faster one only while N_aux^2 N_s / 16 is
-// small (N_aux 32, N_s 8: 41 us a series against 57 of the grid form; N_aux 200,
-// N_s 2: 75 against 48; N_aux 240, N_s 7: 246 against 73).  The grid form has all
-// its blocks resident at once (the launch guarantees it or fails) and must be
+// column, and every lane of a row's warp waits for its FP64 instructions, so the
+// cluster form is the faster one only for one or two states while N_aux^2 N_s / 16
+// is small (us a series, cluster against grid: N_aux 64, N_s 1 28.3 / 33.3; N_aux 32,
+// N_s 2 25.8 / 30.7; with rows for 16 warps a block N_aux 100, N_s 2 45.6 / 38.4, N_aux
+// 176, N_s 1 52.7 / 43.5, N_aux 24, N_s 4 34.2 / 33.3, N_aux 32, N_s 8 45.5 / 41.1).  The grid form has all its
+// blocks resident at once (the launch guarantees it or fails) and must be
 // capturable in a graph on this driver.
-#define CL_WORK 2000
+#define CL_WORK 256
 int prepare_cheb_coop(const StepArgs& a0, cudaStream_t s, int* cl) {
     int dev = 0, coop = 0, nsm = 0;
     *cl = 0;
     if (a0.ns > 8 || a0.naux > 4 * CS_THREADS) return 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     StepArgs a = a0;
-    if (a.naux >= CL_N && a.naux <= CL_MAXN && (a.naux + CL_N - 1) / CL_N * a.naux * a.ns <= CL_WORK) {
-        const void* f = cheb_cl_fn(a);
+    if (a.ns <= CL_MAXS && a.naux >= CL_N && a.naux <= CL_MAXN && (a.naux + CL_N - 1) / CL_N * a.naux * a.ns <= CL_WORK) {
+        const void* f = cheb_cl_fn();
         const size_t sm = cheb_cl_smem(a, RTD_MAX_TERMS);
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
