@@ -8,13 +8,20 @@
 // Oishi and Rump, Numer. Algorithms 59, 2012).  Digits are exact in fp16, a
 // product of two is at most 2^16, and the FP32 accumulator of tcgen05.mma
 // holds the sum of a group (the pairs i + j = s) exactly up to 2^24: over 256
-// reals of K for s = 10 (one pair), 128 for s = 9, 64 for s = 8 and 7.  s = 6 is
-// read out every 128, s = 5 and 4 every 512: their sums pass 2^24 only where
-// nearly all digits have the largest size and one sign, by a rounding of 2^-52
-// of the scale where the result itself is 2^5 of it.  The groups s = 4 .. 10
-// are kept (26 of 36 pairs; the dropped ones are below the 2^-54 of the cut
-// itself), read out and added up as integers, so a result does not depend on
-// the order of the sums or on the number of K slices.
+// reals of K for s = 10 (one pair), 128 for s = 9, 64 for s = 8 and 7, the lengths
+// after which these are read out.  s = 6 (5 pairs) is read out every 128 reals, s = 5
+// and 4 (6 and 5 pairs) every 512: their sums can reach 2^25.3, 2^27.6 and 2^27.3
+// and are rounded past 2^24, as constant operands often do for s = 5 and 4.  Were every
+// product of the largest size and one sign, with the accumulator's last bit lost at
+// each, that were 2^-51.6 of K times the row's and the column's largest entries for s
+// = 6 and 2^-58 for the others; the cut of the operands is 2^-53 of it at most.
+// (Read out every 64 reals, s = 6 still passes 2^24, for a seventh more read-outs,
+// which bound the large products.)  The groups s = 4 .. 10 are kept (26 of 36 pairs;
+// the dropped ones are below the 2^-54 of the cut itself), read out and added up as
+// 64-bit integers: what order the K slices meet in changes nothing, how many there are
+// only what s = 4 to 6 round.  The accuracy is relative to the largest entries of a row
+// and a column: a column that decays over six decades comes out of the direct sum
+// with 1.4 to 1.8 times FP64's error in the norm, a flat one with about half of it.
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 

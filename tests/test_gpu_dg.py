@@ -175,3 +175,31 @@ def test_a_k_point_that_is_not_finite_stays_alone(n_aux, n_s):
     assert np.linalg.norm(ctx.get_state(keep) - want[keep]) < 1e-12 * np.sqrt(n_s)
     assert np.all(np.isnan(ctx.get_state(1 - keep)))
     ctx.close()
+
+
+@pytest.mark.parametrize("n_g,n_s", [(512, 2), (700, 16), (2600, 2)])
+def test_coherent_digits(n_g, n_s):
+    """Constant operands (every digit of one sign) and columns whose leading digits
+    cancel while the low ones add up, in the direct sum: H x = |G|^2/2 x + c sum x for a
+    table that is c everywhere.  2 N_G products a part, each with at most 2^-53 from the
+    cut and 2^-51.6 from the accumulators: below 2^-49 of N_G |c| max|x|."""
+    from systems import free_electron_system
+    s = free_electron_system(n_g=n_g, n_s=n_s, n_aux=n_s)
+    rng = np.random.default_rng(n_g)
+    sign = np.where(np.arange(n_g) % 2 == 0, 1.0, -1.0)
+    sign[-1] = 0.0 if n_g % 2 else sign[-1]
+    for _ in range(4):
+        c = rng.uniform(0.1, 1.0)
+        s["vtab"] = np.full_like(s["vtab"], c)
+        z = rng.uniform(-1, 1, 16) + 1j * rng.uniform(-1, 1, 16)
+        x = np.outer(np.ones(n_g), z)
+        x[:, 8:] = np.outer(sign, z[8:]) + rng.uniform(0, 1, 8) * 2.0 ** -rng.integers(1, 40, 8)
+        ctx = Context(s)
+        got = ctx.apply(0, x)[0]
+        ctx.close()
+        kin = 0.5 * np.sum(s["gk"][0].astype(np.longdouble) ** 2, axis=1)
+        xl = x.astype(np.clongdouble)
+        want = kin[:, None] * xl + np.longdouble(c) * np.sum(xl, axis=0)
+        err = np.abs(got - want).astype(float)
+        size = n_g * c * np.max(np.abs(x), axis=0) + kin.astype(float)[:, None] * np.abs(x)
+        assert np.max(err / size) < 2.0 ** -49
