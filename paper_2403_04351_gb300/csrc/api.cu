@@ -1057,6 +1057,7 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
         ctx->d_st = dalloc<DevState>(ctx, 1);
         CK(cudaMemset(ctx->d_st, 0, sizeof(DevState)));
         ctx->d_flag = dalloc<int>(ctx, 1);
+        CK(cudaMemset(ctx->d_flag, 0, sizeof(int)));
         ctx->d_cheb_sync = dalloc<unsigned char>(ctx, cheb_sync_bytes(nk, naux));
         CK(cudaMemset(ctx->d_cheb_sync, 0, cheb_sync_bytes(nk, naux)));
         ctx->d_rec = dalloc<double>(ctx, (size_t)o->max_record * RTD_REC_STRIDE);

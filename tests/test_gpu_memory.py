@@ -125,3 +125,19 @@ def test_fp64_form_without_the_memory_for_its_digits(route, n_s):
     assert "split_reduce_forward" in names or "tc_backprojection" not in names
     for g, w in zip(got, want):
         assert np.max(np.abs(g - w)) < 1e-11 * np.linalg.norm(w)
+
+
+def test_error_flag_starts_clear():
+    """A context that takes its basis as given reads no flag of the memory's last owner:
+    contexts of other shapes come and go between, and none of its waits has run out."""
+    from oracle import Oracle
+    s = make_system(tiny_config(n_g=300, n_atoms=1, lmax=1, n_lo_per_atom=1, n_s=3, n_aux=20))
+    kp = Oracle(s).kp[0]
+    a = pulse_samples(s, n_steps=2, a0=5.0)
+    for n in (200, 400, 800):
+        other = Context(make_system(tiny_config(n_g=n, n_atoms=1, lmax=1, n_lo_per_atom=1, n_s=5, n_aux=30)), precision="bf16x3")
+        other.close()
+        ctx = Context(s, aux_mode="given", caux=[kp["caux"]], eps=[kp["eps"]])
+        ctx.step(a)
+        assert len(ctx.observables()["t"]) == 2
+        ctx.close()
