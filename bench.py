@@ -62,6 +62,7 @@ TRAFFIC = {}
 # 16-bit products of one FP64 multiply-add in the exact digit products (k_dg.cu):
 # six digits a factor, the 26 pairs that reach the result
 DIGIT_PAIRS = 26
+DIGIT_SLOTS = ("gemm_expand", "gemm_project", "gemm_forward", "toeplitz", "tc_backprojection", "local_mt")  # FP64 form
 DIGIT_SERIES_MIN_NS = 9  # states from which the Chebyshev series runs as digit products
 
 
@@ -86,7 +87,7 @@ def _bf16_peak():
 
 def _src_hash():
     h = hashlib.sha256()
-    for f in ("k_linalg.cu", "k_step.cu", "k_tc.cu", "k_fft.cu", "common.cuh", "rtd.h"):
+    for f in ("k_linalg.cu", "k_step.cu", "k_tc.cu", "k_dg.cu", "k_fft.cu", "common.cuh", "tcgen05.cuh", "dg.h", "rtd.h"):
         with open(os.path.join(ROOT, "paper_2403_04351_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -162,7 +163,10 @@ def algorithmic_work(name, sysd, prec, nterms=1):
         if name == "toeplitz_and_backprojection":
             fl += 8 * ns * (ng * ng + 2 * ng * ma)
             by += ma * ng * cb + ng * ns * 16 * 2
-        elif name == "backprojection":
+        elif name == "toeplitz":
+            fl += 8 * ns * ng * ng
+            by += ng * ns * 16 * 2
+        elif name in ("backprojection", "tc_backprojection"):
             fl += 8 * ns * 2 * ng * ma
             by += ma * ng * cb + ng * ns * 16 * 2
         elif name == "tc_interstitial_and_forward":
@@ -305,8 +309,13 @@ def roofline_of(name, tr, s, prec, nterms):
         ach = fl / dur / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak, "peak_source": src + " (cuBLAS bf16 burst)"}
+    elif name == "tc_backprojection" and prec != "fp64":
+        peak, src = _bf16_peak()
+        ach = 3 * fl / dur / 1e12
+        roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
+                "frac": ach / peak, "peak_source": src + " (cuBLAS bf16 burst; three 16-bit products)"}
     elif (name == "chebyshev_series" and int(s["n_s"]) >= DIGIT_SERIES_MIN_NS) or \
-            (prec == "fp64" and name in ("gemm_expand", "gemm_project", "gemm_forward")):
+            (prec == "fp64" and name in DIGIT_SLOTS):
         peak, src = _bf16_peak()
         ach = DIGIT_PAIRS * fl / dur / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
@@ -314,7 +323,7 @@ def roofline_of(name, tr, s, prec, nterms):
     else:
         if prec == "fp64" or name in ("chebyshev_term", "chebyshev_series"):
             peak = FP64_PEAK_TFLOPS
-            src = "FP64 nominal (the series and the FP64 transforms run in 64-bit integers)"
+            src = "FP64 nominal (the series' products and the FP64 transforms run in integers)"
         else:
             peak = SM_COUNT * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12
             src = "152 SM x 128 FP32 lanes x 2 x 2070 MHz"

@@ -98,7 +98,6 @@ struct DevState {
     double cur_s;       // potential-change scale of the current step
     double cur_aa;      // |A|^2 / (2 c^2)
     int err;            // nonzero: a device iteration limit ran out
-    unsigned bar;       // arrival counter of the grid barrier (zeroed by k_hsub and k_finalize)
     unsigned fin;       // arrival counter of k_finalize's blocks (wraps to zero)
 };
 

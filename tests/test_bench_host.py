@@ -50,6 +50,21 @@ def test_roofline_entry_of_the_fft_slot():
     assert roof64["peak"] == bench.FP64_PEAK_TFLOPS
 
 
+def test_roofline_entries_of_the_digit_products():
+    """Every slot of the FP64 form that runs as digit products has its work and is
+    held against the tensor rate, 26 products for one; the split form's
+    back-projection against three."""
+    s = make_system("tiny400", with_amat=False)
+    peak, _ = bench._bf16_peak()
+    for name in bench.DIGIT_SLOTS:
+        fl, _ = bench.algorithmic_work(name, s, "fp64")
+        roof = bench.roofline_of(name, {name: [0.5, 10]}, s, "fp64", 14)
+        assert fl > 0 and roof["bound"] == "tensor" and roof["peak"] == peak
+        assert np.isclose(roof["achieved"], 26 * fl / 0.05e-3 / 1e12)
+    roof = bench.roofline_of("tc_backprojection", {"tc_backprojection": [0.5, 10]}, s, "bf16x3", 14)
+    assert np.isclose(roof["achieved"], 3 * bench.algorithmic_work("tc_backprojection", s, "bf16x3")[0] / 0.05e-3 / 1e12)
+
+
 def test_density_feedback_is_not_sharded():
     """A k-point shard or subset of a density-feedback run would feed back a
     partial density: the benchmark refuses it before any GPU work; the forms
