@@ -1571,13 +1571,13 @@ int rttddft_setup(const rttddft_system* s, const rttddft_options* opt_in, void* 
             // the subspace current of many states: PP theta on the tensor cores
             std::vector<DgMat> pm(nk);
             std::vector<DgRight> pr(nk);
-            ctx->d_jw = dalloc<zd>(ctx, (size_t)nk * 3 * naux * ns);
+            ctx->d_jw = dtry<zd>(ctx, (size_t)nk * 3 * naux * ns);
             for (int k = 0; k < nk; ++k) {
                 KDev& K = ctx->hkd[k];
                 pm[k] = DgMat{K.psub, (size_t)naux, 1, 1, 3 * naux, naux};  // PP is Hermitian: rows from the stored columns
                 pr[k] = DgRight{K.theta, naux, naux, ctx->d_jw + (size_t)k * 3 * naux * ns, 3 * naux};
             }
-            ctx->dgl_pp = dg_left_create(nk, pm.data(), ctx->stream);
+            if (ctx->d_jw) ctx->dgl_pp = dg_left_create(nk, pm.data(), ctx->stream);
             if (ctx->dgl_pp) ctx->dg_j = dg_gemm_create(ctx->dgl_pp, nk, pr.data(), ns, ctx->d_flag);
         }
         // ---- theta(0)
@@ -2504,9 +2504,14 @@ int rttddft_adjoint(rttddft_ctx* ctx, int nsteps, const double* a_samples, const
             if (pass) break;
             if (off > ctx->adj_cap) {
                 dfree(ctx, ctx->adj_ws);
-                ctx->adj_ws = nullptr;
                 ctx->adj_cap = 0;
-                ctx->adj_ws = dalloc<unsigned char>(ctx, off);
+                ctx->adj_ws = dtry<unsigned char>(ctx, off);
+                if (!ctx->adj_ws && fast) {  // one step's vectors at a time take less
+                    fast = false;
+                    pass = -1;
+                    continue;
+                }
+                if (!ctx->adj_ws) fail(ctx, RTTDDFT_ERR_OOM, "device memory of the adjoint");
                 ctx->adj_cap = off;
             }
             ws = ctx->adj_ws;

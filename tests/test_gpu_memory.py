@@ -141,3 +141,21 @@ def test_error_flag_starts_clear():
         ctx.step(a)
         assert len(ctx.observables()["t"]) == 2
         ctx.close()
+
+
+def test_adjoint_without_the_memory_for_its_history():
+    """The Chebyshev vectors of a whole segment (22 MiB) are optional: without them the
+    sweep forms one step's at a time.  Gradients to 1e-9 of the largest, the bound of
+    both against the oracle."""
+    s = make_system(tiny_config(n_g=300, n_atoms=1, lmax=1, n_lo_per_atom=1, n_s=8, n_aux=200))
+    a = pulse_samples(s, n_steps=60, a0=5.0)
+    g = np.array([0.3, -0.5, 0.8])
+    ctx = Context(s)
+    with Full(16 * MIB):
+        got, dmu = ctx.adjoint(a, g, ckpt_every=60)
+    ctx.close()
+    ctx = Context(s)
+    want, dmu_want = ctx.adjoint(a, g, ckpt_every=60)
+    ctx.close()
+    assert np.max(np.abs(got - want)) < 1e-9 * np.max(np.abs(want))
+    assert np.max(np.abs(dmu - dmu_want)) < 1e-9 * np.max(np.abs(dmu_want))
