@@ -68,9 +68,10 @@ extern "C" {
 #define RTTDDFT_PROP_CN 2        /* Crank-Nicolson (I + i dt/2 HH)^{-1} (I - i dt/2 HH), by its Chebyshev series */
 
 /* precision of the full-basis contractions (expand, operator, project);
- * the subspace propagation and every reduction stay FP64, or exact digit
- * products and 64-bit fixed point of that accuracy, as do the contractions and
- * transforms of the FP64 form */
+ * the subspace propagation and every reduction stay FP64.  Products of FP64
+ * accuracy (the FP64 form's contractions and transforms, the propagation's
+ * products off the diagonal of HH) may run as digit products or in 64-bit fixed
+ * point, cut at 2^-54 of the largest entries of a row and of a column */
 #define RTTDDFT_PREC_FP64 0
 #define RTTDDFT_PREC_FP32 1
 /* split-BF16 on the tensor cores: the interstitial convolution and the

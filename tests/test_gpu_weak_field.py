@@ -30,7 +30,7 @@ def extended_step(eps, pp, a, c, dt, theta):
 
 
 @pytest.mark.parametrize("a0", [0.05, 1e-4, 1e-6])
-@pytest.mark.parametrize("n_aux,n_s,n_k", [(16, 1, 2), (64, 1, 1), (32, 2, 1), (40, 4, 1), (33, 8, 2), (130, 7, 1), (200, 2, 1), (270, 2, 1), (60, 12, 1), (140, 33, 2)])
+@pytest.mark.parametrize("n_aux,n_s,n_k", [(16, 1, 2), (64, 1, 1), (32, 2, 1), (40, 4, 1), (33, 8, 2), (130, 7, 1), (200, 2, 1), (270, 2, 1), (60, 12, 1), (40, 10, 2), (129, 17, 1)])
 def test_excited_amplitudes_of_a_weak_field(n_aux, n_s, n_k, a0):
     """The root-mean-square of the amplitudes outside the occupied block.  A
     step has about 20 terms of a few roundings each, so STEPS steps keep
