@@ -156,14 +156,16 @@ __global__ void __launch_bounds__(128) k_cheb(StepArgs a, int nt, int last) {
 // the N_s entries of a row have their diagonal, recurrence and sum in FP64 (a
 // series of N_aux 200, N_s 2: 82 -> 50 us; N_aux 240, N_s 7: 111 -> 75 us).
 // H~ = (HH - lam_c) / lam_h is its diagonal plus the rest of the row in units of
-// 2^-59 of a power of two above the row's 2-norm; y_n goes into the products in
-// units of 2^-57 of the power of two above its column's 2-norm (which bounds every
-// y_n).  An operand is held as hi 2^28 + lo; a product keeps hi hi and hi lo + lo
-// hi (the dropped lo lo is below 2^-60), summed exactly in 64 bits.  So what a term
-// loses is 2^-54 of the largest off-diagonal entry of its row: an amplitude that a
-// weak field feeds keeps FP64's relative accuracy, as small as it is (with the
-// diagonal in the same units, and the recurrence in them, it kept 2^-58 of the
-// column's norm: 5e-10 of the excited amplitudes at A = 1e-4).
+// 2^-59 of a power of two (cs_rowexp); y_n goes into the products in units of 2^-57
+// of the power of two above its column's 2-norm (which bounds every y_n).  An
+// operand is held as hi 2^28 + lo; a product keeps hi hi and hi lo + lo hi (the
+// dropped lo lo is below 2^-60), summed exactly in 64 bits.  So what a term loses is
+// 2^-56 of the largest off-diagonal entry of its row, or less: an amplitude that a
+// weak field feeds keeps FP64's relative accuracy, as small as it is, and where its
+// state couples to others a hundred times more strongly than to the occupied ones
+// (with the diagonal in the same units, and the recurrence in them, it kept 2^-58 of
+// the column's norm: 5e-10 of the excited amplitudes at A = 1e-4; with rows cut
+// four times coarser 1.9e-15 at N_aux 200, where FP64 has 0.7e-15 and this 0.8e-15).
 //
 // Per term y_n goes around through L2 (two slots of 16 bytes per entry) and a
 // grid barrier follows.  The barrier has CS_CNT arrival counters on lines of
@@ -275,11 +277,13 @@ __device__ __forceinline__ zd cs_hentry(const StepArgs& a, const KDev& K, const 
     if (i == j) v.x += (K.eps[i] + p.diag) * p.ilh;
     return v;
 }
-// the power of two above the 2-norm of a row of n entries whose parts' largest high word is hw
+// the power of two that a row of n entries, whose parts' largest high word is hw, is cut
+// relative to: its 2-norm is below four times that (a product's sum below 2^62), its largest
+// part below half
 __device__ __forceinline__ int cs_rowexp(int hw, int n) {
-    int h = 1;
+    int h = 3;
     while ((1 << (2 * h)) < 2 * n) ++h;  // 2^h >= sqrt(2 n)
-    return max((hw >> 20) - 1022 + h, -900);
+    return max((hw >> 20) - 1022 + h - 2, -900);
 }
 // an entry cut at 2^-59 of 2^e: (re hi, re lo, im hi, im lo)
 __device__ __forceinline__ int4 cs_hcut(zd v, int e) {
