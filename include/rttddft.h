@@ -71,7 +71,7 @@ extern "C" {
  * the subspace propagation and every reduction stay FP64.  Products of FP64
  * accuracy (the FP64 form's contractions and transforms, the propagation's
  * products off the diagonal of HH) may run as digit products or in 64-bit fixed
- * point, cut at 2^-54 of the largest entries of a row and of a column */
+ * point, cut at 2^-54 of the largest entries of a row and of a column or finer */
 #define RTTDDFT_PREC_FP64 0
 #define RTTDDFT_PREC_FP32 1
 /* split-BF16 on the tensor cores: the interstitial convolution and the

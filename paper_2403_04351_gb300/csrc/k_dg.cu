@@ -37,31 +37,40 @@
 
 namespace cg = cooperative_groups;
 
-#define DG_P 6              // digits
+#define DG_P 6              // digits of an operand: 54 bits
+#define DG_PS 7             // in the Chebyshev series: 63 bits
 #define DG_KS 32            // reals per stage: 64 bytes of fp16, one row of the 64-byte swizzle
 #define DG_BM 128           // rows per tile
-#define DG_S0 4             // smallest i + j kept
-#define DG_G 7              // groups kept, s = DG_S0 + g, NT columns of tensor memory each
+// smallest i + j kept with P digits, and the groups kept, s = dg_s0(P) + g, of NT columns of tensor memory each
+__host__ __device__ constexpr int dg_s0(int P) { return P - 2; }
+__host__ __device__ constexpr int dg_ng(int P) { return 2 * (P - 1) - dg_s0(P) + 1; }
 #define DG_THREADS 320      // 8 read-out warps, one product warp, one copy warp
 // and 256 (16 columns) or 128 threads that generate the left operand (GEN): with more columns the
 // read-out's integers need the registers
 __host__ __device__ constexpr int dg_gen(int NT) { return NT == 16 ? 256 : 128; }
 #define DG_A_PL (DG_BM * 64)
 
-// slices of 64 reals that a group collects before it is read out
-__host__ __device__ constexpr int dg_run(int g) { return g == 6 ? 4 : (g == 5 || g == 2 ? 2 : (g < 2 ? 8 : 1)); }
+// slices of 64 reals that a group collects before it is read out; g counted from the largest s (of
+// 1, 2, 3, ... pairs), the two smallest ones last
+__host__ __device__ constexpr int dg_run(int P, int g) {
+    const int t = dg_ng(P) - 1 - g;
+    return t == 0 ? 4 : (t == 1 ? 2 : (g < 2 ? 8 : (P == 6 && t == 4 ? 2 : 1)));
+}
 
 typedef long long i64;
 
 // ------------------------------------------------------------ digits
-// q = sum_i d_i 512^i with |q| <= 2^53, returned as the six biased values
+// q = sum_i d_i 512^i with |q| <= 2^(9 P - 1), returned as the P biased values
 // d_i + 256 (0 .. 512)
+template <int P>
 __device__ __forceinline__ void dg_cut(i64 q, uint32_t* d) {
-    const i64 bias = 256ll * (1ll + (1ll << 9) + (1ll << 18) + (1ll << 27) + (1ll << 36) + (1ll << 45));
-    const i64 u = q + bias;
+    unsigned long long bias = 0ull;
 #pragma unroll
-    for (int i = 0; i < DG_P - 1; ++i) d[i] = (uint32_t)(u >> (9 * i)) & 511u;
-    d[DG_P - 1] = (uint32_t)(u >> 45);
+    for (int i = 0; i < P; ++i) bias += 256ull << (9 * i);
+    const unsigned long long u = (unsigned long long)q + bias;
+#pragma unroll
+    for (int i = 0; i < P - 1; ++i) d[i] = (uint32_t)(u >> (9 * i)) & 511u;
+    d[P - 1] = (uint32_t)(u >> (9 * (P - 1)));
 }
 // fp16 pair (x - 256, y - 256) of biased digits: 1024 + x is exact in fp16
 __device__ __forceinline__ uint32_t dg_pair(uint32_t x, uint32_t y) {
@@ -87,26 +96,27 @@ __device__ __forceinline__ DgScale dg_scale(int e) {
 }
 __device__ __forceinline__ i64 dg_int(double x, DgScale s) { return __double2ll_rn((x * s.p1) * s.p2); }
 
-// (hi 2^27 + lo) 2^e as a double with integer arithmetic (the conversions of
+// (hi 2^SH + lo) 2^e as a double with integer arithmetic (the conversions of
 // the FP64 pipe would cost more than the products of a short K)
+template <int SH>
 __device__ __forceinline__ double dg_double(i64 hi, i64 lo, int e) {
-    i64 m = hi + (lo >> 27);
-    uint32_t r = (uint32_t)lo & ((1u << 27) - 1u);
+    i64 m = hi + (lo >> SH);
+    unsigned long long r = (unsigned long long)lo & ((1ull << SH) - 1ull);
     const bool neg = m < 0;
     if (neg) {
-        const bool b = r != 0u;
+        const bool b = r != 0ull;
         m = -m - (b ? 1 : 0);
-        r = b ? (1u << 27) - r : 0u;
+        r = b ? (1ull << SH) - r : 0ull;
     }
-    // keep the leading 63 bits of m 2^27 + r
+    // keep the leading 63 bits of m 2^SH + r
     const int lz = __clzll(m);
-    const int k = lz > 27 ? 27 : lz - 1;
-    const unsigned long long x = ((unsigned long long)m << k) | (r >> (27 - k));
+    const int k = lz > SH ? SH : lz - 1;
+    const unsigned long long x = ((unsigned long long)m << k) | (r >> (SH - k));
     if (x == 0ull) return 0.0;
     const int z = __clzll(x);
     const unsigned long long t = ((x << z) + (1ull << 10));  // the carry out of a value of all ones:
     const bool cy = t < (1ull << 10);
-    const int ex = e + (27 - k) + 63 - z + (cy ? 1 : 0) + 1023;
+    const int ex = e + (SH - k) + 63 - z + (cy ? 1 : 0) + 1023;
     const unsigned long long man = cy ? 0ull : (t >> 11) & ((1ull << 52) - 1ull);
     double v;
     if (ex >= 1 && ex <= 2046) {
@@ -120,23 +130,25 @@ __device__ __forceinline__ double dg_double(i64 hi, i64 lo, int e) {
 }
 
 // Operands lie tile by tile as a block of k_dg takes them: per tile of RT rows
-// and stage of 16 complex k, six planes of RT rows of 64 bytes, the 16-byte
+// and stage of 16 complex k, P planes of RT rows of 64 bytes, the 16-byte
 // chunks of a row permuted as the 64-byte swizzle wants them.  A stage is one
 // contiguous copy (as boxes of a row-major array, 64 bytes a row, the copies
 // gave 4.9 TB/s over the chip).  Word (two fp16) of row r, complex k, plane 0;
 // the planes are RT 16 words apart.
+template <int P>
 __host__ __device__ __forceinline__ size_t dg_word(int r, int k, int RT, int nst) {
     const int rr = r % RT;
-    return (((size_t)(r / RT) * nst + (k >> 4)) * DG_P * RT + rr) * 16 + ((((k >> 2) & 3) ^ ((rr >> 1) & 3)) << 2) + (k & 3);
+    return (((size_t)(r / RT) * nst + (k >> 4)) * P * RT + rr) * 16 + ((((k >> 2) & 3) ^ ((rr >> 1) & 3)) << 2) + (k & 3);
 }
 // rows 2n: [Re, -Im] and 2n + 1: [Im, Re] of a right operand, entry k of complex column n
+template <int P>
 __device__ __forceinline__ void dg_put_col(uint32_t* b, int NT, int nst, int n, int k, i64 qr, i64 qi) {
-    uint32_t dr[DG_P], di[DG_P];
-    dg_cut(qr, dr);
-    dg_cut(qi, di);
-    b += dg_word(2 * n, k, NT, nst);
+    uint32_t dr[P], di[P];
+    dg_cut<P>(qr, dr);
+    dg_cut<P>(qi, di);
+    b += dg_word<P>(2 * n, k, NT, nst);
 #pragma unroll
-    for (int i = 0; i < DG_P; ++i) {
+    for (int i = 0; i < P; ++i) {
         const uint32_t p = dg_pair(dr[i], di[i]);
         b[(size_t)i * NT * 16] = p ^ (DG_NEG << 16);
         b[(size_t)i * NT * 16 + 16] = (p >> 16) | (p << 16);
@@ -201,9 +213,13 @@ __device__ __forceinline__ void dg_ld(uint32_t taddr, uint32_t* r) {
             : "r"(taddr));
     }
 }
+// digits of a mode's operands, and stages of shared memory
+__host__ __device__ constexpr int dg_p(int mode) { return mode == 1 ? DG_PS : DG_P; }
+__host__ __device__ constexpr int dg_stages(int NT, int mode) { return mode == 1 ? (NT == 64 ? 2 : 3) : (NT == 16 ? 4 : 3); }
+
 // One 128-row x NT-column tile of D = A^ B^^T over this split's K stages (NT
 // real columns: Re and Im of NT / 2 complex ones).  The copy warp brings the
-// six digit planes of both operands of a stage with one bulk copy each.  A group has
+// P digit planes of both operands of a stage with one bulk copy each.  A group has
 // its own NT columns of tensor memory in the order of s, and X's digit planes
 // lie one after another in shared memory, so digit i of A meets a run of X's
 // digits in one product of up to N = 256 (9 instructions per 16 reals for
@@ -220,14 +236,16 @@ __device__ __forceinline__ void dg_ld(uint32_t taddr, uint32_t* r) {
 template <int NT, int MODE, bool GEN>
 __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(const DgArgs g) {
     extern __shared__ unsigned char dgsm[];
-    constexpr int STAGES = NT == 16 ? 4 : 3;
+    constexpr int P = dg_p(MODE), T = P - 1, S0 = dg_s0(P), G = dg_ng(P);  // digits, the largest one, groups
+    constexpr int STAGES = dg_stages(NT, MODE);
     constexpr int B_PL = NT * 64;
-    constexpr int STAGE = DG_P * (DG_A_PL + B_PL);
+    constexpr int STAGE = P * (DG_A_PL + B_PL);
     constexpr int CP = NT / 2;  // columns per read-out thread
-    constexpr uint32_t NCOLS = DG_G * NT <= 128 ? 128 : (DG_G * NT <= 256 ? 256 : 512);
+    constexpr uint32_t NCOLS = G * NT <= 128 ? 128 : (G * NT <= 256 ? 256 : 512);
+    constexpr int GH = G - 4, SH = 9 * GH;  // groups GH .. go to hi, in units of 2^SH of lo's
     unsigned char* smem = dgsm + ((1024u - (smem_u32(dgsm) & 1023u)) & 1023u);
     constexpr int THREADS = DG_THREADS + (GEN ? dg_gen(NT) : 0);
-    __shared__ __align__(8) uint64_t full[STAGES], fullA[STAGES], empty[STAGES], gfull[DG_G], gfree[DG_G], done;
+    __shared__ __align__(8) uint64_t full[STAGES], fullA[STAGES], empty[STAGES], gfull[G], gfree[G], done;
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
     __shared__ int is_last;
@@ -247,7 +265,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
             mbar_init(&fullA[s], dg_gen(NT) / 32);
             mbar_init(&empty[s], 1);
         }
-        for (int s = 0; s < DG_G; ++s) {
+        for (int s = 0; s < G; ++s) {
             mbar_init(&gfull[s], 1);
             mbar_init(&gfree[s], 8);
         }
@@ -271,9 +289,9 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
     if (warp == 9) {
         if (lane == 0) {
             int issued = 0;
-            const unsigned char* ga = o.A + ((size_t)m_i * o.nsta + st0) * (DG_P * DG_A_PL);
+            const unsigned char* ga = o.A + ((size_t)m_i * o.nsta + st0) * (P * DG_A_PL);
             const unsigned char* gb = (MODE == 0 ? o.B : (const unsigned char*)g.ch[z].Bn[(g.term - 1) & 1]) +
-                                      ((size_t)nt_i * o.nst + st0) * (DG_P * B_PL);
+                                      ((size_t)nt_i * o.nst + st0) * (P * B_PL);
             for (int t = 0; t < nk; ++t) {
                 const int s = t % STAGES;
                 if (t >= STAGES && !mbar_wait(&empty[s], (uint32_t)((t / STAGES - 1) & 1))) {
@@ -283,9 +301,9 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                 }
                 if (abort_flag) break;
                 unsigned char* sa = smem + s * STAGE;
-                mbar_expect_tx(&full[s], GEN ? DG_P * B_PL : STAGE);
-                if (!GEN) dg_copy(sa, ga + (size_t)t * (DG_P * DG_A_PL), DG_P * DG_A_PL, &full[s]);
-                dg_copy(sa + DG_P * DG_A_PL, gb + (size_t)t * (DG_P * B_PL), DG_P * B_PL, &full[s]);
+                mbar_expect_tx(&full[s], GEN ? P * B_PL : STAGE);
+                if (!GEN) dg_copy(sa, ga + (size_t)t * (P * DG_A_PL), P * DG_A_PL, &full[s]);
+                dg_copy(sa + P * DG_A_PL, gb + (size_t)t * (P * B_PL), P * B_PL, &full[s]);
                 issued = t + 1;
             }
             // nothing may still be on its way into shared memory when the block ends
@@ -296,7 +314,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
         if (lane == 0) {
             // kind::f16, fp16 operands, FP32 accumulator, both K-major
             const uint32_t idesc0 = (1u << 4) | ((uint32_t)(DG_BM >> 4) << 24);
-            constexpr int WMAX = 256 / NT < DG_P ? 256 / NT : DG_P;  // digits of X per product
+            constexpr int WMAX = 256 / NT < P ? 256 / NT : P;  // digits of X per product
             bool ok = true;
             for (int t = 0; t < nk && ok; ++t) {
                 const int s = t % STAGES;
@@ -309,10 +327,10 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                 const bool first = (t & 1) == 0, lastp = !first || t == nk - 1;
                 const int sl = t >> 1;
                 const uint64_t da = dg_desc(smem_u32(smem + s * STAGE));
-                const uint64_t db = dg_desc(smem_u32(smem + s * STAGE + DG_P * DG_A_PL));
+                const uint64_t db = dg_desc(smem_u32(smem + s * STAGE + P * DG_A_PL));
                 // digit i of A times the digits j .. j + w - 1 of X in one product of N = w NT
                 auto mma = [&](int kk, int i, int j, int w, uint32_t acc) {
-                    umma_bf16(tmem + (uint32_t)((i + j - DG_S0) * NT), da + (uint64_t)((i * DG_A_PL + kk * 32) >> 4),
+                    umma_bf16(tmem + (uint32_t)((i + j - S0) * NT), da + (uint64_t)((i * DG_A_PL + kk * 32) >> 4),
                               db + (uint64_t)((j * B_PL + kk * 32) >> 4),
                               idesc0 | ((uint32_t)((w * NT) >> 3) << 17), acc);
                 };
@@ -320,37 +338,37 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                     // the slice's first products, a group at a time: a group that starts anew waits
                     // for its read-out and overwrites its columns
 #pragma unroll
-                    for (int q = DG_G - 1; q >= 0; --q) {
-                        const bool anew = (sl & (dg_run(q) - 1)) == 0;
+                    for (int q = G - 1; q >= 0; --q) {
+                        const bool anew = (sl & (dg_run(P, q) - 1)) == 0;
                         if (anew && sl > 0) {
-                            if (!mbar_wait(&gfree[q], (uint32_t)((sl / dg_run(q) - 1) & 1))) {
+                            if (!mbar_wait(&gfree[q], (uint32_t)((sl / dg_run(P, q) - 1) & 1))) {
                                 ok = false;
                                 break;
                             }
                             tc_fence_after();
                         }
-                        if (q > 0) mma(0, 5, q + DG_S0 - 5, 1, anew ? 0u : 1u);
-                        else mma(0, 4, 0, 1, anew ? 0u : 1u);
+                        if (q > 0) mma(0, T, q + S0 - T, 1, anew ? 0u : 1u);
+                        else mma(0, T - 1, 0, 1, anew ? 0u : 1u);
                     }
                     if (!ok) break;
                 }
 #pragma unroll
-                for (int i = DG_P - 1; i >= 0; --i) {
+                for (int i = T; i >= 0; --i) {
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk) {
-                        int j = i < DG_S0 ? DG_S0 - i : 0;
+                        int j = i < S0 ? S0 - i : 0;
                         if (first && kk == 0) {
-                            if (i == 5) continue;
-                            if (i == 4) j = 1;
+                            if (i == T) continue;
+                            if (i == T - 1) j = 1;
                         }
 #pragma unroll
-                        for (; j < DG_P; j += WMAX) mma(kk, i, j, DG_P - j < WMAX ? DG_P - j : WMAX, 1u);
+                        for (; j < P; j += WMAX) mma(kk, i, j, P - j < WMAX ? P - j : WMAX, 1u);
                     }
                     // the largest group that digit i reaches is complete (the smallest two with digit 0)
                     if (lastp) {
-                        const int q = i + DG_P - 1 - DG_S0;
-                        if (t == nk - 1 || (sl & (dg_run(q) - 1)) == dg_run(q) - 1) umma_commit(&gfull[q]);
-                        if (i == 0 && (t == nk - 1 || (sl & (dg_run(0) - 1)) == dg_run(0) - 1)) umma_commit(&gfull[0]);
+                        const int q = i + T - S0;
+                        if (t == nk - 1 || (sl & (dg_run(P, q) - 1)) == dg_run(P, q) - 1) umma_commit(&gfull[q]);
+                        if (i == 0 && (t == nk - 1 || (sl & (dg_run(P, 0) - 1)) == dg_run(P, 0) - 1)) umma_commit(&gfull[0]);
                     }
                 }
                 umma_commit(&empty[s]);
@@ -438,10 +456,10 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
         bool ok = true;
         for (int sl = 0; sl < nsl && ok; ++sl) {
 #pragma unroll
-            for (int gi = DG_G - 1; gi >= 0; --gi) {
-                if (sl != nsl - 1 && (sl & (dg_run(gi) - 1)) != dg_run(gi) - 1) continue;
+            for (int gi = G - 1; gi >= 0; --gi) {
+                if (sl != nsl - 1 && (sl & (dg_run(P, gi) - 1)) != dg_run(P, gi) - 1) continue;
                 // the warp's lanes leave together: the loads below take all of them
-                if (__any_sync(0xffffffffu, !mbar_wait(&gfull[gi], (uint32_t)((sl / dg_run(gi)) & 1)) || abort_flag)) {
+                if (__any_sync(0xffffffffu, !mbar_wait(&gfull[gi], (uint32_t)((sl / dg_run(P, gi)) & 1)) || abort_flag)) {
                     ok = false;
                     break;
                 }
@@ -461,8 +479,8 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
 #pragma unroll
                     for (int c = 0; c < W; ++c) {
                         const i64 v = (i64)__float2int_rn(__uint_as_float(r[c]));
-                        if (gi >= 3) hi[c0 + c] += v << (9 * (gi - 3));  // units of s = 7
-                        else lo[c0 + c] += v << (9 * gi);                // units of s = 4
+                        if (gi >= GH) hi[c0 + c] += v << (9 * (gi - GH));  // units of s = S0 + GH
+                        else lo[c0 + c] += v << (9 * gi);                  // units of s = S0
                     }
                 }
             }
@@ -522,6 +540,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
             __syncthreads();
         }
     }
+    constexpr int E0 = 2 * (9 * P - 1) - 9 * S0;  // lo's unit is 2^(er + ec - E0)
     if (mine) {
         for (int it = tid; it < items / 2; it += THREADS) {
             const int rl = it & (DG_BM - 1), row = m0 + rl, c = (it / DG_BM) * 2, n = (n0 + c0 + c) >> 1;
@@ -549,8 +568,8 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                 if (ec >= 2048 || er >= 2048) {
                     v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
                 } else {
-                    v.x = dg_double(hv[0], lv[0], er + ec - 70);
-                    v.y = dg_double(hv[1], lv[1], er + ec - 70);
+                    v.x = dg_double<SH>(hv[0], lv[0], er + ec - E0);
+                    v.y = dg_double<SH>(hv[1], lv[1], er + ec - E0);
                 }
                 if (o.scale) v = zscale(v, *o.scale);
                 zd* p = o.C + row + (size_t)n * o.ldc;
@@ -564,7 +583,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                 const int er = o.er[row], ec = o.ec[n];
                 const zd yp = ((g.term & 1) ? ch.y0 : ch.y1)[e];
                 const double d = ch.diag[row];
-                zd y = zmk(fma(d, yp.x, dg_double(hv[0], lv[0], er + ec - 70)), fma(d, yp.y, dg_double(hv[1], lv[1], er + ec - 70)));
+                zd y = zmk(fma(d, yp.x, dg_double<SH>(hv[0], lv[0], er + ec - E0)), fma(d, yp.y, dg_double<SH>(hv[1], lv[1], er + ec - E0)));
                 if (g.term > 1) {
                     const zd y2 = yb[e];
                     y = zmk(fma(2.0, y.x, -y2.x), fma(2.0, y.y, -y2.y));
@@ -574,7 +593,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                 ch.acc[e] = sm;
                 if (!g.last) {
                     yb[e] = y;
-                    dg_put_col(ch.Bn[g.term & 1], NT, ch.nst, n, row, fix64(y.x, ec, 53), fix64(y.y, ec, 53));
+                    dg_put_col<P>(ch.Bn[g.term & 1], NT, ch.nst, n, row, fix64(y.x, ec, 9 * P - 1), fix64(y.y, ec, 9 * P - 1));
                 }
             }
         }
@@ -651,10 +670,10 @@ __global__ void k_dg_pack_a(const DgSrc* d) {
         const int e = s.er[r];
         const DgScale sc = dg_scale(e >= 2048 ? 0 : e);
         uint32_t dr[DG_P], di[DG_P];
-        dg_cut(e >= 2048 ? 0 : dg_int(v.x, sc), dr);
-        dg_cut(e >= 2048 ? 0 : dg_int(v.y, sc), di);
+        dg_cut<DG_P>(e >= 2048 ? 0 : dg_int(v.x, sc), dr);
+        dg_cut<DG_P>(e >= 2048 ? 0 : dg_int(v.y, sc), di);
         for (int i = 0; i < DG_P; ++i)
-            s.dst[dg_word(r, k, DG_BM, s.nst) + (size_t)i * DG_BM * 16] = dg_pair(dr[i], di[i]);
+            s.dst[dg_word<DG_P>(r, k, DG_BM, s.nst) + (size_t)i * DG_BM * 16] = dg_pair(dr[i], di[i]);
     }
 }
 
@@ -708,7 +727,7 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(DG_PB_T) k_dg_pack_b
     const bool bad = e >= 2048;
     const DgScale sc = dg_scale(bad ? 0 : e);
     auto put = [&](int k, zd w) {
-        dg_put_col(s.dst, s.NT, s.nst, n, k, bad ? 0 : dg_int(w.x, sc), bad ? 0 : dg_int(w.y, sc));
+        dg_put_col<DG_P>(s.dst, s.NT, s.nst, n, k, bad ? 0 : dg_int(w.x, sc), bad ? 0 : dg_int(w.y, sc));
     };
 #pragma unroll
     for (int u = 0; u < DG_PB_E; ++u) {
@@ -747,15 +766,17 @@ struct DgPool {  // device memory of a plan
 static int dg_up(int n, int m) { return (n + m - 1) / m * m; }
 static int dg_nt(int ncol) { return 2 * ncol <= 16 ? 16 : (2 * ncol <= 32 ? 32 : 64); }
 static int dg_nst(int K) { return (2 * K + DG_KS - 1) / DG_KS; }
-static size_t dg_bytes(int rows, int K) { return (size_t)DG_P * rows * dg_nst(K) * 64; }
+static size_t dg_bytes(int rows, int K, int P = DG_P) { return (size_t)P * rows * dg_nst(K) * 64; }
 
-template <int NT>
+// the stages, or a block's integers and its share of a cluster's sum of them
+template <int NT, int MODE>
 static constexpr int dg_smem() {
-    return (NT == 16 ? 4 : 3) * DG_P * (DG_A_PL + NT * 64) + 1024;
+    const int st = dg_stages(NT, MODE) * dg_p(MODE) * (DG_A_PL + NT * 64), ep = 3 * NT * DG_BM * 8;
+    return (st > ep ? st : ep) + 1024;
 }
 template <int MODE, bool GEN>
 static const void* dg_fn(int NT, int* smem) {
-    *smem = NT == 16 ? dg_smem<16>() : (NT == 32 ? dg_smem<32>() : dg_smem<64>());
+    *smem = NT == 16 ? dg_smem<16, MODE>() : (NT == 32 ? dg_smem<32, MODE>() : dg_smem<64, MODE>());
     if constexpr (GEN) return NT == 16 ? (const void*)k_dg<16, MODE, true> : (const void*)k_dg<32, MODE, true>;
     else
         return NT == 16 ? (const void*)k_dg<16, MODE, false>
@@ -983,8 +1004,8 @@ __global__ void __launch_bounds__(256) k_dg_tab_cut(const zd* __restrict__ tab, 
     if (i >= n) return;
     const DgScale sc = dg_scale(e >= 2048 ? 0 : e);
     uint32_t dr[DG_P], di[DG_P], p[DG_P];
-    dg_cut(e >= 2048 ? 0 : dg_int(tab[i].x, sc), dr);
-    dg_cut(e >= 2048 ? 0 : dg_int(tab[i].y, sc), di);
+    dg_cut<DG_P>(e >= 2048 ? 0 : dg_int(tab[i].x, sc), dr);
+    dg_cut<DG_P>(e >= 2048 ? 0 : dg_int(tab[i].y, sc), di);
 #pragma unroll
     for (int q = 0; q < DG_P; ++q) p[q] = dg_pair(dr[q], di[q]);
     t4[i] = make_uint4(p[0], p[1], p[2], p[3]);
@@ -1050,15 +1071,16 @@ int launch_dg_toep(const DgToep* t, int which, int kofs, int nk, cudaStream_t s)
 // The series with H~ y_{n-1} as digit products, one launch per term, for more
 // states or rows than k_cheb_coop takes.  In FP64 its rate was the FP64 pipe's (16
 // k-points of N_aux 300, N_s 60: 9.0 GFLOP in 8.3 ms; 2 k-points 1.91 ms); here the
-// 2 k-points take 0.26 ms, bound by the 14 launches of a few stages each.
+// 2 k-points take 0.28 ms, bound by the 14 launches of a few stages each.
 // H~ = (HH - lam_c) / lam_h is its diagonal, which multiplies y in FP64, and the
 // rest as digits, a power of two above the largest entry for each row; a column of
 // y takes the power of two above theta's 2-norm, which bounds every y_n (H~ has
-// norm <= 1).  The recurrence and the sum are FP64.  So the cut is 2^-54 of what
-// couples an amplitude to the others, and an amplitude that a weak field feeds
-// keeps FP64's relative accuracy (with the diagonal among the digits and y_n in
-// integers it kept 2^-54 of the column's norm: 1e-8 of the excited amplitudes at
-// A = 1e-4).
+// norm <= 1).  The recurrence and the sum are FP64.  Seven digits, 63 bits: the cut
+// is 2^-63 of what couples an amplitude to the others, and an amplitude that a weak
+// field feeds keeps FP64's relative accuracy, also where a state couples to others a
+// hundred times more strongly than to the occupied ones (with the diagonal among the
+// digits and y_n in integers it kept 2^-54 of the column's norm, 1e-8 of the excited
+// amplitudes at A = 1e-4; with six digits 2.5e-15 where FP64 has 0.8e-15).
 struct DgSeriesK {
     uint32_t* A;     // digits of H~ off its diagonal, tiles of 128 rows
     int nst, NT;
@@ -1146,12 +1168,12 @@ __global__ void __launch_bounds__(128) k_dg_hsub(StepArgs a, const DgSeriesK* sk
         S.er[i] = e;
     }
     auto put = [&](int j, zd v) {
-        uint32_t dr[DG_P], di[DG_P];
-        dg_cut(fix64(v.x, e, 53), dr);
-        dg_cut(-fix64(v.y, e, 53), di);
+        uint32_t dr[DG_PS], di[DG_PS];
+        dg_cut<DG_PS>(fix64(v.x, e, 9 * DG_PS - 1), dr);
+        dg_cut<DG_PS>(-fix64(v.y, e, 9 * DG_PS - 1), di);
 #pragma unroll
-        for (int q = 0; q < DG_P; ++q)
-            S.A[dg_word(i, j, DG_BM, S.nst) + (size_t)q * DG_BM * 16] = dg_pair(dr[q], di[q]);
+        for (int q = 0; q < DG_PS; ++q)
+            S.A[dg_word<DG_PS>(i, j, DG_BM, S.nst) + (size_t)q * DG_BM * 16] = dg_pair(dr[q], di[q]);
     };
 #pragma unroll
     for (int u = 0; u < DG_HS_E; ++u) {
@@ -1204,7 +1226,7 @@ __global__ void __launch_bounds__(128) k_dg_y0(StepArgs a, const DgSeriesK* sk, 
         const size_t x = (size_t)c * n + i;
         ch.y0[x] = y;
         ch.acc[x] = zmul(c0, y);
-        dg_put_col(ch.Bn[0], S.NT, ch.nst, c, i, fix64(y.x, e, 53), fix64(y.y, e, 53));
+        dg_put_col<DG_PS>(ch.Bn[0], S.NT, ch.nst, c, i, fix64(y.x, e, 9 * DG_PS - 1), fix64(y.y, e, 9 * DG_PS - 1));
     }
 }
 
@@ -1244,7 +1266,7 @@ DgSeries* dg_series_create(int nk, int n, int ns, const zd* const* coef) {
     std::vector<DgCheb> ch(nk);
     std::vector<DgSeriesK> sk(nk);
     for (int k = 0; k < nk; ++k) {
-        sk[k].A = (uint32_t*)g->pool.get(dg_bytes(g->mt * DG_BM, n), true);
+        sk[k].A = (uint32_t*)g->pool.get(dg_bytes(g->mt * DG_BM, n, DG_PS), true);
         sk[k].nst = nst;
         sk[k].NT = g->NT;
         sk[k].bad = (int*)g->pool.get(n * sizeof(int), true);
@@ -1257,7 +1279,7 @@ DgSeries* dg_series_create(int nk, int n, int ns, const zd* const* coef) {
         c.y1 = (zd*)g->pool.get((size_t)ns * n * sizeof(zd), true);
         c.acc = (zd*)g->pool.get((size_t)ns * n * sizeof(zd), true);
         c.diag = sk[k].diag;
-        for (int q = 0; q < 2; ++q) c.Bn[q] = (uint32_t*)g->pool.get(dg_bytes(np, n), true);
+        for (int q = 0; q < 2; ++q) c.Bn[q] = (uint32_t*)g->pool.get(dg_bytes(np, n, DG_PS), true);
         c.nst = nst;
         c.coef = coef[k];
         out[k] = DgOut{};
