@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
         };
         if (AHEAD && nk > 0) load(0, 0);
         bool ok = true;
-        for (int t = 0; t < nk && ok; ++t) {
+        for (int t = 0; t < nk; ++t) {
             const int s = t % STAGES;
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
@@ -421,13 +421,12 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                     if (b + 1 < NB) load(t, b + 1);
                     else if (t + 1 < nk) load(t + 1, 0);
                 }
-                if (b == 0 && t >= STAGES && !mbar_wait(&empty[s], (uint32_t)((t / STAGES - 1) & 1))) {
-                    abort_flag = 1;
-                    if (lane == 0) atomicOr(g.flag, 8);
-                }
-                if (__any_sync(0xffffffffu, abort_flag)) {  // the warp's lanes leave together
+                // after a wait that ran out no lane waits again, and none leaves the warp: what is
+                // written then is not used
+                if (b == 0 && t >= STAGES && ok && (!mbar_wait(&empty[s], (uint32_t)((t / STAGES - 1) & 1)) || abort_flag)) {
                     ok = false;
-                    break;
+                    abort_flag = 1;
+                    atomicOr(g.flag, 8);
                 }
                 unsigned char* d = smem + s * STAGE + r * 64;
 #pragma unroll
@@ -444,7 +443,6 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
                     *(uint4*)(p + 5 * DG_A_PL) = make_uint4(v[0].y, v[1].y, v[2].y, v[3].y);
                 }
             }
-            if (!ok) break;
             // the planes are read by the products' proxy
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -454,15 +452,14 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
         const int nsl = (nk + 1) >> 1;
         const uint32_t tb = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * CP);
         bool ok = true;
-        for (int sl = 0; sl < nsl && ok; ++sl) {
+        for (int sl = 0; sl < nsl; ++sl) {
 #pragma unroll
             for (int gi = G - 1; gi >= 0; --gi) {
                 if (sl != nsl - 1 && (sl & (dg_run(P, gi) - 1)) != dg_run(P, gi) - 1) continue;
-                // the warp's lanes leave together: the loads below take all of them
-                if (__any_sync(0xffffffffu, !mbar_wait(&gfull[gi], (uint32_t)((sl / dg_run(P, gi)) & 1)) || abort_flag)) {
-                    ok = false;
-                    break;
-                }
+                // after a wait that ran out no lane waits again, and none leaves the warp, whose loads
+                // below take all of them (a vote, or the block's flag, at each read-out took 2 to 6%
+                // of the large products' time)
+                if (ok && !mbar_wait(&gfull[gi], (uint32_t)((sl / dg_run(P, gi)) & 1))) ok = false;
                 tc_fence_after();
                 constexpr int W = CP >= 16 ? 16 : 8;
 #pragma unroll
@@ -487,7 +484,7 @@ __global__ void __launch_bounds__(DG_THREADS + (GEN ? dg_gen(NT) : 0), 1) k_dg(c
         }
         if (!ok) {
             abort_flag = 1;
-            if (lane == 0) atomicOr(g.flag, 8);
+            atomicOr(g.flag, 8);
         }
     }
     __syncthreads();
