@@ -60,7 +60,7 @@ SM_COUNT, SM_MAX_MHZ, FP32_LANES = 152, 2070.0, 128
 # k-points (--k-subset 0,1), 663.4 MB, scaled by sum_k N_G (6.833x): the streams of the
 # interstitial and matching-row products are the matching coefficients and the packed C_G.
 TRAFFIC = {
-    ("tc_interstitial_and_forward", "bf16x3", "mos2_16k", "32b0f03646b7f329"): 4533000000.0,
+    ("tc_interstitial_and_forward", "bf16x3", "mos2_16k", "5e4b4dbf0b3a7687"): 4533000000.0,
 }
 
 # 16-bit products of one FP64 multiply-add in the exact digit products (k_dg.cu):

@@ -38,7 +38,9 @@
 namespace cg = cooperative_groups;
 
 #define DG_P 6              // digits of an operand: 54 bits
-#define DG_PS 7             // in the Chebyshev series: 63 bits
+// in the Chebyshev series, 63 bits: 34 of 49 pairs, s = 5 .. 12, of which s = 9 and above are
+// exact, s = 8 and 7 read out every 64 reals and rounded past 2^24
+#define DG_PS 7
 #define DG_KS 32            // reals per stage: 64 bytes of fp16, one row of the 64-byte swizzle
 #define DG_BM 128           // rows per tile
 // smallest i + j kept with P digits, and the groups kept, s = dg_s0(P) + g, of NT columns of tensor memory each
